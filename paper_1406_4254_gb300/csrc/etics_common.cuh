@@ -90,9 +90,6 @@ struct BasisTables {
     // knorm / (l-m)!: the normalisation of the factorial-scaled harmonics
     // (l-m)! Z_l^m that the coefficient passes evaluate (harm_level_exact)
     double knorm_fact[(kLmaxLimit + 1) * (kLmaxLimit + 2) / 2];
-    // MEX weights 4pi/(2l+1) K_lm^2 = (l-m)!/(l+m)! (times 2 for m > 0)
-    float mexw_f[(kLmaxLimit + 1) * (kLmaxLimit + 2) / 2];
-    double mexw_d[(kLmaxLimit + 1) * (kLmaxLimit + 2) / 2];
     // 1/J_nl, J_nl = -K_nl (n+4l+2)!/n! / (2^(8l+6) (n+2l+3/2) pi prod_{k=0}^{2l}(k+1/2)^2),
     // K_nl = n(n+4l+3)/2 + (l+1)(2l+1)
     double inv_j[kNmaxLimit + 1][kLmaxLimit + 1];
@@ -139,9 +136,6 @@ constexpr BasisTables make_tables() {
             double fact = 1.0;   // (l-m)!
             for (int k = 2; k <= l - m; ++k) fact *= (double)k;
             t.knorm_fact[idx] = t.knorm[idx] / fact;
-            const double w = ratio * (m > 0 ? 2.0 : 1.0);
-            t.mexw_d[idx] = w;
-            t.mexw_f[idx] = (float)w;
         }
     }
     for (int n = 0; n <= kNmaxLimit; ++n) {
@@ -249,9 +243,6 @@ struct RadialSeed {
         }
     }
 };
-template <typename R> __device__ __forceinline__ R mex_w(int idx);
-template <> __device__ __forceinline__ float mex_w<float>(int idx) { return c_tab.mexw_f[idx]; }
-template <> __device__ __forceinline__ double mex_w<double>(int idx) { return c_tab.mexw_d[idx]; }
 
 // ---------------------------------------------------------------------------
 // Unnormalised solid harmonics at a point u (used at the unit vector):

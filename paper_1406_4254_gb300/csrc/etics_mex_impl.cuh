@@ -7,66 +7,139 @@
 // and a_i = -grad Phi_i at fixed q, p.
 //
 // GB300 design (the paper ran one library scan per (l, m) and direction):
-//   pass 1  gathers the particles in radial order (sorted copy), and reduces
+//   pass 1  gathers the particles in radial order (sorted copy) and reduces
 //           each tile's moments m rho^l Y and m rho^-(l+1) Y (rho = r / s_t,
-//           s_t a power of two per tile, so FP32 never overflows) to FP64.
-//           It also scans each thread's sums over its kMexP particles inside
-//           the tile and stores every thread's exclusive prefix (inner) and
-//           suffix (outer).
+//           s_t a power of two per tile, so FP32 never overflows) to one FP64
+//           sum per component.
 //   carry   scans the per-tile FP64 sums in a fixed order: exclusive forward
 //           for the inner moments, exclusive reverse (a true suffix sum) for
 //           the outer ones -- deterministic.
-//   pass 2  adds the tile carry to those per-thread prefixes and suffixes,
-//           evaluates the field at every particle from the exclusive q and p
-//           in a forward and a reverse sweep, and scatters (a, Phi) back to
-//           the caller's order.
-// All harmonics are the unnormalised Cartesian solid harmonics of
-// etics_common.cuh; the MEX weights (l-m)!/(l+m)! (x2 for m > 0) restore the
-// orthonormal normalisation and the 4pi/(2l+1) factor at once.
+//   pass 2  forms the moments of the tile again, scans them in shared memory
+//           from the tile carry (forward and reverse) and evaluates the field
+//           at every particle from its exclusive q and p together; (a, Phi)
+//           is scattered back to the caller's order.
+//
+// A thread owns two neighbouring particles of the sorted list and runs them
+// as the two halves of paired FP32 instructions; it walks the levels one
+// after the other, so that only two levels of harmonics and one level of
+// sums are live, whatever l_max is.  The per-thread moment sums go through
+// shared memory (one row of kMexThreads values per component, padded so that
+// both access patterns, thread = particle pair and thread = component, are
+// free of bank conflicts); one thread per component then runs down its row.
+// Nothing per particle but the sorted copy reaches memory between the passes.
+// What bounds them: instruction issue (pass 2), the gather's latency (pass 1).
+// Measured against the form it replaced (seven particles per thread, all 98
+// sums of l_max = 6 in registers, every thread's prefix sums through memory):
+// N = 2^20, l_max = 6: pass 1 51 -> 37 us, pass 2 61 -> 52 us; N = 500009,
+// l_max = 10 (the whole call): 291 -> 167 us; N = 100003, l_max = 6, FP64:
+// 450 -> 341 us (256-particle tiles also fill the SMs more evenly).
+//
+// Harmonics: R_lm(kappa u) = kappa^l Z_lm(u) / (l+m)! at the unit vector u,
+// with Z the unnormalised solid harmonics of etics_common.cuh and kappa = 8
+// (a power of two: the values stay near 1 up to l = 10 where Z alone or
+// Z / (l+m)! would spread over 2^60).  In this scaling the gradient ladder has
+// no constants:
+//   d/dz R_l^m = R_{l-1}^m,  (d/dx -+ i d/dy) R_l^m = +-R_{l-1}^{m-+1},
+// and the product of an evaluated and a summed harmonic needs the weight
+// (l-m)!(l+m)! kappa^-2l (twice that for m > 0: the twos are applied to the
+// sums over m > 0 as a whole).
 #pragma once
+
+#include <atomic>
 
 #include "etics_internal.h"
 
 namespace etics {
 
 constexpr int kMexThreads = 128;
-// particles per thread (consecutive).  7 rather than 8: at N = 2^20 the 1171
-// tiles of 896 particles fill 1.93 waves of the 608 resident blocks instead
-// of 1.68 (1024 tiles), measured pass 1 57.3 -> 53.3 us, pass 2 67.5 -> 61.5 us
-constexpr int kMexP = 7;
-constexpr int kMexTile = kMexThreads * kMexP;     // 896
+constexpr int kMexTile = 2 * kMexThreads;         // particles per tile, two per thread
 constexpr int kMexLB = kMexLmaxLimit;             // compiled level bound (10)
 constexpr int kMexNC = 49;                        // components of one level group, at most
+constexpr int kMexRow = kMexThreads + 4;          // row stride of the shared rows (conflict-free
+                                                  // for 16-byte reads down a row)
+constexpr int kMexKappa = 8;
 
-// Level groups: the per-thread moment arrays hold the components of one group
-// of levels, so that l_max up to kMexLB needs no more registers than l_max = 6.
-// A group's harmonics are recurred from level 0 (cheap next to the sums).
+// Level groups: the shared rows hold the components of one group of levels,
+// so that l_max up to kMexLB leaves room for several blocks per SM.  A group's
+// harmonics are recurred from level 0 (cheap next to the sums).
 constexpr int kMexGroups = 3;
 __host__ __device__ constexpr int mex_group_l0(int g) { return g == 0 ? 0 : (g == 1 ? 7 : 9); }
 __host__ __device__ constexpr int mex_group_l1(int g) { return g == 0 ? 6 : (g == 1 ? 8 : 10); }
 __host__ __device__ constexpr int mex_ncomp(int l_max) { return (l_max + 1) * (l_max + 1); }
-// components per side in the buffers: the l_max <= 6 kernels always use the
-// full 49 (zeros above l_max), so that their strides and loops are constants
+// components per side in the buffers: one layout for all l_max <= 6
 __host__ __device__ constexpr int mex_layout_ncomp(int l_max) {
     return l_max <= 6 ? kMexNC : mex_ncomp(l_max);
 }
 static_assert(mex_group_l1(kMexGroups - 1) == kMexLB, "groups cover the compiled levels");
 static_assert(mex_ncomp(6) <= kMexNC && mex_ncomp(8) - mex_ncomp(6) <= kMexNC &&
               mex_ncomp(10) - mex_ncomp(8) <= kMexNC, "group size");
+static_assert(2 * kMexNC <= kMexThreads, "one thread per component and side");
 inline int mex_ngroups(int l_max) {
     int g = 1;
     while (g < kMexGroups && mex_group_l0(g) <= l_max) ++g;
     return g;
 }
+// components per side of the largest group present
+inline int mex_row_comps(int l_max) {
+    int most = 0;
+    for (int g = 0; g < mex_ngroups(l_max); ++g) {
+        const int l1 = mex_group_l1(g) < l_max ? mex_group_l1(g) : l_max;
+        const int n = mex_ncomp(l1) - mex_group_l0(g) * mex_group_l0(g);
+        if (n > most) most = n;
+    }
+    return most;
+}
 
 inline int mex_tiles(int64_t N) { return (int)((N + kMexTile - 1) / kMexTile); }
 
-// shared-memory slot of tile particle i (thread i / kMexP owns particles
-// i..i+kMexP-1): stored particle-major so that a warp reading its threads'
-// k-th particles touches consecutive 16-byte words (no bank conflicts)
-__host__ __device__ constexpr int mex_slot(int i) {
-    return (i % kMexP) * kMexThreads + i / kMexP;
+// ---- pairs ------------------------------------------------------------------
+// two particles of one thread: paired FP32 instructions, or two FP64 ones
+template <typename R> struct PairT;
+template <> struct PairT<float> { using type = float2; };
+template <> struct PairT<double> { using type = double2; };
+template <typename R> using Pair = typename PairT<R>::type;
+__device__ __forceinline__ float2 mk2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ double2 mk2(double a, double b) { return make_double2(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double2 mul2(double2 a, double2 b) {
+    return make_double2(a.x * b.x, a.y * b.y);
 }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
+    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+__device__ __forceinline__ double2 add2(double2 a, double2 b) {
+    return make_double2(a.x + b.x, a.y + b.y);
+}
+// a constant in both halves: an immediate or broadcast operand, no extra
+// instruction (nor is the negation of an operand)
+template <typename R> __device__ __forceinline__ Pair<R> splat(R a) { return mk2(a, a); }
+template <typename P> __device__ __forceinline__ P neg2(P a) { return mk2(-a.x, -a.y); }
+template <typename P> __device__ __forceinline__ P sub2(P a, P b) { return add2(a, neg2(b)); }
+
+// (l-m)!(l+m)! kappa^-2l, the weight of component (l, m)
+struct MexWeights {
+    double w[(kMexLB + 1) * (kMexLB + 2) / 2];
+    float wf[(kMexLB + 1) * (kMexLB + 2) / 2];
+};
+constexpr MexWeights make_mex_weights() {
+    MexWeights t{};
+    for (int l = 0; l <= kMexLB; ++l)
+        for (int m = 0; m <= l; ++m) {
+            double v = 1.0;
+            for (int k = 2; k <= l - m; ++k) v *= (double)k;
+            for (int k = 2; k <= l + m; ++k) v *= (double)k;
+            for (int k = 0; k < l; ++k) v /= (double)(kMexKappa * kMexKappa);
+            t.w[l * (l + 1) / 2 + m] = v;
+            t.wf[l * (l + 1) / 2 + m] = (float)v;
+        }
+    return t;
+}
+static __constant__ MexWeights c_mex_w = make_mex_weights();
+template <typename R> __device__ __forceinline__ R mex_w(int idx);
+template <> __device__ __forceinline__ float mex_w<float>(int idx) { return c_mex_w.wf[idx]; }
+template <> __device__ __forceinline__ double mex_w<double>(int idx) { return c_mex_w.w[idx]; }
 
 // tile scale exponent: s_t = 2^e with e halfway (in log2) between the first
 // and last radius of the tile (first radius 0 -> use the last)
@@ -84,311 +157,316 @@ __device__ __forceinline__ R radius(R x, R y, R z) {
     return sqrt(x * x + y * y + z * z);
 }
 
+// x 2^k, exact unless the result leaves the normal range: the exponent field
+// is edited in place (FP64 instructions are slow on this GPU)
+__device__ __forceinline__ double scale_pow2(double x, int k) {
+    const int hi = __double2hiint(x);
+    const int ef = (hi >> 20) & 0x7ff;
+    if (ef != 0 && ef + k > 0 && ef + k < 0x7ff)
+        return __hiloint2double(hi + (k << 20), __double2loint(x));
+    return ldexp(x, k);
+}
+
+// the tile's two particles of a thread, in tile units: v = kappa u, rho = r / s
 template <typename R>
-struct MexParticle {
-    R ux, uy, uz, uu, rho, m;
-    bool origin;
-    __device__ __forceinline__ void init(const Vec4<R>& v, R scale) {
-        const R r = radius<R>(v.x, v.y, v.z);
-        origin = !(r > R(0));
-        const R inv = origin ? R(0) : R(1) / r;
-        ux = v.x * inv; uy = v.y * inv; uz = v.z * inv;
-        uu = ux * ux + uy * uy + uz * uz;
-        rho = r * scale;
-        m = v.w;
+struct MexPair {
+    Pair<R> x, y, z, rho, irho, m;
+    __device__ __forceinline__ void init(const Vec4<R>& a, const Vec4<R>& b, R scale, R iscale) {
+        const R ra = radius<R>(a.x, a.y, a.z), rb = radius<R>(b.x, b.y, b.z);
+        // a particle at the origin: no direction, no outer moment, rho = 0
+        const R ia = ra > R(0) ? R(1) / ra : R(0), ib = rb > R(0) ? R(1) / rb : R(0);
+        const R ka = R(kMexKappa) * ia, kb = R(kMexKappa) * ib;
+        x = mk2(a.x * ka, b.x * kb);
+        y = mk2(a.y * ka, b.y * kb);
+        z = mk2(a.z * ka, b.z * kb);
+        rho = mk2(ra * scale, rb * scale);
+        irho = mk2(ia * iscale, ib * iscale);
+        m = mk2(a.w, b.w);
     }
 };
 
-// moment of column c of level L: index L*L + c
-template <typename R, int L>
-__device__ __forceinline__ R harm_col(const R* C, const R* S, int c) {
-    return c == 0 ? C[0] : ((c & 1) ? C[(c + 1) / 2] : S[c / 2]);
+// The two walks over the levels (moments, field) and the walks of later level
+// groups evaluate the same harmonics; without this the compiler keeps the
+// first walk's values for the second, far more than the registers hold
+// (l_max > 6: 2 KB of spills per thread).
+__device__ __forceinline__ void opaque(float& v) { asm volatile("" : "+f"(v)); }
+__device__ __forceinline__ void opaque(double& v) { asm volatile("" : "+d"(v)); }
+template <typename R> __device__ __forceinline__ void opaque_pair(MexPair<R>& p) {
+    opaque(p.x.x); opaque(p.x.y);
+    opaque(p.y.x); opaque(p.y.y);
+    opaque(p.z.x); opaque(p.z.y);
+    opaque(p.rho.x); opaque(p.rho.y);
+    opaque(p.irho.x); opaque(p.irho.y);
 }
 
-// ---- moments of one particle added to (ain, aout): levels L0..L1 of the
-// group (component L*L + c at index L*L + c - L0*L0), levels below L0 only
-// recurred
+// level L of R_lm(kappa u) from levels L-1 and L-2 (|kappa u|^2 = kappa^2)
+template <typename R, int L>
+__device__ __forceinline__ void mex_harm(const Pair<R>* C1, const Pair<R>* S1, const Pair<R>* C2,
+                                         const Pair<R>* S2, const MexPair<R>& p, Pair<R>* C,
+                                         Pair<R>* S) {
+    using P = Pair<R>;
+    if constexpr (L == 0) {
+        C[0] = splat(R(1));
+        S[0] = splat(R(0));
+    } else if constexpr (L == 1) {
+        C[0] = p.z;
+        S[0] = splat(R(0));
+        C[1] = mul2(p.x, splat(R(0.5)));
+        S[1] = mul2(p.y, splat(R(0.5)));
+    } else {
+        // kappa^2 = |kappa u|^2 taken out of the recursion:
+        //   (L^2 - m^2) R_L = kappa^2 [ (2L-1)/kappa^2 v_z R_{L-1} - R_{L-2} ]
+        constexpr R d = R(1.0 / (2 * L)), k2 = R(kMexKappa * kMexKappa);
+        const P xd = mul2(p.x, splat(d)), yd = mul2(p.y, splat(d));
+        C[L] = fma2(xd, C1[L - 1], neg2(mul2(yd, S1[L - 1])));
+        S[L] = fma2(xd, S1[L - 1], mul2(yd, C1[L - 1]));
+        C[L - 1] = mul2(p.z, C1[L - 1]);
+        S[L - 1] = mul2(p.z, S1[L - 1]);
+        S[0] = splat(R(0));
+        const P zl = mul2(p.z, splat(R(2 * L - 1) / k2));
+#pragma unroll
+        for (int m = 0; m + 2 <= L; ++m) {
+            const P f = splat(k2 / R(L * L - m * m));
+            C[m] = mul2(fma2(zl, C1[m], neg2(C2[m])), f);
+            if (m > 0) S[m] = mul2(fma2(zl, S1[m], neg2(S2[m])), f);
+        }
+    }
+}
+
+// moments of the pair summed, component c = l*l + 2m-1 (cos) / 2m (sin) of
+// levels L0..L1 into this thread's column of the rows (inner components first,
+// outer ones nc rows further)
 template <typename R, int L0, int L1, int L>
-__device__ __forceinline__ void mex_moments(R (&C)[3][L1 + 1], R (&S)[3][L1 + 1],
-                                            const MexParticle<R>& pt, int l_max, R win, R wout,
-                                            R irho, R (&ain)[kMexNC], R (&aout)[kMexNC]) {
+__device__ __forceinline__ void mex_moments(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3][L1 + 1],
+                                            const MexPair<R>& p, int l_max, Pair<R> win,
+                                            Pair<R> wout, R* col, int nc) {
     if constexpr (L <= L1) {
         if (L > l_max) return;
         constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
-        harm_level<R, L>(C[s1], S[s1], C[s2], S[s2], pt.ux, pt.uy, pt.uz, pt.uu, C[s0], S[s0]);
+        mex_harm<R, L>(C[s1], S[s1], C[s2], S[s2], p, C[s0], S[s0]);
         if constexpr (L >= L0) {
             constexpr int o = L * L - L0 * L0;
 #pragma unroll
             for (int c = 0; c <= 2 * L; ++c) {
-                const R y = harm_col<R, L>(C[s0], S[s0], c);
-                ain[o + c] = fma(win, y, ain[o + c]);
-                aout[o + c] = fma(wout, y, aout[o + c]);
+                const Pair<R> h = c == 0 ? C[s0][0] : ((c & 1) ? C[s0][(c + 1) / 2] : S[s0][c / 2]);
+                col[(o + c) * kMexRow] = fma(win.y, h.y, win.x * h.x);
+                col[(nc + o + c) * kMexRow] = fma(wout.y, h.y, wout.x * h.x);
             }
         }
-        mex_moments<R, L0, L1, L + 1>(C, S, pt, l_max, win * pt.rho, wout * irho, irho, ain,
-                                      aout);
+        mex_moments<R, L0, L1, L + 1>(C, S, p, l_max, mul2(win, p.rho), mul2(wout, p.irho), col,
+                                      nc);
     }
 }
 
-template <typename R, int L0, int L1>
-__device__ __forceinline__ void particle_moments(const MexParticle<R>& pt, int l_max,
-                                                 R (&ain)[kMexNC], R (&aout)[kMexNC]) {
-    R C[3][L1 + 1], S[3][L1 + 1];
-    const R irho = pt.origin ? R(0) : R(1) / pt.rho;
-    // a particle at the origin has no outer moment (nothing lies inside it)
-    mex_moments<R, L0, L1, 0>(C, S, pt, l_max, pt.m, pt.origin ? R(0) : pt.m * irho, irho, ain,
-                              aout);
+template <typename R, int G>
+__device__ __forceinline__ void mex_group_moments(const MexPair<R>& p, int l_max, R* col, int nc) {
+    constexpr int L0 = mex_group_l0(G), L1 = mex_group_l1(G);
+    Pair<R> C[3][L1 + 1], S[3][L1 + 1];
+    mex_moments<R, L0, L1, 0>(C, S, p, l_max, p.m, mul2(p.m, p.irho), col, nc);
 }
 
-// ---- forward sweep, one particle: inner (q) part of the field, then q += own
-// inner moment.  On entry q is the inner sum over the particles before this
-// one (exclusive).  In tile units (rho = r / s):
-//   Phi_q = -(1/s) sum_l rho^-(l+1) sum_m w_lm q Y
-//   a_q   = (1/s^2) sum_l rho^-(l+2) sum_m w_lm q [G - (2l+1) Y u]
-// with Y, G the unnormalised harmonic and its gradient at the unit vector u.
+// field of the pair, in tile units (rho = r / s), of levels L0..L1 from the
+// weighted exclusive sums in this thread's column.  With s_lm = q rho^-(l+2)
+// + p rho^(l-1) (both already weighted), l >= 1:
+//   Phi = -(1/s) [ rho sum s R + q_00 / rho + p_00 ]
+//   a   = (1/s^2) [ kappa sum s grad R - u (sum (2l+1) q rho^-(l+2) R + q_00 / rho^2) ]
+// so one gradient contraction serves both parts.  The column holds the sums
+// over the particles before (after) the pair; the second particle's q also
+// holds the first, the first one's p the second (own: the first particle's
+// m rho^l and the second one's m rho^-(l+1); ownf: their factors per level).
+template <typename R>
+struct MexField {
+    using P = Pair<R>;
+    P s0, s1;             // sum s R: m = 0, m > 0 (the latter counts twice)
+    P rad;                // sum (2l+1) q rho^-(l+2) R
+    P vx, vy, vz0, vz1;   // sum s grad R (vz1: k > 0, counts twice)
+    P pot0;               // level 0
+};
+
 template <typename R, int L0, int L1, int L, bool ACC>
-__device__ __forceinline__ void mex_fwd(R (&C)[3][L1 + 1], R (&S)[3][L1 + 1],
-                                        const MexParticle<R>& pt, int l_max, R win, R rinv,
-                                        R irho, R (&q)[kMexNC], R& pot, R& ax, R& ay, R& az) {
+__device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3][L1 + 1],
+                                         const MexPair<R>& p, int l_max, Pair<R> a, Pair<R> b,
+                                         Pair<R> own, Pair<R> ownf, const R* col, int nc,
+                                         MexField<R>& f) {
+    using P = Pair<R>;
     if constexpr (L <= L1) {
         if (L > l_max) return;
         constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
-        harm_level<R, L>(C[s1], S[s1], C[s2], S[s2], pt.ux, pt.uy, pt.uz, pt.uu, C[s0], S[s0]);
+        mex_harm<R, L>(C[s1], S[s1], C[s2], S[s2], p, C[s0], S[s0]);
         if constexpr (L >= L0) {
             constexpr int o = L * L - L0 * L0;
-            if (!pt.origin) {
-                R P = R(0), vx = R(0), vy = R(0), vz = R(0);
-                R qc[L + 1], qs[L + 1];
+            if constexpr (L == 0) {
+                const R q = col[0], pp = col[nc * kMexRow];
+                const P q2 = mk2(q, q + own.x), p2 = mk2(pp + own.y, pp);
+                f.pot0 = fma2(q2, p.irho, p2);
+                if (ACC) f.rad = mul2(q2, a);
+            } else {
+                P ac[L + 1], as[L + 1];
+                P r0 = splat(R(0)), r1 = splat(R(0));
 #pragma unroll
-                for (int mm = 0; mm <= L; ++mm) {
-                    const R w = mex_w<R>(L * (L + 1) / 2 + mm);
-                    const int cc = o + (mm == 0 ? 0 : 2 * mm - 1);
-                    qc[mm] = w * q[cc];
-                    P = fma(qc[mm], C[s0][mm], P);
-                    qs[mm] = R(0);
-                    if (mm > 0) {
-                        qs[mm] = w * q[cc + 1];
-                        P = fma(qs[mm], S[s0][mm], P);
+                for (int m = 0; m <= L; ++m) {
+                    const R w = mex_w<R>(L * (L + 1) / 2 + m);
+                    const P wm = mul2(own, splat(w));
+                    {
+                        const int cc = o + (m == 0 ? 0 : 2 * m - 1);
+                        const R q = col[cc * kMexRow], pp = col[(nc + cc) * kMexRow];
+                        const P h = C[s0][m];
+                        const P qa = mul2(mk2(q, fma(wm.x, h.x, q)), a);
+                        ac[m] = fma2(mk2(fma(wm.y, h.y, pp), pp), b, qa);
+                        if (m == 0) f.s0 = fma2(ac[m], h, f.s0);
+                        else f.s1 = fma2(ac[m], h, f.s1);
+                        if (ACC) {
+                            if (m == 0) r0 = mul2(qa, h);
+                            else r1 = fma2(qa, h, r1);
+                        }
+                    }
+                    as[m] = splat(R(0));
+                    if (m > 0) {
+                        const int cc = o + 2 * m;
+                        const R q = col[cc * kMexRow], pp = col[(nc + cc) * kMexRow];
+                        const P h = S[s0][m];
+                        const P qa = mul2(mk2(q, fma(wm.x, h.x, q)), a);
+                        as[m] = fma2(mk2(fma(wm.y, h.y, pp), pp), b, qa);
+                        f.s1 = fma2(as[m], h, f.s1);
+                        if (ACC) r1 = fma2(qa, h, r1);
                     }
                 }
-                if (ACC && L >= 1) grad_contract<R, L>(C[s1], S[s1], qc, qs, vx, vy, vz);
-                pot = fma(rinv, P, pot);
                 if (ACC) {
-                    const R f = rinv * irho;
-                    const R k = R(2 * L + 1) * P;
-                    ax = fma(f, vx - k * pt.ux, ax);
-                    ay = fma(f, vy - k * pt.uy, ay);
-                    az = fma(f, vz - k * pt.uz, az);
+                    f.rad = fma2(splat(R(2 * L + 1)), r0, f.rad);
+                    f.rad = fma2(splat(R(2 * (2 * L + 1))), r1, f.rad);
+                    // gradient from the level below (the ladder regrouped by the
+                    // harmonic it multiplies)
+                    const P* C1 = C[s1];
+                    const P* S1 = S[s1];
+#pragma unroll
+                    for (int k = 0; k <= L - 1; ++k) {
+                        const P xc = k >= 1 ? sub2(ac[k + 1], ac[k - 1]) : ac[k + 1];
+                        const P yc = k >= 2 ? add2(as[k + 1], as[k - 1]) : as[k + 1];
+                        f.vx = fma2(xc, C1[k], f.vx);
+                        f.vy = fma2(yc, C1[k], f.vy);
+                        if (k == 0) f.vz0 = fma2(ac[k], C1[k], f.vz0);
+                        if (k >= 1) {
+                            const P xs = k >= 2 ? sub2(as[k + 1], as[k - 1]) : as[k + 1];
+                            const P ys = add2(ac[k + 1], ac[k - 1]);
+                            f.vz1 = fma2(ac[k], C1[k], f.vz1);
+                            f.vx = fma2(xs, S1[k], f.vx);
+                            f.vy = fma2(neg2(ys), S1[k], f.vy);
+                            f.vz1 = fma2(as[k], S1[k], f.vz1);
+                        }
+                    }
                 }
             }
-#pragma unroll
-            for (int c = 0; c <= 2 * L; ++c)
-                q[o + c] = fma(win, harm_col<R, L>(C[s0], S[s0], c), q[o + c]);
         }
-        mex_fwd<R, L0, L1, L + 1, ACC>(C, S, pt, l_max, win * pt.rho, rinv * irho, irho, q, pot,
-                                       ax, ay, az);
+        // a_l = rho^-(l+2); b_l = rho^(l-1), b_1 = 1
+        const P bn = L == 0 ? b : mul2(b, p.rho);
+        mex_eval<R, L0, L1, L + 1, ACC>(C, S, p, l_max, mul2(a, p.irho), bn, mul2(own, ownf), ownf,
+                                        col, nc, f);
     }
 }
 
-// ---- reverse sweep, one particle: outer (p) part of the field, then p += own
-// outer moment.  On entry p is the outer sum over the particles after this one:
-//   Phi_p = -(1/s) sum_l rho^l sum_m w_lm p Y,   a_p = (1/s^2) sum_l rho^(l-1) sum_m w_lm p G
-template <typename R, int L0, int L1, int L, bool ACC>
-__device__ __forceinline__ void mex_rev(R (&C)[3][L1 + 1], R (&S)[3][L1 + 1],
-                                        const MexParticle<R>& pt, int l_max, R wout, R rl,
-                                        R rlm1, R irho, R (&p)[kMexNC], R& pot, R& ax, R& ay,
-                                        R& az) {
-    if constexpr (L <= L1) {
-        if (L > l_max) return;
-        constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
-        harm_level<R, L>(C[s1], S[s1], C[s2], S[s2], pt.ux, pt.uy, pt.uz, pt.uu, C[s0], S[s0]);
-        if constexpr (L >= L0) {
-            constexpr int o = L * L - L0 * L0;
-            R P = R(0), vx = R(0), vy = R(0), vz = R(0);
-            R pc[L + 1], ps[L + 1];
-#pragma unroll
-            for (int mm = 0; mm <= L; ++mm) {
-                const R w = mex_w<R>(L * (L + 1) / 2 + mm);
-                const int cc = o + (mm == 0 ? 0 : 2 * mm - 1);
-                pc[mm] = w * p[cc];
-                P = fma(pc[mm], C[s0][mm], P);
-                ps[mm] = R(0);
-                if (mm > 0) {
-                    ps[mm] = w * p[cc + 1];
-                    P = fma(ps[mm], S[s0][mm], P);
-                }
-            }
-            if (ACC && L >= 1) grad_contract<R, L>(C[s1], S[s1], pc, ps, vx, vy, vz);
-            pot = fma(rl, P, pot);
-            if (ACC && L >= 1) {
-                ax = fma(rlm1, vx, ax);
-                ay = fma(rlm1, vy, ay);
-                az = fma(rlm1, vz, az);
-            }
-#pragma unroll
-            for (int c = 0; c <= 2 * L; ++c)
-                p[o + c] = fma(wout, harm_col<R, L>(C[s0], S[s0], c), p[o + c]);
-        }
-        mex_rev<R, L0, L1, L + 1, ACC>(C, S, pt, l_max, wout * irho, rl * pt.rho, rl, irho, p,
-                                       pot, ax, ay, az);
-    }
+template <typename R, int G, bool ACC>
+__device__ __forceinline__ void mex_group_eval(const MexPair<R>& p, int l_max, const R* col, int nc,
+                                               MexField<R>& f) {
+    constexpr int L0 = mex_group_l0(G), L1 = mex_group_l1(G);
+    Pair<R> C[3][L1 + 1], S[3][L1 + 1];
+    mex_eval<R, L0, L1, 0, ACC>(C, S, p, l_max, mul2(p.irho, p.irho), splat(R(1)),
+                                mk2(p.m.x, p.m.y * p.irho.y), mk2(p.rho.x, p.irho.y), col, nc, f);
 }
 
-// Exclusive scan over the 32 lanes of a warp of each of the kMexNC components
-// in v (forward: prefix in lane order; backward: suffix), in two rounds of at
-// most kMexScanHalf components.  buf: the warp's 32 x kMexScanHalf slots (row
-// = lane; the odd row length keeps both access patterns free of bank
-// conflicts).  total[c] receives the warp's sum of component c.
-constexpr int kMexScanHalf = (kMexNC + 1) / 2;
-static_assert(kMexScanHalf % 2 == 1, "row length must be odd");
-template <typename R, bool kForward, int C0, int NC>
-__device__ __forceinline__ void scan_rows_part(R (&v)[kMexNC], R* buf, R* total, int lane) {
-#pragma unroll
-    for (int j = 0; j < NC; ++j) buf[lane * kMexScanHalf + j] = v[C0 + j];
-    __syncwarp();
-    if (lane < NC) {
-        R run = R(0);
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            const int r = kForward ? t : 31 - t;
-            const R x = buf[r * kMexScanHalf + lane];
-            buf[r * kMexScanHalf + lane] = run;
-            run += x;
-        }
-        total[C0 + lane] = run;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < NC; ++j) v[C0 + j] = buf[lane * kMexScanHalf + j];
-    __syncwarp();
+// level of component c
+__device__ __forceinline__ int comp_level(int c) {
+    int l = 0;
+    while ((l + 1) * (l + 1) <= c) ++l;
+    return l;
 }
-template <typename R, bool kForward>
-__device__ __forceinline__ void scan_rows(R (&v)[kMexNC], R* buf, R* total, int lane) {
-    scan_rows_part<R, kForward, 0, kMexScanHalf>(v, buf, total, lane);
-    scan_rows_part<R, kForward, kMexScanHalf, kMexNC - kMexScanHalf>(v, buf, total, lane);
+
+// tile frame shared by both passes: this thread's two particles and the
+// tile's scale exponent
+template <typename R>
+__device__ __forceinline__ int mex_tile_exponent(const Vec4<R>& a, const Vec4<R>& b, int nt, R* s_end) {
+    const int tid = threadIdx.x;
+    if (tid == 0) s_end[0] = radius<R>(a.x, a.y, a.z);
+    if (2 * tid == nt - 1) s_end[1] = radius<R>(a.x, a.y, a.z);
+    if (2 * tid + 1 == nt - 1) s_end[1] = radius<R>(b.x, b.y, b.z);
+    __syncthreads();
+    return tile_exponent<R>(s_end[0], s_end[1]);
 }
+
+// resident blocks per SM the registers are sized for
+// (FP32 pass 2: 118 registers for l_max <= 6, 158 with the later level groups)
+template <typename R>
+constexpr int mex_pass1_blocks() { return sizeof(R) == 4 ? 4 : 2; }
+template <typename R, int NG>
+constexpr int mex_pass2_blocks() { return sizeof(R) == 4 ? (NG == 1 ? 4 : 3) : 2; }
 
 // ---------------------------------------------------------------------------
 // pass 1: gather into radial order + per-tile FP64 moment sums
 // ---------------------------------------------------------------------------
-// resident blocks per SM the kernels' registers are sized for: FP32 with one
-// level group 4 (16 warps hide the gather latency); the multi-group kernels
-// and FP64 need more registers (FP64 pass 2 at 4 blocks spilled ~1 KB)
 template <typename R, int NG>
-constexpr int mex_pass1_blocks() { return sizeof(R) == 4 ? (NG == 1 ? 4 : 3) : 1; }
-template <typename R, int NG>
-constexpr int mex_pass2_blocks() { return sizeof(R) == 4 ? (NG == 1 ? 4 : 2) : (NG == 1 ? 2 : 1); }
-
-template <typename R, int NG>
-__global__ void __launch_bounds__(kMexThreads, mex_pass1_blocks<R, NG>())
+__global__ void __launch_bounds__(kMexThreads, mex_pass1_blocks<R>())
 mex_pass1_kernel(const Vec4<R>* __restrict__ posm, const uint32_t* __restrict__ perm, int64_t N,
-                 int l_max, Vec4<R>* __restrict__ sorted, double* __restrict__ tile_agg,
-                 R* __restrict__ thread_sums, unsigned* err) {
-    __shared__ Vec4<R> s_pt[kMexTile];
-    __shared__ R s_red[kMexThreads / 32][2 * kMexNC];
+                 int l_max, Vec4<R>* __restrict__ sorted, double* __restrict__ tile_agg, int stride,
+                 unsigned* err) {
+    extern __shared__ __align__(16) unsigned char mex_smem[];
+    R* rows = reinterpret_cast<R*>(mex_smem);
+    __shared__ R s_end[2];
     pdl_wait();
     const int tid = threadIdx.x;
     const int64_t base = (int64_t)blockIdx.x * kMexTile;
     const int64_t rem = N - base;
     const int nt = (int)(rem < kMexTile ? rem : kMexTile);
-    // gather in radial order: coalesced index loads, independent particle loads
-    uint32_t idx[kMexP];
+    uint32_t idx[2];
+    Vec4<R> v[2];
 #pragma unroll
-    for (int j = 0; j < kMexP; ++j) {
-        const int i = tid + j * kMexThreads;
-        idx[j] = i < nt ? perm[base + i] : 0u;
+    for (int j = 0; j < 2; ++j) idx[j] = 2 * tid + j < nt ? perm[base + 2 * tid + j] : 0u;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        v[j] = mk4<R>(R(0), R(0), R(0), R(0));
+        // an index >= N can only come from a sort whose lookback timed
+        // out (already reported): it gathers a massless particle at 0
+        if (2 * tid + j < nt && (int64_t)idx[j] < N) v[j] = ld4(posm + idx[j]);
     }
 #pragma unroll
-    for (int j = 0; j < kMexP; ++j) {
-        const int i = tid + j * kMexThreads;
-        Vec4<R> v = mk4<R>(R(0), R(0), R(0), R(0));
-        if (i < nt) {
-            // an index >= N can only come from a sort whose lookback timed
-            // out (already reported): it gathers a massless particle at 0
-            if ((int64_t)idx[j] < N) {
-                v = ld4(posm + idx[j]);
-                if (!finite4(v.x, v.y, v.z, v.w)) {
-                    report(err, ETICS_ERR_NONFINITE);
-                    v = mk4<R>(R(0), R(0), R(0), R(0));
-                }
-            }
-            st4(sorted + base + i, v);
+    for (int j = 0; j < 2; ++j) {
+        if (!finite4(v[j].x, v[j].y, v[j].z, v[j].w)) {
+            report(err, ETICS_ERR_NONFINITE);
+            v[j] = mk4<R>(R(0), R(0), R(0), R(0));
         }
-        st4(&s_pt[mex_slot(i)], v);
+        if (2 * tid + j < nt) st4(sorted + base + 2 * tid + j, v[j]);
     }
-    __syncthreads();
-    int e;
-    {
-        const Vec4<R> a = s_pt[mex_slot(0)], b = s_pt[mex_slot(nt - 1)];
-        e = tile_exponent<R>(radius<R>(a.x, a.y, a.z), radius<R>(b.x, b.y, b.z));
-    }
-    const R scale = ldexp(R(1), -e);
-    const int lane = tid & 31, warp = tid >> 5;
-    // One level group per iteration: this thread's moment sums over its kMexP
-    // particles; their exclusive prefix (inner) and suffix (outer) over the
-    // tile, by a transposed scan through shared memory (every thread writes
-    // its row of sums, each lane scans one component serially down the 32
-    // rows in lane order, every thread reads its row back; the rows live
-    // where the particles were); every thread's prefix and suffix stored, the
-    // tile's FP64 sums (tile scale undone) stored.  l_max <= 6 is the single
-    // group with constant sizes.
-    const int ncomp = NG == 1 ? kMexNC : mex_layout_ncomp(l_max);
+    const int e = mex_tile_exponent<R>(v[0], v[1], nt, s_end);
+    MexPair<R> p;
+    p.init(v[0], v[1], ldexp(R(1), -e), ldexp(R(1), e));
+    const int ncomp = mex_layout_ncomp(l_max);
     for (int g = 0; g < NG; ++g) {
         const int L0 = mex_group_l0(g), L1 = mex_group_l1(g);
         if (L0 > l_max) break;
-        if (g > 0) {
-            // the previous group's scan rows overwrote the particles
-            __syncthreads();
-            for (int i = tid; i < kMexTile; i += kMexThreads)
-                st4(&s_pt[mex_slot(i)],
-                    i < nt ? ld4(sorted + base + i) : mk4<R>(R(0), R(0), R(0), R(0)));
-            __syncthreads();
-        }
         const int c0 = L0 * L0;
-        const int gn = NG == 1 ? kMexNC : mex_ncomp(L1 < l_max ? L1 : l_max) - c0;
-        R ain[kMexNC], aout[kMexNC];
-#pragma unroll
-        for (int c = 0; c < kMexNC; ++c) { ain[c] = R(0); aout[c] = R(0); }
-#pragma unroll 1
-        for (int k = 0; k < kMexP; ++k) {
-            MexParticle<R> pt;
-            pt.init(s_pt[k * kMexThreads + tid], scale);
-            if (NG == 1 || g == 0) particle_moments<R, 0, 6>(pt, l_max, ain, aout);
-            else if (g == 1) particle_moments<R, 7, 8>(pt, l_max, ain, aout);
-            else particle_moments<R, 9, 10>(pt, l_max, ain, aout);
-        }
-        static_assert(kMexThreads / 32 * 32 * kMexScanHalf * sizeof(R) <= sizeof(s_pt), "rows");
+        const int nc = mex_ncomp(L1 < l_max ? L1 : l_max) - c0;
+        if (g > 0) __syncthreads();   // the previous group's rows have been read
+        opaque_pair(p);
+        if (NG == 1 || g == 0) mex_group_moments<R, 0>(p, l_max, rows + tid, nc);
+        else if (g == 1) mex_group_moments<R, 1>(p, l_max, rows + tid, nc);
+        else mex_group_moments<R, 2>(p, l_max, rows + tid, nc);
         __syncthreads();
-        R* rows = reinterpret_cast<R*>(s_pt) + warp * 32 * kMexScanHalf;
-        scan_rows<R, true>(ain, rows, &s_red[warp][0], lane);
-        scan_rows<R, false>(aout, rows, &s_red[warp][kMexNC], lane);
-        __syncthreads();
-        {
-            R* ts = thread_sums + (size_t)blockIdx.x * 2 * ncomp * kMexThreads + tid;
-#pragma unroll
-            for (int c = 0; c < kMexNC; ++c) {
-                if (c < gn) {
-                    R q = R(0), pp = R(0);
-                    for (int w = 0; w < warp; ++w) q += s_red[w][c];
-                    for (int w = kMexThreads / 32 - 1; w > warp; --w) pp += s_red[w][kMexNC + c];
-                    ts[(size_t)(c0 + c) * kMexThreads] = q + ain[c];
-                    ts[(size_t)(ncomp + c0 + c) * kMexThreads] = pp + aout[c];
-                }
+        if (tid < 2 * nc) {
+            // one thread per component: four interleaved sums down the row
+            const Vec4<R>* row = reinterpret_cast<const Vec4<R>*>(rows + tid * kMexRow);
+            Vec4<R> s = ld4(row);
+#pragma unroll 8
+            for (int i = 1; i < kMexThreads / 4; ++i) {
+                const Vec4<R> t = ld4(row + i);
+                s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
             }
-        }
-        for (int c = tid; c < 2 * gn; c += kMexThreads) {
-            const bool inner = c < gn;
-            const int lc = inner ? c : c - gn;
-            double sum = 0.0;
-            for (int w = 0; w < kMexThreads / 32; ++w)
-                sum += (double)s_red[w][(inner ? 0 : kMexNC) + lc];
-            const int cc = c0 + lc;
-            int l = 0;
-            while ((l + 1) * (l + 1) <= cc) ++l;
-            // undo the tile scale: inner moments scale as s^l, outer as s^-(l+1)
-            sum = inner ? ldexp(sum, l * e) : ldexp(sum, -(l + 1) * e);
+            const R sum = (s.x + s.y) + (s.z + s.w);
             if (!isfinite(sum)) report(err, ETICS_ERR_NONFINITE);
-            tile_agg[(size_t)blockIdx.x * 2 * ncomp + (inner ? 0 : ncomp) + cc] = sum;
+            const bool inner = tid < nc;
+            const int cc = c0 + (inner ? tid : tid - nc);
+            const int l = comp_level(cc);
+            // undo the tile scale: inner moments scale as s^l, outer as s^-(l+1)
+            const double d = scale_pow2((double)sum, inner ? l * e : -(l + 1) * e);
+            if (!isfinite(d)) report(err, ETICS_ERR_NONFINITE);
+            tile_agg[(size_t)((inner ? 0 : ncomp) + cc) * stride + blockIdx.x] = d;
         }
     }
 }
@@ -396,189 +474,232 @@ mex_pass1_kernel(const Vec4<R>* __restrict__ posm, const uint32_t* __restrict__ 
 // ---------------------------------------------------------------------------
 // carry: exclusive scans of the tile sums over tiles, one block per
 // component; forward for inner moments, reverse for outer (fixed order).
-// FP64 arithmetic is slow on this GPU (about 1/76 of the FP32 rate), so the scan
-// keeps the FP64 additions per block near the minimum: thread t owns a
-// contiguous run of scan positions, adds them in order, the run totals are
-// scanned by one warp-shuffle scan per warp and one over the warp totals,
-// then each thread writes its positions' exclusive sums.  Every addition
-// order depends only on (ntiles, ncomp): deterministic.
+// The sums of a component lie next to each other ([component][tile]), so a
+// thread takes kCarryRun neighbouring ones with wide loads, all in flight at
+// once, adds them in order, the run totals are scanned by one warp-shuffle
+// scan per warp and one over the warp totals, and each thread writes its
+// positions' exclusive sums; longer lists go segment by segment.  FP64
+// additions are slow on this GPU (about 1/76 of the FP32 rate): two per sum.
+// Every addition order depends only on ntiles: deterministic.
 // ---------------------------------------------------------------------------
 constexpr int kCarryThreads = 256;
 constexpr int kCarryWarps = kCarryThreads / 32;
+constexpr int kCarryRun = 16;
 static __global__ void __launch_bounds__(kCarryThreads)
-mex_carry_kernel(const double* __restrict__ tile_agg, int ntiles, int ncomp,
+mex_carry_kernel(const double* __restrict__ tile_agg, int ntiles, int stride, int ncomp,
                  double* __restrict__ carry) {
-    __shared__ double s_w[kCarryWarps];
+    __shared__ double s_w[kCarryWarps + 1];
     pdl_wait();   // the tile sums come from pass 1
     const int c = blockIdx.x;
     const bool rev = c >= ncomp;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int chunk = (ntiles + kCarryThreads - 1) / kCarryThreads;
-    const int o0 = tid * chunk;
-    const int o1 = o0 + chunk < ntiles ? o0 + chunk : ntiles;
-    const size_t stride = (size_t)2 * ncomp;
-    auto at = [&](int o) { return (size_t)(rev ? ntiles - 1 - o : o) * stride + c; };
-    // this thread's run, in scan order (read coherently after the wait)
-    double local = 0.0;
-#pragma unroll 4
-    for (int o = o0; o < o1; ++o) local += __ldcg(tile_agg + at(o));
-    // inclusive scan of the run totals over the warp
-    double x = local;
+    const double* src = tile_agg + (size_t)c * stride;
+    double* dst = carry + (size_t)c * stride;
+    double before = 0.0;   // sum of the earlier segments
+    // scan position o of the component is tile o (forward) or ntiles-1-o
+    for (int s0 = 0; s0 < ntiles; s0 += kCarryThreads * kCarryRun) {
+        const int left = ntiles - s0;
+        const int run = left >= kCarryThreads * kCarryRun
+                            ? kCarryRun : (left + kCarryThreads - 1) / kCarryThreads;
+        const int o0 = s0 + tid * run;
+        double v[kCarryRun];   // read coherently after the wait
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const double t = __shfl_up_sync(0xffffffffu, x, d);
-        if (lane >= d) x += t;
-    }
-    double ex = __shfl_up_sync(0xffffffffu, x, 1);
-    if (lane == 0) ex = 0.0;
-    if (lane == 31) s_w[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        // exclusive scan of the warp totals, in warp order
-        double w = lane < kCarryWarps ? s_w[lane] : 0.0;
-#pragma unroll
-        for (int d = 1; d < kCarryWarps; d <<= 1) {
-            const double t = __shfl_up_sync(0xffffffffu, w, d);
-            if (lane >= d) w += t;
+        for (int k = 0; k < kCarryRun; ++k) {
+            const int o = o0 + k;
+            v[k] = k < run && o < ntiles ? __ldcg(src + (rev ? ntiles - 1 - o : o)) : 0.0;
         }
-        double we = __shfl_up_sync(0xffffffffu, w, 1);
-        if (lane == 0) we = 0.0;
-        __syncwarp();
-        if (lane < kCarryWarps) s_w[lane] = we;
-    }
-    __syncthreads();
-    double run = warp == 0 ? ex : s_w[warp] + ex;
-    for (int o = o0; o < o1; ++o) {
-        const size_t i = at(o);
-        carry[i] = run;
-        run += __ldcg(tile_agg + i);
+        double local = v[0];
+#pragma unroll
+        for (int k = 1; k < kCarryRun; ++k)
+            if (k < run) local += v[k];
+        // inclusive scan of the run totals over the warp
+        double x = local;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const double t = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += t;
+        }
+        double ex = __shfl_up_sync(0xffffffffu, x, 1);
+        if (lane == 0) ex = 0.0;
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        if (warp == 0) {
+            // exclusive scan of the warp totals, in warp order; the last slot
+            // gets the segment's total
+            double w = lane < kCarryWarps ? s_w[lane] : 0.0;
+#pragma unroll
+            for (int d = 1; d <= kCarryWarps; d <<= 1) {
+                const double t = __shfl_up_sync(0xffffffffu, w, d);
+                if (lane >= d) w += t;
+            }
+            double we = __shfl_up_sync(0xffffffffu, w, 1);
+            if (lane == 0) we = 0.0;
+            __syncwarp();
+            if (lane <= kCarryWarps) s_w[lane] = we;
+        }
+        __syncthreads();
+        double at = (before + s_w[warp]) + ex;
+#pragma unroll
+        for (int k = 0; k < kCarryRun; ++k) {
+            const int o = o0 + k;
+            if (k < run && o < ntiles) {
+                dst[rev ? ntiles - 1 - o : o] = at;
+                at += v[k];
+            }
+        }
+        before += s_w[kCarryWarps];
+        __syncthreads();   // s_w is written again
     }
 }
 
 // ---------------------------------------------------------------------------
 // pass 2: field from the exclusive sums, per level group
 // ---------------------------------------------------------------------------
-// Group G: this thread's exclusive inner sum (tile carry + in-tile prefix from
-// pass 1), the forward sweep (inner part of the field, added to s_f), its
-// exclusive outer sum (a true suffix sum, never total minus prefix), the
-// reverse sweep (outer part); the last group present completes each
-// particle's field and scatters it back to the caller's order.
-template <typename R, int NG, int G, bool ACC>
-__device__ __forceinline__ void mex_pass2_group(const Vec4<R>* s_pt, Vec4<R>* s_f, R* s_q0,
-                                                R* s_p0, const double* carry,
-                                                const R* thread_sums, const uint32_t* perm,
-                                                int64_t base, int64_t N, int l_max, int e,
-                                                R scale, bool last, Vec4<R>* out, int out_mask,
-                                                unsigned* err) {
-    constexpr int L0 = mex_group_l0(G), L1 = mex_group_l1(G);
-    if (L0 > l_max) return;
-    const int tid = threadIdx.x;
-    const int ncomp = NG == 1 ? kMexNC : mex_layout_ncomp(l_max);
-    const int c0 = L0 * L0;
-    const int gn = NG == 1 ? kMexNC : mex_ncomp(L1 < l_max ? L1 : l_max) - c0;
-    if (G > 0) __syncthreads();   // the previous group's readers of s_q0 / s_p0 are done
-    for (int c = tid; c < 2 * gn; c += kMexThreads) {
-        const bool inner = c < gn;
-        const int lc = inner ? c : c - gn;
-        const int cc = c0 + lc;
-        int l = 0;
-        while ((l + 1) * (l + 1) <= cc) ++l;
-        const double v = carry[(size_t)blockIdx.x * 2 * ncomp + (inner ? 0 : ncomp) + cc];
-        if (inner) s_q0[lc] = (R)ldexp(v, -l * e);
-        else s_p0[lc] = (R)ldexp(v, (l + 1) * e);
-    }
-    __syncthreads();
-    const R* ts = thread_sums + (size_t)blockIdx.x * 2 * ncomp * kMexThreads + tid;
-    R a[kMexNC];
-#pragma unroll
-    for (int c = 0; c < kMexNC; ++c)
-        a[c] = c < gn ? s_q0[c] + ts[(size_t)(c0 + c) * kMexThreads] : R(0);
-#pragma unroll 1
-    for (int k = 0; k < kMexP; ++k) {
-        MexParticle<R> pt;
-        pt.init(s_pt[k * kMexThreads + tid], scale);
-        const R irho = pt.origin ? R(0) : R(1) / pt.rho;
-        R C[3][L1 + 1], S[3][L1 + 1];
-        R pot = R(0), ax = R(0), ay = R(0), az = R(0);
-        if (G > 0) {
-            const Vec4<R> f = s_f[k * kMexThreads + tid];
-            ax = f.x; ay = f.y; az = f.z; pot = f.w;
-        }
-        mex_fwd<R, L0, L1, 0, ACC>(C, S, pt, l_max, pt.m, irho, irho, a, pot, ax, ay, az);
-        st4(&s_f[k * kMexThreads + tid], mk4<R>(ax, ay, az, pot));
-    }
-    R b[kMexNC];
-#pragma unroll
-    for (int c = 0; c < kMexNC; ++c)
-        b[c] = c < gn ? s_p0[c] + ts[(size_t)(ncomp + c0 + c) * kMexThreads] : R(0);
-    const R s1 = scale, s2 = scale * scale;
-#pragma unroll 1
-    for (int k = kMexP - 1; k >= 0; --k) {
-        MexParticle<R> pt;
-        pt.init(s_pt[k * kMexThreads + tid], scale);
-        const R irho = pt.origin ? R(0) : R(1) / pt.rho;
-        R C[3][L1 + 1], S[3][L1 + 1];
-        const Vec4<R> f = s_f[k * kMexThreads + tid];
-        R pot = f.w, ax = f.x, ay = f.y, az = f.z;
-        const R wout = pt.origin ? R(0) : pt.m * irho;
-        mex_rev<R, L0, L1, 0, ACC>(C, S, pt, l_max, wout, R(1), R(0), irho, b, pot, ax, ay, az);
-        if (!last) {
-            st4(&s_f[k * kMexThreads + tid], mk4<R>(ax, ay, az, pot));
-            continue;
-        }
-        const int64_t i = base + (int64_t)tid * kMexP + k;
-        // perm[i] >= N only after a timed-out sort (reported): no store
-        if (i < N && (int64_t)perm[i] < N) {
-            const R potv = (out_mask & ETICS_OUT_POT) ? -pot * s1 : R(0);
-            const R fx = ACC ? ax * s2 : R(0);
-            const R fy = ACC ? ay * s2 : R(0);
-            const R fz = ACC ? az * s2 : R(0);
-            if (!finite4(fx, fy, fz, potv)) report(err, ETICS_ERR_NONFINITE);
-            st4(out + perm[i], mk4<R>(fx, fy, fz, potv));
-        }
+// exclusive sums of one component over four neighbouring pairs: the values
+// before (inner) or after (outer) each of them, of the sum `run` over what
+// lies on the other side of the four; then times the component's weight w on
+// top of the weighted tile carry `base`.  `run` takes in the four.
+template <typename R, bool kInner>
+__device__ __forceinline__ Vec4<R> mex_scan4(const Vec4<R>& t, R& run, R w, R base) {
+    const R b = fma(w, run, base);
+    if constexpr (kInner) {
+        const R t2 = t.x + t.y, t3 = t2 + t.z;
+        run += t2 + (t.z + t.w);
+        return mk4<R>(b, fma(w, t.x, b), fma(w, t2, b), fma(w, t3, b));
+    } else {
+        const R t2 = t.w + t.z, t3 = t2 + t.y;
+        run += t2 + (t.y + t.x);
+        return mk4<R>(fma(w, t3, b), fma(w, t2, b), fma(w, t.w, b), b);
     }
 }
 
-template <typename R, int NG, int G, bool ACC>
-__device__ __forceinline__ void mex_pass2_groups(const Vec4<R>* s_pt, Vec4<R>* s_f, R* s_q0,
-                                                 R* s_p0, const double* carry,
-                                                 const R* thread_sums, const uint32_t* perm,
-                                                 int64_t base, int64_t N, int l_max, int e,
-                                                 R scale, Vec4<R>* out, int out_mask,
-                                                 unsigned* err) {
-    if constexpr (G < NG) {
-        const bool last = G + 1 == NG || mex_group_l0(G + 1) > l_max;
-        mex_pass2_group<R, NG, G, ACC>(s_pt, s_f, s_q0, s_p0, carry, thread_sums, perm, base,
-                                       N, l_max, e, scale, last, out, out_mask, err);
-        mex_pass2_groups<R, NG, G + 1, ACC>(s_pt, s_f, s_q0, s_p0, carry, thread_sums, perm,
-                                            base, N, l_max, e, scale, out, out_mask, err);
+// one thread down the row of its component: forward for inner, reverse for
+// outer components (a true suffix sum, never total minus prefix)
+template <typename R>
+__device__ __forceinline__ void mex_scan_row(Vec4<R>* row, bool inner, R q0, R w) {
+    R run = R(0);
+    const R base = w * q0;
+    if (inner) {
+#pragma unroll 4
+        for (int i = 0; i < kMexThreads / 4; ++i)
+            st4(row + i, mex_scan4<R, true>(ld4(row + i), run, w, base));
+    } else {
+#pragma unroll 4
+        for (int i = kMexThreads / 4 - 1; i >= 0; --i)
+            st4(row + i, mex_scan4<R, false>(ld4(row + i), run, w, base));
     }
 }
+
+// one warp over the row of one component (four pairs per lane)
+template <typename R>
+__device__ __forceinline__ void mex_scan_row_warp(Vec4<R>* row, bool inner, R q0, R w, int lane) {
+    static_assert(kMexThreads == 128, "four pairs per lane");
+    const Vec4<R> t = ld4(row + lane);
+    R x = (t.x + t.y) + (t.z + t.w);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const R o = inner ? __shfl_up_sync(0xffffffffu, x, d) : __shfl_down_sync(0xffffffffu, x, d);
+        if (inner ? lane >= d : lane + d < 32) x += o;
+    }
+    R run = inner ? __shfl_up_sync(0xffffffffu, x, 1) : __shfl_down_sync(0xffffffffu, x, 1);
+    if (lane == (inner ? 0 : 31)) run = R(0);
+    const R base = w * q0;
+    st4(row + lane, inner ? mex_scan4<R, true>(t, run, w, base) : mex_scan4<R, false>(t, run, w, base));
+}
+
+// Components left over after whole warps of 32: up to this many go to the
+// next warp one after the other, all its lanes on one row (l_max = 6: 96 + 2
+// components; a fourth warp walking two rows serially would cost as much as
+// the other three).
+constexpr int kMexLeftover = 8;
 
 template <typename R, int NG, bool ACC>
 __global__ void __launch_bounds__(kMexThreads, mex_pass2_blocks<R, NG>())
 mex_pass2_kernel(const Vec4<R>* __restrict__ sorted, const uint32_t* __restrict__ perm, int64_t N,
-                 int l_max, const double* __restrict__ carry, const R* __restrict__ thread_sums,
+                 int l_max, const double* __restrict__ carry, int stride,
                  Vec4<R>* __restrict__ out, int out_mask, unsigned* err) {
-    __shared__ Vec4<R> s_pt[kMexTile];
-    __shared__ Vec4<R> s_f[kMexTile];   // each particle's field so far
-    __shared__ R s_q0[kMexNC], s_p0[kMexNC];
+    extern __shared__ __align__(16) unsigned char mex_smem[];
+    R* rows = reinterpret_cast<R*>(mex_smem);
+    __shared__ R s_end[2];
     pdl_wait();
     const int tid = threadIdx.x;
     const int64_t base = (int64_t)blockIdx.x * kMexTile;
     const int64_t rem = N - base;
     const int nt = (int)(rem < kMexTile ? rem : kMexTile);
-    for (int i = tid; i < kMexTile; i += kMexThreads)
-        st4(&s_pt[mex_slot(i)], i < nt ? ld4(sorted + base + i) : mk4<R>(R(0), R(0), R(0), R(0)));
-    __syncthreads();
-    int e;
-    {
-        const Vec4<R> a = s_pt[mex_slot(0)], b = s_pt[mex_slot(nt - 1)];
-        e = tile_exponent<R>(radius<R>(a.x, a.y, a.z), radius<R>(b.x, b.y, b.z));
-    }
+    Vec4<R> v[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+        v[j] = 2 * tid + j < nt ? ld4(sorted + base + 2 * tid + j) : mk4<R>(R(0), R(0), R(0), R(0));
+    uint32_t dst[2];   // in flight until the end
+#pragma unroll
+    for (int j = 0; j < 2; ++j) dst[j] = 2 * tid + j < nt ? perm[base + 2 * tid + j] : 0u;
+    const int e = mex_tile_exponent<R>(v[0], v[1], nt, s_end);
     const R scale = ldexp(R(1), -e);
-    mex_pass2_groups<R, NG, 0, ACC>(s_pt, s_f, s_q0, s_p0, carry, thread_sums, perm, base, N,
-                                    l_max, e, scale, out, out_mask, err);
+    MexPair<R> p;
+    p.init(v[0], v[1], scale, ldexp(R(1), e));
+    MexField<R> f;
+    const Pair<R> zero = splat(R(0));
+    f.s0 = f.s1 = f.rad = f.vx = f.vy = f.vz0 = f.vz1 = f.pot0 = zero;
+    const int ncomp = mex_layout_ncomp(l_max);
+    for (int g = 0; g < NG; ++g) {
+        const int L0 = mex_group_l0(g), L1 = mex_group_l1(g);
+        if (L0 > l_max) break;
+        const int c0 = L0 * L0;
+        const int nc = mex_ncomp(L1 < l_max ? L1 : l_max) - c0;
+        // this component's carry, in flight during the moments
+        const bool scanner = tid < 2 * nc, inner = tid < nc;
+        const int cc = c0 + (inner ? tid : tid - nc);
+        double cv = 0.0;
+        if (scanner) cv = carry[(size_t)((inner ? 0 : ncomp) + cc) * stride + blockIdx.x];
+        if (g > 0) __syncthreads();   // the previous group's rows have been read
+        opaque_pair(p);
+        if (NG == 1 || g == 0) mex_group_moments<R, 0>(p, l_max, rows + tid, nc);
+        else if (g == 1) mex_group_moments<R, 1>(p, l_max, rows + tid, nc);
+        else mex_group_moments<R, 2>(p, l_max, rows + tid, nc);
+        __syncthreads();
+        {
+            const int left = (2 * nc) & 31, whole = left <= kMexLeftover ? 2 * nc - left : 2 * nc;
+            R q0 = R(0), w = R(0);
+            if (scanner) {
+                const int l = comp_level(cc), am = (cc - l * l + 1) / 2;
+                q0 = (R)scale_pow2(cv, inner ? -l * e : (l + 1) * e);
+                w = mex_w<R>(l * (l + 1) / 2 + am);
+            }
+            if (tid < whole) {
+                mex_scan_row<R>(reinterpret_cast<Vec4<R>*>(rows + tid * kMexRow), inner, q0, w);
+            } else if ((tid & ~31) == whole) {   // whole is a multiple of 32 here
+                for (int j = 0; j < 2 * nc - whole; ++j)
+                    mex_scan_row_warp<R>(reinterpret_cast<Vec4<R>*>(rows + (whole + j) * kMexRow),
+                                         whole + j < nc, __shfl_sync(0xffffffffu, q0, j),
+                                         __shfl_sync(0xffffffffu, w, j), tid & 31);
+            }
+        }
+        __syncthreads();
+        opaque_pair(p);
+        if (NG == 1 || g == 0) mex_group_eval<R, 0, ACC>(p, l_max, rows + tid, nc, f);
+        else if (g == 1) mex_group_eval<R, 1, ACC>(p, l_max, rows + tid, nc, f);
+        else mex_group_eval<R, 2, ACC>(p, l_max, rows + tid, nc, f);
+    }
+    const R s1 = scale, s2 = scale * scale;
+    const R two = R(2), kap = R(kMexKappa), ikap = R(1) / R(kMexKappa);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        auto at = [&](const Pair<R>& q) { return j == 0 ? q.x : q.y; };
+        const int i = 2 * tid + j;
+        if (i >= nt) continue;
+        const R pot = fma(at(p.rho), fma(two, at(f.s1), at(f.s0)), at(f.pot0));
+        const R potv = (out_mask & ETICS_OUT_POT) ? -pot * s1 : R(0);
+        R fx = R(0), fy = R(0), fz = R(0);
+        if (ACC) {
+            const R k = at(f.rad) * ikap;
+            fx = s2 * fma(-k, at(p.x), kap * at(f.vx));
+            fy = s2 * fma(-k, at(p.y), kap * at(f.vy));
+            fz = s2 * fma(-k, at(p.z), kap * fma(two, at(f.vz1), at(f.vz0)));
+        }
+        if (!finite4(fx, fy, fz, potv)) report(err, ETICS_ERR_NONFINITE);
+        // an entry >= N only after a timed-out sort (reported): no store
+        if ((int64_t)dst[j] < N) st4(out + dst[j], mk4<R>(fx, fy, fz, potv));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -588,9 +709,8 @@ template <typename R>
 struct MexBuffers {
     SortBuffers sort;
     Vec4<R>* sorted;
-    double* tile_agg;    // [tile][2 * ncomp]: inner then outer sums (ncomp: mex_layout_ncomp)
-    double* carry;       // [tile][2 * ncomp]
-    R* thread_sums;      // [tile][2 * ncomp][kMexThreads], in-tile exclusive prefix / suffix
+    double* tile_agg;    // [2 * ncomp][tile]: inner then outer sums (ncomp: mex_layout_ncomp)
+    double* carry;       // [2 * ncomp][tile]
 };
 
 // ncomp = mex_layout_ncomp(l_max) components per side
@@ -611,7 +731,6 @@ inline MexBuffers<R> mex_buffers(void* ws, int64_t N, int l_max, size_t* total) 
     b.sorted = reinterpret_cast<Vec4<R>*>(take(n * sizeof(Vec4<R>)));
     b.tile_agg = reinterpret_cast<double*>(take(nt * 2 * nc * sizeof(double)));
     b.carry = reinterpret_cast<double*>(take(nt * 2 * nc * sizeof(double)));
-    b.thread_sums = reinterpret_cast<R*>(take(nt * 2 * nc * kMexThreads * sizeof(R)));
     if (total) *total = off;
     return b;
 }
@@ -623,31 +742,49 @@ inline size_t mex_workspace_impl(int64_t N, int l_max) {
     return total;
 }
 
+// the passes' shared memory: rows of one level group (above 48 KB the kernel
+// has to be told once per device)
+template <typename R, typename K>
+inline cudaError_t mex_allow_smem(K kernel, std::atomic<uint64_t>& done, size_t bytes) {
+    int dev = 0;
+    const cudaError_t ge = cudaGetDevice(&dev);
+    if (ge != cudaSuccess) return ge;
+    const uint64_t bit = uint64_t(1) << (dev & 63);
+    if (done.load() & bit) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done.fetch_or(bit);
+    return e;
+}
+
 template <typename R, int NG>
 inline int mex_passes(const MexBuffers<R>& b, const Vec4<R>* pp, int64_t N, int l_max, void* out,
                       int out_mask, const LaunchCtx& ctx) {
     const int nt = mex_tiles(N);
     const int ncomp = mex_layout_ncomp(l_max);
-    if (launch_pdl(mex_pass1_kernel<R, NG>, dim3(nt), dim3(kMexThreads), 0, ctx.stream, pp,
-                   (const uint32_t*)b.sort.vals_a, N, l_max, b.sorted, b.tile_agg, b.thread_sums,
-                   ctx.err))
+    constexpr size_t smem_max = (size_t)2 * kMexNC * kMexRow * sizeof(R);
+    const size_t smem = (size_t)2 * mex_row_comps(l_max) * kMexRow * sizeof(R);
+    static std::atomic<uint64_t> done1{0}, done2{0}, done3{0};
+    auto k1 = mex_pass1_kernel<R, NG>;
+    if (mex_allow_smem<R>(k1, done1, smem_max)) return ETICS_ERR_CUDA;
+    if (launch_pdl(k1, dim3(nt), dim3(kMexThreads), smem, ctx.stream, pp,
+                   (const uint32_t*)b.sort.vals_a, N, l_max, b.sorted, b.tile_agg, nt, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     stage_event(ctx, 3);
     if (launch_pdl(mex_carry_kernel, dim3(2 * ncomp), dim3(kCarryThreads), 0, ctx.stream,
-                   (const double*)b.tile_agg, nt, ncomp, b.carry))
+                   (const double*)b.tile_agg, nt, nt, ncomp, b.carry))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     stage_event(ctx, 4);
     Vec4<R>* op = reinterpret_cast<Vec4<R>*>(out);
-    const cudaError_t le = (out_mask & ETICS_OUT_ACC)
-        ? launch_pdl(mex_pass2_kernel<R, NG, true>, dim3(nt), dim3(kMexThreads), 0, ctx.stream,
-                     (const Vec4<R>*)b.sorted, (const uint32_t*)b.sort.vals_a, N, l_max,
-                     (const double*)b.carry, (const R*)b.thread_sums, op, out_mask, ctx.err)
-        : launch_pdl(mex_pass2_kernel<R, NG, false>, dim3(nt), dim3(kMexThreads), 0, ctx.stream,
-                     (const Vec4<R>*)b.sorted, (const uint32_t*)b.sort.vals_a, N, l_max,
-                     (const double*)b.carry, (const R*)b.thread_sums, op, out_mask, ctx.err);
-    if (le) return ETICS_ERR_CUDA;
+    const bool acc = out_mask & ETICS_OUT_ACC;
+    auto k2 = acc ? mex_pass2_kernel<R, NG, true> : mex_pass2_kernel<R, NG, false>;
+    if (mex_allow_smem<R>(k2, acc ? done2 : done3, smem_max)) return ETICS_ERR_CUDA;
+    if (launch_pdl(k2, dim3(nt), dim3(kMexThreads), smem, ctx.stream, (const Vec4<R>*)b.sorted,
+                   (const uint32_t*)b.sort.vals_a, N, l_max, (const double*)b.carry, nt, op, out_mask,
+                   ctx.err))
+        return ETICS_ERR_CUDA;
     ++*ctx.launches;
     stage_event(ctx, 5);
     return ETICS_OK;

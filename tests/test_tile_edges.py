@@ -1,0 +1,35 @@
+"""Sizes at the edges of the kernels' tiles, against the FP64 oracle: one
+particle more or less than a tile, a thread's pair or a bucket holds, and
+the smallest sizes.  Tolerances are those of the parity tests (eq. 23 errors
+of the mixed path; FP64 relative to the largest force, as in their edge
+cases: with few particles single forces nearly vanish)."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import device_particles, hernquist, rounded
+from paper_1406_4254_gb300 import etics
+
+pytestmark = pytest.mark.gpu
+
+
+def close(o, acc_ref, pot_ref, precision, what):
+    tol = 1e-11 if precision == "fp64" else 2e-5
+    amax = np.max(np.linalg.norm(acc_ref, axis=1))
+    assert np.max(np.abs(o[:, :3] - acc_ref)) <= tol * amax, what
+    assert np.max(np.abs(o[:, 3] - pot_ref)) <= tol * np.max(np.abs(pot_ref)), what
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("l_max", [0, 3, 6, 7, 10])
+def test_mex_tile_edges(precision, l_max):
+    """MEX tiles hold 256 particles, two per thread; 0, 3, 6: one level group
+    with 2, 32 and 98 components (a part of a warp, whole warps, a leftover
+    pair), 7 and 10: two and three groups."""
+    for n in (2, 255, 256, 257, 511, 513, 769):
+        pm = hernquist(n, seed=n)
+        ref = rounded(pm, precision)
+        acc, pot, _ = oracle.mex_field(ref[:, :3], ref[:, 3], l_max)
+        o = etics.mex_field(device_particles(pm, precision), l_max).cpu().numpy()
+        etics.check_error()
+        close(o, acc, pot, precision, (n, l_max))
