@@ -38,10 +38,14 @@ int scf_field_cb_f64(const void* posm, int64_t N, int n_max, int l_max, const do
 
 // ---- radial sort (etics_sort.cu) -------------------------------------------
 struct SortBuffers {
-    uint32_t *keys_a, *keys_b, *vals_a, *vals_b;
+    uint32_t *vals_a, *vals_b;           // the order; spare values
+    // radix path
+    uint32_t *keys_a, *keys_b;
     uint32_t *hist, *status, *counters;
     void* zero_base;
     size_t zero_bytes;
+    // sample path: bucket contents, splitters, ticket, flag and bucket sizes
+    uint32_t *region, *splitters, *part;
 };
 // carve the sort buffers from ws (ws may be null to only compute *total)
 SortBuffers sort_buffers(void* ws, int64_t N, size_t* total);
@@ -49,9 +53,10 @@ int sort_tiles(int64_t N);
 // the 32-bit sort keys alone
 template <typename R>
 int radial_keys_impl(const void* posm, int64_t N, uint32_t* keys, const LaunchCtx& ctx);
-// keys + 4 radix passes + tie fix-up; the order ends in vals_a
+// the radial order, into vals_a; sorted (nullable): the particles in that order
 template <typename R>
-int radial_sort_impl(const void* posm, int64_t N, const SortBuffers& b, const LaunchCtx& ctx);
+int radial_sort_impl(const void* posm, int64_t N, const SortBuffers& b, void* sorted,
+                     const LaunchCtx& ctx);
 
 // the bounded waits made to run out (etics_test_wait_timeout): one radix pass
 // over kTimeoutProbeN keys whose only block takes tile 1 while tile 0 never

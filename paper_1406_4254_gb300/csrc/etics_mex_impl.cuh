@@ -7,10 +7,9 @@
 // and a_i = -grad Phi_i at fixed q, p.
 //
 // GB300 design (the paper ran one library scan per (l, m) and direction):
-//   pass 1  gathers the particles in radial order (sorted copy) and reduces
-//           each tile's moments m rho^l Y and m rho^-(l+1) Y (rho = r / s_t,
-//           s_t a power of two per tile, so FP32 never overflows) to one FP64
-//           sum per component.
+//   pass 1  reduces each tile of the sorted particles' moments m rho^l Y and
+//           m rho^-(l+1) Y (rho = r / s_t, s_t a power of two per tile, so
+//           FP32 never overflows) to one FP64 sum per component.
 //   carry   scans the per-tile FP64 sums in a fixed order: exclusive forward
 //           for the inner moments, exclusive reverse (a true suffix sum) for
 //           the outer ones -- deterministic.
@@ -400,13 +399,12 @@ template <typename R, int NG>
 constexpr int mex_pass2_blocks() { return sizeof(R) == 4 ? (NG == 1 ? 4 : 3) : 2; }
 
 // ---------------------------------------------------------------------------
-// pass 1: gather into radial order + per-tile FP64 moment sums
+// pass 1: per-tile FP64 moment sums
 // ---------------------------------------------------------------------------
 template <typename R, int NG>
 __global__ void __launch_bounds__(kMexThreads, mex_pass1_blocks<R>())
-mex_pass1_kernel(const Vec4<R>* __restrict__ posm, const uint32_t* __restrict__ perm, int64_t N,
-                 int l_max, Vec4<R>* __restrict__ sorted, double* __restrict__ tile_agg, int stride,
-                 unsigned* err) {
+mex_pass1_kernel(const Vec4<R>* __restrict__ sorted, int64_t N, int l_max,
+                 double* __restrict__ tile_agg, int stride, unsigned* err) {
     extern __shared__ __align__(16) unsigned char mex_smem[];
     R* rows = reinterpret_cast<R*>(mex_smem);
     __shared__ R s_end[2];
@@ -415,25 +413,10 @@ mex_pass1_kernel(const Vec4<R>* __restrict__ posm, const uint32_t* __restrict__ 
     const int64_t base = (int64_t)blockIdx.x * kMexTile;
     const int64_t rem = N - base;
     const int nt = (int)(rem < kMexTile ? rem : kMexTile);
-    uint32_t idx[2];
     Vec4<R> v[2];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) idx[j] = 2 * tid + j < nt ? perm[base + 2 * tid + j] : 0u;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        v[j] = mk4<R>(R(0), R(0), R(0), R(0));
-        // an index >= N can only come from a sort whose lookback timed
-        // out (already reported): it gathers a massless particle at 0
-        if (2 * tid + j < nt && (int64_t)idx[j] < N) v[j] = ld4(posm + idx[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        if (!finite4(v[j].x, v[j].y, v[j].z, v[j].w)) {
-            report(err, ETICS_ERR_NONFINITE);
-            v[j] = mk4<R>(R(0), R(0), R(0), R(0));
-        }
-        if (2 * tid + j < nt) st4(sorted + base + 2 * tid + j, v[j]);
-    }
+    for (int j = 0; j < 2; ++j)
+        v[j] = 2 * tid + j < nt ? ld4(sorted + base + 2 * tid + j) : mk4<R>(R(0), R(0), R(0), R(0));
     const int e = mex_tile_exponent<R>(v[0], v[1], nt, s_end);
     MexPair<R> p;
     p.init(v[0], v[1], ldexp(R(1), -e), ldexp(R(1), e));
@@ -758,8 +741,8 @@ inline cudaError_t mex_allow_smem(K kernel, std::atomic<uint64_t>& done, size_t 
 }
 
 template <typename R, int NG>
-inline int mex_passes(const MexBuffers<R>& b, const Vec4<R>* pp, int64_t N, int l_max, void* out,
-                      int out_mask, const LaunchCtx& ctx) {
+inline int mex_passes(const MexBuffers<R>& b, int64_t N, int l_max, void* out, int out_mask,
+                      const LaunchCtx& ctx) {
     const int nt = mex_tiles(N);
     const int ncomp = mex_layout_ncomp(l_max);
     constexpr size_t smem_max = (size_t)2 * kMexNC * kMexRow * sizeof(R);
@@ -767,8 +750,8 @@ inline int mex_passes(const MexBuffers<R>& b, const Vec4<R>* pp, int64_t N, int 
     static std::atomic<uint64_t> done1{0}, done2{0}, done3{0};
     auto k1 = mex_pass1_kernel<R, NG>;
     if (mex_allow_smem<R>(k1, done1, smem_max)) return ETICS_ERR_CUDA;
-    if (launch_pdl(k1, dim3(nt), dim3(kMexThreads), smem, ctx.stream, pp,
-                   (const uint32_t*)b.sort.vals_a, N, l_max, b.sorted, b.tile_agg, nt, ctx.err))
+    if (launch_pdl(k1, dim3(nt), dim3(kMexThreads), smem, ctx.stream, (const Vec4<R>*)b.sorted, N,
+                   l_max, b.tile_agg, nt, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     stage_event(ctx, 3);
@@ -796,13 +779,12 @@ inline int mex_field_impl(const void* posm, int64_t N, int l_max, void* out, int
     if (N == 0) return ETICS_OK;
     MexBuffers<R> b = mex_buffers<R>(ws, N, l_max, nullptr);
     stage_event(ctx, 0);
-    int rc = radial_sort_impl<R>(posm, N, b.sort, ctx);
+    int rc = radial_sort_impl<R>(posm, N, b.sort, b.sorted, ctx);
     if (rc) return rc;
     stage_event(ctx, 2);
-    const Vec4<R>* pp = reinterpret_cast<const Vec4<R>*>(posm);
     // l_max <= 6: one level group (the kernels specialised for it)
-    if (mex_ngroups(l_max) == 1) return mex_passes<R, 1>(b, pp, N, l_max, out, out_mask, ctx);
-    return mex_passes<R, kMexGroups>(b, pp, N, l_max, out, out_mask, ctx);
+    if (mex_ngroups(l_max) == 1) return mex_passes<R, 1>(b, N, l_max, out, out_mask, ctx);
+    return mex_passes<R, kMexGroups>(b, N, l_max, out, out_mask, ctx);
 }
 
 template <typename R>
@@ -810,7 +792,7 @@ inline int radial_order_impl(const void* posm, int64_t N, uint32_t* order, void*
                              const LaunchCtx& ctx) {
     if (N == 0) return ETICS_OK;
     MexBuffers<R> b = mex_buffers<R>(ws, N, 0, nullptr);
-    int rc = radial_sort_impl<R>(posm, N, b.sort, ctx);
+    int rc = radial_sort_impl<R>(posm, N, b.sort, nullptr, ctx);
     if (rc) return rc;
     if (cudaMemcpyAsync(order, b.sort.vals_a, (size_t)N * 4, cudaMemcpyDeviceToDevice, ctx.stream))
         return ETICS_ERR_CUDA;

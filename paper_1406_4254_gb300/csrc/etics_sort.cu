@@ -2,17 +2,30 @@
 // sums need the particles ordered by radius; Sec. 3.2 used a library merge
 // sort).
 //
-// GB300 design: a hand-written stable LSD radix sort (4 passes of 8 bits) of
+// GB300 design, two paths that give the same order, the exact FP64 order
+// (r^2 = (x*x + y*y) + z*z rounded as a CPU does, ties by index):
+//
+// Up to kSampleMaxN particles, a sample sort: one partition of the indices
+// into buckets of about 1024 particles (splitters from a sorted sample), then one
+// block per bucket sorts it in shared memory by the 64-bit pattern of r^2 and
+// writes the order and the particles themselves.  Up to 8192 particles the
+// last kernel alone does it.  Two dependent launches instead of the radix
+// path's six, and three passes over the particles instead of ten over keys.
+//
+// Above, a hand-written stable LSD radix sort (4 passes of 8 bits) of
 // the high 32 bits of the FP64 r^2 bit pattern, one kernel per pass
 // ("one-sweep": per-tile digit ranking with warp ballots, the tile's keys
 // placed in digit order in shared memory, a decoupled lookback over tiles for
 // the digit offsets, coalesced writes of digit runs).  Runs of equal high
-// words are then ordered by the low 32 bits and the particle index, which
-// reproduces the exact FP64 order (r^2 = (x*x + y*y) + z*z rounded as a CPU
-// does, ties by index).  The passes and the tie fix-up are launched with
-// programmatic dependent launch, so each launch overlaps its predecessor's
-// tail.
+// words are then ordered by the low 32 bits and the particle index, and the
+// particles are gathered into that order.
+//
+// All kernels are launched with programmatic dependent launch, so each launch
+// overlaps its predecessor's tail.
+#include <atomic>
+
 #include "etics_internal.h"
+#include "etics_r2.h"
 
 namespace etics {
 
@@ -209,6 +222,55 @@ __device__ __forceinline__ void rank_in_warp(const uint32_t (&d)[kSortKpt], uint
     }
 }
 
+// Decoupled lookback over the earlier tiles of one digit or bucket (st: this
+// tile's status word, stride: words per tile): a window of predecessors is
+// read at once; flags become bit masks; counts are summed up to the first
+// inclusive prefix, or up to the first predecessor that has not published
+// (then that one word is polled before the next window).  The status array
+// holds kStatusPad zeroed (never published) tiles before tile 0, so a window
+// may reach below tile 0 without a bounds test: tile 0 always publishes an
+// inclusive prefix, which ends every walk first.  A tile takes its number from
+// a counter, so the tiles waited for have started.  The poll gives up after
+// spin_limit tries: the error word records ETICS_ERR_TIMEOUT and the partial
+// sum (at most the true one) is returned.
+__device__ __forceinline__ uint32_t lookback(const uint32_t* st, size_t stride, int64_t spin_limit,
+                                             unsigned* err) {
+    uint32_t excl = 0;
+    const uint32_t* p = st - stride;   // tile - 1
+    int64_t spins = 0;
+    for (;;) {
+        uint32_t w[kLookbackWindow];
+#pragma unroll
+        for (int j = 0; j < kLookbackWindow; ++j) w[j] = ld_volatile(p - j * stride);
+        uint32_t pub = 0, inc = 0;
+#pragma unroll
+        for (int j = 0; j < kLookbackWindow; ++j) {
+            const uint32_t f = w[j] >> 30;
+            pub |= (f != 0u ? 1u : 0u) << j;
+            inc |= (f == (kFlagInc >> 30) ? 1u : 0u) << j;
+        }
+        const int first_wait = ~pub ? __ffs(~pub) - 1 : kLookbackWindow;
+        const int first_inc = inc ? __ffs(inc) - 1 : kLookbackWindow;
+        const bool done = first_inc < first_wait;
+        const int used = done ? first_inc + 1 : first_wait;
+        const uint32_t take = used >= 32 ? 0xffffffffu : ((1u << used) - 1u);
+#pragma unroll
+        for (int j = 0; j < kLookbackWindow; ++j)
+            if ((take >> j) & 1u) excl += w[j] & kCountMask;
+        if (done) break;
+        p -= (size_t)used * stride;
+        if (used < kLookbackWindow) {
+            bool timed_out = false;
+            while ((ld_volatile(p) >> 30) == 0u) {
+                if (++spins > spin_limit) { timed_out = true; break; }
+                __nanosleep(32);
+            }
+            if (timed_out) { report(err, ETICS_ERR_TIMEOUT); break; }
+        }
+    }
+    return excl;
+}
+
 // One pass of the stable LSD radix sort (8-bit digit at `shift`) over tiles
 // of kSortTile keys.  Order of work in a tile: load and rank; publish the
 // tile's digit counts (status word: flag | count); scan the global histogram
@@ -283,8 +345,8 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     }
     // publish at once: tile 0 (and any digit no key has) as inclusive
     uint32_t* st = status + (size_t)(tile + kStatusPad) * 256 + dig;
-    const bool lookback = tile != 0 && gcount != 0u;
-    st_volatile(st, (lookback ? kFlagAgg : kFlagInc) | count);
+    const bool look = tile != 0 && gcount != 0u;
+    st_volatile(st, (look ? kFlagAgg : kFlagInc) | count);
     // exclusive scans of the global histogram (start of each digit) and of
     // the tile counts (start of each digit in the tile), together
     uint32_t xa = gcount, xb = count;
@@ -309,49 +371,13 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
             s_vals[pos] = v[s];
         }
     }
-    // decoupled lookback over earlier tiles for this digit: a window of
-    // predecessors is read at once; flags become bit masks; counts are summed
-    // up to the first inclusive prefix, or up to the first predecessor that
-    // has not published (then that one word is polled before the next window).
-    // The poll gives up after spin_limit tries: the error word records
-    // ETICS_ERR_TIMEOUT and the tile goes on with the partial prefix (at most
-    // the true one), so its output positions stay below N; keys that no
-    // longer match the histogram (a later pass of a timed-out sort) can
-    // compute a position >= N, and such a store is skipped below.
+    // the sum over earlier tiles of this digit; after a wait that gave up (a
+    // partial sum, at most the true one) the output positions stay below N;
+    // keys that no longer match the histogram (a later pass of a timed-out
+    // sort) can compute a position >= N, and such a store is skipped below
     uint32_t excl = 0;
-    if (lookback) {
-        const uint32_t* p = st - 256;   // tile - 1
-        int64_t spins = 0;
-        for (;;) {
-            uint32_t w[kLookbackWindow];
-#pragma unroll
-            for (int j = 0; j < kLookbackWindow; ++j) w[j] = ld_volatile(p - j * 256);
-            uint32_t pub = 0, inc = 0;
-#pragma unroll
-            for (int j = 0; j < kLookbackWindow; ++j) {
-                const uint32_t f = w[j] >> 30;
-                pub |= (f != 0u ? 1u : 0u) << j;
-                inc |= (f == (kFlagInc >> 30) ? 1u : 0u) << j;
-            }
-            const int first_wait = ~pub ? __ffs(~pub) - 1 : kLookbackWindow;
-            const int first_inc = inc ? __ffs(inc) - 1 : kLookbackWindow;
-            const bool done = first_inc < first_wait;
-            const int used = done ? first_inc + 1 : first_wait;
-            const uint32_t take = used >= 32 ? 0xffffffffu : ((1u << used) - 1u);
-#pragma unroll
-            for (int j = 0; j < kLookbackWindow; ++j)
-                if ((take >> j) & 1u) excl += w[j] & kCountMask;
-            if (done) break;
-            p -= (size_t)used * 256;
-            if (used < kLookbackWindow) {
-                bool timed_out = false;
-                while ((ld_volatile(p) >> 30) == 0u) {
-                    if (++spins > spin_limit) { timed_out = true; break; }
-                    __nanosleep(32);
-                }
-                if (timed_out) { report(err, ETICS_ERR_TIMEOUT); break; }
-            }
-        }
+    if (look) {
+        excl = lookback(st, 256, spin_limit, err);
         st_volatile(st, kFlagInc | (excl + count));
     }
     s_gbase[dig] = hexcl + excl;
@@ -602,6 +628,569 @@ tie_fixup_kernel(const uint32_t* __restrict__ key, const Vec4<R>* __restrict__ p
         sort_run_block<R>(posm, N, val, tmp, s_long_s[r], s_long_n[r], s_cnt, s_off, s_wsum);
 }
 
+// the particles in radial order (radix path; an index >= N, only after a
+// timed-out sort, gives a massless particle at the origin, as does a
+// non-finite one, which is reported)
+template <typename R>
+__device__ __forceinline__ Vec4<R> gather_particle(const Vec4<R>* posm, uint32_t i, int64_t N,
+                                                   unsigned* err) {
+    Vec4<R> v = mk4<R>(R(0), R(0), R(0), R(0));
+    if ((int64_t)i < N) {
+        v = ld4(posm + i);
+        if (!finite4(v.x, v.y, v.z, v.w)) {
+            report(err, ETICS_ERR_NONFINITE);
+            v = mk4<R>(R(0), R(0), R(0), R(0));
+        }
+    }
+    return v;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256)
+gather_kernel(const Vec4<R>* __restrict__ posm, const uint32_t* perm, int64_t N,
+              Vec4<R>* __restrict__ sorted, unsigned* err) {
+    pdl_wait();   // the order comes from the kernel before
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) st4(sorted + i, gather_particle<R>(posm, __ldcg(perm + i), N, err));
+}
+
+// ---------------------------------------------------------------------------
+// sample sort
+// ---------------------------------------------------------------------------
+// the whole FP64 bit pattern of r^2; a non-finite particle sorts last
+__device__ __forceinline__ uint64_t r2_bits(const float4& v) {
+    uint64_t b;
+    if (!finite4(v.x, v.y, v.z, v.w)) return ~uint64_t(0);
+    if (!r2_bits_from_f32(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), b))
+        b = (uint64_t)__double_as_longlong(r2_fp64((double)v.x, (double)v.y, (double)v.z));
+    return b;
+}
+__device__ __forceinline__ uint64_t r2_bits(const dvec4& v) {
+    if (!finite4(v.x, v.y, v.z, v.w)) return ~uint64_t(0);
+    return (uint64_t)__double_as_longlong(r2_fp64(v.x, v.y, v.z));
+}
+
+// Bucket sizes: a bucket's mean is a quarter of what a block sorts in shared
+// memory.  With kOversample random samples per bucket a bucket four times the
+// mean has a probability of about 1e-7 (the sum of eight exponential spacings);
+// it is sorted all the same, by the slower sort_bucket_global.
+constexpr int kOversample = 8;
+constexpr int kMaxBuckets = 1024;
+constexpr int kPartThreads = 1024;          // one thread per bucket
+constexpr int kBucketSmall = 4096, kBucketLarge = 8192;
+constexpr int kBucketKpt = 16;              // pairs per thread at capacity
+static_assert(kOversample * kMaxBuckets <= 8 * kPartThreads, "one block sorts the sample");
+
+// How many buckets, of which capacity, and how many particles per thread of
+// the partition: enough tiles for the SMs at each size (2^20: 128 tiles of
+// 8192).  Above kSampleMaxN the sample (sorted by one block) would get too
+// small for the number of buckets: the radix path.
+constexpr int64_t kSampleMaxN = int64_t(kMaxBuckets) * (kBucketLarge / 4);
+struct SamplePlan { int nbuckets, cap, kpt, ntiles; };
+SamplePlan sample_plan(int64_t N) {
+    SamplePlan p{};
+    if (N > kSampleMaxN) return p;
+    p.cap = N > kBucketLarge && N <= int64_t(kMaxBuckets) * kBucketSmall / 4 ? kBucketSmall
+                                                                              : kBucketLarge;
+    p.nbuckets = N <= p.cap ? 1 : (int)((N + p.cap / 4 - 1) / (p.cap / 4));
+    p.kpt = N <= (int64_t(1) << 18) ? 2 : N <= (int64_t(1) << 19) ? 4 : 8;
+    p.ntiles = (int)((N + (int64_t)kPartThreads * p.kpt - 1) / ((int64_t)kPartThreads * p.kpt));
+    return p;
+}
+
+// Sorts n <= TH KPT pairs (32-bit key, id) of a block, thread t holding the
+// pairs t, t + TH, ... in k[], id[]: each key is mapped linearly from the
+// block's key range to one of 8 TH bins, the bins are counted and scanned, and
+// the pairs placed in bin order in s_key / s_id; within a bin (half a pair on
+// average at a bucket's mean size) count_less() counts the smaller keys.
+// Equal keys are told apart by the caller, who fills s_low and passes how.
+constexpr int kBinLimit = 48;
+template <int TH, int KPT>
+struct BlockSort {
+    static constexpr int CAP = TH * KPT, NB = 8 * TH;
+    static constexpr size_t kSmem = (size_t)CAP * 14 + (size_t)NB * 4;   // with a 16-bit list
+    uint32_t *s_key, *s_id, *s_low, *s_bin;
+    uint32_t kmin, mult;
+    int n;
+    bool crowded;   // a bin holds more than kBinLimit pairs
+
+    __device__ __forceinline__ explicit BlockSort(unsigned char* smem)
+        : s_key(reinterpret_cast<uint32_t*>(smem)), s_id(s_key + CAP), s_low(s_id + CAP),
+          s_bin(s_low + CAP) {}
+
+    __device__ __forceinline__ int bin_of(uint32_t key) const {
+        return (int)(mult ? __umulhi(key - kmin, mult) : key - kmin);
+    }
+
+    // (s_low is not touched; low: placed along when not null)
+    __device__ __forceinline__ void place(const uint32_t (&k)[KPT], const uint32_t (&id)[KPT],
+                                          const uint32_t* low, int count) {
+        __shared__ uint32_t s_lo, s_hi, s_sum[32];
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        n = count;
+        if (tid == 0) { s_lo = 0xffffffffu; s_hi = 0u; }
+        uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+        for (int s = 0; s < KPT; ++s)
+            if (tid + s * TH < n) {
+                lo = k[s] < lo ? k[s] : lo;
+                hi = k[s] > hi ? k[s] : hi;
+            }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        uint4* bins4 = reinterpret_cast<uint4*>(s_bin);
+        bins4[tid] = make_uint4(0, 0, 0, 0);
+        bins4[tid + TH] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        if (lane == 0) {
+            atomicMin(&s_lo, lo);
+            atomicMax(&s_hi, hi);
+        }
+        __syncthreads();
+        // (key - lo) NB / (range + 1); a range below NB is its own bin number
+        kmin = s_lo;
+        const uint32_t range = s_hi - kmin;
+        mult = range < (uint32_t)NB ? 0u : (uint32_t)(((uint64_t)NB << 32) / ((uint64_t)range + 1));
+        uint32_t at[KPT];   // bin, then rank within it (16 bits each)
+#pragma unroll
+        for (int s = 0; s < KPT; ++s)
+            if (tid + s * TH < n) {
+                const int b = bin_of(k[s]);
+                at[s] = (uint32_t)b | (atomicAdd(&s_bin[b], 1u) << 16);
+            }
+        __syncthreads();
+        // exclusive scan of the bins, eight neighbouring ones per thread
+        uint4 c0 = bins4[2 * tid], c1 = bins4[2 * tid + 1];
+        const uint32_t most = max(max(max(c0.x, c0.y), max(c0.z, c0.w)),
+                                  max(max(c1.x, c1.y), max(c1.z, c1.w)));
+        const uint32_t h0 = c0.x + c0.y + c0.z + c0.w, sum = h0 + c1.x + c1.y + c1.z + c1.w;
+        uint32_t x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += t;
+        }
+        if (lane == 31) s_sum[warp] = x;
+        crowded = __syncthreads_or(most > (uint32_t)kBinLimit);
+        uint32_t at0 = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? s_sum[lane] : 0u);
+        bins4[2 * tid] = make_uint4(at0, at0 + c0.x, at0 + c0.x + c0.y, at0 + c0.x + c0.y + c0.z);
+        at0 += h0;
+        bins4[2 * tid + 1] = make_uint4(at0, at0 + c1.x, at0 + c1.x + c1.y, at0 + c1.x + c1.y + c1.z);
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < KPT; ++s)
+            if (tid + s * TH < n) {
+                const uint32_t pos = s_bin[at[s] & 0xffffu] + (at[s] >> 16);
+                s_key[pos] = k[s];
+                s_id[pos] = id[s];
+                if (low) s_low[pos] = low[s];
+            }
+        __syncthreads();
+    }
+
+    // the pairs [0, n) sorted by (key, low, id), padded to a power of two (at
+    // most CAP): where keys crowd, a network instead of the bins
+    __device__ __noinline__ void bitonic() {
+        int p2 = 2;
+        while (p2 < n) p2 <<= 1;
+        for (int i = n + threadIdx.x; i < p2; i += TH) s_key[i] = s_low[i] = s_id[i] = 0xffffffffu;
+        __syncthreads();
+        for (int k = 2; k <= p2; k <<= 1)
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int t = threadIdx.x; t < p2 / 2; t += TH) {
+                    const int i = 2 * t - (t & (j - 1)), l = i + j;
+                    const uint32_t a = s_key[i], b = s_key[l], la = s_low[i], lb = s_low[l],
+                                   ia = s_id[i], ib = s_id[l];
+                    const bool after = a > b || (a == b && (la > lb || (la == lb && ia > ib)));
+                    if (after == ((i & k) == 0)) {
+                        s_key[i] = b; s_key[l] = a;
+                        s_low[i] = lb; s_low[l] = la;
+                        s_id[i] = ib; s_id[l] = ia;
+                    }
+                }
+                __syncthreads();
+            }
+    }
+
+    // bounds of the bin of the pair at p
+    __device__ __forceinline__ void bin_range(uint32_t key, int& s, int& e) const {
+        const int b = bin_of(key);
+        s = (int)s_bin[b];
+        e = b + 1 < NB ? (int)s_bin[b + 1] : n;
+    }
+};
+
+__device__ __forceinline__ uint32_t mix32(uint32_t x) {
+    x = (x ^ (x >> 16)) * 0x45d9f3bu;
+    x = (x ^ (x >> 16)) * 0x45d9f3bu;
+    return x ^ (x >> 16);
+}
+
+// the 32-bit key of a particle (r2_key); non-finite ones come last
+template <typename R>
+__device__ __forceinline__ uint32_t sort_key(const Vec4<R>& v) {
+    return finite4(v.x, v.y, v.z, v.w) ? r2_key(v.x, v.y, v.z) : 0xffffffffu;
+}
+
+// The splitters: every kOversample-th key of a sorted sample of kOversample
+// nbuckets particles, one at a random place of each of as many equal stretches
+// of the array (a regular stride could fall in step with an order of the
+// particles).  stride: N / (number of samples), 32.32 fixed point.
+using SplitterSort = BlockSort<kPartThreads, 8>;
+template <typename R>
+__device__ __forceinline__ void make_splitters(const Vec4<R>* posm, int64_t N, int nbuckets,
+                                               uint64_t stride, uint32_t* splitters,
+                                               unsigned char* smem) {
+    const int tid = threadIdx.x, ns = kOversample * nbuckets;
+    uint32_t k[8], id[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+        const uint32_t i = (uint32_t)(tid + s * kPartThreads);
+        if ((int)i < ns) {
+            const int64_t a = (int64_t)((i * stride) >> 32);
+            int64_t b = (int64_t)(((i + 1) * stride) >> 32);
+            if (b <= a) b = a + 1;
+            const int64_t g = a + (int64_t)__umulhi(mix32(i + 1), (uint32_t)(b - a));
+            k[s] = sort_key<R>(ld4(posm + (g < N ? g : N - 1)));
+            id[s] = i;
+        }
+    }
+    SplitterSort sort(smem);
+    sort.place(k, id, nullptr, ns);
+    if (sort.crowded) {
+        for (int p = tid; p < ns; p += kPartThreads) sort.s_low[p] = 0u;
+        sort.bitonic();
+    }
+    for (int p = tid; p < ns; p += kPartThreads) {
+        int r = p;
+        const uint32_t key = sort.s_key[p];
+        if (!sort.crowded) {
+            int s, e;
+            sort.bin_range(key, s, e);
+            r = s;
+            const uint32_t own = sort.s_id[p];
+            for (int j = s; j < e; ++j)
+                r += sort.s_key[j] < key || (sort.s_key[j] == key && sort.s_id[j] < own);
+        }
+        if (r % kOversample == 0) splitters[r / kOversample] = r == 0 ? 0u : key;
+    }
+}
+
+// bucket of a key: the last splitter not above it (s_split padded with
+// 0xffffffff to 1024 entries, splitter 0 is 0)
+__device__ __forceinline__ int bucket_of(const uint32_t* s_split, uint32_t key, int nbuckets) {
+    int b = 0;
+#pragma unroll
+    for (int h = kMaxBuckets / 2; h > 0; h >>= 1)
+        if (s_split[b + h] <= key) b += h;
+    return b < nbuckets ? b : nbuckets - 1;
+}
+
+// Partition.  Blocks take tickets; the block with the first one makes the
+// splitters and raises the flag, the others load their tile's particles and
+// evaluate the keys meanwhile and wait for it (bounded; the tickets' order
+// makes sure that the block waited for has started).  A tile then counts its
+// particles per bucket in shared memory, takes its places in the buckets with
+// one addition per bucket to the bucket sizes, and writes the particles'
+// indices to region[b * cap + place].  The order inside a bucket's region is
+// whatever the additions give: the bucket sort orders by (r^2, index).  A place
+// beyond the capacity is not written (sort_bucket_global finds those particles
+// again).  A tile whose wait runs out (ETICS_ERR_TIMEOUT) counts its particles
+// in bucket 0: the sizes still add up to N, so that everything after stays
+// inside the buffers.
+// part (zero at launch): [0] ticket counter, [1] flag, from word kPartHeader
+// on the bucket sizes.
+constexpr int kPartHeader = 64;
+template <typename R, int KPT>
+__global__ void __launch_bounds__(kPartThreads, 1)
+partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int cap,
+                 uint64_t stride, uint32_t* splitters, uint32_t* part,
+                 uint32_t* __restrict__ region, int64_t spin_limit, unsigned* err) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    __shared__ uint32_t s_split[kMaxBuckets];
+    __shared__ uint32_t s_hist[kMaxBuckets];
+    __shared__ uint32_t s_ticket;
+    __shared__ int s_ok;
+    const int tid = threadIdx.x;
+    s_hist[tid] = 0u;
+    pdl_wait();
+    if (tid == 0) s_ticket = atomicAdd(part, 1u);
+    __syncthreads();
+    if (s_ticket == 0u) {
+        make_splitters<R>(posm, N, nbuckets, stride, splitters, sort_smem);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) st_volatile(part + 1, 1u);
+        return;
+    }
+    const int64_t start = (int64_t)(s_ticket - 1u) * kPartThreads * KPT;
+    Vec4<R> v[KPT];
+#pragma unroll
+    for (int s = 0; s < KPT; ++s) {
+        const int64_t i = start + s * kPartThreads + tid;
+        if (i < N) v[s] = ld4(posm + i);
+    }
+    uint32_t key[KPT];
+#pragma unroll
+    for (int s = 0; s < KPT; ++s) {
+        key[s] = 0u;
+        if (start + s * kPartThreads + tid < N) {
+            key[s] = sort_key<R>(v[s]);
+            if (key[s] == 0xffffffffu) report(err, ETICS_ERR_NONFINITE);
+        }
+    }
+    if (tid == 0) {
+        int64_t spins = 0;
+        int ok = 1;
+        while (ld_volatile(part + 1) == 0u) {
+            if (++spins > spin_limit) { ok = 0; break; }
+            __nanosleep(32);
+        }
+        if (!ok) report(err, ETICS_ERR_TIMEOUT);
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    s_split[tid] = tid < nbuckets && s_ok ? __ldcg(splitters + tid) : (tid ? 0xffffffffu : 0u);
+    __syncthreads();
+    uint32_t at[KPT];   // bucket, then place within the tile's share (16 bits each)
+#pragma unroll
+    for (int s = 0; s < KPT; ++s) {
+        at[s] = 0u;
+        if (start + s * kPartThreads + tid < N) {
+            const int b = bucket_of(s_split, key[s], s_ok ? nbuckets : 1);
+            at[s] = (uint32_t)b | (atomicAdd(&s_hist[b], 1u) << 16);
+        }
+    }
+    __syncthreads();
+    if (tid < nbuckets && s_hist[tid])
+        s_hist[tid] = atomicAdd(part + kPartHeader + tid, s_hist[tid]);
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < KPT; ++s) {
+        const int64_t i = start + s * kPartThreads + tid;
+        if (i < N) {
+            const uint32_t b = at[s] & 0xffffu, slot = s_hist[b] + (at[s] >> 16);
+            if (slot < (uint32_t)cap) region[(size_t)b * cap + slot] = (uint32_t)i;
+        }
+    }
+}
+
+// A bucket larger than a block's shared memory (keys that crowd on one high
+// word, or, rarely, an unlucky sample): the block collects its members in
+// index order from all particles, then sorts them in place by the 64-bit
+// pattern with stable 8-bit passes (sort_run_block's, over both words),
+// passes whose digit is the same for all members left out.
+template <typename R, int TH>
+__device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, uint32_t key_lo,
+                                                uint32_t key_hi, bool last, uint32_t* val,
+                                                uint32_t* tmp, int64_t len, uint32_t* scratch) {
+    constexpr int NW = TH / 32;
+    uint32_t (*s_cnt)[256] = reinterpret_cast<uint32_t (*)[256]>(scratch);   // [NW][256]
+    uint32_t* s_off = scratch + NW * 256;                                    // [256]
+    uint32_t* s_wsum = s_off + 256;                                          // [NW]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t found = 0;
+    for (int64_t c0 = 0; c0 < N; c0 += TH) {
+        bool mine = false;
+        if (c0 + tid < N) {
+            const uint32_t k = sort_key<R>(ld4(posm + c0 + tid));
+            mine = k >= key_lo && (last || k < key_hi);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, mine);
+        if (lane == 0) s_wsum[warp] = (uint32_t)__popc(bal);
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+        for (int w = 0; w < NW; ++w) {
+            if (w < warp) before += s_wsum[w];
+            total += s_wsum[w];
+        }
+        const int64_t pos = found + before + __popc(bal & ((1u << lane) - 1u));
+        if (mine && pos < len) val[pos] = (uint32_t)(c0 + tid);
+        found += total;
+        __syncthreads();
+    }
+    auto digit = [&](uint32_t i, int shift) -> uint32_t {
+        const uint64_t b = (int64_t)i < N ? r2_bits(ld4(posm + i)) : ~uint64_t(0);
+        return (uint32_t)(b >> shift) & 255u;
+    };
+    uint32_t *src = val, *dst = tmp;
+    for (int pass = 0; pass < 8; ++pass) {
+        const int shift = 8 * pass;
+        for (int i = tid; i < NW * 256; i += TH) (&s_cnt[0][0])[i] = 0u;
+        __syncthreads();
+        for (int64_t i = tid; i < len; i += TH) atomicAdd(&s_cnt[0][digit(src[i], shift)], 1u);
+        __syncthreads();
+        const uint32_t c = tid < 256 ? s_cnt[0][tid] : 0u;
+        if (__syncthreads_or(tid < 256 && (int64_t)c == len)) continue;   // one digit only
+        uint32_t x = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += t;
+        }
+        if (lane == 31) s_wsum[warp] = x;
+        __syncthreads();
+        if (tid < 256) {
+            uint32_t b = 0;
+            for (int w = 0; w < warp; ++w) b += s_wsum[w];
+            s_off[tid] = b + x - c;
+            s_cnt[0][tid] = 0u;
+        }
+        __syncthreads();
+        for (int64_t c0 = 0; c0 < len; c0 += TH) {
+            const bool valid = c0 + tid < len;
+            const uint32_t v = valid ? src[c0 + tid] : 0u;
+            const uint32_t d = valid ? digit(v, shift) : 256u;
+            const unsigned vb = __ballot_sync(0xffffffffu, valid);
+            unsigned mask = valid ? vb : ~vb;
+#pragma unroll
+            for (int bit = 0; bit < 8; ++bit) {
+                const bool on = (d >> bit) & 1u;
+                const unsigned bal = __ballot_sync(0xffffffffu, on);
+                mask &= on ? bal : ~bal;
+            }
+            const unsigned lower = mask & ((1u << lane) - 1u);
+            if (valid && lower == 0u) s_cnt[warp][d] = (uint32_t)__popc(mask);
+            __syncthreads();
+            uint32_t total = 0;   // thread = digit: exclusive prefix over the warps
+            if (tid < 256)
+                for (int w = 0; w < NW; ++w) {
+                    const uint32_t t = s_cnt[w][tid];
+                    s_cnt[w][tid] = total;
+                    total += t;
+                }
+            __syncthreads();
+            if (valid) dst[s_off[d] + s_cnt[warp][d] + (uint32_t)__popc(lower)] = v;
+            __syncthreads();
+            if (tid < 256) {
+                s_off[tid] += total;
+                for (int w = 0; w < NW; ++w) s_cnt[w][tid] = 0u;
+            }
+            __syncthreads();
+        }
+        uint32_t* t = src;
+        src = dst;
+        dst = t;
+    }
+    if (src != val) {
+        for (int64_t i = tid; i < len; i += TH) val[i] = src[i];
+        __syncthreads();
+    }
+}
+
+// One block per bucket: its place in the order from the bucket sizes, the sort
+// of its members by (64-bit pattern of r^2, index), the order and (sorted not
+// null) the particles.  nbuckets == 1: the particles 0..N-1 themselves (at
+// most TH kBucketKpt), no partition before.
+// The members are sorted by the high word of the pattern (the cheap 32-bit
+// key); the low word is evaluated only for members that share their high word
+// with another one (a few in a hundred), collected first so that whole warps
+// do it.
+template <typename R, int TH>
+__global__ void __launch_bounds__(TH)
+bucket_sort_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets,
+                   const uint32_t* splitters, const uint32_t* sizes, const uint32_t* region,
+                   uint32_t* perm, uint32_t* tmp, Vec4<R>* __restrict__ sorted, unsigned* err) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    constexpr int KPT = kBucketKpt;
+    using Sort = BlockSort<TH, KPT>;
+    constexpr int CAP = Sort::CAP;
+    __shared__ uint32_t s_base[TH / 32];
+    __shared__ int s_ntie;
+    pdl_wait();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
+    int64_t base = 0, len = N;
+    if (tid == 0) s_ntie = 0;
+    if (nbuckets > 1) {
+        uint32_t before = 0;
+        for (int i = tid; i < b; i += TH) before += __ldcg(sizes + i);
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0) s_base[warp] = before;
+        len = __ldcg(sizes + b);
+        __syncthreads();
+        base = __reduce_add_sync(0xffffffffu, lane < TH / 32 ? s_base[lane] : 0u);
+        if (base > N) base = N;   // (the sizes add up to N)
+        if (base + len > N) len = N - base;
+    }
+    if (len == 0) return;
+    if (len > CAP) {
+        sort_bucket_global<R, TH>(posm, N, __ldcg(splitters + b),
+                                  b + 1 < nbuckets ? __ldcg(splitters + b + 1) : 0u,
+                                  b + 1 == nbuckets, perm + base, tmp + base, len,
+                                  reinterpret_cast<uint32_t*>(sort_smem));
+        if (sorted)
+            for (int64_t i = tid; i < len; i += TH)
+                st4(sorted + base + i, gather_particle<R>(posm, perm[base + i], N, err));
+        return;
+    }
+    const int n = (int)len;
+    Sort sort(sort_smem);
+    {
+        uint32_t k[KPT], id[KPT];
+#pragma unroll
+        for (int s = 0; s < KPT; ++s) {
+            const int i = tid + s * TH;
+            if (i < n) id[s] = nbuckets > 1 ? __ldcg(region + (size_t)b * CAP + i) : (uint32_t)i;
+        }
+#pragma unroll
+        for (int s = 0; s < KPT; ++s)
+            if (tid + s * TH < n)
+                k[s] = (int64_t)id[s] < N ? sort_key<R>(ld4(posm + id[s])) : 0xffffffffu;
+        sort.place(k, id, nullptr, n);
+    }
+    auto low_word = [&](uint32_t i) -> uint32_t {
+        return (int64_t)i < N ? (uint32_t)r2_bits(ld4(posm + i)) : 0xffffffffu;
+    };
+    if (sort.crowded) {
+        for (int p = tid; p < n; p += TH) sort.s_low[p] = low_word(sort.s_id[p]);
+        __syncthreads();
+        sort.bitonic();
+        for (int p = tid; p < n; p += TH) {
+            const uint32_t i = sort.s_id[p];
+            perm[base + p] = i;
+            if (sorted) st4(sorted + base + p, gather_particle<R>(posm, i, N, err));
+        }
+        return;
+    }
+    // a pair's place is the start of its bin plus the smaller ones in it; those
+    // with an equal key in the bin go to the list, get their low words and are
+    // placed by all of (key, low word, index)
+    uint16_t* s_tie = reinterpret_cast<uint16_t*>(sort.s_bin + Sort::NB);
+    auto put = [&](int r, uint32_t i) {
+        perm[base + r] = i;
+        if (sorted) st4(sorted + base + r, gather_particle<R>(posm, i, N, err));
+    };
+    for (int p = tid; p < n; p += TH) {
+        const uint32_t key = sort.s_key[p];
+        int s, e;
+        sort.bin_range(key, s, e);
+        int r = s, same = 0;
+        for (int j = s; j < e; ++j) {
+            r += sort.s_key[j] < key;
+            same += sort.s_key[j] == key;
+        }
+        if (same > 1) s_tie[atomicAdd(&s_ntie, 1)] = (uint16_t)p;
+        else put(r, sort.s_id[p]);
+    }
+    __syncthreads();
+    const int ntie = s_ntie;
+    for (int q = tid; q < ntie; q += TH) sort.s_low[s_tie[q]] = low_word(sort.s_id[s_tie[q]]);
+    __syncthreads();
+    for (int q = tid; q < ntie; q += TH) {
+        const int p = s_tie[q];
+        const uint32_t key = sort.s_key[p], low = sort.s_low[p], id = sort.s_id[p];
+        int s, e;
+        sort.bin_range(key, s, e);
+        int r = s;
+        for (int j = s; j < e; ++j) {
+            const uint32_t kj = sort.s_key[j];
+            r += kj < key || (kj == key && (sort.s_low[j] < low || (sort.s_low[j] == low && sort.s_id[j] < id)));
+        }
+        put(r, id);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -615,10 +1204,12 @@ SortBuffers sort_buffers(void* ws, int64_t N, size_t* total) {
         return q;
     };
     const size_t n4 = (size_t)(N > 0 ? N : 1) * 4;
-    b.keys_a = reinterpret_cast<uint32_t*>(take(n4));
-    b.keys_b = reinterpret_cast<uint32_t*>(take(n4));
     b.vals_a = reinterpret_cast<uint32_t*>(take(n4));
     b.vals_b = reinterpret_cast<uint32_t*>(take(n4));
+    // the two paths' own buffers lie over each other
+    const size_t shared = off;
+    b.keys_a = reinterpret_cast<uint32_t*>(take(n4));
+    b.keys_b = reinterpret_cast<uint32_t*>(take(n4));
     const size_t nst = (size_t)sort_tiles(N);
     b.zero_bytes = (4 * 256 + 4 * (nst + kStatusPad) * 256 + 64) * 4;
     b.zero_bytes = (b.zero_bytes + 255) / 256 * 256;
@@ -627,18 +1218,94 @@ SortBuffers sort_buffers(void* ws, int64_t N, size_t* total) {
     b.status = b.hist ? b.hist + 4 * 256 : nullptr;
     b.counters = b.status ? b.status + 4 * (nst + kStatusPad) * 256 : nullptr;
     b.zero_base = z;
+    const size_t radix_end = off;
+    off = shared;
+    const SamplePlan sp = sample_plan(N);
+    if (sp.nbuckets > 1) {
+        b.region = reinterpret_cast<uint32_t*>(take((size_t)sp.nbuckets * sp.cap * 4));
+        b.splitters = reinterpret_cast<uint32_t*>(take(kMaxBuckets * 4));
+        b.part = reinterpret_cast<uint32_t*>(take((kPartHeader + kMaxBuckets) * 4));
+    }
+    if (radix_end > off) off = radix_end;
     if (total) *total = off;
     return b;
 }
 
+// dynamic shared memory above 48 KB: allowed once per kernel and device.  The
+// carve-out is left alone: a larger one for a third resident block of the
+// bucket sort costs its second gather the L1 cache (MEX at 2^20: 158 -> 170 us)
+template <typename K>
+static int allow_smem(K kernel, std::atomic<uint64_t>& done, size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev)) return ETICS_ERR_CUDA;
+    const uint64_t bit = uint64_t(1) << (dev & 63);
+    if (done.load() & bit) return ETICS_OK;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))
+        return ETICS_ERR_CUDA;
+    done.fetch_or(bit);
+    return ETICS_OK;
+}
+
+template <typename R, int KPT>
+static int launch_partition(const Vec4<R>* pp, int64_t N, const SamplePlan& sp,
+                            const SortBuffers& b, const LaunchCtx& ctx) {
+    static std::atomic<uint64_t> done{0};
+    auto k = partition_kernel<R, KPT>;
+    constexpr size_t smem = SplitterSort::kSmem;
+    if (allow_smem(k, done, smem)) return ETICS_ERR_CUDA;
+    if (cudaMemsetAsync(b.part, 0, (kPartHeader + sp.nbuckets) * 4, ctx.stream)) return ETICS_ERR_CUDA;
+    const uint64_t stride = ((uint64_t)N << 32) / (uint64_t)(kOversample * sp.nbuckets);
+    if (launch_pdl(k, dim3(sp.ntiles + 1), dim3(kPartThreads), smem, ctx.stream, pp, N, sp.nbuckets,
+                   sp.cap, stride, b.splitters, b.part, b.region,
+                   ctx.wait_limit > 0 ? ctx.wait_limit : kSpinLimit, ctx.err))
+        return ETICS_ERR_CUDA;
+    ++*ctx.launches;
+    return ETICS_OK;
+}
+
+template <typename R, int CAP>
+static int launch_buckets(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, const SortBuffers& b,
+                          Vec4<R>* sorted, const LaunchCtx& ctx) {
+    static std::atomic<uint64_t> done{0};
+    constexpr int TH = CAP / kBucketKpt;
+    constexpr size_t smem = BlockSort<TH, kBucketKpt>::kSmem;
+    auto k = bucket_sort_kernel<R, TH>;
+    if (allow_smem(k, done, smem)) return ETICS_ERR_CUDA;
+    if (launch_pdl(k, dim3(sp.nbuckets), dim3(TH), smem, ctx.stream, pp, N, sp.nbuckets,
+                   (const uint32_t*)b.splitters,
+                   (const uint32_t*)(b.part ? b.part + kPartHeader : nullptr),
+                   (const uint32_t*)b.region, b.vals_a, b.vals_b, sorted, ctx.err))
+        return ETICS_ERR_CUDA;
+    ++*ctx.launches;
+    return ETICS_OK;
+}
+
 template <typename R>
-int radial_sort_impl(const void* posm, int64_t N, const SortBuffers& b, const LaunchCtx& ctx) {
+static int sample_sort(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, const SortBuffers& b,
+                       Vec4<R>* sorted, const LaunchCtx& ctx) {
+    if (sp.nbuckets > 1) {
+        const int rc = sp.kpt == 2   ? launch_partition<R, 2>(pp, N, sp, b, ctx)
+                       : sp.kpt == 4 ? launch_partition<R, 4>(pp, N, sp, b, ctx)
+                                     : launch_partition<R, 8>(pp, N, sp, b, ctx);
+        if (rc) return rc;
+    }
+    stage_event(ctx, 1);
+    return sp.cap == kBucketSmall ? launch_buckets<R, kBucketSmall>(pp, N, sp, b, sorted, ctx)
+                                  : launch_buckets<R, kBucketLarge>(pp, N, sp, b, sorted, ctx);
+}
+
+template <typename R>
+int radial_sort_impl(const void* posm, int64_t N, const SortBuffers& b, void* sorted,
+                     const LaunchCtx& ctx) {
+    const Vec4<R>* pp = reinterpret_cast<const Vec4<R>*>(posm);
+    Vec4<R>* sp_out = reinterpret_cast<Vec4<R>*>(sorted);
+    const SamplePlan sp = sample_plan(N);
+    if (sp.nbuckets > 0) return sample_sort<R>(pp, N, sp, b, sp_out, ctx);
     if (cudaMemsetAsync(b.zero_base, 0, b.zero_bytes, ctx.stream)) return ETICS_ERR_CUDA;
     // few, long-lived blocks: each zeroes and merges 8 private histograms
     int kg = (int)((N + 256 * kKeygenIlp - 1) / (256 * kKeygenIlp));
     if (kg > ctx.num_sms * 2) kg = ctx.num_sms * 2;
-    keygen_kernel<R><<<kg, 256, 0, ctx.stream>>>(reinterpret_cast<const Vec4<R>*>(posm), N,
-                                                  b.keys_a, b.hist, ctx.err);
+    keygen_kernel<R><<<kg, 256, 0, ctx.stream>>>(pp, N, b.keys_a, b.hist, ctx.err);
     if (cudaGetLastError()) return ETICS_ERR_CUDA;
     ++*ctx.launches;
     stage_event(ctx, 1);
@@ -660,10 +1327,15 @@ int radial_sort_impl(const void* posm, int64_t N, const SortBuffers& b, const La
     // after 4 passes the sorted keys/values are back in keys_a / vals_a
     const int fg = (int)((N + kFixTile - 1) / kFixTile);
     if (launch_pdl(tie_fixup_kernel<R>, dim3(fg), dim3(kFixThreads), 0, ctx.stream,
-                   (const uint32_t*)b.keys_a, reinterpret_cast<const Vec4<R>*>(posm), b.vals_a,
-                   b.vals_b, N, ctx.err))
+                   (const uint32_t*)b.keys_a, pp, b.vals_a, b.vals_b, N, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
+    if (sp_out) {
+        if (launch_pdl(gather_kernel<R>, dim3((unsigned)((N + 255) / 256)), dim3(256), 0, ctx.stream,
+                       pp, (const uint32_t*)b.vals_a, N, sp_out, ctx.err))
+            return ETICS_ERR_CUDA;
+        ++*ctx.launches;
+    }
     return ETICS_OK;
 }
 
@@ -698,7 +1370,9 @@ int lookback_timeout_probe(void* ws, int64_t spins, const LaunchCtx& ctx) {
     return ETICS_OK;
 }
 
-template int radial_sort_impl<float>(const void*, int64_t, const SortBuffers&, const LaunchCtx&);
-template int radial_sort_impl<double>(const void*, int64_t, const SortBuffers&, const LaunchCtx&);
+template int radial_sort_impl<float>(const void*, int64_t, const SortBuffers&, void*,
+                                     const LaunchCtx&);
+template int radial_sort_impl<double>(const void*, int64_t, const SortBuffers&, void*,
+                                      const LaunchCtx&);
 
 }  // namespace etics

@@ -33,3 +33,32 @@ def test_mex_tile_edges(precision, l_max):
         o = etics.mex_field(device_particles(pm, precision), l_max).cpu().numpy()
         etics.check_error()
         close(o, acc, pot, precision, (n, l_max))
+
+
+def order_of(pm):
+    x = pm[:, :3]
+    r2 = (x[:, 0] * x[:, 0] + x[:, 1] * x[:, 1]) + x[:, 2] * x[:, 2]
+    return np.lexsort((np.arange(len(x)), r2))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_radial_order_across_the_sort_paths(precision):
+    """The order is exact on both sides of every line the sort draws by size:
+    one block up to 8192, buckets of mean 1024 up to 2^20 and of mean 2048 up
+    to 2^21, the radix passes above; particles already in radial order, in two
+    interleaved populations, and with one radius crowding (more equal keys
+    than a bucket or a bin holds)."""
+    rng = np.random.default_rng(3)
+    for n in (1023, 8191, 8192, 8193, 9217, (1 << 18) + 1, (1 << 20) + 1, (1 << 21) + 1):
+        pm = hernquist(n, seed=5)
+        if n == 8193:
+            pm = pm[order_of(pm)]                      # sorted already
+        if n == 9217:
+            pm[::2, :3] *= 1e-3                        # two interleaved populations
+        if n == (1 << 18) + 1:
+            u = rng.normal(size=(20000, 3))            # a shell: r^2 within a few ulps of 4
+            pm[1000:21000, :3] = 2.0 * u / np.linalg.norm(u, axis=1, keepdims=True)
+            pm[30000:30300, :3] = pm[30000, :3]        # one point, 300 times
+        got = etics.radial_order(device_particles(pm, precision)).cpu().numpy()
+        etics.check_error()
+        assert np.array_equal(got, order_of(rounded(pm, precision))), n
