@@ -125,8 +125,10 @@ int etics_scf_field(const void* posm, int64_t N, int n_max, int l_max, int preci
     if (rc) return rc;
     etics::stage_event(h.ctx, 0);
     rc = precision == ETICS_MIXED
-             ? etics::scf_field_f32(posm, N, n_max, l_max, coeffs, accpot, out_mask, h.ctx)
-             : etics::scf_field_f64(posm, N, n_max, l_max, coeffs, accpot, out_mask, h.ctx);
+             ? etics::scf_field_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, coeffs, accpot, out_mask,
+                                    {}, h.ctx)
+             : etics::scf_field_f64(posm, N, n_max, l_max, ETICS_BASIS_HO, coeffs, accpot, out_mask,
+                                    {}, h.ctx);
     etics::stage_event(h.ctx, 1);
     return rc;
 }
@@ -173,8 +175,9 @@ int etics_scf_field_basis(const void* posm, int64_t N, int n_max, int l_max, int
     if (rc) return rc;
     etics::stage_event(h.ctx, 0);
     rc = precision == ETICS_MIXED
-             ? etics::scf_field_cb_f32(posm, N, n_max, l_max, coeffs, accpot, out_mask, h.ctx)
-             : etics::scf_field_cb_f64(posm, N, n_max, l_max, coeffs, accpot, out_mask, h.ctx);
+             ? etics::scf_field_f32(posm, N, n_max, l_max, basis, coeffs, accpot, out_mask, {}, h.ctx)
+             : etics::scf_field_f64(posm, N, n_max, l_max, basis, coeffs, accpot, out_mask, {},
+                                    h.ctx);
     etics::stage_event(h.ctx, 1);
     return rc;
 }
@@ -250,8 +253,12 @@ int etics_leapfrog_step(void* posm, void* vel, void* accpot, int64_t N, double d
         rc = mixed ? etics::scf_coeffs_f32(posm, N, n_max, l_max, c, ws, h.ctx)
                    : etics::scf_coeffs_f64(posm, N, n_max, l_max, c, ws, h.ctx);
         if (rc) return rc;
-        rc = mixed ? etics::scf_field_f32(posm, N, n_max, l_max, c, accpot, 3, h.ctx)
-                   : etics::scf_field_f64(posm, N, n_max, l_max, c, accpot, 3, h.ctx);
+        // the field pass does the second kick with the acceleration at hand
+        const etics::FieldKick kick{vel, 0.5 * (mixed ? (double)(float)dt : dt)};
+        return mixed ? etics::scf_field_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, c, accpot, 3,
+                                            kick, h.ctx)
+                     : etics::scf_field_f64(posm, N, n_max, l_max, ETICS_BASIS_HO, c, accpot, 3,
+                                            kick, h.ctx);
     } else {
         rc = mixed ? etics::mex_field_f32(posm, N, l_max, accpot, 3, ws, h.ctx)
                    : etics::mex_field_f64(posm, N, l_max, accpot, 3, ws, h.ctx);
@@ -276,11 +283,11 @@ int etics_leapfrog_step_coeffs(void* posm, void* vel, void* accpot, int64_t N, d
     rc = mixed ? etics::kick_drift_f32(posm, vel, accpot, N, dt, h.ctx)
                : etics::kick_drift_f64(posm, vel, accpot, N, dt, h.ctx);
     if (rc) return rc;
-    rc = mixed ? etics::scf_field_f32(posm, N, n_max, l_max, coeffs, accpot, 3, h.ctx)
-               : etics::scf_field_f64(posm, N, n_max, l_max, coeffs, accpot, 3, h.ctx);
-    if (rc) return rc;
-    return mixed ? etics::kick_f32(vel, accpot, N, dt, h.ctx)
-                 : etics::kick_f64(vel, accpot, N, dt, h.ctx);
+    const etics::FieldKick kick{vel, 0.5 * (mixed ? (double)(float)dt : dt)};
+    return mixed ? etics::scf_field_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, coeffs, accpot, 3,
+                                        kick, h.ctx)
+                 : etics::scf_field_f64(posm, N, n_max, l_max, ETICS_BASIS_HO, coeffs, accpot, 3,
+                                        kick, h.ctx);
 }
 
 // ---- coefficient-forecasting MLP ---------------------------------------------

@@ -21,6 +21,7 @@
 // tuning parameters (etics_batch_tuning) chosen by the autotuner.
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "etics_batch_layout.h"
@@ -492,11 +493,18 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
 // ---------------------------------------------------------------------------
 // 3. field: one work item (a chunk of one instance) per block iteration
 // ---------------------------------------------------------------------------
-template <typename R, bool ACC>
-__global__ void __launch_bounds__(256)
-batch_field_kernel(const Vec4<R>* __restrict__ posm, const void* __restrict__ plan,
-                   const double* __restrict__ coeffs, Vec4<R>* __restrict__ out, int out_mask,
-                 unsigned* err) {
+// (three blocks of 128 threads per SM at 168 registers: with one of 256 the
+// kernel takes 210 registers and leaves 8 warps per SM.  256 systems, 17
+// million particles: 1300 us with one particle per thread, 1200 with two and
+// 256 threads, 1160 so.)
+constexpr int kBatchFieldThreads = 128;
+template <typename P, bool ACC>
+__global__ void __launch_bounds__(kBatchFieldThreads, 3)
+batch_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm,
+                   const void* __restrict__ plan, const double* coeffs,
+                   Vec4<typename FieldLane<P>::R>* __restrict__ out, int out_mask, unsigned* err) {
+    using R = typename FieldLane<P>::R;
+    constexpr int NP = FieldLane<P>::kParticles;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* cs = reinterpret_cast<R*>(smem_raw);
     const BatchHeader hd = *plan_table<BatchHeader>(plan, 0);
@@ -506,52 +514,29 @@ batch_field_kernel(const Vec4<R>* __restrict__ posm, const void* __restrict__ pl
         const BatchField it = items[w];
         const BatchInst in = insts[it.inst];
         const int ncols = col_total(in.l_max);
-        const int nj = (in.l_max + 1) * (in.l_max + 1);
         __syncthreads();
         for (int e = threadIdx.x; e < (in.n_max + 1) * ncols; e += blockDim.x) {
             const int n = e / ncols;
-            int c = e % ncols, l = 0;
-            while (c >= ncol_pad(l)) { c -= ncol_pad(l); ++l; }
-            R v = R(0);
-            if (c < 2 * l + 1) {
-                const int m = (c == 0) ? 0 : ((c & 1) ? (c + 1) / 2 : -(c / 2));
-                const int am = m < 0 ? -m : m;
-                v = (R)(coeffs[in.coef_offset + (int64_t)n * nj + l * l + l + m] *
-                        c_tab.knorm[l * (l + 1) / 2 + am] * geg_gamma(0, l, n));
-            }
-            cs[e] = v;
+            cs[e] = field_coeff<R>(coeffs + in.coef_offset, ETICS_BASIS_HO, n, e - n * ncols, in.l_max);
         }
         __syncthreads();
-        for (int k = threadIdx.x; k < it.count; k += blockDim.x) {
+        for (int k = threadIdx.x * NP; k < it.count; k += blockDim.x * NP) {
             const int64_t i = in.offset + it.begin + k;
-            const Vec4<R> pv = ld4(posm + i);
-            if (!finite4(pv.x, pv.y, pv.z, pv.w)) report(err, ETICS_ERR_NONFINITE);
-            FieldEval<R, kBatchLM, ACC, 0> f;
-            const R r = sqrt(pv.x * pv.x + pv.y * pv.y + pv.z * pv.z);
-            const R inv = r > R(0) ? R(1) / r : R(0);
-            f.ux = pv.x * inv; f.uy = pv.y * inv; f.uz = pv.z * inv;
-            f.uu = f.ux * f.ux + f.uy * f.uy + f.uz * f.uz;
-            f.t = R(1) / (R(1) + r);
-            f.st = r * f.t * f.t;
-            f.xi = R(1) - R(2) * f.t;
-            f.dxdr = R(2) * f.t * f.t;
-            f.pre = -f.t;
-            f.preR = -f.t * f.t * f.t;
-            f.pot = f.gr = f.gx = f.gy = f.gz = R(0);
-            f.cs = cs;
-            f.ncols = ncols;
-            f.n_max = in.n_max;
-            f.l_max = in.l_max;
-            f.template level<0>();
-            R ax = R(0), ay = R(0), az = R(0);
-            if (ACC) {
-                ax = -(f.gr * f.ux + f.gx);
-                ay = -(f.gr * f.uy + f.gy);
-                az = -(f.gr * f.uz + f.gz);
+            Vec4<R> pv[NP], res[NP];
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                pv[j] = k + j < it.count ? ld4(posm + i + j) : mk4<R>(R(0), R(0), R(0), R(0));
+                if (!finite4(pv[j].x, pv[j].y, pv[j].z, pv[j].w)) report(err, ETICS_ERR_NONFINITE);
             }
-            const R pot = (out_mask & ETICS_OUT_POT) ? f.pot : R(0);
-            if (!finite4(ax, ay, az, pot)) report(err, ETICS_ERR_NONFINITE);
-            st4(out + i, mk4<R>(ax, ay, az, pot));
+            field_eval<P, kBatchLM, ACC, 0, 0>(pv, cs, ncols, in.n_max, in.l_max, ~0u, res);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                if (k + j >= it.count) continue;
+                if (!(out_mask & ETICS_OUT_POT)) res[j].w = R(0);
+                if (!finite4(res[j].x, res[j].y, res[j].z, res[j].w))
+                    report(err, ETICS_ERR_NONFINITE);
+                st4(out + i + j, res[j]);
+            }
         }
     }
 }
@@ -805,22 +790,24 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
     }
     stage_event(ctx, 2);
     if (out && hd.nfield > 0) {
+        using FieldP = std::conditional_t<sizeof(R) == 4, float2, double>;
         const size_t smem = (size_t)(kBatchNR) * col_total(kBatchLM) * sizeof(R);
         int grid = hd.nfield < ctx.num_sms * 8 ? hd.nfield : ctx.num_sms * 8;
+        const int threads = std::min(hd.field_threads, kBatchFieldThreads);
         if (out_mask & ETICS_OUT_ACC) {
-            auto k = batch_field_kernel<R, true>;
+            auto k = batch_field_kernel<FieldP, true>;
             if (smem > 48 * 1024 &&
                 cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
                 return ETICS_ERR_CUDA;
-            k<<<grid, hd.field_threads, smem, ctx.stream>>>(
+            k<<<grid, threads, smem, ctx.stream>>>(
                 reinterpret_cast<const Vec4<R>*>(posm), plan_dev, coeffs,
                 reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err);
         } else {
-            auto k = batch_field_kernel<R, false>;
+            auto k = batch_field_kernel<FieldP, false>;
             if (smem > 48 * 1024 &&
                 cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
                 return ETICS_ERR_CUDA;
-            k<<<grid, hd.field_threads, smem, ctx.stream>>>(
+            k<<<grid, threads, smem, ctx.stream>>>(
                 reinterpret_cast<const Vec4<R>*>(posm), plan_dev, coeffs,
                 reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err);
         }

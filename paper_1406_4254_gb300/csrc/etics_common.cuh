@@ -207,6 +207,10 @@ template <typename R, int B = 0> __device__ __forceinline__ R geg_bs(int l, int 
     if constexpr (sizeof(R) == 4) return c_tab.gbs_f[B][l][n];
     else return c_tab.gbs_d[B][l][n];
 }
+template <typename R> __device__ __forceinline__ R geg_bs_of(int basis, int l, int n) {
+    if constexpr (sizeof(R) == 4) return c_tab.gbs_f[basis][l][n];
+    else return c_tab.gbs_d[basis][l][n];
+}
 __device__ __forceinline__ double geg_gamma(int basis, int l, int n) { return c_tab.ggam[basis][l][n]; }
 __device__ __forceinline__ double inv_j_of(int basis, int n, int l) {
     return basis == 0 ? c_tab.inv_j[n][l] : c_tab.inv_j_cb[n][l];

@@ -1,0 +1,12 @@
+// etics_field_f32_ho_low.cu -- the SCF field pass (etics_scf_field.cuh),
+// mixed precision, Hernquist-Ostriker basis (paper Sec. 2.5), l_max <= 6: its own translation unit so that
+// the instantiations compile in parallel.
+#include "etics_scf_field.cuh"
+
+namespace etics {
+int scf_field_f32_ho_low(const void* posm, int64_t N, int n_max, int l_max,
+                          const double* coeffs, void* out, int out_mask, FieldKick kick,
+                          const LaunchCtx& ctx) {
+    return scf_field_low<float2, 0>(posm, N, n_max, l_max, coeffs, out, out_mask, kick, ctx);
+}
+}  // namespace etics

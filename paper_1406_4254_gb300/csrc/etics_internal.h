@@ -21,20 +21,34 @@ int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, double* co
                    const LaunchCtx& ctx);
 int scf_coeffs_f64(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
                    const LaunchCtx& ctx);
-int scf_field_f32(const void* posm, int64_t N, int n_max, int l_max, const double* coeffs,
-                  void* out, int out_mask, const LaunchCtx& ctx);
-int scf_field_f64(const void* posm, int64_t N, int n_max, int l_max, const double* coeffs,
-                  void* out, int out_mask, const LaunchCtx& ctx);
+
+// field pass, basis ETICS_BASIS_HO or ETICS_BASIS_CB; kick: the second kick
+// of a leapfrog step, v += factor a, done along with it (vel null: none)
+struct FieldKick { void* vel; double factor; };
+int scf_field_f32(const void* posm, int64_t N, int n_max, int l_max, int basis,
+                  const double* coeffs, void* out, int out_mask, FieldKick kick,
+                  const LaunchCtx& ctx);
+int scf_field_f64(const void* posm, int64_t N, int n_max, int l_max, int basis,
+                  const double* coeffs, void* out, int out_mask, FieldKick kick,
+                  const LaunchCtx& ctx);
+#define ETICS_FIELD_PART(name)                                                          \
+    int name(const void* posm, int64_t N, int n_max, int l_max, const double* coeffs, void* out, \
+             int out_mask, FieldKick kick, const LaunchCtx& ctx)
+ETICS_FIELD_PART(scf_field_f32_ho_low);
+ETICS_FIELD_PART(scf_field_f32_ho_high);
+ETICS_FIELD_PART(scf_field_f32_cb_low);
+ETICS_FIELD_PART(scf_field_f32_cb_high);
+ETICS_FIELD_PART(scf_field_f64_ho_low);
+ETICS_FIELD_PART(scf_field_f64_ho_high);
+ETICS_FIELD_PART(scf_field_f64_cb_low);
+ETICS_FIELD_PART(scf_field_f64_cb_high);
+#undef ETICS_FIELD_PART
 
 // ---- SCF with the Clutton-Brock radial basis (etics_scf_cb_f32/f64.cu) ------
 int scf_coeffs_cb_f32(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
                       const LaunchCtx& ctx);
 int scf_coeffs_cb_f64(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
                       const LaunchCtx& ctx);
-int scf_field_cb_f32(const void* posm, int64_t N, int n_max, int l_max, const double* coeffs,
-                     void* out, int out_mask, const LaunchCtx& ctx);
-int scf_field_cb_f64(const void* posm, int64_t N, int n_max, int l_max, const double* coeffs,
-                     void* out, int out_mask, const LaunchCtx& ctx);
 
 // ---- radial sort (etics_sort.cu) -------------------------------------------
 struct SortBuffers {

@@ -33,20 +33,16 @@
 // l_max = 10 (the whole call): 291 -> 167 us; N = 100003, l_max = 6, FP64:
 // 450 -> 341 us (256-particle tiles also fill the SMs more evenly).
 //
-// Harmonics: R_lm(kappa u) = kappa^l Z_lm(u) / (l+m)! at the unit vector u,
-// with Z the unnormalised solid harmonics of etics_common.cuh and kappa = 8
-// (a power of two: the values stay near 1 up to l = 10 where Z alone or
-// Z / (l+m)! would spread over 2^60).  In this scaling the gradient ladder has
-// no constants:
-//   d/dz R_l^m = R_{l-1}^m,  (d/dx -+ i d/dy) R_l^m = +-R_{l-1}^{m-+1},
-// and the product of an evaluated and a summed harmonic needs the weight
-// (l-m)!(l+m)! kappa^-2l (twice that for m > 0: the twos are applied to the
-// sums over m > 0 as a whole).
+// Harmonics: the scaled ones of etics_pair.cuh, at kappa u.  The product of an
+// evaluated and a summed harmonic needs the weight (l-m)!(l+m)! kappa^-2l
+// (twice that for m > 0: the twos are applied to the sums over m > 0 as a
+// whole).
 #pragma once
 
 #include <atomic>
 
 #include "etics_internal.h"
+#include "etics_pair.cuh"
 
 namespace etics {
 
@@ -56,7 +52,6 @@ constexpr int kMexLB = kMexLmaxLimit;             // compiled level bound (10)
 constexpr int kMexNC = 49;                        // components of one level group, at most
 constexpr int kMexRow = kMexThreads + 4;          // row stride of the shared rows (conflict-free
                                                   // for 16-byte reads down a row)
-constexpr int kMexKappa = 8;
 
 // Level groups: the shared rows hold the components of one group of levels,
 // so that l_max up to kMexLB leaves room for several blocks per SM.  A group's
@@ -91,32 +86,6 @@ inline int mex_row_comps(int l_max) {
 
 inline int mex_tiles(int64_t N) { return (int)((N + kMexTile - 1) / kMexTile); }
 
-// ---- pairs ------------------------------------------------------------------
-// two particles of one thread: paired FP32 instructions, or two FP64 ones
-template <typename R> struct PairT;
-template <> struct PairT<float> { using type = float2; };
-template <> struct PairT<double> { using type = double2; };
-template <typename R> using Pair = typename PairT<R>::type;
-__device__ __forceinline__ float2 mk2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 mk2(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ double2 mul2(double2 a, double2 b) {
-    return make_double2(a.x * b.x, a.y * b.y);
-}
-__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
-    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
-__device__ __forceinline__ double2 add2(double2 a, double2 b) {
-    return make_double2(a.x + b.x, a.y + b.y);
-}
-// a constant in both halves: an immediate or broadcast operand, no extra
-// instruction (nor is the negation of an operand)
-template <typename R> __device__ __forceinline__ Pair<R> splat(R a) { return mk2(a, a); }
-template <typename P> __device__ __forceinline__ P neg2(P a) { return mk2(-a.x, -a.y); }
-template <typename P> __device__ __forceinline__ P sub2(P a, P b) { return add2(a, neg2(b)); }
-
 // (l-m)!(l+m)! kappa^-2l, the weight of component (l, m)
 struct MexWeights {
     double w[(kMexLB + 1) * (kMexLB + 2) / 2];
@@ -129,7 +98,7 @@ constexpr MexWeights make_mex_weights() {
             double v = 1.0;
             for (int k = 2; k <= l - m; ++k) v *= (double)k;
             for (int k = 2; k <= l + m; ++k) v *= (double)k;
-            for (int k = 0; k < l; ++k) v /= (double)(kMexKappa * kMexKappa);
+            for (int k = 0; k < l; ++k) v /= (double)(kKappa * kKappa);
             t.w[l * (l + 1) / 2 + m] = v;
             t.wf[l * (l + 1) / 2 + m] = (float)v;
         }
@@ -174,7 +143,7 @@ struct MexPair {
         const R ra = radius<R>(a.x, a.y, a.z), rb = radius<R>(b.x, b.y, b.z);
         // a particle at the origin: no direction, no outer moment, rho = 0
         const R ia = ra > R(0) ? R(1) / ra : R(0), ib = rb > R(0) ? R(1) / rb : R(0);
-        const R ka = R(kMexKappa) * ia, kb = R(kMexKappa) * ib;
+        const R ka = R(kKappa) * ia, kb = R(kKappa) * ib;
         x = mk2(a.x * ka, b.x * kb);
         y = mk2(a.y * ka, b.y * kb);
         z = mk2(a.z * ka, b.z * kb);
@@ -185,51 +154,14 @@ struct MexPair {
 };
 
 // The two walks over the levels (moments, field) and the walks of later level
-// groups evaluate the same harmonics; without this the compiler keeps the
-// first walk's values for the second, far more than the registers hold
-// (l_max > 6: 2 KB of spills per thread).
-__device__ __forceinline__ void opaque(float& v) { asm volatile("" : "+f"(v)); }
-__device__ __forceinline__ void opaque(double& v) { asm volatile("" : "+d"(v)); }
+// groups must not keep one another's harmonics (l_max > 6: 2 KB of spills per
+// thread without this).
 template <typename R> __device__ __forceinline__ void opaque_pair(MexPair<R>& p) {
     opaque(p.x.x); opaque(p.x.y);
     opaque(p.y.x); opaque(p.y.y);
     opaque(p.z.x); opaque(p.z.y);
     opaque(p.rho.x); opaque(p.rho.y);
     opaque(p.irho.x); opaque(p.irho.y);
-}
-
-// level L of R_lm(kappa u) from levels L-1 and L-2 (|kappa u|^2 = kappa^2)
-template <typename R, int L>
-__device__ __forceinline__ void mex_harm(const Pair<R>* C1, const Pair<R>* S1, const Pair<R>* C2,
-                                         const Pair<R>* S2, const MexPair<R>& p, Pair<R>* C,
-                                         Pair<R>* S) {
-    using P = Pair<R>;
-    if constexpr (L == 0) {
-        C[0] = splat(R(1));
-        S[0] = splat(R(0));
-    } else if constexpr (L == 1) {
-        C[0] = p.z;
-        S[0] = splat(R(0));
-        C[1] = mul2(p.x, splat(R(0.5)));
-        S[1] = mul2(p.y, splat(R(0.5)));
-    } else {
-        // kappa^2 = |kappa u|^2 taken out of the recursion:
-        //   (L^2 - m^2) R_L = kappa^2 [ (2L-1)/kappa^2 v_z R_{L-1} - R_{L-2} ]
-        constexpr R d = R(1.0 / (2 * L)), k2 = R(kMexKappa * kMexKappa);
-        const P xd = mul2(p.x, splat(d)), yd = mul2(p.y, splat(d));
-        C[L] = fma2(xd, C1[L - 1], neg2(mul2(yd, S1[L - 1])));
-        S[L] = fma2(xd, S1[L - 1], mul2(yd, C1[L - 1]));
-        C[L - 1] = mul2(p.z, C1[L - 1]);
-        S[L - 1] = mul2(p.z, S1[L - 1]);
-        S[0] = splat(R(0));
-        const P zl = mul2(p.z, splat(R(2 * L - 1) / k2));
-#pragma unroll
-        for (int m = 0; m + 2 <= L; ++m) {
-            const P f = splat(k2 / R(L * L - m * m));
-            C[m] = mul2(fma2(zl, C1[m], neg2(C2[m])), f);
-            if (m > 0) S[m] = mul2(fma2(zl, S1[m], neg2(S2[m])), f);
-        }
-    }
 }
 
 // moments of the pair summed, component c = l*l + 2m-1 (cos) / 2m (sin) of
@@ -242,7 +174,7 @@ __device__ __forceinline__ void mex_moments(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S
     if constexpr (L <= L1) {
         if (L > l_max) return;
         constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
-        mex_harm<R, L>(C[s1], S[s1], C[s2], S[s2], p, C[s0], S[s0]);
+        harm_scaled<R, L>(C[s1], S[s1], C[s2], S[s2], p.x, p.y, p.z, C[s0], S[s0]);
         if constexpr (L >= L0) {
             constexpr int o = L * L - L0 * L0;
 #pragma unroll
@@ -291,7 +223,7 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
     if constexpr (L <= L1) {
         if (L > l_max) return;
         constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
-        mex_harm<R, L>(C[s1], S[s1], C[s2], S[s2], p, C[s0], S[s0]);
+        harm_scaled<R, L>(C[s1], S[s1], C[s2], S[s2], p.x, p.y, p.z, C[s0], S[s0]);
         if constexpr (L >= L0) {
             constexpr int o = L * L - L0 * L0;
             if constexpr (L == 0) {
@@ -301,11 +233,11 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                 if (ACC) f.rad = mul2(q2, a);
             } else {
                 P ac[L + 1], as[L + 1];
-                P r0 = splat(R(0)), r1 = splat(R(0));
+                P r0 = splat<Pair<R>>(R(0)), r1 = splat<Pair<R>>(R(0));
 #pragma unroll
                 for (int m = 0; m <= L; ++m) {
                     const R w = mex_w<R>(L * (L + 1) / 2 + m);
-                    const P wm = mul2(own, splat(w));
+                    const P wm = mul2(own, splat<P>(w));
                     {
                         const int cc = o + (m == 0 ? 0 : 2 * m - 1);
                         const R q = col[cc * kMexRow], pp = col[(nc + cc) * kMexRow];
@@ -319,7 +251,7 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                             else r1 = fma2(qa, h, r1);
                         }
                     }
-                    as[m] = splat(R(0));
+                    as[m] = splat<Pair<R>>(R(0));
                     if (m > 0) {
                         const int cc = o + 2 * m;
                         const R q = col[cc * kMexRow], pp = col[(nc + cc) * kMexRow];
@@ -331,8 +263,8 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                     }
                 }
                 if (ACC) {
-                    f.rad = fma2(splat(R(2 * L + 1)), r0, f.rad);
-                    f.rad = fma2(splat(R(2 * (2 * L + 1))), r1, f.rad);
+                    f.rad = fma2(splat<Pair<R>>(R(2 * L + 1)), r0, f.rad);
+                    f.rad = fma2(splat<Pair<R>>(R(2 * (2 * L + 1))), r1, f.rad);
                     // gradient from the level below (the ladder regrouped by the
                     // harmonic it multiplies)
                     const P* C1 = C[s1];
@@ -368,7 +300,7 @@ __device__ __forceinline__ void mex_group_eval(const MexPair<R>& p, int l_max, c
                                                MexField<R>& f) {
     constexpr int L0 = mex_group_l0(G), L1 = mex_group_l1(G);
     Pair<R> C[3][L1 + 1], S[3][L1 + 1];
-    mex_eval<R, L0, L1, 0, ACC>(C, S, p, l_max, mul2(p.irho, p.irho), splat(R(1)),
+    mex_eval<R, L0, L1, 0, ACC>(C, S, p, l_max, mul2(p.irho, p.irho), splat<Pair<R>>(R(1)),
                                 mk2(p.m.x, p.m.y * p.irho.y), mk2(p.rho.x, p.irho.y), col, nc, f);
 }
 
@@ -621,7 +553,7 @@ mex_pass2_kernel(const Vec4<R>* __restrict__ sorted, const uint32_t* __restrict_
     MexPair<R> p;
     p.init(v[0], v[1], scale, ldexp(R(1), e));
     MexField<R> f;
-    const Pair<R> zero = splat(R(0));
+    const Pair<R> zero = splat<Pair<R>>(R(0));
     f.s0 = f.s1 = f.rad = f.vx = f.vy = f.vz0 = f.vz1 = f.pot0 = zero;
     const int ncomp = mex_layout_ncomp(l_max);
     for (int g = 0; g < NG; ++g) {
@@ -664,7 +596,7 @@ mex_pass2_kernel(const Vec4<R>* __restrict__ sorted, const uint32_t* __restrict_
         else mex_group_eval<R, 2, ACC>(p, l_max, rows + tid, nc, f);
     }
     const R s1 = scale, s2 = scale * scale;
-    const R two = R(2), kap = R(kMexKappa), ikap = R(1) / R(kMexKappa);
+    const R two = R(2), kap = R(kKappa), ikap = R(1) / R(kKappa);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         auto at = [&](const Pair<R>& q) { return j == 0 ? q.x : q.y; };

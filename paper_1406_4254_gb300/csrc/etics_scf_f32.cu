@@ -21,8 +21,13 @@ int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, double* co
     if (n_max == 14 && l_max == 8) return scf_coeffs_bins148_f32(posm, N, coeffs, ws, ctx);
     return scf_coeffs_launch<float>(posm, N, n_max, l_max, coeffs, ws, ctx);
 }
-int scf_field_f32(const void* posm, int64_t N, int n_max, int l_max, const double* coeffs,
-                  void* out, int out_mask, const LaunchCtx& ctx) {
-    return scf_field_launch<float>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
+int scf_field_f32(const void* posm, int64_t N, int n_max, int l_max, int basis,
+                  const double* coeffs, void* out, int out_mask, FieldKick kick,
+                  const LaunchCtx& ctx) {
+    if (N == 0) return ETICS_OK;
+    const auto run = basis == ETICS_BASIS_HO
+                         ? (l_max <= 6 ? scf_field_f32_ho_low : scf_field_f32_ho_high)
+                         : (l_max <= 6 ? scf_field_f32_cb_low : scf_field_f32_cb_high);
+    return run(posm, N, n_max, l_max, coeffs, out, out_mask, kick, ctx);
 }
 }  // namespace etics

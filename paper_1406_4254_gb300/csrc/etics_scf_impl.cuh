@@ -1,6 +1,6 @@
-// etics_scf_impl.cuh -- SCF coefficient and field kernels (templated on the
-// arithmetic type; instantiated for float in etics_scf_f32.cu and for double
-// in etics_scf_f64.cu).
+// etics_scf_impl.cuh -- SCF coefficient kernel (templated on the arithmetic
+// type; instantiated for float in etics_scf_f32.cu and for double in
+// etics_scf_f64.cu).  The field pass is in etics_scf_field.cuh.
 //
 // Method (paper Sec. 2.4 eq. 18, basis of Sec. 2.5, two passes of Sec. 3.3):
 //   c_nlm = (1/J_nl) sum_k m_k phi_nl(r_k) Y_lm(x_k)             (coefficients)
@@ -18,13 +18,9 @@
 //     shared load).  FP32 partial sums are flushed into per-block FP64
 //     accumulators every few tiles; per-block FP64 partials are summed in a
 //     fixed order by a finalize kernel (deterministic).
-//   * field pass: one thread per particle; coefficients (pre-multiplied by the
-//     harmonic normalisation) broadcast from shared memory; the gradient of
-//     phi_nl(r) Y_lm is built from the Cartesian gradient of the solid
-//     harmonic, which is regular on the z axis and at the origin.
 #pragma once
 
-#include "etics_common.cuh"
+#include "etics_scf_field.cuh"
 
 namespace etics {
 
@@ -37,7 +33,6 @@ template <> struct ScfCfg<double> {
     static constexpr int kThreads = 128;
     static constexpr int kTile = 64;
 };
-constexpr int kFieldThreads = 256;
 constexpr int kFlushTiles = 16;
 
 struct ScfCoeffParams {
@@ -52,12 +47,6 @@ struct ScfCoeffParams {
     unsigned* err;
 };
 
-__host__ __device__ constexpr int ncol_pad_c(int l) { return ((2 * l + 1 + 3) / 4) * 4; }
-__host__ __device__ constexpr int col_offset_c(int l) {
-    int o = 0;
-    for (int k = 0; k < l; ++k) o += ncol_pad_c(k);
-    return o;
-}
 __host__ __device__ inline int scf_items(int l_max) { return col_total(l_max) / 4; }
 
 // shared-memory bytes of the coefficient kernel
@@ -284,199 +273,6 @@ static __global__ void scf_finalize_kernel(const double* __restrict__ partial, i
 }
 
 // ---------------------------------------------------------------------------
-// field pass
-// ---------------------------------------------------------------------------
-// NM1 > 0: specialised for n_max + 1 == NM1 and l_max == LM (n loop unrolled,
-// coefficient row stride and recursion constants known at compile time);
-// NM1 == 0: generic, n_max and l_max <= LM at run time.
-template <typename R, int LM, bool ACC, int NM1, int BASIS = 0>
-struct FieldEval {
-    using V4 = Vec4<R>;
-    R C[3][LM + 1], S[3][LM + 1];
-    // t: the basis's tau (radial derivative factor), see RadialSeed
-    R ux, uy, uz, uu, t, xi, dxdr, st, pre, preR;
-    R pot, gr, gx, gy, gz;
-    const R* cs;
-    int ncols, n_max, l_max;
-
-    template <int L>
-    __device__ __forceinline__ void level() {
-        if constexpr (L <= LM) {
-            if (NM1 == 0 && L > l_max) return;
-            constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
-            harm_level<R, L>(C[s1], S[s1], C[s2], S[s2], ux, uy, uz, uu, C[s0], S[s0]);
-            constexpr int NC = 2 * L + 1;
-            constexpr int NQ = ncol_pad_c(L) / 4;
-            constexpr int CO = col_offset_c(L);
-            R A[NC], B[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) { A[c] = R(0); B[c] = R(0); }
-            // FP32: the column sums run as packed pairs (columns 2i, 2i+1:
-            // one paired FMA for two columns; the padded table has a zero
-            // partner for the last, odd column)
-            constexpr int NP = (NC + 1) / 2;
-            float2 A2[NP], B2[NP];
-#pragma unroll
-            for (int i = 0; i < NP; ++i) { A2[i] = make_float2(0.f, 0.f); B2[i] = make_float2(0.f, 0.f); }
-            R cm1 = R(0), cn = R(1), dm1 = R(0), dn = R(0);
-            constexpr int kStride = NM1 > 0 ? col_offset_c(LM + 1) : 0;
-            const int stride = NM1 > 0 ? kStride : ncols;
-            const int nlim = NM1 > 0 ? NM1 - 1 : n_max;
-            const R* row = cs + CO;
-#pragma unroll (NM1 > 0 ? NM1 : 4)
-            for (int n = 0; n <= nlim; ++n, row += stride) {
-                if (n > 0) {
-                    // rescaled polynomials (the table holds gam_n c_nlm)
-                    const R bs = geg_bs<R, BASIS>(L, n);
-                    const R cnew = fma(xi, cn, -bs * cm1);
-                    if (ACC) {
-                        const R dnew = fma(-bs, dm1, fma(xi, dn, cn));
-                        dm1 = dn;
-                        dn = dnew;
-                    }
-                    cm1 = cn;
-                    cn = cnew;
-                }
-                if constexpr (sizeof(R) == 4) {
-                    // a pair whose second column is the padding (the last,
-                    // odd column) runs as one scalar FMA
-                    const float2 cc = make_float2(cn, cn), dd = make_float2(dn, dn);
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) {
-                        const V4 v = ld4(reinterpret_cast<const V4*>(row) + q);
-                        if (4 * q + 1 < NC) {
-                            A2[2 * q] = __ffma2_rn(make_float2(v.x, v.y), cc, A2[2 * q]);
-                            if (ACC) B2[2 * q] = __ffma2_rn(make_float2(v.x, v.y), dd, B2[2 * q]);
-                        } else if (4 * q < NC) {
-                            A2[2 * q].x = fmaf(v.x, cn, A2[2 * q].x);
-                            if (ACC) B2[2 * q].x = fmaf(v.x, dn, B2[2 * q].x);
-                        }
-                        if (4 * q + 3 < NC) {
-                            A2[2 * q + 1] = __ffma2_rn(make_float2(v.z, v.w), cc, A2[2 * q + 1]);
-                            if (ACC) B2[2 * q + 1] = __ffma2_rn(make_float2(v.z, v.w), dd, B2[2 * q + 1]);
-                        } else if (4 * q + 2 < NC) {
-                            A2[2 * q + 1].x = fmaf(v.z, cn, A2[2 * q + 1].x);
-                            if (ACC) B2[2 * q + 1].x = fmaf(v.z, dn, B2[2 * q + 1].x);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) {
-                        const V4 v = ld4(reinterpret_cast<const V4*>(row) + q);
-                        const R vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int c = 4 * q + e;
-                            if (c < NC) {
-                                A[c] = fma(vv[e], cn, A[c]);
-                                if (ACC) B[c] = fma(vv[e], dn, B[c]);
-                            }
-                        }
-                    }
-                }
-            }
-            if constexpr (sizeof(R) == 4) {
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    A[c] = (c & 1) ? A2[c / 2].y : A2[c / 2].x;
-                    B[c] = (c & 1) ? B2[c / 2].y : B2[c / 2].x;
-                }
-            }
-            // angular sums with the level's harmonics
-            R P = A[0] * C[s0][0];
-            R Q = ACC ? B[0] * C[s0][0] : R(0);
-#pragma unroll
-            for (int m = 1; m <= L; ++m) {
-                P = fma(A[2 * m - 1], C[s0][m], P);
-                P = fma(A[2 * m], S[s0][m], P);
-                if (ACC) {
-                    Q = fma(B[2 * m - 1], C[s0][m], Q);
-                    Q = fma(B[2 * m], S[s0][m], Q);
-                }
-            }
-            pot = fma(pre, P, pot);
-            if (ACC) {
-                gr = fma(pre, R(-(2 * L + 1)) * t * P + dxdr * Q, gr);
-                if constexpr (L >= 1) {
-                    R vx = R(0), vy = R(0), vz = R(0);
-                    R ac[L + 1], as[L + 1];
-#pragma unroll
-                    for (int m = 0; m <= L; ++m) {
-                        ac[m] = A[m == 0 ? 0 : 2 * m - 1];
-                        as[m] = m == 0 ? R(0) : A[2 * m];
-                    }
-                    grad_contract<R, L>(C[s1], S[s1], ac, as, vx, vy, vz);
-                    gx = fma(preR, vx, gx);
-                    gy = fma(preR, vy, gy);
-                    gz = fma(preR, vz, gz);
-                    preR *= st;
-                }
-            }
-            pre *= st;
-            level<L + 1>();
-        }
-    }
-};
-
-template <typename R, int LM, bool ACC, int NM1, int B = 0>
-__global__ void __launch_bounds__(kFieldThreads, 2)
-scf_field_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int n_max, int l_max,
-                 const double* __restrict__ coeffs, Vec4<R>* __restrict__ out, int out_mask,
-                 unsigned* err) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R* cs = reinterpret_cast<R*>(smem_raw);
-    const int ncols = col_total(l_max);
-    const int nj = (l_max + 1) * (l_max + 1);
-    pdl_wait();   // the coefficients come from the previous kernel
-    for (int e = threadIdx.x; e < (n_max + 1) * ncols; e += blockDim.x) {
-        const int n = e / ncols;
-        int c = e % ncols, l = 0;
-        while (c >= ncol_pad(l)) { c -= ncol_pad(l); ++l; }
-        R v = R(0);
-        if (c < 2 * l + 1) {
-            const int m = (c == 0) ? 0 : ((c & 1) ? (c + 1) / 2 : -(c / 2));
-            const int am = m < 0 ? -m : m;
-            v = (R)(coeffs[(size_t)n * nj + l * l + l + m] * c_tab.knorm[l * (l + 1) / 2 + am] *
-                    geg_gamma(B, l, n));
-        }
-        cs[e] = v;
-    }
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const Vec4<R> pv = ld4(posm + i);
-        if (!finite4(pv.x, pv.y, pv.z, pv.w)) report(err, ETICS_ERR_NONFINITE);
-        FieldEval<R, LM, ACC, NM1, B> f;
-        const R r = sqrt(pv.x * pv.x + pv.y * pv.y + pv.z * pv.z);
-        const R inv = r > R(0) ? R(1) / r : R(0);
-        f.ux = pv.x * inv; f.uy = pv.y * inv; f.uz = pv.z * inv;
-        f.uu = f.ux * f.ux + f.uy * f.uy + f.uz * f.uz;
-        const RadialSeed<R, B> rs(r);
-        f.t = rs.tau;
-        f.st = rs.st;
-        f.xi = rs.xi;
-        f.dxdr = rs.dxdr;
-        f.pre = rs.pre0;
-        f.preR = rs.pre0 * rs.q;
-        f.pot = f.gr = f.gx = f.gy = f.gz = R(0);
-        f.cs = cs;
-        f.ncols = ncols;
-        f.n_max = n_max;
-        f.l_max = l_max;
-        f.template level<0>();
-        R ax = R(0), ay = R(0), az = R(0);
-        if (ACC) {
-            ax = -(f.gr * f.ux + f.gx);
-            ay = -(f.gr * f.uy + f.gy);
-            az = -(f.gr * f.uz + f.gz);
-        }
-        const R pot = (out_mask & ETICS_OUT_POT) ? f.pot : R(0);
-        if (!finite4(ax, ay, az, pot)) report(err, ETICS_ERR_NONFINITE);
-        st4(out + i, mk4<R>(ax, ay, az, pot));
-    }
-}
-
-// ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
 template <typename R>
@@ -588,78 +384,6 @@ inline int scf_coeffs_launch(const void* posm, int64_t N, int n_max, int l_max, 
     if (cudaGetLastError() != cudaSuccess) return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;
-}
-
-template <typename R, int LM, int NM1 = 0, int B = 0>
-inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
-                           const double* coeffs, void* out, int out_mask, const LaunchCtx& ctx) {
-    const size_t smem = (size_t)(n_max + 1) * col_total(l_max) * sizeof(R);
-    // at most 4 blocks per SM (two resident at a time): each block builds the
-    // FP32 coefficient table once (FP64 multiplies, slow on this GPU) and then
-    // walks its particles; 8 per SM measured 5% slower at N = 2^20
-    int64_t want = (N + kFieldThreads - 1) / kFieldThreads;
-    const int64_t cap = (int64_t)ctx.num_sms * 4;
-    int grid = (int)(want < cap ? want : cap);
-    if (grid < 1) grid = 1;
-    const Vec4<R>* pp = reinterpret_cast<const Vec4<R>*>(posm);
-    Vec4<R>* op = reinterpret_cast<Vec4<R>*>(out);
-    // launched as a programmatic dependent of the coefficient finalize (or
-    // whatever precedes it): its launch overlaps the predecessor's tail
-    cudaError_t e;
-    if (out_mask & ETICS_OUT_ACC) {
-        auto k = scf_field_kernel<R, LM, true, NM1, B>;
-        if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-            return ETICS_ERR_CUDA;
-        e = launch_pdl(k, dim3(grid), dim3(kFieldThreads), smem, ctx.stream, pp, N, n_max, l_max,
-                       coeffs, op, out_mask, ctx.err);
-    } else {
-        auto k = scf_field_kernel<R, LM, false, NM1, B>;
-        if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-            return ETICS_ERR_CUDA;
-        e = launch_pdl(k, dim3(grid), dim3(kFieldThreads), smem, ctx.stream, pp, N, n_max, l_max,
-                       coeffs, op, out_mask, ctx.err);
-    }
-    if (e != cudaSuccess) return ETICS_ERR_CUDA;
-    ++*ctx.launches;
-    return ETICS_OK;
-}
-
-// the generic field kernels for radial basis B
-template <typename R, int B>
-inline int scf_field_launch_generic(const void* posm, int64_t N, int n_max, int l_max,
-                                    const double* coeffs, void* out, int out_mask,
-                                    const LaunchCtx& ctx) {
-    if (N == 0) return ETICS_OK;
-    if (l_max <= 2)
-        return launch_field_lm<R, 2, 0, B>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 4)
-        return launch_field_lm<R, 4, 0, B>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 6)
-        return launch_field_lm<R, 6, 0, B>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 8)
-        return launch_field_lm<R, 8, 0, B>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 10)
-        return launch_field_lm<R, 10, 0, B>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    return launch_field_lm<R, 14, 0, B>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-}
-
-template <typename R>
-inline int scf_field_launch(const void* posm, int64_t N, int n_max, int l_max,
-                            const double* coeffs, void* out, int out_mask, const LaunchCtx& ctx) {
-    if (N == 0) return ETICS_OK;
-    // specialised instantiations for the configurations of the paper's tests
-    if (n_max == 10 && l_max == 6)
-        return launch_field_lm<R, 6, 11>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (n_max == 14 && l_max == 8)
-        return launch_field_lm<R, 8, 15>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 2) return launch_field_lm<R, 2>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 4) return launch_field_lm<R, 4>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 6) return launch_field_lm<R, 6>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 8) return launch_field_lm<R, 8>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    if (l_max <= 10) return launch_field_lm<R, 10>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
-    return launch_field_lm<R, 14>(posm, N, n_max, l_max, coeffs, out, out_mask, ctx);
 }
 
 }  // namespace etics

@@ -62,3 +62,24 @@ def test_radial_order_across_the_sort_paths(precision):
         got = etics.radial_order(device_particles(pm, precision)).cpu().numpy()
         etics.check_error()
         assert np.array_equal(got, order_of(rounded(pm, precision))), n
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("basis", [0, 1])
+def test_scf_field_edges(precision, basis):
+    """The field pass takes two particles per thread (one in FP64), two radial
+    rows per round and, while a quarter of the threads would do (about 38000
+    particles at l_max <= 6, 19000 above 8), splits the levels from 2 up over
+    four warps: odd counts, odd and even n_max, either side of the split, each
+    register class of l_max, and (10, 6), (14, 8) with their unrolled rows."""
+    sizes = [(1, 0, 0), (2, 1, 1), (3, 2, 2), (65, 0, 4), (257, 3, 6), (303, 10, 6), (304, 11, 7),
+             (305, 14, 8), (1215, 5, 10), (77, 2, 14), (20001, 2, 9), (38911, 10, 6), (38913, 10, 6)]
+    for n, n_max, l_max in sizes:
+        pm = hernquist(n, seed=n)
+        ref = rounded(pm, precision)
+        c = oracle.scf_coeffs(ref[:, :3], ref[:, 3], n_max, l_max, basis=basis)
+        acc, pot = oracle.scf_field(ref[:, :3], n_max, l_max, c, basis=basis)
+        d = device_particles(pm, precision)
+        o, _ = etics.scf_force(d, n_max, l_max, basis=basis)
+        etics.check_error()
+        close(o.cpu().numpy(), acc, pot, precision, (n, n_max, l_max))
