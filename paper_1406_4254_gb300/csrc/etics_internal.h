@@ -58,8 +58,10 @@ struct SortBuffers {
     uint32_t *hist, *status, *counters;
     void* zero_base;
     size_t zero_bytes;
-    // sample path: bucket contents, splitters, ticket, flag and bucket sizes
-    uint32_t *region, *splitters, *part;
+    // sample path: bucket contents, table of the keys' distribution, and
+    // ticket, flag and bucket sizes
+    uint8_t *region, *cdf;
+    uint32_t* part;
 };
 // carve the sort buffers from ws (ws may be null to only compute *total)
 SortBuffers sort_buffers(void* ws, int64_t N, size_t* total);

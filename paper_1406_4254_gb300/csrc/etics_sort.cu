@@ -5,12 +5,13 @@
 // GB300 design, two paths that give the same order, the exact FP64 order
 // (r^2 = (x*x + y*y) + z*z rounded as a CPU does, ties by index):
 //
-// Up to kSampleMaxN particles, a sample sort: one partition of the indices
-// into buckets of about 1024 particles (splitters from a sorted sample), then one
-// block per bucket sorts it in shared memory by the 64-bit pattern of r^2 and
-// writes the order and the particles themselves.  Up to 8192 particles the
-// last kernel alone does it.  Two dependent launches instead of the radix
-// path's six, and three passes over the particles instead of ten over keys.
+// Up to kSampleMaxN particles, a sample sort: one partition of the particles
+// into buckets of about 1024 (by a table of the keys' cumulative distribution,
+// from a sample), then one block per bucket sorts it in shared memory by the
+// 64-bit pattern of r^2 and writes the order and the particles themselves.  Up
+// to 8192 particles the last kernel alone does it.  Two dependent launches
+// instead of the radix path's six, and three passes over the particles instead
+// of ten over keys.
 //
 // Above, a hand-written stable LSD radix sort (4 passes of 8 bits) of
 // the high 32 bits of the FP64 r^2 bit pattern, one kernel per pass
@@ -23,6 +24,7 @@
 // All kernels are launched with programmatic dependent launch, so each launch
 // overlaps its predecessor's tail.
 #include <atomic>
+#include <cstddef>
 
 #include "etics_internal.h"
 #include "etics_r2.h"
@@ -670,29 +672,30 @@ __device__ __forceinline__ uint64_t r2_bits(const dvec4& v) {
     return (uint64_t)__double_as_longlong(r2_fp64(v.x, v.y, v.z));
 }
 
-// Bucket sizes: a bucket's mean is a quarter of what a block sorts in shared
-// memory.  With kOversample random samples per bucket a bucket four times the
-// mean has a probability of about 1e-7 (the sum of eight exponential spacings);
+// Bucket sizes: a bucket's mean is a third of what a block sorts in shared
+// memory.  With kOversample random samples per bucket a bucket three times the
+// mean has a probability below 1e-7 (the sum of sixteen exponential spacings);
 // it is sorted all the same, by the slower sort_bucket_global.
-constexpr int kOversample = 8;
+constexpr int kOversample = 16;
 constexpr int kMaxBuckets = 1024;
 constexpr int kPartThreads = 1024;          // one thread per bucket
-constexpr int kBucketSmall = 4096, kBucketLarge = 8192;
-constexpr int kBucketKpt = 16;              // pairs per thread at capacity
-static_assert(kOversample * kMaxBuckets <= 8 * kPartThreads, "one block sorts the sample");
+constexpr int kBucketKpt = 12;              // members per thread at capacity
+constexpr int kSmallThreads = 256, kLargeThreads = 512;
+constexpr int kSmallMean = 1024, kLargeMean = 2048;
+static_assert(3 * kSmallMean == kSmallThreads * kBucketKpt && 3 * kLargeMean == kLargeThreads * kBucketKpt,
+              "a bucket's capacity is three times its mean");
+constexpr int kSingleMax = 8192, kSingleKpt = kSingleMax / kLargeThreads;   // one block, no partition
 
-// How many buckets, of which capacity, and how many particles per thread of
-// the partition: enough tiles for the SMs at each size (2^20: 128 tiles of
-// 8192).  Above kSampleMaxN the sample (sorted by one block) would get too
-// small for the number of buckets: the radix path.
-constexpr int64_t kSampleMaxN = int64_t(kMaxBuckets) * (kBucketLarge / 4);
-struct SamplePlan { int nbuckets, cap, kpt, ntiles; };
+// How many buckets, of which mean, and how many particles per thread of the
+// partition: enough tiles for the SMs at each size (2^20: 128 tiles of 8192).
+// Above kSampleMaxN: the radix path.
+constexpr int64_t kSampleMaxN = int64_t(kMaxBuckets) * kLargeMean;
+struct SamplePlan { int nbuckets, mean, kpt, ntiles; };
 SamplePlan sample_plan(int64_t N) {
     SamplePlan p{};
     if (N > kSampleMaxN) return p;
-    p.cap = N > kBucketLarge && N <= int64_t(kMaxBuckets) * kBucketSmall / 4 ? kBucketSmall
-                                                                              : kBucketLarge;
-    p.nbuckets = N <= p.cap ? 1 : (int)((N + p.cap / 4 - 1) / (p.cap / 4));
+    p.mean = N <= int64_t(kMaxBuckets) * kSmallMean ? kSmallMean : kLargeMean;
+    p.nbuckets = N <= kSingleMax ? 1 : (int)((N + p.mean - 1) / p.mean);
     p.kpt = N <= (int64_t(1) << 18) ? 2 : N <= (int64_t(1) << 19) ? 4 : 8;
     p.ntiles = (int)((N + (int64_t)kPartThreads * p.kpt - 1) / ((int64_t)kPartThreads * p.kpt));
     return p;
@@ -702,29 +705,32 @@ SamplePlan sample_plan(int64_t N) {
 // pairs t, t + TH, ... in k[], id[]: each key is mapped linearly from the
 // block's key range to one of 8 TH bins, the bins are counted and scanned, and
 // the pairs placed in bin order in s_key / s_id; within a bin (half a pair on
-// average at a bucket's mean size) count_less() counts the smaller keys.
-// Equal keys are told apart by the caller, who fills s_low and passes how.
+// average at a bucket's mean size) the caller counts the smaller keys.
+// Equal keys are told apart by the caller.
 constexpr int kBinLimit = 48;
 template <int TH, int KPT>
 struct BlockSort {
     static constexpr int CAP = TH * KPT, NB = 8 * TH;
-    static constexpr size_t kSmem = (size_t)CAP * 14 + (size_t)NB * 4;   // with a 16-bit list
+    // keys, ids, bins, and a 16-bit list; s_low (bitonic() only) lies over the
+    // last two
+    static constexpr size_t kSmem = (size_t)CAP * 10 + (size_t)NB * 4;
+    static_assert((size_t)CAP * 4 <= (size_t)CAP * 2 + (size_t)NB * 4, "room for the low words");
     uint32_t *s_key, *s_id, *s_low, *s_bin;
+    uint16_t* s_list;
     uint32_t kmin, mult;
     int n;
     bool crowded;   // a bin holds more than kBinLimit pairs
 
     __device__ __forceinline__ explicit BlockSort(unsigned char* smem)
         : s_key(reinterpret_cast<uint32_t*>(smem)), s_id(s_key + CAP), s_low(s_id + CAP),
-          s_bin(s_low + CAP) {}
+          s_bin(s_id + CAP), s_list(reinterpret_cast<uint16_t*>(s_bin + NB)) {}
 
     __device__ __forceinline__ int bin_of(uint32_t key) const {
         return (int)(mult ? __umulhi(key - kmin, mult) : key - kmin);
     }
 
-    // (s_low is not touched; low: placed along when not null)
     __device__ __forceinline__ void place(const uint32_t (&k)[KPT], const uint32_t (&id)[KPT],
-                                          const uint32_t* low, int count) {
+                                          int count) {
         __shared__ uint32_t s_lo, s_hi, s_sum[32];
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
         n = count;
@@ -783,26 +789,28 @@ struct BlockSort {
                 const uint32_t pos = s_bin[at[s] & 0xffffu] + (at[s] >> 16);
                 s_key[pos] = k[s];
                 s_id[pos] = id[s];
-                if (low) s_low[pos] = low[s];
             }
         __syncthreads();
     }
 
-    // the pairs [0, n) sorted by (key, low, id), padded to a power of two (at
-    // most CAP): where keys crowd, a network instead of the bins
+    // the pairs [0, n) sorted by (key, s_low, id): where keys crowd, a network
+    // (of a power of two of places, those from n on taken as infinite: a pair
+    // with one of them is never exchanged, as the larger value always belongs
+    // to the upper place in the form used, first step mirrored)
     __device__ __noinline__ void bitonic() {
         int p2 = 2;
         while (p2 < n) p2 <<= 1;
-        for (int i = n + threadIdx.x; i < p2; i += TH) s_key[i] = s_low[i] = s_id[i] = 0xffffffffu;
         __syncthreads();
         for (int k = 2; k <= p2; k <<= 1)
             for (int j = k >> 1; j > 0; j >>= 1) {
                 for (int t = threadIdx.x; t < p2 / 2; t += TH) {
-                    const int i = 2 * t - (t & (j - 1)), l = i + j;
+                    const int i = 2 * t - (t & (j - 1));
+                    const int l = j == (k >> 1) ? (i ^ (k - 1)) : i + j;
+                    if (l >= n) continue;
                     const uint32_t a = s_key[i], b = s_key[l], la = s_low[i], lb = s_low[l],
                                    ia = s_id[i], ib = s_id[l];
                     const bool after = a > b || (a == b && (la > lb || (la == lb && ia > ib)));
-                    if (after == ((i & k) == 0)) {
+                    if (after) {
                         s_key[i] = b; s_key[l] = a;
                         s_low[i] = lb; s_low[l] = la;
                         s_id[i] = ib; s_id[l] = ia;
@@ -832,67 +840,169 @@ __device__ __forceinline__ uint32_t sort_key(const Vec4<R>& v) {
     return finite4(v.x, v.y, v.z, v.w) ? r2_key(v.x, v.y, v.z) : 0xffffffffu;
 }
 
-// The splitters: every kOversample-th key of a sorted sample of kOversample
-// nbuckets particles, one at a random place of each of as many equal stretches
+// The cumulative distribution of the keys, from a sample of kOversample
+// nbuckets particles: one at a random place of each of as many equal stretches
 // of the array (a regular stride could fall in step with an order of the
-// particles).  stride: N / (number of samples), 32.32 fixed point.
-using SplitterSort = BlockSort<kPartThreads, 8>;
+// particles).  kCdfBins bins of equal width over the sample's key range hold
+// the number of samples below them; a bin with more than kCdfCrowd samples is
+// divided once more into 256 (kCdfFine of them at most).  Within a bin the
+// distribution is taken as linear, so that a key's bucket comes from two table
+// entries instead of a search among splitters (the binary search cost 12 us at
+// 2^20, sorting the sample for splitters another 8).  How good the table is
+// only decides how even the buckets are.
+constexpr int kCdfBins = 8192, kCdfCrowd = 32, kCdfFine = 64, kCdfFineRow = 264;
+struct KeyCdf {                      // 16-byte pieces, copied to shared memory as a whole
+    uint32_t kmin, range, mult, nfine;
+    uint16_t below[kCdfBins + 8];    // samples below bin b; [kCdfBins]: all of them
+    uint8_t fine[kCdfBins];          // row of a divided bin, 255: none
+    uint16_t row[kCdfFine][kCdfFineRow];   // samples of the bin below its part
+};
+static_assert(sizeof(KeyCdf) % 16 == 0 && kOversample * kMaxBuckets < 65536, "table layout");
+
+__device__ __forceinline__ int bucket_of(const KeyCdf& t, uint32_t key, int nbuckets) {
+    if (key < t.kmin) return 0;
+    if (key - t.kmin > t.range) return nbuckets - 1;
+    // bin and place in it (32-bit fraction); mult 0: a bin per key
+    const uint64_t p = t.mult ? (uint64_t)(key - t.kmin) * t.mult : (uint64_t)(key - t.kmin) << 32;
+    const int b = (int)(p >> 32);
+    uint32_t frac = (uint32_t)p, lo = t.below[b], hi = t.below[b + 1];
+    if (hi - lo > (uint32_t)kCdfCrowd && t.fine[b] != 255) {
+        const uint16_t* r = t.row[t.fine[b]] + (frac >> 24);
+        frac <<= 8;
+        hi = lo + r[1];
+        lo += r[0];
+    }
+    // in sixteenths of a sample
+    const uint32_t c = lo * 16u + (((hi - lo) * (frac >> 16)) >> 12);
+    const int k = (int)(c / (16u * kOversample));
+    return k < nbuckets ? k : nbuckets - 1;
+}
+
+// one block; scratch: (kCdfBins + kCdfFine 256) words of shared memory.
+// stride: N / (number of samples), 32.32 fixed point.
+constexpr size_t kCdfSmem = ((size_t)kCdfBins + (size_t)kCdfFine * 256) * 4;
+static_assert(kCdfSmem >= sizeof(KeyCdf), "the tiles copy the table there");
 template <typename R>
-__device__ __forceinline__ void make_splitters(const Vec4<R>* posm, int64_t N, int nbuckets,
-                                               uint64_t stride, uint32_t* splitters,
-                                               unsigned char* smem) {
-    const int tid = threadIdx.x, ns = kOversample * nbuckets;
-    uint32_t k[8], id[8];
+__device__ __forceinline__ void make_cdf(const Vec4<R>* posm, int64_t N, int nbuckets,
+                                         uint64_t stride, KeyCdf* out, uint32_t* scratch) {
+    constexpr int TH = kPartThreads, KPT = kOversample * kMaxBuckets / TH;
+    static_assert(kCdfBins == 8 * TH, "eight bins per thread");
+    __shared__ uint32_t s_lo, s_hi, s_nfine, s_sum[32];
+    uint32_t *s_bin = scratch, *s_part = scratch + kCdfBins;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ns = kOversample * nbuckets;
+    uint4* bins4 = reinterpret_cast<uint4*>(s_bin);
+    bins4[tid] = bins4[tid + TH] = make_uint4(0, 0, 0, 0);
+    if (tid == 0) { s_lo = 0xffffffffu; s_hi = 0u; s_nfine = 0u; }
+    uint32_t k[KPT], lo = 0xffffffffu, hi = 0u;
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-        const uint32_t i = (uint32_t)(tid + s * kPartThreads);
+    for (int s = 0; s < KPT; ++s) {
+        const uint32_t i = (uint32_t)(tid + s * TH);
         if ((int)i < ns) {
             const int64_t a = (int64_t)((i * stride) >> 32);
             int64_t b = (int64_t)(((i + 1) * stride) >> 32);
             if (b <= a) b = a + 1;
             const int64_t g = a + (int64_t)__umulhi(mix32(i + 1), (uint32_t)(b - a));
             k[s] = sort_key<R>(ld4(posm + (g < N ? g : N - 1)));
-            id[s] = i;
+            lo = k[s] < lo ? k[s] : lo;
+            hi = k[s] > hi ? k[s] : hi;
         }
     }
-    SplitterSort sort(smem);
-    sort.place(k, id, nullptr, ns);
-    if (sort.crowded) {
-        for (int p = tid; p < ns; p += kPartThreads) sort.s_low[p] = 0u;
-        sort.bitonic();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    __syncthreads();
+    if (lane == 0) {
+        atomicMin(&s_lo, lo);
+        atomicMax(&s_hi, hi);
     }
-    for (int p = tid; p < ns; p += kPartThreads) {
-        int r = p;
-        const uint32_t key = sort.s_key[p];
-        if (!sort.crowded) {
-            int s, e;
-            sort.bin_range(key, s, e);
-            r = s;
-            const uint32_t own = sort.s_id[p];
-            for (int j = s; j < e; ++j)
-                r += sort.s_key[j] < key || (sort.s_key[j] == key && sort.s_id[j] < own);
-        }
-        if (r % kOversample == 0) splitters[r / kOversample] = r == 0 ? 0u : key;
-    }
-}
-
-// bucket of a key: the last splitter not above it (s_split padded with
-// 0xffffffff to 1024 entries, splitter 0 is 0)
-__device__ __forceinline__ int bucket_of(const uint32_t* s_split, uint32_t key, int nbuckets) {
-    int b = 0;
+    __syncthreads();
+    const uint32_t kmin = s_lo, range = s_hi - kmin;
+    const uint32_t mult = range < (uint32_t)kCdfBins
+                              ? 0u : (uint32_t)(((uint64_t)kCdfBins << 32) / ((uint64_t)range + 1));
+    auto place = [&](uint32_t key) {
+        return mult ? (uint64_t)(key - kmin) * mult : (uint64_t)(key - kmin) << 32;
+    };
 #pragma unroll
-    for (int h = kMaxBuckets / 2; h > 0; h >>= 1)
-        if (s_split[b + h] <= key) b += h;
-    return b < nbuckets ? b : nbuckets - 1;
+    for (int s = 0; s < KPT; ++s)
+        if (tid + s * TH < ns) atomicAdd(&s_bin[(uint32_t)(place(k[s]) >> 32)], 1u);
+    __syncthreads();
+    // this thread's eight bins: rows for the crowded ones, counts to sums
+    uint32_t c[8];
+    *reinterpret_cast<uint4*>(c) = bins4[2 * tid];
+    *reinterpret_cast<uint4*>(c + 4) = bins4[2 * tid + 1];
+    uint32_t rows[2] = {0u, 0u}, sum = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        uint32_t r = 255u;
+        if (c[j] > (uint32_t)kCdfCrowd) {
+            r = atomicAdd(&s_nfine, 1u);
+            if (r >= (uint32_t)kCdfFine) r = 255u;
+        }
+        rows[j / 4] |= r << (8 * (j % 4));
+        const uint32_t v = c[j];
+        c[j] = sum;
+        sum += v;
+    }
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+    }
+    if (lane == 31) s_sum[warp] = x;
+    for (int i = tid; i < kCdfFine * 256; i += TH) s_part[i] = 0u;
+    __syncthreads();
+    const uint32_t before = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? s_sum[lane] : 0u);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        out->below[8 * tid + j] = (uint16_t)(before + c[j]);
+        // the bin's row for the second count, in place of its count
+        s_bin[8 * tid + j] = (rows[j / 4] >> (8 * (j % 4))) & 255u;
+    }
+    *reinterpret_cast<uint2*>(out->fine + 8 * tid) = make_uint2(rows[0], rows[1]);
+    const int nfine = min((int)s_nfine, kCdfFine);
+    if (tid == 0) {
+        out->below[kCdfBins] = (uint16_t)ns;
+        out->kmin = kmin;
+        out->range = range;
+        out->mult = mult;
+        out->nfine = (uint32_t)nfine;
+    }
+    __syncthreads();
+    if (nfine == 0) return;
+#pragma unroll
+    for (int s = 0; s < KPT; ++s)
+        if (tid + s * TH < ns) {
+            const uint64_t p = place(k[s]);
+            const uint32_t r = s_bin[(uint32_t)(p >> 32)];
+            if (r != 255u) atomicAdd(&s_part[r * 256u + ((uint32_t)p >> 24)], 1u);
+        }
+    __syncthreads();
+    for (int r = warp; r < nfine; r += TH / 32) {
+        uint32_t v[8], t = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            v[j] = t;
+            t += s_part[r * 256 + 8 * lane + j];
+        }
+        uint32_t y = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += u;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) out->row[r][8 * lane + j] = (uint16_t)(y - t + v[j]);
+        if (lane == 31) out->row[r][256] = (uint16_t)y;
+    }
 }
 
 // Partition.  Blocks take tickets; the block with the first one makes the
-// splitters and raises the flag, the others load their tile's particles and
+// table and raises the flag, the others load their tile's particles and
 // evaluate the keys meanwhile and wait for it (bounded; the tickets' order
 // makes sure that the block waited for has started).  A tile then counts its
 // particles per bucket in shared memory, takes its places in the buckets with
-// one addition per bucket to the bucket sizes, and writes the particles'
-// indices to region[b * cap + place].  The order inside a bucket's region is
+// one addition per bucket to the bucket sizes, and writes the particles' keys
+// and indices to region[b * cap + place].  The order inside a bucket's region is
 // whatever the additions give: the bucket sort orders by (r^2, index).  A place
 // beyond the capacity is not written (sort_bucket_global finds those particles
 // again).  A tile whose wait runs out (ETICS_ERR_TIMEOUT) counts its particles
@@ -904,10 +1014,9 @@ constexpr int kPartHeader = 64;
 template <typename R, int KPT>
 __global__ void __launch_bounds__(kPartThreads, 1)
 partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int cap,
-                 uint64_t stride, uint32_t* splitters, uint32_t* part,
-                 uint32_t* __restrict__ region, int64_t spin_limit, unsigned* err) {
+                 uint64_t stride, KeyCdf* cdf, uint32_t* part, uint2* __restrict__ region,
+                 int64_t spin_limit, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
-    __shared__ uint32_t s_split[kMaxBuckets];
     __shared__ uint32_t s_hist[kMaxBuckets];
     __shared__ uint32_t s_ticket;
     __shared__ int s_ok;
@@ -917,7 +1026,7 @@ partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int 
     if (tid == 0) s_ticket = atomicAdd(part, 1u);
     __syncthreads();
     if (s_ticket == 0u) {
-        make_splitters<R>(posm, N, nbuckets, stride, splitters, sort_smem);
+        make_cdf<R>(posm, N, nbuckets, stride, cdf, reinterpret_cast<uint32_t*>(sort_smem));
         __threadfence();
         __syncthreads();
         if (tid == 0) st_volatile(part + 1, 1u);
@@ -951,14 +1060,22 @@ partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int 
         s_ok = ok;
     }
     __syncthreads();
-    s_split[tid] = tid < nbuckets && s_ok ? __ldcg(splitters + tid) : (tid ? 0xffffffffu : 0u);
+    const bool ok = s_ok;
+    KeyCdf& t = *reinterpret_cast<KeyCdf*>(sort_smem);
+    if (ok) {
+        // without the rows of divided bins that are not there
+        const uint32_t nfine = __ldcg(&cdf->nfine);
+        const int pieces = (int)((offsetof(KeyCdf, row) + nfine * sizeof(t.row[0])) / 16);
+        for (int i = tid; i < pieces; i += kPartThreads)
+            reinterpret_cast<uint4*>(&t)[i] = __ldcg(reinterpret_cast<const uint4*>(cdf) + i);
+    }
     __syncthreads();
     uint32_t at[KPT];   // bucket, then place within the tile's share (16 bits each)
 #pragma unroll
     for (int s = 0; s < KPT; ++s) {
         at[s] = 0u;
         if (start + s * kPartThreads + tid < N) {
-            const int b = bucket_of(s_split, key[s], s_ok ? nbuckets : 1);
+            const int b = ok ? bucket_of(t, key[s], nbuckets) : 0;
             at[s] = (uint32_t)b | (atomicAdd(&s_hist[b], 1u) << 16);
         }
     }
@@ -971,7 +1088,7 @@ partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int 
         const int64_t i = start + s * kPartThreads + tid;
         if (i < N) {
             const uint32_t b = at[s] & 0xffffu, slot = s_hist[b] + (at[s] >> 16);
-            if (slot < (uint32_t)cap) region[(size_t)b * cap + slot] = (uint32_t)i;
+            if (slot < (uint32_t)cap) region[(size_t)b * cap + slot] = make_uint2(key[s], (uint32_t)i);
         }
     }
 }
@@ -982,8 +1099,8 @@ partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int 
 // pattern with stable 8-bit passes (sort_run_block's, over both words),
 // passes whose digit is the same for all members left out.
 template <typename R, int TH>
-__device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, uint32_t key_lo,
-                                                uint32_t key_hi, bool last, uint32_t* val,
+__device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, const KeyCdf* cdf,
+                                                int nbuckets, int bucket, uint32_t* val,
                                                 uint32_t* tmp, int64_t len, uint32_t* scratch) {
     constexpr int NW = TH / 32;
     uint32_t (*s_cnt)[256] = reinterpret_cast<uint32_t (*)[256]>(scratch);   // [NW][256]
@@ -993,10 +1110,8 @@ __device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, 
     int64_t found = 0;
     for (int64_t c0 = 0; c0 < N; c0 += TH) {
         bool mine = false;
-        if (c0 + tid < N) {
-            const uint32_t k = sort_key<R>(ld4(posm + c0 + tid));
-            mine = k >= key_lo && (last || k < key_hi);
-        }
+        if (c0 + tid < N)
+            mine = bucket_of(*cdf, sort_key<R>(ld4(posm + c0 + tid)), nbuckets) == bucket;
         const unsigned bal = __ballot_sync(0xffffffffu, mine);
         if (lane == 0) s_wsum[warp] = (uint32_t)__popc(bal);
         __syncthreads();
@@ -1082,112 +1197,127 @@ __device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, 
 // One block per bucket: its place in the order from the bucket sizes, the sort
 // of its members by (64-bit pattern of r^2, index), the order and (sorted not
 // null) the particles.  nbuckets == 1: the particles 0..N-1 themselves (at
-// most TH kBucketKpt), no partition before.
+// most TH KPT), no partition before.
 // The members are sorted by the high word of the pattern (the cheap 32-bit
 // key); the low word is evaluated only for members that share their high word
-// with another one (a few in a hundred), collected first so that whole warps
-// do it.
-template <typename R, int TH>
+// with another one (a few in a hundred), listed first so that whole warps do
+// it.  Latency-bound: a chain of loads and block-wide steps, about 12 us per
+// block whatever its size, hidden only by other blocks.
+template <typename R, int TH, int KPT>
 __global__ void __launch_bounds__(TH)
-bucket_sort_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets,
-                   const uint32_t* splitters, const uint32_t* sizes, const uint32_t* region,
-                   uint32_t* perm, uint32_t* tmp, Vec4<R>* __restrict__ sorted, unsigned* err) {
+bucket_sort_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, const KeyCdf* cdf,
+                   const uint32_t* sizes, const uint2* region, uint32_t* perm, uint32_t* tmp,
+                   Vec4<R>* __restrict__ sorted, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
-    constexpr int KPT = kBucketKpt;
     using Sort = BlockSort<TH, KPT>;
     constexpr int CAP = Sort::CAP;
+    constexpr int kAhead = 5;   // members per thread loaded before the size is known
     __shared__ uint32_t s_base[TH / 32];
     __shared__ int s_ntie;
     pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
     int64_t base = 0, len = N;
     if (tid == 0) s_ntie = 0;
+    uint32_t k[KPT], id[KPT];
     if (nbuckets > 1) {
+        const uint2* mem = region + (size_t)b * CAP + tid;
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s) {
+            const uint2 m = __ldcg(mem + s * TH);
+            k[s] = m.x;
+            id[s] = m.y;
+        }
         uint32_t before = 0;
         for (int i = tid; i < b; i += TH) before += __ldcg(sizes + i);
+        len = __ldcg(sizes + b);
         before = __reduce_add_sync(0xffffffffu, before);
         if (lane == 0) s_base[warp] = before;
-        len = __ldcg(sizes + b);
         __syncthreads();
         base = __reduce_add_sync(0xffffffffu, lane < TH / 32 ? s_base[lane] : 0u);
         if (base > N) base = N;   // (the sizes add up to N)
         if (base + len > N) len = N - base;
-    }
-    if (len == 0) return;
-    if (len > CAP) {
-        sort_bucket_global<R, TH>(posm, N, __ldcg(splitters + b),
-                                  b + 1 < nbuckets ? __ldcg(splitters + b + 1) : 0u,
-                                  b + 1 == nbuckets, perm + base, tmp + base, len,
-                                  reinterpret_cast<uint32_t*>(sort_smem));
-        if (sorted)
-            for (int64_t i = tid; i < len; i += TH)
-                st4(sorted + base + i, gather_particle<R>(posm, perm[base + i], N, err));
-        return;
-    }
-    const int n = (int)len;
-    Sort sort(sort_smem);
-    {
-        uint32_t k[KPT], id[KPT];
+        if (len == 0) return;
+        if (len > CAP) {
+            sort_bucket_global<R, TH>(posm, N, cdf, nbuckets, b, perm + base, tmp + base, len,
+                                      reinterpret_cast<uint32_t*>(sort_smem));
+            if (sorted)
+                for (int64_t i = tid; i < len; i += TH)
+                    st4(sorted + base + i, gather_particle<R>(posm, perm[base + i], N, err));
+            return;
+        }
+#pragma unroll
+        for (int s = kAhead; s < KPT; ++s)
+            if (tid + s * TH < (int)len) {
+                const uint2 m = __ldcg(mem + s * TH);
+                k[s] = m.x;
+                id[s] = m.y;
+            }
+    } else {
 #pragma unroll
         for (int s = 0; s < KPT; ++s) {
             const int i = tid + s * TH;
-            if (i < n) id[s] = nbuckets > 1 ? __ldcg(region + (size_t)b * CAP + i) : (uint32_t)i;
+            if (i < (int)len) {
+                k[s] = sort_key<R>(ld4(posm + i));
+                id[s] = (uint32_t)i;
+            }
         }
-#pragma unroll
-        for (int s = 0; s < KPT; ++s)
-            if (tid + s * TH < n)
-                k[s] = (int64_t)id[s] < N ? sort_key<R>(ld4(posm + id[s])) : 0xffffffffu;
-        sort.place(k, id, nullptr, n);
     }
+    const int n = (int)len;
+    Sort sort(sort_smem);
+    sort.place(k, id, n);
     auto low_word = [&](uint32_t i) -> uint32_t {
         return (int64_t)i < N ? (uint32_t)r2_bits(ld4(posm + i)) : 0xffffffffu;
     };
-    if (sort.crowded) {
-        for (int p = tid; p < n; p += TH) sort.s_low[p] = low_word(sort.s_id[p]);
-        __syncthreads();
-        sort.bitonic();
-        for (int p = tid; p < n; p += TH) {
-            const uint32_t i = sort.s_id[p];
-            perm[base + p] = i;
-            if (sorted) st4(sorted + base + p, gather_particle<R>(posm, i, N, err));
-        }
-        return;
-    }
-    // a pair's place is the start of its bin plus the smaller ones in it; those
-    // with an equal key in the bin go to the list, get their low words and are
-    // placed by all of (key, low word, index)
-    uint16_t* s_tie = reinterpret_cast<uint16_t*>(sort.s_bin + Sort::NB);
     auto put = [&](int r, uint32_t i) {
         perm[base + r] = i;
         if (sorted) st4(sorted + base + r, gather_particle<R>(posm, i, N, err));
     };
-    for (int p = tid; p < n; p += TH) {
-        const uint32_t key = sort.s_key[p];
-        int s, e;
-        sort.bin_range(key, s, e);
-        int r = s, same = 0;
-        for (int j = s; j < e; ++j) {
-            r += sort.s_key[j] < key;
-            same += sort.s_key[j] == key;
+    // a pair's place is the start of its bin plus the smaller ones in it; those
+    // with an equal key in the bin go to the list and are placed by (key, low
+    // word, index).  Where keys crowd in one bin, or a quarter of the members
+    // share their key (comparing those in pairs would be quadratic), the
+    // network sorts them all.
+    bool net = sort.crowded;
+    if (!net) {
+        for (int p = tid; p < n; p += TH) {
+            const uint32_t key = sort.s_key[p];
+            int s, e;
+            sort.bin_range(key, s, e);
+            int r = s, same = 0;
+            for (int j = s; j < e; ++j) {
+                r += sort.s_key[j] < key;
+                same += sort.s_key[j] == key;
+            }
+            if (same > 1) sort.s_list[atomicAdd(&s_ntie, 1)] = (uint16_t)p;
+            else put(r, sort.s_id[p]);
         }
-        if (same > 1) s_tie[atomicAdd(&s_ntie, 1)] = (uint16_t)p;
-        else put(r, sort.s_id[p]);
+        __syncthreads();
+        net = 4 * s_ntie > n;
     }
-    __syncthreads();
+    if (net) {
+        // (s_low lies over the bins and the list, neither needed any more)
+        for (int p = tid; p < n; p += TH) sort.s_low[p] = low_word(sort.s_id[p]);
+        sort.bitonic();
+        for (int p = tid; p < n; p += TH) put(p, sort.s_id[p]);
+        return;
+    }
     const int ntie = s_ntie;
-    for (int q = tid; q < ntie; q += TH) sort.s_low[s_tie[q]] = low_word(sort.s_id[s_tie[q]]);
-    __syncthreads();
     for (int q = tid; q < ntie; q += TH) {
-        const int p = s_tie[q];
-        const uint32_t key = sort.s_key[p], low = sort.s_low[p], id = sort.s_id[p];
+        const int p = sort.s_list[q];
+        const uint32_t key = sort.s_key[p], own = sort.s_id[p], low = low_word(own);
         int s, e;
         sort.bin_range(key, s, e);
         int r = s;
         for (int j = s; j < e; ++j) {
             const uint32_t kj = sort.s_key[j];
-            r += kj < key || (kj == key && (sort.s_low[j] < low || (sort.s_low[j] == low && sort.s_id[j] < id)));
+            if (kj < key) {
+                ++r;
+            } else if (kj == key && j != p) {
+                const uint32_t lj = low_word(sort.s_id[j]);
+                r += lj < low || (lj == low && sort.s_id[j] < own);
+            }
         }
-        put(r, id);
+        put(r, own);
     }
 }
 
@@ -1222,8 +1352,8 @@ SortBuffers sort_buffers(void* ws, int64_t N, size_t* total) {
     off = shared;
     const SamplePlan sp = sample_plan(N);
     if (sp.nbuckets > 1) {
-        b.region = reinterpret_cast<uint32_t*>(take((size_t)sp.nbuckets * sp.cap * 4));
-        b.splitters = reinterpret_cast<uint32_t*>(take(kMaxBuckets * 4));
+        b.region = take((size_t)sp.nbuckets * 3 * sp.mean * sizeof(uint2));
+        b.cdf = take(sizeof(KeyCdf));
         b.part = reinterpret_cast<uint32_t*>(take((kPartHeader + kMaxBuckets) * 4));
     }
     if (radix_end > off) off = radix_end;
@@ -1251,30 +1381,29 @@ static int launch_partition(const Vec4<R>* pp, int64_t N, const SamplePlan& sp,
                             const SortBuffers& b, const LaunchCtx& ctx) {
     static std::atomic<uint64_t> done{0};
     auto k = partition_kernel<R, KPT>;
-    constexpr size_t smem = SplitterSort::kSmem;
+    constexpr size_t smem = kCdfSmem;
     if (allow_smem(k, done, smem)) return ETICS_ERR_CUDA;
     if (cudaMemsetAsync(b.part, 0, (kPartHeader + sp.nbuckets) * 4, ctx.stream)) return ETICS_ERR_CUDA;
     const uint64_t stride = ((uint64_t)N << 32) / (uint64_t)(kOversample * sp.nbuckets);
     if (launch_pdl(k, dim3(sp.ntiles + 1), dim3(kPartThreads), smem, ctx.stream, pp, N, sp.nbuckets,
-                   sp.cap, stride, b.splitters, b.part, b.region,
-                   ctx.wait_limit > 0 ? ctx.wait_limit : kSpinLimit, ctx.err))
+                   3 * sp.mean, stride, reinterpret_cast<KeyCdf*>(b.cdf), b.part,
+                   reinterpret_cast<uint2*>(b.region), ctx.wait_limit > 0 ? ctx.wait_limit : kSpinLimit, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;
 }
 
-template <typename R, int CAP>
+template <typename R, int TH, int KPT>
 static int launch_buckets(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, const SortBuffers& b,
                           Vec4<R>* sorted, const LaunchCtx& ctx) {
     static std::atomic<uint64_t> done{0};
-    constexpr int TH = CAP / kBucketKpt;
-    constexpr size_t smem = BlockSort<TH, kBucketKpt>::kSmem;
-    auto k = bucket_sort_kernel<R, TH>;
+    constexpr size_t smem = BlockSort<TH, KPT>::kSmem;
+    auto k = bucket_sort_kernel<R, TH, KPT>;
     if (allow_smem(k, done, smem)) return ETICS_ERR_CUDA;
     if (launch_pdl(k, dim3(sp.nbuckets), dim3(TH), smem, ctx.stream, pp, N, sp.nbuckets,
-                   (const uint32_t*)b.splitters,
+                   reinterpret_cast<const KeyCdf*>(b.cdf),
                    (const uint32_t*)(b.part ? b.part + kPartHeader : nullptr),
-                   (const uint32_t*)b.region, b.vals_a, b.vals_b, sorted, ctx.err))
+                   reinterpret_cast<const uint2*>(b.region), b.vals_a, b.vals_b, sorted, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;
@@ -1290,8 +1419,11 @@ static int sample_sort(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, const
         if (rc) return rc;
     }
     stage_event(ctx, 1);
-    return sp.cap == kBucketSmall ? launch_buckets<R, kBucketSmall>(pp, N, sp, b, sorted, ctx)
-                                  : launch_buckets<R, kBucketLarge>(pp, N, sp, b, sorted, ctx);
+    if (sp.nbuckets == 1)
+        return launch_buckets<R, kLargeThreads, kSingleKpt>(pp, N, sp, b, sorted, ctx);
+    return sp.mean == kSmallMean
+               ? launch_buckets<R, kSmallThreads, kBucketKpt>(pp, N, sp, b, sorted, ctx)
+               : launch_buckets<R, kLargeThreads, kBucketKpt>(pp, N, sp, b, sorted, ctx);
 }
 
 template <typename R>
