@@ -13,9 +13,17 @@
 // back-propagated errors) and accumulates in FP32; biases, tanh, the loss, its
 // gradient and Adam run in FP32; the feature / update glue in FP64.
 //
-// Products run as C_part[s] = op(A) op(B) over K-slice s (split-K, slices
-// written to separate buffers) followed by an epilogue kernel that sums the
-// slices in a fixed order, so every result is deterministic.
+// A product whose K is not split finishes in its own kernel (bias, tanh or its
+// derivative, bf16 copies, column sums for the bias gradient: etics_tc.cuh).
+// Split products write one slice each, C_part[s] = op(A) op(B) over K-slice s,
+// summed in a fixed order afterwards, so every result is deterministic.
+// Layers at most kThin wide on one side are no work for a 64- or 128-wide tile
+// and have kernels of their own: the output layer with the loss, its backward
+// step, and the weight gradient of a narrow input.  The training step of the
+// shared network (8 -> 256 -> 256 -> 3, 19440 rows) went from 25 launches and
+// 437 us to 9 launches and 112 us (per kernel, cold: forward products 12 and
+// 14, output layer 12, its backward step 14, dH 10, dW 19, narrow dW 10,
+// reductions 18, Adam 4).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -175,7 +183,7 @@ __global__ void mlp_epilogue_kernel(const float* __restrict__ part, int splits, 
 }
 
 // dY = 2 (Y - T) / count (FP32 and bf16); per-block FP64 partial sums of
-// (Y - T)^2 in a fixed grid, summed by mlp_loss_final_kernel
+// (Y - T)^2 in a fixed grid, summed by mlp_reduce_kernel
 __global__ void __launch_bounds__(256)
 mlp_mse_kernel(const float* __restrict__ y, const float* __restrict__ tg, int64_t count,
                float scale, float* __restrict__ dy, bf16* __restrict__ dyb,
@@ -201,17 +209,8 @@ mlp_mse_kernel(const float* __restrict__ y, const float* __restrict__ tg, int64_
     }
 }
 
-__global__ void mlp_loss_final_kernel(const double* __restrict__ block_sums, int n,
-                                      double inv_count, double* __restrict__ loss) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += block_sums[i];
-        *loss = s * inv_count;
-    }
-}
-
-// db[n] = sum over rows of dz[m][n] in two deterministic stages: FP64 sums
-// of row chunk blockIdx.y (rows in order), then the chunk sums in order
+// column sums of dz over row chunk blockIdx.y in FP64 (rows in order), added by
+// mlp_reduce_kernel
 constexpr int kColChunks = 128;
 
 __global__ void mlp_colsum_partial_kernel(const float* __restrict__ dz, int M, int N, int rows,
@@ -224,13 +223,302 @@ __global__ void mlp_colsum_partial_kernel(const float* __restrict__ dz, int M, i
     part[(size_t)blockIdx.y * N + n] = s;
 }
 
-__global__ void mlp_colsum_final_kernel(const double* __restrict__ part, int chunks, int N,
-                                        float* __restrict__ db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += part[(size_t)c * N + n];
-    db[n] = (float)s;
+// ---- layers at most kThin wide on one side ----------------------------------
+constexpr int kThin = 8;
+constexpr int kThinBlocks = kTargetBlocks;   // row chunks, and so partial sums, at most
+constexpr int kThinInputs = 1024;            // inputs of a narrow output layer, at most
+
+__device__ __forceinline__ float bf(bf16 v) { return __bfloat162float(v); }
+
+// y = a W + bias for dout <= kThin outputs on m16n8k16 MMAs, one warp per 16
+// rows, the K slices and the order inside them those of mlp_gemm_kernel (the
+// same bits).  With a target: dy = scale (y - t) in bf16 and per block the sums
+// of (y - t)^2 and of dy (FP32 pairs); else y itself.
+__global__ void __launch_bounds__(256)
+mlp_narrow_out_kernel(const bf16* __restrict__ a, const bf16* __restrict__ W,
+                      const float* __restrict__ bias, const float* __restrict__ target, int B,
+                      int din, int dout, int kslice, float scale, float* __restrict__ y,
+                      bf16* __restrict__ dyb, double* __restrict__ loss_part,
+                      double* __restrict__ db_part) {
+    __shared__ __align__(16) bf16 s_w[kThin][kThinInputs + kPadK];   // [output][input]
+    __shared__ double s_loss[8], s_db[8][kThin];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    for (int i = tid; i < din * kThin; i += 256) {
+        const int n = i % kThin, k = i / kThin;
+        s_w[n][k] = n < dout ? W[(size_t)k * dout + n] : __float2bfloat16_rn(0.0f);
+    }
+    __syncthreads();
+    const float b0 = 2 * t < dout ? bias[2 * t] : 0.0f, b1 = 2 * t + 1 < dout ? bias[2 * t + 1] : 0.0f;
+    float ls = 0.0f, le = 0.0f, gs[2] = {0.0f, 0.0f}, ge[2] = {0.0f, 0.0f};
+    for (int r0 = ((int)blockIdx.x * 8 + warp) * 16; r0 < B; r0 += (int)gridDim.x * 8 * 16) {
+        const bool v0 = r0 + g < B, v1 = r0 + g + 8 < B;
+        const bf16* p0 = a + (size_t)(r0 + g) * din + 2 * t;
+        const bf16* p1 = p0 + (size_t)8 * din;
+        float total[4];
+        for (int kb = 0; kb < din; kb += kslice) {
+            const int ke = min(din, kb + kslice);
+            float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+            for (int k = kb; k < ke; k += 16) {
+                uint32_t af[4], bfr[2];
+                af[0] = v0 ? *reinterpret_cast<const uint32_t*>(p0 + k) : 0u;
+                af[1] = v1 ? *reinterpret_cast<const uint32_t*>(p1 + k) : 0u;
+                af[2] = v0 ? *reinterpret_cast<const uint32_t*>(p0 + k + 8) : 0u;
+                af[3] = v1 ? *reinterpret_cast<const uint32_t*>(p1 + k + 8) : 0u;
+                bfr[0] = *reinterpret_cast<const uint32_t*>(&s_w[g][k + 2 * t]);
+                bfr[1] = *reinterpret_cast<const uint32_t*>(&s_w[g][k + 2 * t + 8]);
+                mma_16816(acc, af, bfr);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) total[e] = kb == 0 ? acc[e] : total[e] + acc[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int row = r0 + g + (e >= 2 ? 8 : 0), n = 2 * t + (e & 1);
+            if (row >= B || n >= dout) continue;
+            const size_t at = (size_t)row * dout + n;
+            const float v = total[e] + ((e & 1) ? b1 : b0);
+            if (target) {
+                const float d = v - target[at], gr = scale * d, sq = d * d;
+                dyb[at] = __float2bfloat16_rn(gr);
+                tc::add_exact(ls, le, sq);
+                le += fmaf(d, d, -sq);
+                tc::add_exact(gs[e & 1], ge[e & 1], gr);
+            } else {
+                y[at] = v;
+            }
+        }
+    }
+    if (!target) return;
+    double l = (double)ls + (double)le;
+    double db[2] = {(double)gs[0] + (double)ge[0], (double)gs[1] + (double)ge[1]};
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) {   // over the rows (lanes of equal t)
+        l += __shfl_xor_sync(0xffffffffu, l, o);
+        db[0] += __shfl_xor_sync(0xffffffffu, db[0], o);
+        db[1] += __shfl_xor_sync(0xffffffffu, db[1], o);
+    }
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    if (lane == 0) s_loss[warp] = l;
+    if (lane < 4) {
+        s_db[warp][2 * lane] = db[0];
+        s_db[warp][2 * lane + 1] = db[1];
+    }
+    __syncthreads();
+    if (tid < dout) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += s_db[w][tid];
+        db_part[(size_t)blockIdx.x * dout + tid] = s;
+    }
+    if (tid == 32) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += s_loss[w];
+        loss_part[blockIdx.x] = s;
+    }
+}
+
+// The backward kernels below take four neighbouring columns per thread and four
+// groups of 64 threads on alternate rows (wide loads, many in flight: they are
+// bound by the latency of the activations), added in group order at the end.
+constexpr int kThinRows = 128;   // rows of dy (or x) staged at a time
+
+__device__ __forceinline__ void load4(const bf16* p, float (&v)[4]) {
+    const uint2 raw = *reinterpret_cast<const uint2*>(p);
+    const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.x));
+    const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.y));
+    v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
+}
+
+// Backward step of a narrow output layer over the rows of chunk blockIdx.y, per
+// input column m: dW[m][o] = sum a[b][m] dy[b][o], and (h not null) dz[b][m] =
+// (sum_o dy[b][o] W[m][o]) (1 - h^2) in bf16 with its column sum.  One pass over
+// the rows for all three.  din a multiple of 4.
+template <int DO>
+__global__ void __launch_bounds__(256)
+mlp_narrow_back_kernel(const bf16* __restrict__ a, const float* __restrict__ h,
+                       const bf16* __restrict__ W, const bf16* __restrict__ dyb, int B, int din,
+                       int rows, bf16* __restrict__ dzb, float* __restrict__ dw_part,
+                       double* __restrict__ db_part) {
+    __shared__ float s_dy[kThinRows][DO];
+    __shared__ float s_acc[3][64][4][DO];
+    __shared__ double s_db[3][64][4];
+    const int cg = threadIdx.x & 63, rg = threadIdx.x >> 6;
+    const int m = (blockIdx.x * 64 + cg) * 4;
+    const int r0 = blockIdx.y * rows, r1 = min(B, r0 + rows);
+    const bool on = m < din;
+    float w[4][DO], acc[4][DO], cs[4], ce[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        cs[j] = ce[j] = 0.0f;
+#pragma unroll
+        for (int o = 0; o < DO; ++o) {
+            w[j][o] = on ? bf(W[(size_t)(m + j) * DO + o]) : 0.0f;
+            acc[j][o] = 0.0f;
+        }
+    }
+    for (int c0 = r0; c0 < r1; c0 += kThinRows) {
+        const int n = min(kThinRows, r1 - c0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < n * DO; i += 256)
+            (&s_dy[0][0])[i] = bf(dyb[(size_t)c0 * DO + i]);
+        __syncthreads();
+        if (!on) continue;
+#pragma unroll 4
+        for (int r = rg; r < n; r += 4) {
+            const size_t at = (size_t)(c0 + r) * din + m;
+            float av[4], hv[4];
+            load4(a + at, av);
+            if (h) {
+                const float4 t = *reinterpret_cast<const float4*>(h + at);
+                hv[0] = t.x; hv[1] = t.y; hv[2] = t.z; hv[3] = t.w;
+            }
+            float z[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                z[j] = 0.0f;
+#pragma unroll
+                for (int o = 0; o < DO; ++o) {
+                    const float g = s_dy[r][o];
+                    acc[j][o] = fmaf(av[j], g, acc[j][o]);
+                    z[j] = fmaf(g, w[j][o], z[j]);
+                }
+                if (h) {
+                    z[j] *= 1.0f - hv[j] * hv[j];
+                    tc::add_exact(cs[j], ce[j], z[j]);
+                }
+            }
+            if (h) {
+                __nv_bfloat162 b2[2] = {__floats2bfloat162_rn(z[0], z[1]),
+                                        __floats2bfloat162_rn(z[2], z[3])};
+                *reinterpret_cast<uint2*>(dzb + at) = *reinterpret_cast<uint2*>(b2);
+            }
+        }
+    }
+    if (rg > 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int o = 0; o < DO; ++o) s_acc[rg - 1][cg][j][o] = acc[j][o];
+            s_db[rg - 1][cg][j] = (double)cs[j] + (double)ce[j];
+        }
+    }
+    __syncthreads();
+    if (rg > 0 || !on) return;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int o = 0; o < DO; ++o)
+            dw_part[((size_t)blockIdx.y * din + m + j) * DO + o] =
+                ((acc[j][o] + s_acc[0][cg][j][o]) + s_acc[1][cg][j][o]) + s_acc[2][cg][j][o];
+        if (h)
+            db_part[(size_t)blockIdx.y * din + m + j] =
+                (((double)cs[j] + (double)ce[j]) + s_db[0][cg][j]) + (s_db[1][cg][j] + s_db[2][cg][j]);
+    }
+}
+
+// dW[i][n] = sum over the rows of chunk blockIdx.y of x[b][i] dz[b][n] for DI
+// inputs; dout a multiple of 4
+template <int DI>
+__global__ void __launch_bounds__(256)
+mlp_narrow_in_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dzb, int B, int dout,
+                     int rows, float* __restrict__ dw_part) {
+    __shared__ float s_x[kThinRows][DI];
+    __shared__ float s_acc[3][64][4][DI];
+    const int cg = threadIdx.x & 63, rg = threadIdx.x >> 6;
+    const int n = (blockIdx.x * 64 + cg) * 4;
+    const int r0 = blockIdx.y * rows, r1 = min(B, r0 + rows);
+    const bool on = n < dout;
+    float acc[4][DI];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < DI; ++i) acc[j][i] = 0.0f;
+    for (int c0 = r0; c0 < r1; c0 += kThinRows) {
+        const int cnt = min(kThinRows, r1 - c0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < cnt * DI; i += 256)
+            (&s_x[0][0])[i] = bf(x[(size_t)c0 * DI + i]);
+        __syncthreads();
+        if (!on) continue;
+#pragma unroll 8
+        for (int r = rg; r < cnt; r += 4) {
+            float g[4];
+            load4(dzb + (size_t)(c0 + r) * dout + n, g);
+#pragma unroll
+            for (int i = 0; i < DI; ++i) {
+                const float xv = s_x[r][i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[j][i] = fmaf(xv, g[j], acc[j][i]);
+            }
+        }
+    }
+    if (rg > 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < DI; ++i) s_acc[rg - 1][cg][j][i] = acc[j][i];
+    }
+    __syncthreads();
+    if (rg > 0 || !on) return;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < DI; ++i)
+            dw_part[((size_t)blockIdx.y * DI + i) * dout + n + j] =
+                ((acc[j][i] + s_acc[0][cg][j][i]) + s_acc[1][cg][j][i]) + s_acc[2][cg][j][i];
+}
+
+// The partial sums of one call, all in one launch: item k's output j is the sum
+// over its parts p of src[p n + j].  A block takes 32 neighbouring outputs of
+// one item; its 8 warps take the parts p = warp, warp + 8, ... and are added in
+// warp order.
+struct ReduceItem {
+    const void* src;
+    void* dst;
+    int64_t n;
+    int parts, block0;
+    int wide;        // src: 0 float, 1 double
+    double scale;    // dst is a double, sum * scale, if not 0; else a float
+};
+constexpr int kReduceItems = 2 * ETICS_MLP_MAX_LAYERS + 1;
+struct ReduceList {
+    ReduceItem item[kReduceItems];
+    int count, blocks;
+};
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const __grid_constant__ ReduceList list) {
+    __shared__ double s_d[8][32];
+    __shared__ float s_f[8][32];
+    int k = 0;
+    while (k + 1 < list.count && (int)blockIdx.x >= list.item[k + 1].block0) ++k;
+    const ReduceItem it = list.item[k];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t j = (int64_t)((int)blockIdx.x - it.block0) * 32 + lane;
+    double d = 0.0;
+    float f = 0.0f;
+    if (j < it.n) {
+        if (it.wide) {
+            const double* p = static_cast<const double*>(it.src) + j;
+#pragma unroll 8
+            for (int i = warp; i < it.parts; i += 8) d += p[(size_t)i * it.n];
+        } else {
+            const float* p = static_cast<const float*>(it.src) + j;
+#pragma unroll 8
+            for (int i = warp; i < it.parts; i += 8) f += p[(size_t)i * it.n];
+        }
+    }
+    s_d[warp][lane] = d;
+    s_f[warp][lane] = f;
+    __syncthreads();
+    if (warp != 0 || j >= it.n) return;
+    if (it.wide) {
+        for (int w = 1; w < 8; ++w) d += s_d[w][lane];
+        if (it.scale != 0.0) static_cast<double*>(it.dst)[j] = d * it.scale;
+        else static_cast<float*>(it.dst)[j] = (float)d;
+    } else {
+        for (int w = 1; w < 8; ++w) f += s_f[w][lane];
+        static_cast<float*>(it.dst)[j] = f;
+    }
 }
 
 __global__ void mlp_adam_kernel(float* __restrict__ p, const float* __restrict__ g,
@@ -633,8 +921,14 @@ struct MlpLayout {
     int64_t nparam;
     int dmax;
     // workspace offsets (bytes)
-    size_t h32[5], hb[5], y32, dz32[2], dzb[2], part, loss_blocks, colsum, total;
+    size_t h32[5], hb[5], y32, dz32[2], dzb[2], part, loss_blocks, colsum;
+    size_t wpart[5], bpart[5];         // a layer's partial weight and bias gradients
+    size_t total;
+    bool narrow_out;                   // the output layer runs on the narrow kernels
 };
+
+// whether the weight gradient of layer i runs on the narrow kernel
+bool narrow_in(const MlpLayout& o, int i) { return o.d[i] <= kThin && o.d[i + 1] % 4 == 0; }
 
 bool valid_shape(const etics_mlp_shape* s) {
     if (!s || s->nlayers < 1 || s->nlayers > ETICS_MLP_MAX_LAYERS) return false;
@@ -672,6 +966,16 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
         o.dz32[k] = off; off += al256(Bz * o.dmax * 4);
         o.dzb[k] = off;  off += al256(Bz * o.dmax * 2);
     }
+    o.narrow_out = o.d[o.L] <= kThin && o.d[o.L - 1] % 16 == 0 && o.d[o.L - 1] <= kThinInputs;
+    for (int i = 0; i < o.L; ++i) {
+        const GemmShape w = gemm_shape(o.d[i], o.d[i + 1], (int)Bz);
+        const size_t parts = (size_t)std::max(w.splits, kThinBlocks);
+        const bool narrow = narrow_in(o, i) || (i == o.L - 1 && o.narrow_out);
+        o.wpart[i] = off;
+        off += al256((narrow ? parts : (size_t)w.splits) * o.d[i] * o.d[i + 1] * 4);
+        o.bpart[i] = off;
+        off += al256(std::max((size_t)kThinBlocks, (Bz + tc::kM - 1) / tc::kM) * o.d[i + 1] * 8);
+    }
     // the largest split-K partial buffer over all products
     size_t pmax = 0;
     for (int i = 0; i < o.L; ++i) {
@@ -685,7 +989,7 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
         }
     }
     o.part = off; off += al256(pmax * 4);
-    o.loss_blocks = off; off += al256(kLossBlocks * 8);
+    o.loss_blocks = off; off += al256(std::max(kLossBlocks, kThinBlocks) * 8);
     o.colsum = off; off += al256((size_t)kColChunks * o.dmax * 8);
     o.total = off;
     return o;
@@ -738,22 +1042,43 @@ bool operand_map(CUtensorMap* map, const bf16* X, int64_t ld, int R, int K, bool
            CUDA_SUCCESS;
 }
 
-// product + epilogue
+// product + epilogue.  colsum (nullable): where the column sums of the result
+// go, one row per row of 128-row tiles; *colsum_rows is set to that number, or
+// to 0 where this product does not make them (the caller sums the columns).
+// part_only: a split product is left as its slices in part (their number in
+// *splits); an unsplit one goes to out.
+struct GemmOut {
+    const float* bias = nullptr;
+    int act = 0;
+    const float* h = nullptr;
+    float* out = nullptr;
+    bf16* out_b = nullptr;
+    double* colsum = nullptr;
+    int* colsum_rows = nullptr;
+    int* splits = nullptr;   // not null: part_only
+};
+
 template <bool TA, bool TB>
 int gemm(const bf16* A, int64_t lda, const bf16* Bm, int64_t ldb, int M, int N, int K, float* part,
-         const float* bias, int act, const float* h, float* out, bf16* out_b,
-         const LaunchCtx& ctx) {
+         const GemmOut& g, const LaunchCtx& ctx) {
     const GemmShape s = gemm_shape(M, N, K);
     stage_event(ctx, 0);
+    if (g.colsum_rows) *g.colsum_rows = 0;
+    if (g.splits) *g.splits = s.splits;
     CUtensorMap ma, mb;
+    tc::Epilogue ep{};
     if (s.tc && operand_map(&ma, A, lda, M, K, TA) && operand_map(&mb, Bm, ldb, N, K, TB)) {
         auto k = tc::gemm_tma_kernel<TA, TB>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tc::kSmemTmaBytes))
             return ETICS_ERR_CUDA;
-        dim3 grid((N + tc::kN - 1) / tc::kN, (M + tc::kM - 1) / tc::kM, s.splits);
-        k<<<grid, tc::kThreads, tc::kSmemTmaBytes, ctx.stream>>>(ma, mb, part, M, N, K, s.kslice,
-                                                                 ctx.err);
+        const dim3 grid((N + tc::kN - 1) / tc::kN, (M + tc::kM - 1) / tc::kM, s.splits);
+        if (s.splits == 1) {
+            ep = tc::Epilogue{1, g.act, g.bias, g.h, g.out, g.out_b, g.colsum};
+            if (g.colsum && g.colsum_rows) *g.colsum_rows = (int)grid.y;
+        }
+        k<<<grid, tc::kTmaThreads, tc::kSmemTmaBytes, ctx.stream>>>(ma, mb, part, M, N, K, s.kslice,
+                                                                    ep, ctx.err);
     } else if (s.tc) {
         auto k = tc::gemm_kernel<TA, TB>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -768,29 +1093,71 @@ int gemm(const bf16* A, int64_t lda, const bf16* Bm, int64_t ldb, int M, int N, 
                                                                       N, K, s.kslice);
     }
     if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    ++*ctx.launches;
     stage_event(ctx, 1);
-    mlp_epilogue_kernel<<<grid_1d((int64_t)M * N, ctx), 256, 0, ctx.stream>>>(
-        part, s.splits, M, N, bias, act, h, out, out_b);
-    if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    if (!ep.on && !(g.splits && s.splits > 1)) {
+        mlp_epilogue_kernel<<<grid_1d((int64_t)M * N, ctx), 256, 0, ctx.stream>>>(
+            part, s.splits, M, N, g.bias, g.act, g.h, g.out, g.out_b);
+        if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        ++*ctx.launches;
+    }
     stage_event(ctx, 2);
-    *ctx.launches += 2;
     return ETICS_OK;
 }
 
-// forward pass; activations stay in ws for the backward pass
+// the narrow kernels for the run-time width W (1..kThin)
+#define ETICS_NARROW(W, KERNEL, ...)                                        \
+    switch (W) {                                                            \
+        case 1: KERNEL<1> __VA_ARGS__; break;                               \
+        case 2: KERNEL<2> __VA_ARGS__; break;                               \
+        case 3: KERNEL<3> __VA_ARGS__; break;                               \
+        case 4: KERNEL<4> __VA_ARGS__; break;                               \
+        case 5: KERNEL<5> __VA_ARGS__; break;                               \
+        case 6: KERNEL<6> __VA_ARGS__; break;                               \
+        case 7: KERNEL<7> __VA_ARGS__; break;                               \
+        default: KERNEL<8> __VA_ARGS__; break;                              \
+    }
+
+// the narrow output layer: y, or with a target the loss and dy
+int narrow_out(const MlpLayout& o, const float* params, const bf16* pb, const bf16* a, int B,
+               const float* target, float scale, float* y, bf16* dyb, void* ws, int* parts,
+               const LaunchCtx& ctx) {
+    const int i = o.L - 1;
+    const int blocks = std::min((B + 127) / 128, kThinBlocks);
+    mlp_narrow_out_kernel<<<blocks, 256, 0, ctx.stream>>>(
+        a, pb + o.woff[i], params + o.boff[i], target, B, o.d[i], o.d[o.L],
+        gemm_shape(B, o.d[o.L], o.d[i]).kslice, scale, y, dyb, at<double>(ws, o.loss_blocks),
+        at<double>(ws, o.bpart[i]));
+    if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    ++*ctx.launches;
+    *parts = blocks;
+    return ETICS_OK;
+}
+
+// forward pass of layers 0..last; activations stay in ws for the backward
+// pass; the output layer (if included) writes y
 int forward_impl(const MlpLayout& o, const float* params, const bf16* pb, const bf16* x, int B,
-                 float* y, void* ws, const LaunchCtx& ctx) {
+                 int layers, float* y, void* ws, const LaunchCtx& ctx) {
     const bf16* a = x;
-    for (int i = 0; i < o.L; ++i) {
+    for (int i = 0; i < layers; ++i) {
         const bool last = i == o.L - 1;
-        int rc = gemm<false, true>(a, o.d[i], pb + o.woff[i], o.d[i + 1], B, o.d[i + 1], o.d[i],
-                                   at<float>(ws, o.part), params + o.boff[i], last ? 0 : 1,
-                                   nullptr, last ? y : at<float>(ws, o.h32[i]),
-                                   last ? nullptr : at<bf16>(ws, o.hb[i]), ctx);
+        GemmOut g;
+        g.bias = params + o.boff[i];
+        g.act = last ? 0 : 1;
+        g.out = last ? y : at<float>(ws, o.h32[i]);
+        g.out_b = last ? nullptr : at<bf16>(ws, o.hb[i]);
+        const int rc = gemm<false, true>(a, o.d[i], pb + o.woff[i], o.d[i + 1], B, o.d[i + 1],
+                                         o.d[i], at<float>(ws, o.part), g, ctx);
         if (rc) return rc;
         if (!last) a = at<bf16>(ws, o.hb[i]);
     }
     return ETICS_OK;
+}
+
+// whether the narrow output kernels take this call (their loads of the layer's
+// input are up to 8 bytes wide: the caller's x may be less aligned)
+bool narrow_now(const MlpLayout& o, const bf16* x) {
+    return o.narrow_out && (o.L > 1 || (reinterpret_cast<uintptr_t>(x) & 7) == 0);
 }
 
 }  // namespace
@@ -812,8 +1179,14 @@ int mlp_forward(const etics_mlp_shape* s, const float* params, const uint16_t* p
     const MlpLayout o = mlp_layout(s, B);
     if (ws_bytes < o.total) return ETICS_ERR_WORKSPACE;
     if (B == 0) return ETICS_OK;
-    return forward_impl(o, params, reinterpret_cast<const bf16*>(pb),
-                        reinterpret_cast<const bf16*>(x), B, y, ws, ctx);
+    const bf16* w = reinterpret_cast<const bf16*>(pb);
+    const bf16* xb = reinterpret_cast<const bf16*>(x);
+    if (!narrow_now(o, xb)) return forward_impl(o, params, w, xb, B, o.L, y, ws, ctx);
+    const int rc = forward_impl(o, params, w, xb, B, o.L - 1, y, ws, ctx);
+    if (rc) return rc;
+    int parts = 0;
+    return narrow_out(o, params, w, o.L > 1 ? at<bf16>(ws, o.hb[o.L - 2]) : xb, B, nullptr, 0.0f, y,
+                      nullptr, ws, &parts, ctx);
 }
 
 int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t* pbits,
@@ -824,49 +1197,110 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
     if (B == 0) return ETICS_ERR_ARG;
     const bf16* pb = reinterpret_cast<const bf16*>(pbits);
     const bf16* x = reinterpret_cast<const bf16*>(xbits);
-    float* y = at<float>(ws, o.y32);
-    int rc = forward_impl(o, params, pb, x, B, y, ws, ctx);
-    if (rc) return rc;
     const int L = o.L;
     const int64_t count = (int64_t)B * o.d[L];
+    const float scale = (float)(2.0 / (double)count);
+    const bool narrow = narrow_now(o, x);
+    float* y = at<float>(ws, o.y32);
+    int rc = forward_impl(o, params, pb, x, B, narrow ? L - 1 : L, y, ws, ctx);
+    if (rc) return rc;
+    // partial sums to be added at the end, all in one launch
+    ReduceList list{};
+    auto reduce = [&](const void* src, void* dst, int64_t n, int parts, int wide, double sc) {
+        list.item[list.count++] = ReduceItem{src, dst, n, parts, list.blocks, wide, sc};
+        list.blocks += (int)((n + 31) / 32);
+    };
+    // rows per chunk of the narrow kernels
+    const int rows = std::max(16, (B + kThinBlocks - 1) / kThinBlocks);
+    const int chunks = (B + rows - 1) / rows;
     int cur = 0;
-    mlp_mse_kernel<<<kLossBlocks, 256, 0, ctx.stream>>>(
-        y, target, count, (float)(2.0 / (double)count), at<float>(ws, o.dz32[cur]),
-        at<bf16>(ws, o.dzb[cur]), at<double>(ws, o.loss_blocks));
-    if (cudaGetLastError()) return ETICS_ERR_CUDA;
-    mlp_loss_final_kernel<<<1, 32, 0, ctx.stream>>>(at<double>(ws, o.loss_blocks), kLossBlocks,
-                                                    1.0 / (double)count, loss);
-    if (cudaGetLastError()) return ETICS_ERR_CUDA;
-    *ctx.launches += 2;
-    for (int i = L - 1; i >= 0; --i) {
+    int top = L - 1;       // the layer whose dz is in dz32/dzb[cur]
+    int sums = 0;          // rows of its column sums in bpart[top]; 0: not made
+    if (narrow) {
+        const int din = o.d[L - 1], dout = o.d[L];
+        const bf16* a = L > 1 ? at<bf16>(ws, o.hb[L - 2]) : x;
+        bf16* dyb = at<bf16>(ws, o.dzb[cur]);
+        int parts = 0;
+        rc = narrow_out(o, params, pb, a, B, target, scale, nullptr, dyb, ws, &parts, ctx);
+        if (rc) return rc;
+        reduce(at<double>(ws, o.loss_blocks), loss, 1, parts, 1, 1.0 / (double)count);
+        reduce(at<double>(ws, o.bpart[L - 1]), grads + o.boff[L - 1], dout, parts, 1, 0.0);
+        const dim3 grid((din + 255) / 256, chunks);   // 64 threads of four columns
+        ETICS_NARROW(dout, mlp_narrow_back_kernel,
+                     <<<grid, 256, 0, ctx.stream>>>(
+                         a, L > 1 ? at<float>(ws, o.h32[L - 2]) : nullptr, pb + o.woff[L - 1], dyb, B,
+                         din, rows, at<bf16>(ws, o.dzb[cur ^ 1]), at<float>(ws, o.wpart[L - 1]),
+                         L > 1 ? at<double>(ws, o.bpart[L - 2]) : nullptr));
+        if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        ++*ctx.launches;
+        reduce(at<float>(ws, o.wpart[L - 1]), grads + o.woff[L - 1], (int64_t)din * dout, chunks, 0, 0.0);
+        cur ^= 1;
+        top = L - 2;
+        sums = chunks;
+    } else {
+        mlp_mse_kernel<<<kLossBlocks, 256, 0, ctx.stream>>>(
+            y, target, count, scale, at<float>(ws, o.dz32[cur]), at<bf16>(ws, o.dzb[cur]),
+            at<double>(ws, o.loss_blocks));
+        if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        ++*ctx.launches;
+        reduce(at<double>(ws, o.loss_blocks), loss, 1, kLossBlocks, 1, 1.0 / (double)count);
+    }
+    for (int i = top; i >= 0; --i) {
         const int din = o.d[i], dout = o.d[i + 1];
         const bf16* a_in = i == 0 ? x : at<bf16>(ws, o.hb[i - 1]);
         const bf16* dzb = at<bf16>(ws, o.dzb[cur]);
         // dW_i = a_in^T dz
-        rc = gemm<true, true>(a_in, din, dzb, dout, din, dout, B, at<float>(ws, o.part), nullptr, 0,
-                              nullptr, grads + o.woff[i], nullptr, ctx);
-        if (rc) return rc;
-        {
-            const int rows = (B + kColChunks - 1) / kColChunks;
-            const int chunks = (B + rows - 1) / rows;
-            const dim3 g1((dout + 127) / 128, chunks);
-            mlp_colsum_partial_kernel<<<g1, 128, 0, ctx.stream>>>(
-                at<float>(ws, o.dz32[cur]), B, dout, rows, at<double>(ws, o.colsum));
-            mlp_colsum_final_kernel<<<(dout + 127) / 128, 128, 0, ctx.stream>>>(
-                at<double>(ws, o.colsum), chunks, dout, grads + o.boff[i]);
+        if (narrow_in(o, i)) {
+            const dim3 grid((dout + 255) / 256, chunks);
+            ETICS_NARROW(din, mlp_narrow_in_kernel,
+                         <<<grid, 256, 0, ctx.stream>>>(a_in, dzb, B, dout, rows,
+                                                        at<float>(ws, o.wpart[i])));
             if (cudaGetLastError()) return ETICS_ERR_CUDA;
-            *ctx.launches += 2;
+            ++*ctx.launches;
+            reduce(at<float>(ws, o.wpart[i]), grads + o.woff[i], (int64_t)din * dout, chunks, 0, 0.0);
+        } else {
+            int splits = 0;
+            GemmOut g;
+            g.out = grads + o.woff[i];
+            g.splits = &splits;
+            rc = gemm<true, true>(a_in, din, dzb, dout, din, dout, B, at<float>(ws, o.wpart[i]), g, ctx);
+            if (rc) return rc;
+            if (splits > 1)
+                reduce(at<float>(ws, o.wpart[i]), grads + o.woff[i], (int64_t)din * dout, splits, 0, 0.0);
         }
+        // db_i: the column sums of dz, made along with it or from its FP32 copy
+        if (sums == 0) {
+            const int crows = (B + kColChunks - 1) / kColChunks;
+            sums = (B + crows - 1) / crows;
+            mlp_colsum_partial_kernel<<<dim3((dout + 127) / 128, sums), 128, 0, ctx.stream>>>(
+                at<float>(ws, o.dz32[cur]), B, dout, crows, at<double>(ws, o.bpart[i]));
+            if (cudaGetLastError()) return ETICS_ERR_CUDA;
+            ++*ctx.launches;
+        }
+        reduce(at<double>(ws, o.bpart[i]), grads + o.boff[i], dout, sums, 1, 0.0);
         if (i > 0) {
             // dz_{i-1} = (dz W_i^T) * (1 - h_{i-1}^2)
             const int nxt = cur ^ 1;
+            GemmOut g;
+            g.h = at<float>(ws, o.h32[i - 1]);
+            // the FP32 copy is read only where the column sums are not made here
+            const GemmShape gs = gemm_shape(B, din, dout);
+            g.out = gs.tc && gs.splits == 1 && din % 8 == 0 && dout % 8 == 0 &&
+                            (reinterpret_cast<uintptr_t>(pb + o.woff[i]) & 15) == 0 && encode_tiled()
+                        ? nullptr : at<float>(ws, o.dz32[nxt]);
+            g.out_b = at<bf16>(ws, o.dzb[nxt]);
+            g.colsum = at<double>(ws, o.bpart[i - 1]);
+            g.colsum_rows = &sums;
             rc = gemm<false, false>(dzb, dout, pb + o.woff[i], dout, B, din, dout,
-                                    at<float>(ws, o.part), nullptr, 0, at<float>(ws, o.h32[i - 1]),
-                                    at<float>(ws, o.dz32[nxt]), at<bf16>(ws, o.dzb[nxt]), ctx);
+                                    at<float>(ws, o.part), g, ctx);
             if (rc) return rc;
+            if (sums == 0 && !g.out) return ETICS_ERR_CUDA;   // not reached: the test above is gemm's own
             cur = nxt;
         }
     }
+    mlp_reduce_kernel<<<list.blocks, 256, 0, ctx.stream>>>(list);
+    if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    ++*ctx.launches;
     return ETICS_OK;
 }
 

@@ -374,10 +374,40 @@ __device__ __forceinline__ uint64_t tile_desc(uint32_t addr, int kk) {
               : make_desc_sw128(addr + (uint32_t)kk * 32u, 16u, 1024u);
 }
 
+// What happens to the product of an unsplit K (on): + bias, tanh, times the
+// tanh derivative 1 - h^2, to FP32 and / or bf16, and the column sums of the
+// FP32 result over the tile's rows (for a bias gradient; double per row of
+// tiles).  In the product kernel it saves writing and reading the FP32 product
+// once and a launch.
+struct Epilogue {
+    int on, act;
+    const float* bias;   // nullable, as all pointers
+    const float* h;
+    float* out;
+    bf16* out_b;
+    double* colsum;      // [row of tiles][N]
+};
+
+// s + e accumulates x with the rounding errors kept (two-sum): as good as an
+// FP64 sum for the lengths here, without FP64 instructions (slow on this GPU)
+__device__ __forceinline__ void add_exact(float& s, float& e, float x) {
+    const float t = s + x, b = t - s;
+    e += (s - (t - b)) + (x - b);
+    s = t;
+}
+
+// Eight warps: the read-back (each warp 32 rows by 64 columns of the tile,
+// staged through shared memory so that every global access covers whole rows
+// of 256 bytes) is what the products of the networks here spend their time
+// on; a row per thread with 128-byte pieces cost 30 us at 19440 x 256 x 256.
+constexpr int kTmaThreads = 256;
+constexpr int kStageRow = kN + 4;   // floats; rows 16 bytes apart in the banks
+
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kTmaThreads, 2)
 gemm_tma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                float* __restrict__ part, int M, int N, int K, int kslice, unsigned* err) {
+                float* __restrict__ part, int M, int N, int K, int kslice, Epilogue ep,
+                unsigned* err) {
     extern __shared__ unsigned char smem_raw[];
     SmemTma& sm = *reinterpret_cast<SmemTma*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~uintptr_t(1023));
@@ -461,24 +491,97 @@ gemm_tma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (!ok && tid == 0) report(err, ETICS_ERR_TIMEOUT);
     tc_fence_after();
     if (ok) {
-        // warp w reads TMEM lanes 32w..32w+31 = tile rows 32w.., 32 columns at a time
-        const int row = m0 + warp * 32 + lane;
-        float* out = part + (size_t)blockIdx.z * M * N;
-#pragma unroll 1
-        for (int c0 = 0; c0 < kN; c0 += 32) {
+        // the ring is idle: every copy has been consumed by a completed MMA
+        static_assert(kM * kStageRow * 4 + 4 * kN * 8 <= 2 * kTmaStages * (int)kTileBytes, "staging");
+        float* stage = reinterpret_cast<float*>(sm.a[0]);
+        double* csum = reinterpret_cast<double*>(stage + kM * kStageRow);   // [4][kN]
+        const int q = warp & 3, half = warp >> 2;   // rows 32q.., columns 64 half..
+#pragma unroll
+        for (int c = 0; c < 64; c += 32) {
             float v[32];
             if (nk > 0) {
-                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 64 + c), v);
             } else {
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] = 0.0f;
             }
-            if (row < M) {
-                float* dst = out + (size_t)row * N + n0 + c0;
+            float4* dst = reinterpret_cast<float4*>(stage + (q * 32 + lane) * kStageRow + half * 64 + c);
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (n0 + c0 + i < N) dst[i] = v[i];
+            for (int i = 0; i < 8; ++i)
+                dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+        __syncwarp();
+        const int cl = half * 64 + (lane & 15) * 4, gc = n0 + cl;
+        float* out = ep.on ? ep.out : part + (size_t)blockIdx.z * M * N;
+        // four columns at once where rows and pointers allow (a weight gradient
+        // may start at any float)
+        const bool vec = (N & 3) == 0 && gc + 4 <= N &&
+                         ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(ep.h) |
+                           2 * reinterpret_cast<uintptr_t>(ep.out_b)) & 15) == 0;
+        float bias[4] = {0.f, 0.f, 0.f, 0.f}, cs[4] = {0.f, 0.f, 0.f, 0.f}, ce[4] = {0.f, 0.f, 0.f, 0.f};
+        if (ep.on && ep.bias) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (gc + j < N) bias[j] = ep.bias[gc + j];
+        }
+#pragma unroll 4
+        for (int i = 0; i < 16; ++i) {
+            const int r = q * 32 + 2 * i + (lane >> 4), row = m0 + r;
+            if (row >= M || gc >= N) continue;
+            const float4 s4 = *reinterpret_cast<const float4*>(stage + r * kStageRow + cl);
+            float s[4] = {s4.x, s4.y, s4.z, s4.w};
+            const size_t at = (size_t)row * N + gc;
+            if (ep.on) {
+                float hv[4];
+                if (ep.h) {
+                    if (vec) {
+                        const float4 t4 = *reinterpret_cast<const float4*>(ep.h + at);
+                        hv[0] = t4.x; hv[1] = t4.y; hv[2] = t4.z; hv[3] = t4.w;
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) hv[j] = gc + j < N ? ep.h[at + j] : 0.0f;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (ep.bias) s[j] += bias[j];
+                    if (ep.act) s[j] = tanhf(s[j]);
+                    if (ep.h) s[j] *= 1.0f - hv[j] * hv[j];
+                    if (ep.colsum) add_exact(cs[j], ce[j], s[j]);
+                }
+                if (ep.out_b) {
+                    if (vec) {
+                        __nv_bfloat162 b2[2] = {__floats2bfloat162_rn(s[0], s[1]),
+                                                __floats2bfloat162_rn(s[2], s[3])};
+                        *reinterpret_cast<uint2*>(ep.out_b + at) = *reinterpret_cast<uint2*>(b2);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (gc + j < N) ep.out_b[at + j] = __float2bfloat16_rn(s[j]);
+                    }
+                }
             }
+            if (out) {
+                if (vec) {
+                    *reinterpret_cast<float4*>(out + at) = make_float4(s[0], s[1], s[2], s[3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (gc + j < N) out[at + j] = s[j];
+                }
+            }
+        }
+        if (ep.on && ep.colsum) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                double d = (double)cs[j] + (double)ce[j];
+                d += __shfl_xor_sync(0xffffffffu, d, 16);
+                if (lane < 16) csum[q * kN + cl + j] = d;
+            }
+            __syncthreads();
+            if (tid < kN && n0 + tid < N)
+                ep.colsum[(size_t)blockIdx.y * N + n0 + tid] =
+                    (csum[tid] + csum[kN + tid]) + (csum[2 * kN + tid] + csum[3 * kN + tid]);
         }
     }
     tc_fence_before();

@@ -303,3 +303,31 @@ def test_forecast_meets_the_stated_budget():
     assert passed_f >= 14, st_f.checks
     assert passed_h <= 2, st_h.checks
     assert st_f.forecasts >= 28, st_f.forecasts
+
+
+# layers at most 8 wide on one side have kernels of their own where the other
+# side is a multiple of 4 (weight gradient of the input) or of 16 up to 1024
+# (output layer): each width class, both sides of the lines, row counts around
+# the 16 rows of a fragment and the 128 of a block
+@pytest.mark.parametrize("dims,batch", [([1, 64, 1], 1), ([3, 68, 8], 129), ([8, 16, 1], 257),
+                                        ([4, 6, 16, 5], 130), ([8, 1024, 2], 33),
+                                        ([8, 1040, 2], 33), ([16, 3], 131), ([64, 64, 7], 4097)])
+def test_narrow_layers_match_oracle(dims, batch):
+    test_forward_matches_oracle(dims, batch)
+    test_gradient_matches_oracle(dims, batch)
+
+
+def test_narrow_output_layer_of_an_unaligned_input():
+    """A one-layer network reads the caller's x, which may start anywhere."""
+    dims, batch = [16, 3], 131
+    net, _ = _net(dims, seed=3)
+    x, _, tg, _ = _data(dims, batch, seed=4)
+    buf = torch.empty(x.numel() + 1, dtype=x.dtype, device="cuda")
+    odd = buf[1:].view(x.shape)
+    odd.copy_(x)
+    y = net.forward(x).clone()
+    loss = net.loss_grad(x, tg).item()
+    g = net.grads.clone()
+    assert torch.allclose(net.forward(odd), y, rtol=1e-5, atol=1e-6)
+    assert abs(net.loss_grad(odd, tg).item() - loss) <= 1e-6 * loss
+    assert _rel(net.grads.cpu().numpy(), g.cpu().numpy()) < 1e-5
