@@ -17,8 +17,18 @@ size_t scf_bins148_workspace_f32(int num_sms);
 int scf_coeffs_bins148_f32(const void* posm, int64_t N, double* coeffs, void* ws,
                            const LaunchCtx& ctx);
 size_t scf_workspace_f64(int64_t N, int n_max, int l_max, int num_sms);
-int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
-                   const LaunchCtx& ctx);
+int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, int basis, double* coeffs,
+                   void* ws, const LaunchCtx& ctx);
+// its parts, by the number of rows (n_max + 1 rounded up to an odd number)
+#define ETICS_COEFF_PART(k)                                                                      \
+    size_t scf_coeffs_f32_##k##_workspace(int rows, int num_sms);                                \
+    int scf_coeffs_f32_##k(int rows, const void* posm, int64_t N, int n_max, int l_max, int basis, \
+                           double* coeffs, void* ws, const LaunchCtx& ctx)
+ETICS_COEFF_PART(a);
+ETICS_COEFF_PART(b);
+ETICS_COEFF_PART(c);
+ETICS_COEFF_PART(d);
+#undef ETICS_COEFF_PART
 int scf_coeffs_f64(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
                    const LaunchCtx& ctx);
 
@@ -45,8 +55,6 @@ ETICS_FIELD_PART(scf_field_f64_cb_high);
 #undef ETICS_FIELD_PART
 
 // ---- SCF with the Clutton-Brock radial basis (etics_scf_cb_f32/f64.cu) ------
-int scf_coeffs_cb_f32(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
-                      const LaunchCtx& ctx);
 int scf_coeffs_cb_f64(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
                       const LaunchCtx& ctx);
 

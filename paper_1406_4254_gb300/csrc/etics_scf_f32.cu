@@ -1,25 +1,37 @@
 // etics_scf_f32.cu -- mixed-precision SCF instantiation (FP32 basis and field
 // sums, FP64 coefficient accumulation).
+#include <algorithm>
+
 #include "etics_internal.h"
-#include "etics_scf_bins.cuh"
+#include "etics_scf_coeffs.cuh"
+#include "etics_scf_impl.cuh"
 
 namespace etics {
 size_t scf_workspace_f32(int64_t N, int n_max, int l_max, int num_sms) {
-    size_t a = scf_workspace<float>(N, n_max, l_max, num_sms);
-    size_t b = 0;
-    if (n_max == 10 && l_max == 6) b = scf_pairs106_workspace_f32(num_sms);
-    if (n_max == 14 && l_max == 8) b = scf_bins148_workspace_f32(num_sms);
-    return a > b ? a : b;
+    const int rows = coeff_rows(n_max);
+    const auto need = rows <= 7 ? scf_coeffs_f32_a_workspace : rows <= 11 ? scf_coeffs_f32_b_workspace
+                      : rows <= 15 ? scf_coeffs_f32_c_workspace : scf_coeffs_f32_d_workspace;
+    // at least what the register-tile kernel takes (the FP64 path's, and this
+    // path's before it ran on particle pairs)
+    size_t most = scf_workspace<float>(N, n_max, l_max, num_sms);
+    most = std::max(most, need(rows, num_sms));
+    if (n_max == 10 && l_max == 6) most = std::max(most, scf_pairs106_workspace_f32(num_sms));
+    if (n_max == 14 && l_max == 8) most = std::max(most, scf_bins148_workspace_f32(num_sms));
+    return most;
 }
-int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, double* coeffs, void* ws,
-                   const LaunchCtx& ctx) {
-    // specialised kernels for the paper's (10, 6) and (14, 8) expansions:
-    // particle pairs on paired FP32 instructions, one level per warp (10, 6);
-    // per-warp bins (14, 8)
-    if (n_max == 10 && l_max == 6)
+int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, int basis, double* coeffs,
+                   void* ws, const LaunchCtx& ctx) {
+    // the paper's (10, 6) and the forecast experiment's (14, 8) expansion have
+    // kernels with their bins known at compile time: (10, 6) at 2^20 54 us
+    // against 72 with the general kernel, (14, 8) at 2^22 560 against 718
+    if (basis == ETICS_BASIS_HO && n_max == 10 && l_max == 6)
         return scf_coeffs_pairs106_f32(posm, N, coeffs, ws, ctx);
-    if (n_max == 14 && l_max == 8) return scf_coeffs_bins148_f32(posm, N, coeffs, ws, ctx);
-    return scf_coeffs_launch<float>(posm, N, n_max, l_max, coeffs, ws, ctx);
+    if (basis == ETICS_BASIS_HO && n_max == 14 && l_max == 8)
+        return scf_coeffs_bins148_f32(posm, N, coeffs, ws, ctx);
+    const int rows = coeff_rows(n_max);
+    const auto run = rows <= 7 ? scf_coeffs_f32_a : rows <= 11 ? scf_coeffs_f32_b
+                     : rows <= 15 ? scf_coeffs_f32_c : scf_coeffs_f32_d;
+    return run(rows, posm, N, n_max, l_max, basis, coeffs, ws, ctx);
 }
 int scf_field_f32(const void* posm, int64_t N, int n_max, int l_max, int basis,
                   const double* coeffs, void* out, int out_mask, FieldKick kick,

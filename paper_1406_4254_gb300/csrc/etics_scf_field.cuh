@@ -383,7 +383,9 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     // blocks on part of the SMs (small N) nor a last round that is nearly
     // empty leaves the GPU idle.  Where a quarter of the threads would do, the
     // levels are split over four warps (mixed precision: the FP64 kernel is
-    // bound by the FP64 pipe at any size, and repeats the harmonics).
+    // bound by the FP64 pipe at any size, and repeats the harmonics): (10, 6)
+    // 13 us up to 38912 particles, 17 with one warp for all levels; (14, 8) 17
+    // to 21 and 23 to 25 around 29184; l_max 10 19 and 27 around 19456.
     constexpr int kMost = field_threads<LM>();
     const int64_t lanes = (N + FieldLane<P>::kParticles - 1) / FieldLane<P>::kParticles;
     const int parts = sizeof(R) == 4 && l_max >= 2 &&
