@@ -105,12 +105,11 @@ struct ScfBinParams {
     unsigned* err;
 };
 
-// contributions of one particle to segment S of bin B: the Gegenbauer values
-// of the segment's level times the (mass and radial prefactor scaled)
-// harmonics of its columns
+// rows of segment S of bin B and the segments after it for one particle: the
+// Gegenbauer values of the segment's level times its columns y (harmonics
+// scaled by mass and radial prefactor)
 template <typename R, int NR, int LM, int B, int S>
-__device__ __forceinline__ void bin_segment(R (&acc)[NR][kBinCap], const R* Ys, int T, int k,
-                                            R xi, R w0, R st) {
+__device__ __forceinline__ void bin_segment(R (&acc)[NR][kBinCap], const R (&y)[kBinCap], R xi) {
     constexpr BinDef bd = BinConst<LM>::plan.bin[B];
     if constexpr (S < bd.nseg) {
         constexpr BinSeg g = bd.seg[S];
@@ -119,73 +118,150 @@ __device__ __forceinline__ void bin_segment(R (&acc)[NR][kBinCap], const R* Ys, 
             for (int s = 0; s < S; ++s) o += BinConst<LM>::plan.bin[B].seg[s].n;
             return o;
         }();
-        // w_l = m * (-(1+r)^-1) * (r/(1+r)^2)^l
-        R w = w0;
-#pragma unroll
-        for (int i = 0; i < g.l; ++i) w *= st;
-        R y[g.n];
-#pragma unroll
-        for (int c = 0; c < g.n; ++c) y[c] = w * Ys[(size_t)(g.l * g.l + g.c0 + c) * T + k];
         R cm1 = R(0), cn = R(1);
 #pragma unroll
         for (int n = 0; n < NR; ++n) {
-            if (n > 0) {
+            if (n == 1) {
+                cm1 = cn;
+                cn = xi;
+            } else if (n > 1) {
                 const R cnew = fma(xi, cn, -geg_bs<R>(g.l, n) * cm1);   // rescaled
                 cm1 = cn;
                 cn = cnew;
             }
 #pragma unroll
-            for (int c = 0; c < g.n; ++c) acc[n][off + c] = fma(cn, y[c], acc[n][off + c]);
+            for (int c = 0; c < g.n; ++c)
+                acc[n][off + c] = n == 0 ? acc[n][off + c] + y[off + c]
+                                         : fma(cn, y[off + c], acc[n][off + c]);
         }
-        bin_segment<R, NR, LM, B, S + 1>(acc, Ys, T, k, xi, w0, st);
+        bin_segment<R, NR, LM, B, S + 1>(acc, y, xi);
+    }
+}
+template <typename R, int LM, int T, int B, int S = 0>
+__device__ __forceinline__ void bin_load(R (&y)[kBinCap], const R* Ys, int k) {
+    constexpr BinDef bd = BinConst<LM>::plan.bin[B];
+    if constexpr (S < bd.nseg) {
+        constexpr BinSeg g = bd.seg[S];
+        constexpr int off = [] {
+            int o = 0;
+            for (int s = 0; s < S; ++s) o += BinConst<LM>::plan.bin[B].seg[s].n;
+            return o;
+        }();
+#pragma unroll
+        for (int c = 0; c < g.n; ++c) y[off + c] = Ys[(g.l * g.l + g.c0 + c) * T + k];
+        bin_load<R, LM, T, B, S + 1>(y, Ys, k);
     }
 }
 
-template <typename R, int NR, int LM, int B>
-__device__ __forceinline__ void bin_tile(R (&acc)[NR][kBinCap], const R* Ys, const Vec4<R>* s_rad,
-                                         int T, int lane) {
+// the lane's particles of one tile; the next one's values are loaded before
+// this one's rows
+template <typename R, int NR, int LM, int T, int B>
+__device__ __forceinline__ void bin_tile(R (&acc)[NR][kBinCap], const R* Ys, const R* Xs, int lane) {
+    R y[kBinCap], xi = Xs[lane];
+    bin_load<R, LM, T, B>(y, Ys, lane);
 #pragma unroll 1
     for (int k = lane; k < T; k += 32) {
-        const Vec4<R> rd = s_rad[k];   // (xi, st, w0, -)
-        bin_segment<R, NR, LM, B, 0>(acc, Ys, T, k, rd.x, rd.z, rd.y);
+        const int kn = k + 32 < T ? k + 32 : lane;
+        R yn[kBinCap];
+        const R xn = Xs[kn];
+        bin_load<R, LM, T, B>(yn, Ys, kn);
+        bin_segment<R, NR, LM, B, 0>(acc, y, xi);
+        xi = xn;
+#pragma unroll
+        for (int c = 0; c < BinConst<LM>::plan.bin[B].ncol; ++c) y[c] = yn[c];
     }
 }
 
-template <typename R, int NR, int LM, int B>
+template <typename R, int NR, int LM, int T, int B>
 __device__ __forceinline__ void bin_dispatch(int warp, R (&acc)[NR][kBinCap], const R* Ys,
-                                             const Vec4<R>* s_rad, int T, int lane) {
+                                             const R* Xs, int lane) {
     if constexpr (B < BinConst<LM>::nbins) {
-        if (warp == B) bin_tile<R, NR, LM, B>(acc, Ys, s_rad, T, lane);
-        else bin_dispatch<R, NR, LM, B + 1>(warp, acc, Ys, s_rad, T, lane);
+        if (warp == B) bin_tile<R, NR, LM, T, B>(acc, Ys, Xs, lane);
+        else bin_dispatch<R, NR, LM, T, B + 1>(warp, acc, Ys, Xs, lane);
     }
 }
 
-// TP: particles per tile (at most one per thread in phase 1; the default,
-// one per thread, keeps every thread busy there; fewer particles per tile
-// keep the two basis buffers of a large l_max within shared memory).
-// MINB: resident blocks per SM the registers are sized for.
+// phase 1: w_l H_l^m of the columns of orders m in [M0, M1] into Ys, order by
+// order (the recursion in l at fixed m of harm_level_exact), so that two
+// threads share a particle and no thread holds more than two levels of one
+// order.  w[l] = m pre0 st^l; (c, s) the sectoral value of order M.
+template <typename R, int LM, int T, int M, int M1>
+__device__ __forceinline__ void bin_orders(const R (&w)[LM + 1], R ux, R uy, R uz, R c, R s, R* Ys) {
+    R c1 = c, s1 = s, c2 = R(0), s2 = R(0);   // level l - 1, l - 2 below
+#pragma unroll
+    for (int l = M; l <= LM; ++l) {
+        if (l > M) {
+            const R d = R(2 * l - 1) * uz, b = R((l + M - 1) * (l - M - 1));
+            const R cn = l == M + 1 ? d * c1 : fma(d, c1, -b * c2);
+            const R sn = l == M + 1 ? d * s1 : fma(d, s1, -b * s2);
+            c2 = c1; s2 = s1;
+            c1 = cn; s1 = sn;
+        }
+        if constexpr (M == 0) {
+            Ys[l * l * T] = w[l] * c1;
+        } else {
+            Ys[(l * l + 2 * M - 1) * T] = w[l] * c1;
+            Ys[(l * l + 2 * M) * T] = w[l] * s1;
+        }
+    }
+    if constexpr (M < M1) {
+        constexpr R d = R(2 * M + 1);
+        bin_orders<R, LM, T, M + 1, M1>(w, ux, uy, uz, d * (ux * c - uy * s), d * (ux * s + uy * c), Ys);
+    }
+}
+// orders 0..half-1 have about half of the columns
 template <int LM>
-constexpr int bins_threads() { return BinConst<LM>::nbins * 32; }
-template <typename R, int NR, int LM, int TP = bins_threads<LM>(), int MINB = 2>
-__global__ void __launch_bounds__(bins_threads<LM>(), MINB)
+__host__ __device__ constexpr int bin_half_order() {
+    int m = 1, cols = LM + 1;
+    while (2 * cols + 2 * (LM + 1 - m) <= (LM + 1) * (LM + 1) + 2) cols += 2 * (LM + 1 - m++);
+    return m;
+}
+
+// warp totals of v[0..K), K a multiple of 32, by a reduce-scatter (each step
+// halves the values a lane still holds): lane j ends with the totals of values
+// j K/32 .. in v[0..K/32)
+template <int K, int O>
+__device__ __forceinline__ void warp_scatter(float* v, int lane) {
+    if constexpr (O >= 1) {
+        const bool up = lane & O;
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) {
+            const float give = up ? v[i] : v[i + K / 2];
+            const float keep = up ? v[i + K / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, O);
+        }
+        warp_scatter<K / 2, O / 2>(v, lane);
+    }
+}
+
+// Two threads per tile particle in phase 1, one warp per bin in phase 2, one
+// block per SM: 105 accumulators a lane leave room for 12 warps.  Bound: FMA
+// issue, NR x 7 updates and a recursion of 2 NR per bin and particle.  (14, 8),
+// 2^24 particles: 2645 us with phase 1 on half of the warps and an FP64
+// addition per column in the flush, 2158 so.
+template <int LM>
+__host__ __device__ constexpr int bins_threads() { return BinConst<LM>::nbins * 32; }
+template <int LM>
+__host__ __device__ constexpr int bins_tile() { return bins_threads<LM>() / 2; }
+template <typename R, int NR, int LM>
+__global__ void __launch_bounds__(bins_threads<LM>(), 1)
 scf_coeff_bins_kernel(ScfBinParams p) {
     constexpr int NB = BinConst<LM>::nbins;
     constexpr int TH = NB * 32;         // threads: one warp per bin
-    constexpr int T = TP;               // particles per tile
-    static_assert(T <= TH && T % 32 == 0, "tile");
+    constexpr int T = bins_tile<LM>();  // particles per tile
+    static_assert(T % 32 == 0, "tile");
     constexpr int NCOL = (LM + 1) * (LM + 1);
     constexpr int NOUT = NB * NR * kBinCap;
     using V4 = Vec4<R>;
     // dynamic shared memory: accd [NOUT] doubles, then two buffers of
-    // s_rad [T] and Ys [NCOL][T]: the basis of the next tile is evaluated into
+    // Ys [NCOL][T] and xi [T]: the basis of the next tile is evaluated into
     // one while the warps contract the current tile from the other
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* accd = reinterpret_cast<double*>(smem_raw);
-    V4* s_rad0 = reinterpret_cast<V4*>(smem_raw + ((NOUT * sizeof(double) + 15) / 16) * 16);
-    R* Ys0 = reinterpret_cast<R*>(s_rad0 + T);
-    V4* s_rad1 = reinterpret_cast<V4*>(Ys0 + (size_t)NCOL * T);
-    R* Ys1 = reinterpret_cast<R*>(s_rad1 + T);
+    R* buf0 = reinterpret_cast<R*>(smem_raw + ((NOUT * sizeof(double) + 15) / 16) * 16);
+    R* buf1 = buf0 + (NCOL + 1) * T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int k1 = tid < T ? tid : tid - T;   // phase 1: this thread's particle
     const V4* posm = reinterpret_cast<const V4*>(p.posm);
     for (int e = tid; e < NOUT; e += TH) accd[e] = 0.0;
     R acc[NR][kBinCap];
@@ -194,43 +270,58 @@ scf_coeff_bins_kernel(ScfBinParams p) {
 #pragma unroll
         for (int c = 0; c < kBinCap; ++c) acc[n][c] = R(0);
 
+    // FP64 additions are slow on this GPU: each total is one lane's, so that a
+    // few warp-wide instructions add them all
     auto flush = [&]() {
-        // butterfly sum over the warp's lanes, lane 0 adds to the FP64 block sums
+        constexpr int kPerWarp = NR * kBinCap, K = (kPerWarp + 31) / 32 * 32;
+        R v[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) v[i] = i < kPerWarp ? acc[i / kBinCap][i % kBinCap] : R(0);
+        warp_scatter<K, 16>(v, lane);
+#pragma unroll
+        for (int i = 0; i < K / 32; ++i) {
+            const int idx = lane * (K / 32) + i;
+            if (idx < kPerWarp) accd[warp * kPerWarp + idx] += (double)v[i];
+        }
 #pragma unroll
         for (int n = 0; n < NR; ++n)
 #pragma unroll
-            for (int c = 0; c < kBinCap; ++c) {
-                R v = acc[n][c];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == 0) accd[(warp * NR + n) * kBinCap + c] += (double)v;
-                acc[n][c] = R(0);
-            }
+            for (int c = 0; c < kBinCap; ++c) acc[n][c] = R(0);
     };
     auto load = [&](int tile) -> V4 {
-        const int64_t gi = (int64_t)tile * T + tid;
-        return (tid < T && tile < p.ntiles && gi < p.N) ? ld4(posm + gi)
-                                                      : mk4<R>(R(0), R(0), R(0), R(0));
+        const int64_t gi = (int64_t)tile * T + k1;
+        return (tile < p.ntiles && gi < p.N) ? ld4(posm + gi) : mk4<R>(R(0), R(0), R(0), R(0));
     };
-    // phase 1: one particle per thread (threads tid < T) -> angular basis +
-    // radial seeds
-    auto basis = [&](const V4& cur, V4* s_rad, R* Ys) {
-        if (T < TH && tid >= T) return;
+    auto basis = [&](const V4& cur, R* Ys) {
         R x = R(0), y = R(0), z = R(0), m = R(0);
         if (finite4(cur.x, cur.y, cur.z, cur.w)) { x = cur.x; y = cur.y; z = cur.z; m = cur.w; }
         else report(p.err, ETICS_ERR_NONFINITE);
         const R r = sqrt(x * x + y * y + z * z);
-        const R t = R(1) / (R(1) + r);
-        s_rad[tid] = mk4<R>(R(1) - R(2) * t, r * t * t, -m * t, R(0));
+        const R t = R(1) / (R(1) + r), st = r * t * t;
         const R inv = r > R(0) ? R(1) / r : R(0);
+        R w[LM + 1];
+        w[0] = -m * t;
+#pragma unroll
+        for (int l = 1; l <= LM; ++l) w[l] = w[l - 1] * st;
+        constexpr int H = bin_half_order<LM>();
         const R ux = x * inv, uy = y * inv, uz = z * inv;
-        const R uu = ux * ux + uy * uy + uz * uz;
-        R C[3][LM + 1], S[3][LM + 1];
-        angular_levels<R, 0, LM, false>(C, S, ux, uy, uz, uu, LM, Ys, T, tid);
+        if (tid < T) {
+            Ys[NCOL * T + k1] = R(1) - R(2) * t;
+            bin_orders<R, LM, T, 0, H - 1>(w, ux, uy, uz, R(1), R(0), Ys + k1);
+        } else {
+            R c = R(1), s = R(0);
+#pragma unroll
+            for (int m1 = 1; m1 <= H; ++m1) {
+                const R cn = R(2 * m1 - 1) * (ux * c - uy * s);
+                s = R(2 * m1 - 1) * (ux * s + uy * c);
+                c = cn;
+            }
+            bin_orders<R, LM, T, H, LM>(w, ux, uy, uz, c, s, Ys + k1);
+        }
     };
 
     V4 cur = load(blockIdx.x);
-    if (blockIdx.x < p.ntiles) basis(cur, s_rad0, Ys0);
+    if (blockIdx.x < p.ntiles) basis(cur, buf0);
     cur = load(blockIdx.x + gridDim.x);
     __syncthreads();
     int since = 0, buf = 0;
@@ -239,11 +330,12 @@ scf_coeff_bins_kernel(ScfBinParams p) {
         // contraction of the previous tile, finished before the last barrier)
         const int nxt = tile + gridDim.x;
         if (nxt < p.ntiles) {
-            basis(cur, buf ? s_rad0 : s_rad1, buf ? Ys0 : Ys1);
+            basis(cur, buf ? buf0 : buf1);
             cur = load(nxt + gridDim.x);
         }
         // phase 2: each warp accumulates its bin over this tile's particles
-        bin_dispatch<R, NR, LM, 0>(warp, acc, buf ? Ys1 : Ys0, buf ? s_rad1 : s_rad0, T, lane);
+        const R* Ys = buf ? buf1 : buf0;
+        bin_dispatch<R, NR, LM, T, 0>(warp, acc, Ys, Ys + NCOL * T, lane);
         __syncthreads();
         if (++since == kBinFlushTiles) { flush(); since = 0; }
     }
@@ -281,28 +373,28 @@ __global__ void scf_finalize_bins_kernel(const double* __restrict__ partial, int
     }
 }
 
-template <typename R, int NR, int LM, int MINB = 2>
+template <typename R, int NR, int LM>
 inline size_t scf_bins_workspace(int num_sms) {
-    return (size_t)MINB * num_sms * BinConst<LM>::nbins * NR * kBinCap * sizeof(double);
+    return (size_t)num_sms * BinConst<LM>::nbins * NR * kBinCap * sizeof(double);
 }
 
-template <typename R, int NR, int LM, int TP = bins_threads<LM>(), int MINB = 2>
+template <typename R, int NR, int LM>
 inline int scf_coeffs_bins_launch(const void* posm, int64_t N, double* coeffs, void* ws,
                                   const LaunchCtx& ctx) {
     constexpr int NB = BinConst<LM>::nbins;
     constexpr int TH = NB * 32;
-    constexpr int T = TP;
+    constexpr int T = bins_tile<LM>();
     const int ntiles = (int)((N + T - 1) / T);
-    int grid = ctx.num_sms * MINB;
+    int grid = ctx.num_sms;
     if (grid > ntiles) grid = ntiles > 0 ? ntiles : 1;
     ScfBinParams p{posm, N, ntiles, reinterpret_cast<double*>(ws), ctx.err};
     constexpr int NOUT = NB * NR * kBinCap;
     constexpr size_t smem = ((NOUT * sizeof(double) + 15) / 16) * 16 +
-                            2 * (T * sizeof(Vec4<R>) + (size_t)(LM + 1) * (LM + 1) * T * sizeof(R));
+                            2 * (size_t)((LM + 1) * (LM + 1) + 1) * T * sizeof(R);
     static_assert(smem <= 227 * 1024, "bins kernel shared memory");
     int nblocks = 0;
     if (ntiles > 0) {
-        auto k = scf_coeff_bins_kernel<R, NR, LM, TP, MINB>;
+        auto k = scf_coeff_bins_kernel<R, NR, LM>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ||
             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100))
             return ETICS_ERR_CUDA;

@@ -10,15 +10,11 @@
 #include "etics_scf_bins.cuh"
 
 namespace etics {
-constexpr int kBins148Tile = 192;
-constexpr int kBins148Blocks = 1;
-
 size_t scf_bins148_workspace_f32(int num_sms) {
-    return scf_bins_workspace<float, 15, 8, kBins148Blocks>(num_sms);
+    return scf_bins_workspace<float, 15, 8>(num_sms);
 }
 int scf_coeffs_bins148_f32(const void* posm, int64_t N, double* coeffs, void* ws,
                            const LaunchCtx& ctx) {
-    return scf_coeffs_bins_launch<float, 15, 8, kBins148Tile, kBins148Blocks>(posm, N, coeffs, ws,
-                                                                              ctx);
+    return scf_coeffs_bins_launch<float, 15, 8>(posm, N, coeffs, ws, ctx);
 }
 }  // namespace etics
