@@ -309,18 +309,6 @@ __device__ __forceinline__ void bp_rows_n(int nrr, float2 (&acc)[kBatchNR][kBpCa
     }
 }
 
-// 16-byte asynchronous global -> shared copies (the next tile's particles)
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
-
 // Blocks claim chunks (at most kBpChunkTiles tiles of one instance, heaviest
 // instances first) from a counter in the workspace; chunk c writes its FP64
 // sums c[n][l*l + col] into segment slot c, so the result does not depend on

@@ -9,12 +9,13 @@
 // etics_scf_impl.cuh (paper Sec. 2.4 eq. 18, Sec. 2.5 basis).
 #pragma once
 
+#include "etics_pair.cuh"
 #include "etics_scf_impl.cuh"
 
 namespace etics {
 
 constexpr int kBinCap = 7;
-constexpr int kBinFlushTiles = 16;
+constexpr int kBinFlushTiles = 5;
 
 struct BinSeg { int l, c0, n; };          // columns c0..c0+n-1 of level l
 struct BinDef { int nseg; BinSeg seg[4]; int ncol; };
@@ -100,7 +101,7 @@ static __constant__ BinIndex<LM> c_bin_index = make_bin_index<LM>();
 struct ScfBinParams {
     const void* posm;
     int64_t N;
-    int ntiles;
+    int64_t per;       // particles per block: block b takes [b per, (b+1) per)
     double* partial;   // [gridDim.x][nbins][NR][kBinCap]
     unsigned* err;
 };
@@ -153,14 +154,15 @@ __device__ __forceinline__ void bin_load(R (&y)[kBinCap], const R* Ys, int k) {
     }
 }
 
-// the lane's particles of one tile; the next one's values are loaded before
-// this one's rows
+// the lane's particles of one tile of n; the next one's values are loaded
+// before this one's rows
 template <typename R, int NR, int LM, int T, int B>
-__device__ __forceinline__ void bin_tile(R (&acc)[NR][kBinCap], const R* Ys, const R* Xs, int lane) {
+__device__ __forceinline__ void bin_tile(R (&acc)[NR][kBinCap], const R* Ys, const R* Xs, int lane,
+                                         int n) {
     R y[kBinCap], xi = Xs[lane];
     bin_load<R, LM, T, B>(y, Ys, lane);
 #pragma unroll 1
-    for (int k = lane; k < T; k += 32) {
+    for (int k = lane; k < n; k += 32) {
         const int kn = k + 32 < T ? k + 32 : lane;
         R yn[kBinCap];
         const R xn = Xs[kn];
@@ -174,10 +176,10 @@ __device__ __forceinline__ void bin_tile(R (&acc)[NR][kBinCap], const R* Ys, con
 
 template <typename R, int NR, int LM, int T, int B>
 __device__ __forceinline__ void bin_dispatch(int warp, R (&acc)[NR][kBinCap], const R* Ys,
-                                             const R* Xs, int lane) {
+                                             const R* Xs, int lane, int n) {
     if constexpr (B < BinConst<LM>::nbins) {
-        if (warp == B) bin_tile<R, NR, LM, T, B>(acc, Ys, Xs, lane);
-        else bin_dispatch<R, NR, LM, T, B + 1>(warp, acc, Ys, Xs, lane);
+        if (warp == B) bin_tile<R, NR, LM, T, B>(acc, Ys, Xs, lane, n);
+        else bin_dispatch<R, NR, LM, T, B + 1>(warp, acc, Ys, Xs, lane, n);
     }
 }
 
@@ -234,34 +236,43 @@ __device__ __forceinline__ void warp_scatter(float* v, int lane) {
     }
 }
 
-// Two threads per tile particle in phase 1, one warp per bin in phase 2, one
-// block per SM: 105 accumulators a lane leave room for 12 warps.  Bound: FMA
-// issue, NR x 7 updates and a recursion of 2 NR per bin and particle.  (14, 8),
-// 2^24 particles: 2645 us with phase 1 on half of the warps and an FP64
-// addition per column in the flush, 2158 so.
+// Two threads per particle in phase 1, one warp per bin in phase 2, one block
+// per SM: 105 accumulators a lane leave room for 12 warps.  Every bin is
+// straight-line code of its own, and so is phase 1: with tiles of 192
+// particles a third of the warps' time went to waiting for instructions (six
+// rounds per lane and bin), so a tile is as large as shared memory holds once
+// and the two phases alternate.  Bound: FMA issue, NR x 7 updates and a
+// recursion of 2 NR per bin and particle.  (14, 8), 2^24 particles: 2645 us
+// with phase 1 on half of the warps and an FP64 addition per column in the
+// flush, 2158 without these and with two buffers of 192, 2050 so.
 template <int LM>
 __host__ __device__ constexpr int bins_threads() { return BinConst<LM>::nbins * 32; }
 template <int LM>
-__host__ __device__ constexpr int bins_tile() { return bins_threads<LM>() / 2; }
+__host__ __device__ constexpr int bins_tile() { return bins_threads<LM>() * 3 / 2; }
+template <typename R, int NR, int LM>
+constexpr size_t bins_smem() {
+    return ((size_t)BinConst<LM>::nbins * NR * kBinCap * sizeof(double) + 15) / 16 * 16 +
+           (size_t)bins_tile<LM>() * (sizeof(Vec4<R>) + ((LM + 1) * (LM + 1) + 1) * sizeof(R));
+}
 template <typename R, int NR, int LM>
 __global__ void __launch_bounds__(bins_threads<LM>(), 1)
 scf_coeff_bins_kernel(ScfBinParams p) {
     constexpr int NB = BinConst<LM>::nbins;
     constexpr int TH = NB * 32;         // threads: one warp per bin
     constexpr int T = bins_tile<LM>();  // particles per tile
-    static_assert(T % 32 == 0, "tile");
+    constexpr int K1 = TH / 2;          // particles per round of phase 1
+    static_assert(T % 32 == 0 && T % K1 == 0, "tile");
     constexpr int NCOL = (LM + 1) * (LM + 1);
     constexpr int NOUT = NB * NR * kBinCap;
     using V4 = Vec4<R>;
-    // dynamic shared memory: accd [NOUT] doubles, then two buffers of
-    // Ys [NCOL][T] and xi [T]: the basis of the next tile is evaluated into
-    // one while the warps contract the current tile from the other
+    // dynamic shared memory: accd [NOUT] doubles, the next tile's particles
+    // P [T], Ys [NCOL][T] and xi [T]
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* accd = reinterpret_cast<double*>(smem_raw);
-    R* buf0 = reinterpret_cast<R*>(smem_raw + ((NOUT * sizeof(double) + 15) / 16) * 16);
-    R* buf1 = buf0 + (NCOL + 1) * T;
+    V4* P = reinterpret_cast<V4*>(smem_raw + ((NOUT * sizeof(double) + 15) / 16) * 16);
+    R* Ys = reinterpret_cast<R*>(P + T);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int k1 = tid < T ? tid : tid - T;   // phase 1: this thread's particle
+    const int k1 = tid < K1 ? tid : tid - K1;   // phase 1: this thread's particle
     const V4* posm = reinterpret_cast<const V4*>(p.posm);
     for (int e = tid; e < NOUT; e += TH) accd[e] = 0.0;
     R acc[NR][kBinCap];
@@ -288,11 +299,18 @@ scf_coeff_bins_kernel(ScfBinParams p) {
 #pragma unroll
             for (int c = 0; c < kBinCap; ++c) acc[n][c] = R(0);
     };
-    auto load = [&](int tile) -> V4 {
-        const int64_t gi = (int64_t)tile * T + k1;
-        return (tile < p.ntiles && gi < p.N) ? ld4(posm + gi) : mk4<R>(R(0), R(0), R(0), R(0));
+    const int64_t lo = (int64_t)blockIdx.x * p.per;
+    const int64_t hi = lo + p.per < p.N ? lo + p.per : p.N;
+    // asynchronous copy of the particles of the tile at `first` (zeros beyond
+    // the block's range); each thread waits for its own before the barrier
+    auto fetch = [&](int64_t first) {
+        for (int i = tid; i < T; i += TH) {
+            if (first + i < hi) cp_async16(P + i, posm + first + i);
+            else st4(P + i, mk4<R>(R(0), R(0), R(0), R(0)));
+        }
+        cp_async_commit();
     };
-    auto basis = [&](const V4& cur, R* Ys) {
+    auto basis = [&](const V4& cur, int k) {
         R x = R(0), y = R(0), z = R(0), m = R(0);
         if (finite4(cur.x, cur.y, cur.z, cur.w)) { x = cur.x; y = cur.y; z = cur.z; m = cur.w; }
         else report(p.err, ETICS_ERR_NONFINITE);
@@ -305,9 +323,9 @@ scf_coeff_bins_kernel(ScfBinParams p) {
         for (int l = 1; l <= LM; ++l) w[l] = w[l - 1] * st;
         constexpr int H = bin_half_order<LM>();
         const R ux = x * inv, uy = y * inv, uz = z * inv;
-        if (tid < T) {
-            Ys[NCOL * T + k1] = R(1) - R(2) * t;
-            bin_orders<R, LM, T, 0, H - 1>(w, ux, uy, uz, R(1), R(0), Ys + k1);
+        if (tid < K1) {
+            Ys[NCOL * T + k] = R(1) - R(2) * t;
+            bin_orders<R, LM, T, 0, H - 1>(w, ux, uy, uz, R(1), R(0), Ys + k);
         } else {
             R c = R(1), s = R(0);
 #pragma unroll
@@ -316,27 +334,21 @@ scf_coeff_bins_kernel(ScfBinParams p) {
                 s = R(2 * m1 - 1) * (ux * s + uy * c);
                 c = cn;
             }
-            bin_orders<R, LM, T, H, LM>(w, ux, uy, uz, c, s, Ys + k1);
+            bin_orders<R, LM, T, H, LM>(w, ux, uy, uz, c, s, Ys + k);
         }
     };
 
-    V4 cur = load(blockIdx.x);
-    if (blockIdx.x < p.ntiles) basis(cur, buf0);
-    cur = load(blockIdx.x + gridDim.x);
-    __syncthreads();
-    int since = 0, buf = 0;
-    for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, buf ^= 1) {
-        // basis of the next tile into the other buffer (its last reader, the
-        // contraction of the previous tile, finished before the last barrier)
-        const int nxt = tile + gridDim.x;
-        if (nxt < p.ntiles) {
-            basis(cur, buf ? buf0 : buf1);
-            cur = load(nxt + gridDim.x);
-        }
-        // phase 2: each warp accumulates its bin over this tile's particles
-        const R* Ys = buf ? buf1 : buf0;
-        bin_dispatch<R, NR, LM, T, 0>(warp, acc, Ys, Ys + NCOL * T, lane);
-        __syncthreads();
+    if (lo < hi) fetch(lo);
+    int since = 0;
+    for (int64_t first = lo; first < hi; first += T) {
+        const int n = hi - first < T ? (int)(hi - first) : T;
+        cp_async_wait_all();
+        __syncthreads();   // P is there; the last tile's columns are read
+#pragma unroll 1
+        for (int k = k1; k < n; k += K1) basis(P[k], k);
+        __syncthreads();   // the columns are there; P is free
+        if (first + T < hi) fetch(first + T);
+        bin_dispatch<R, NR, LM, T, 0>(warp, acc, Ys, Ys + NCOL * T, lane, n);
         if (++since == kBinFlushTiles) { flush(); since = 0; }
     }
     if (since) flush();
@@ -381,19 +393,16 @@ inline size_t scf_bins_workspace(int num_sms) {
 template <typename R, int NR, int LM>
 inline int scf_coeffs_bins_launch(const void* posm, int64_t N, double* coeffs, void* ws,
                                   const LaunchCtx& ctx) {
-    constexpr int NB = BinConst<LM>::nbins;
-    constexpr int TH = NB * 32;
-    constexpr int T = bins_tile<LM>();
-    const int ntiles = (int)((N + T - 1) / T);
-    int grid = ctx.num_sms;
-    if (grid > ntiles) grid = ntiles > 0 ? ntiles : 1;
-    ScfBinParams p{posm, N, ntiles, reinterpret_cast<double*>(ws), ctx.err};
-    constexpr int NOUT = NB * NR * kBinCap;
-    constexpr size_t smem = ((NOUT * sizeof(double) + 15) / 16) * 16 +
-                            2 * (size_t)((LM + 1) * (LM + 1) + 1) * T * sizeof(R);
+    constexpr int TH = bins_threads<LM>();
+    // contiguous equal ranges of at least 64 particles
+    int64_t per = (N + ctx.num_sms - 1) / ctx.num_sms;
+    if (per < 64) per = 64;
+    const int grid = (int)((N + per - 1) / per);
+    ScfBinParams p{posm, N, per, reinterpret_cast<double*>(ws), ctx.err};
+    constexpr size_t smem = bins_smem<R, NR, LM>();
     static_assert(smem <= 227 * 1024, "bins kernel shared memory");
     int nblocks = 0;
-    if (ntiles > 0) {
+    if (N > 0) {
         auto k = scf_coeff_bins_kernel<R, NR, LM>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ||
             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100))

@@ -3,9 +3,8 @@
 // surrogate experiment uses for its bar-perturbed Hernquist sphere (the
 // coefficients of Sec. 2.4 eq. 18 in the basis of Sec. 2.5).  12 bins of at most 7
 // columns: 384 threads, 105 FP32 accumulators per lane, so one block per SM;
-// tiles of 192 particles keep the two 81-column basis buffers within shared
-// memory.  Its own translation unit so that it compiles in parallel with the
-// other SCF kernels.
+// tiles of 576 particles.  Its own translation unit so that it compiles in
+// parallel with the other SCF kernels.
 #include "etics_internal.h"
 #include "etics_scf_bins.cuh"
 

@@ -83,3 +83,23 @@ def test_scf_field_edges(precision, basis):
         o, _ = etics.scf_force(d, n_max, l_max, basis=basis)
         etics.check_error()
         close(o.cpu().numpy(), acc, pot, precision, (n, n_max, l_max))
+
+
+@pytest.mark.parametrize("basis", [0, 1])
+@pytest.mark.parametrize("nl", [(10, 6), (14, 8), (0, 0), (1, 1), (8, 4), (12, 5), (16, 14)])
+def test_scf_coefficient_tile_edges(nl, basis):
+    """Around the tiles of the mixed-precision coefficient kernels (192 to 576
+    particles, pairs of particles per lane) and their flushes.  Tolerance, of
+    the largest coefficient: the parity tests' 2e-6, or what the roundings of
+    one particle's value may add up to (5 per level for the harmonic and the
+    radial prefactor, 2 per row, 10 for radius, xi and direction), as with few
+    particles they do not average out."""
+    n_max, l_max = nl
+    for n in (1, 2, 63, 191, 193, 383, 511, 513, 575, 577, 1153, 90001):
+        pm = hernquist(n, seed=n)
+        ref = rounded(pm, "mixed")
+        want = oracle.scf_coeffs(ref[:, :3], ref[:, 3], n_max, l_max, basis=basis)
+        got = etics.scf_coeffs(device_particles(pm, "mixed"), n_max, l_max, basis=basis).cpu().numpy()
+        etics.check_error()
+        tol = max(2e-6, (10 + 5 * l_max + 2 * n_max) * 2.0 ** -24)
+        assert np.max(np.abs(got.reshape(want.shape) - want)) <= tol * np.max(np.abs(want)), n
