@@ -106,7 +106,7 @@ int etics_scf_coeffs(const void* posm, int64_t N, int n_max, int l_max, int prec
     if (rc) return rc;
     etics::stage_event(h.ctx, 0);
     rc = precision == ETICS_MIXED
-             ? etics::scf_coeffs_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, coeffs, ws, h.ctx)
+             ? etics::scf_coeffs_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, coeffs, ws, {}, h.ctx)
              : etics::scf_coeffs_f64(posm, N, n_max, l_max, coeffs, ws, h.ctx);
     etics::stage_event(h.ctx, 2);
     return rc;
@@ -152,7 +152,7 @@ int etics_scf_coeffs_basis(const void* posm, int64_t N, int n_max, int l_max, in
     if (rc) return rc;
     etics::stage_event(h.ctx, 0);
     rc = precision == ETICS_MIXED
-             ? etics::scf_coeffs_f32(posm, N, n_max, l_max, basis, coeffs, ws, h.ctx)
+             ? etics::scf_coeffs_f32(posm, N, n_max, l_max, basis, coeffs, ws, {}, h.ctx)
              : etics::scf_coeffs_cb_f64(posm, N, n_max, l_max, coeffs, ws, h.ctx);
     etics::stage_event(h.ctx, 2);
     return rc;
@@ -243,14 +243,18 @@ int etics_leapfrog_step(void* posm, void* vel, void* accpot, int64_t N, double d
     int rc = make_ctx(stream, h);
     if (rc) return rc;
     const bool mixed = precision == ETICS_MIXED;
-    rc = mixed ? etics::kick_drift_f32(posm, vel, accpot, N, dt, h.ctx)
-               : etics::kick_drift_f64(posm, vel, accpot, N, dt, h.ctx);
-    if (rc) return rc;
+    // (the mixed-precision coefficient pass does the first half of the step itself)
+    if (!mixed || method != ETICS_SCF) {
+        rc = mixed ? etics::kick_drift_f32(posm, vel, accpot, N, dt, h.ctx)
+                   : etics::kick_drift_f64(posm, vel, accpot, N, dt, h.ctx);
+        if (rc) return rc;
+    }
     if (method == ETICS_SCF) {
         // coefficients go to coeffs_out, or to the end of the workspace
         double* c = coeffs_out ? coeffs_out
                                : reinterpret_cast<double*>(static_cast<uint8_t*>(ws) + need);
-        rc = mixed ? etics::scf_coeffs_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, c, ws, h.ctx)
+        rc = mixed ? etics::scf_coeffs_f32(posm, N, n_max, l_max, ETICS_BASIS_HO, c, ws,
+                                           {posm, vel, accpot, dt}, h.ctx)
                    : etics::scf_coeffs_f64(posm, N, n_max, l_max, c, ws, h.ctx);
         if (rc) return rc;
         // the field pass does the second kick with the acceleration at hand

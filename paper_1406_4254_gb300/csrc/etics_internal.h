@@ -9,16 +9,19 @@ namespace etics {
 // ---- SCF (etics_scf_f32.cu / etics_scf_f64.cu) ----------------------------
 size_t scf_workspace_f32(int64_t N, int n_max, int l_max, int num_sms);
 // particle-pair coefficient pass at (10, 6) (etics_scf_pairs_f32.cu)
+// the first half of a leapfrog step (v += dt/2 a, x += dt v), done by a
+// coefficient pass as it reads the particles (posm null: none)
+struct DriftStep { void* posm; void* vel; const void* acc; double dt; };
 size_t scf_pairs106_workspace_f32(int num_sms);
-int scf_coeffs_pairs106_f32(const void* posm, int64_t N, double* coeffs, void* ws,
+int scf_coeffs_pairs106_f32(const void* posm, int64_t N, double* coeffs, void* ws, DriftStep drift,
                             const LaunchCtx& ctx);
 // per-warp-bin coefficient pass at (14, 8) (etics_scf_bins_f32.cu)
 size_t scf_bins148_workspace_f32(int num_sms);
-int scf_coeffs_bins148_f32(const void* posm, int64_t N, double* coeffs, void* ws,
+int scf_coeffs_bins148_f32(const void* posm, int64_t N, double* coeffs, void* ws, DriftStep drift,
                            const LaunchCtx& ctx);
 size_t scf_workspace_f64(int64_t N, int n_max, int l_max, int num_sms);
 int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, int basis, double* coeffs,
-                   void* ws, const LaunchCtx& ctx);
+                   void* ws, DriftStep drift, const LaunchCtx& ctx);
 // its parts, by the number of rows (n_max + 1 rounded up to an odd number)
 #define ETICS_COEFF_PART(k)                                                                      \
     size_t scf_coeffs_f32_##k##_workspace(int rows, int num_sms);                                \

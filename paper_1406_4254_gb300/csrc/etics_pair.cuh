@@ -105,4 +105,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
+// kick-drift of one particle: v += h a, x += dt v (h = dt / 2)
+template <typename V4, typename R>
+__device__ __forceinline__ void kick_drift(V4& x, V4& v, const V4& a, R h, R dt) {
+    v.x = fma(h, a.x, v.x);
+    v.y = fma(h, a.y, v.y);
+    v.z = fma(h, a.z, v.z);
+    x.x = fma(dt, v.x, x.x);
+    x.y = fma(dt, v.y, x.y);
+    x.z = fma(dt, v.z, x.z);
+}
+
 }  // namespace etics

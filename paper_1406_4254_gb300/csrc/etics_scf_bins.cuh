@@ -9,6 +9,7 @@
 // etics_scf_impl.cuh (paper Sec. 2.4 eq. 18, Sec. 2.5 basis).
 #pragma once
 
+#include "etics_internal.h"
 #include "etics_pair.cuh"
 #include "etics_scf_impl.cuh"
 
@@ -104,6 +105,11 @@ struct ScfBinParams {
     int64_t per;       // particles per block: block b takes [b per, (b+1) per)
     double* partial;   // [gridDim.x][nbins][NR][kBinCap]
     unsigned* err;
+    // the first half of a leapfrog step, if the kernel does it
+    void* drift_posm;
+    void* vel;
+    const void* acc;
+    double dt;
 };
 
 // rows of segment S of bin B and the segments after it for one particle: the
@@ -249,12 +255,15 @@ template <int LM>
 __host__ __device__ constexpr int bins_threads() { return BinConst<LM>::nbins * 32; }
 template <int LM>
 __host__ __device__ constexpr int bins_tile() { return bins_threads<LM>() * 3 / 2; }
-template <typename R, int NR, int LM>
+template <typename R, int NR, int LM, bool DRIFT>
 constexpr size_t bins_smem() {
     return ((size_t)BinConst<LM>::nbins * NR * kBinCap * sizeof(double) + 15) / 16 * 16 +
-           (size_t)bins_tile<LM>() * (sizeof(Vec4<R>) + ((LM + 1) * (LM + 1) + 1) * sizeof(R));
+           (size_t)bins_tile<LM>() * ((DRIFT ? 3 : 1) * sizeof(Vec4<R>) + ((LM + 1) * (LM + 1) + 1) * sizeof(R));
 }
-template <typename R, int NR, int LM>
+// DRIFT: kick and drift the particles as they are read (the copies of a tile's
+// velocities and accelerations are hidden behind the contraction of the tile
+// before; a kick-drift kernel is bound by memory, 188 us at 2^24).
+template <typename R, int NR, int LM, bool DRIFT>
 __global__ void __launch_bounds__(bins_threads<LM>(), 1)
 scf_coeff_bins_kernel(ScfBinParams p) {
     constexpr int NB = BinConst<LM>::nbins;
@@ -266,11 +275,14 @@ scf_coeff_bins_kernel(ScfBinParams p) {
     constexpr int NOUT = NB * NR * kBinCap;
     using V4 = Vec4<R>;
     // dynamic shared memory: accd [NOUT] doubles, the next tile's particles
-    // P [T], Ys [NCOL][T] and xi [T]
+    // P [T], (DRIFT) their velocities and accelerations V [T], A [T], then
+    // Ys [NCOL][T] and xi [T]
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* accd = reinterpret_cast<double*>(smem_raw);
     V4* P = reinterpret_cast<V4*>(smem_raw + ((NOUT * sizeof(double) + 15) / 16) * 16);
-    R* Ys = reinterpret_cast<R*>(P + T);
+    V4* V = P + T;
+    V4* A = V + T;
+    R* Ys = reinterpret_cast<R*>(P + (DRIFT ? 3 : 1) * T);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k1 = tid < K1 ? tid : tid - K1;   // phase 1: this thread's particle
     const V4* posm = reinterpret_cast<const V4*>(p.posm);
@@ -301,14 +313,30 @@ scf_coeff_bins_kernel(ScfBinParams p) {
     };
     const int64_t lo = (int64_t)blockIdx.x * p.per;
     const int64_t hi = lo + p.per < p.N ? lo + p.per : p.N;
-    // asynchronous copy of the particles of the tile at `first` (zeros beyond
-    // the block's range); each thread waits for its own before the barrier
+    // asynchronous copy of the particles of the tile at `first`; each thread
+    // waits for its own before the barrier
     auto fetch = [&](int64_t first) {
         for (int i = tid; i < T; i += TH) {
-            if (first + i < hi) cp_async16(P + i, posm + first + i);
-            else st4(P + i, mk4<R>(R(0), R(0), R(0), R(0)));
+            if (first + i < hi) {
+                cp_async16(P + i, posm + first + i);
+                if (DRIFT) {
+                    cp_async16(V + i, reinterpret_cast<const V4*>(p.vel) + first + i);
+                    cp_async16(A + i, reinterpret_cast<const V4*>(p.acc) + first + i);
+                }
+            }
         }
         cp_async_commit();
+    };
+    // the thread's own copies have arrived: kick, drift, and back to memory
+    auto step = [&](int64_t first) {
+        const R dt = (R)p.dt, h = R(0.5) * dt;
+        for (int i = tid; i < T && first + i < hi; i += TH) {
+            V4 x = P[i], v = V[i];
+            kick_drift(x, v, A[i], h, dt);
+            st4(reinterpret_cast<V4*>(p.vel) + first + i, v);
+            st4(reinterpret_cast<V4*>(p.drift_posm) + first + i, x);
+            P[i] = x;
+        }
     };
     auto basis = [&](const V4& cur, int k) {
         R x = R(0), y = R(0), z = R(0), m = R(0);
@@ -343,6 +371,7 @@ scf_coeff_bins_kernel(ScfBinParams p) {
     for (int64_t first = lo; first < hi; first += T) {
         const int n = hi - first < T ? (int)(hi - first) : T;
         cp_async_wait_all();
+        if (DRIFT) step(first);
         __syncthreads();   // P is there; the last tile's columns are read
 #pragma unroll 1
         for (int k = k1; k < n; k += K1) basis(P[k], k);
@@ -392,18 +421,20 @@ inline size_t scf_bins_workspace(int num_sms) {
 
 template <typename R, int NR, int LM>
 inline int scf_coeffs_bins_launch(const void* posm, int64_t N, double* coeffs, void* ws,
-                                  const LaunchCtx& ctx) {
+                                  DriftStep drift, const LaunchCtx& ctx) {
     constexpr int TH = bins_threads<LM>();
     // contiguous equal ranges of at least 64 particles
     int64_t per = (N + ctx.num_sms - 1) / ctx.num_sms;
     if (per < 64) per = 64;
     const int grid = (int)((N + per - 1) / per);
-    ScfBinParams p{posm, N, per, reinterpret_cast<double*>(ws), ctx.err};
-    constexpr size_t smem = bins_smem<R, NR, LM>();
-    static_assert(smem <= 227 * 1024, "bins kernel shared memory");
+    ScfBinParams p{posm, N, per, reinterpret_cast<double*>(ws), ctx.err,
+                   drift.posm, drift.vel, drift.acc, drift.dt};
+    static_assert(bins_smem<R, NR, LM, true>() <= 227 * 1024, "bins kernel shared memory");
+    const size_t smem = drift.posm ? bins_smem<R, NR, LM, true>() : bins_smem<R, NR, LM, false>();
     int nblocks = 0;
     if (N > 0) {
-        auto k = scf_coeff_bins_kernel<R, NR, LM>;
+        auto k = drift.posm ? scf_coeff_bins_kernel<R, NR, LM, true>
+                            : scf_coeff_bins_kernel<R, NR, LM, false>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ||
             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100))
             return ETICS_ERR_CUDA;

@@ -20,14 +20,17 @@ size_t scf_workspace_f32(int64_t N, int n_max, int l_max, int num_sms) {
     return most;
 }
 int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, int basis, double* coeffs,
-                   void* ws, const LaunchCtx& ctx) {
+                   void* ws, DriftStep drift, const LaunchCtx& ctx) {
     // the paper's (10, 6) and the forecast experiment's (14, 8) expansion have
     // kernels with their bins known at compile time: (10, 6) at 2^20 54 us
     // against 72 with the general kernel, (14, 8) at 2^22 560 against 718
     if (basis == ETICS_BASIS_HO && n_max == 10 && l_max == 6)
-        return scf_coeffs_pairs106_f32(posm, N, coeffs, ws, ctx);
+        return scf_coeffs_pairs106_f32(posm, N, coeffs, ws, drift, ctx);
     if (basis == ETICS_BASIS_HO && n_max == 14 && l_max == 8)
-        return scf_coeffs_bins148_f32(posm, N, coeffs, ws, ctx);
+        return scf_coeffs_bins148_f32(posm, N, coeffs, ws, drift, ctx);
+    // (here several blocks may read the same particle: the drift comes first)
+    if (drift.posm)
+        if (const int rc = kick_drift_f32(drift.posm, drift.vel, drift.acc, N, drift.dt, ctx)) return rc;
     const int rows = coeff_rows(n_max);
     const auto run = rows <= 7 ? scf_coeffs_f32_a : rows <= 11 ? scf_coeffs_f32_b
                      : rows <= 15 ? scf_coeffs_f32_c : scf_coeffs_f32_d;

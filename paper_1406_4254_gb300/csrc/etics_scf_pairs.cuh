@@ -33,6 +33,8 @@
 
 #include <atomic>
 
+#include "etics_internal.h"
+#include "etics_pair.cuh"
 #include "etics_scf_impl.cuh"
 
 namespace etics {
@@ -100,6 +102,11 @@ struct ScfPairParams {
     int64_t per;       // particles per block (even): block b takes [b*per, (b+1)*per)
     double* partial;   // [gridDim.x][nbins][NR][CAP]
     unsigned* err;
+    // the first half of a leapfrog step, if the kernel does it
+    float4* drift_posm;
+    float4* vel;
+    const float4* acc;
+    float dt;
 };
 
 // phase 1 for one particle: xi, and w_l H_l^m of every column (dense layout
@@ -170,14 +177,18 @@ __device__ __forceinline__ void pair_dispatch(int warp, float2 (&acc)[NR][CAP], 
     }
 }
 
-template <int NR, int LM, int CAP>
+template <int NR, int LM, int CAP, bool DRIFT>
 constexpr size_t pair_smem_bytes() {
     constexpr int NB = PairConst<LM, CAP>::nbins;
     return ((size_t)NB * NR * CAP * sizeof(double) + 15) / 16 * 16 +
-           2 * ((size_t)(LM + 1) * (LM + 1) * kPairTile + kPairTile) * sizeof(float);
+           2 * ((size_t)(LM + 1) * (LM + 1) * kPairTile + kPairTile) * sizeof(float) +
+           (DRIFT ? 2 * kPairTile * sizeof(float4) : 0);
 }
 
-template <int NR, int LM, int CAP>
+// DRIFT: kick and drift the particles as they are read (their velocities and
+// accelerations arrive by asynchronous copies during the previous tile; a
+// kick-drift kernel of its own takes 11.5 us at 2^20).
+template <int NR, int LM, int CAP, bool DRIFT>
 __global__ void __launch_bounds__(PairConst<LM, CAP>::threads, 1)
 scf_coeff_pairs_kernel(ScfPairParams p) {
     constexpr int NB = PairConst<LM, CAP>::nbins;
@@ -236,10 +247,27 @@ scf_coeff_pairs_kernel(ScfPairParams p) {
     const int64_t lo = (int64_t)blockIdx.x * p.per;
     const int64_t hi = lo + p.per < p.N ? lo + p.per : p.N;
     const int ntb = hi > lo ? (int)((hi - lo + kPairTile - 1) / kPairTile) : 0;
+    // (DRIFT) this thread's velocity and acceleration of the next tile
+    float4* V = reinterpret_cast<float4*>(buf0 + 2 * kBuf) + tid;
+    float4* A = V + kPairTile;
     auto load = [&](int t) -> float4 {
         const int64_t gi = lo + (int64_t)t * kPairTile + tid;
-        return (tid < kPairTile && t < ntb && gi < hi) ? p.posm[gi]
-                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid >= kPairTile || t >= ntb || gi >= hi) return make_float4(0.f, 0.f, 0.f, 0.f);
+        if (DRIFT) {
+            cp_async16(V, p.vel + gi);
+            cp_async16(A, p.acc + gi);
+            cp_async_commit();
+        }
+        return p.posm[gi];
+    };
+    auto step = [&](int t, float4& x) {
+        const int64_t gi = lo + (int64_t)t * kPairTile + tid;
+        if (tid >= kPairTile || gi >= hi) return;
+        cp_async_wait_all();
+        float4 v = *V;
+        kick_drift(x, v, *A, 0.5f * p.dt, p.dt);
+        p.vel[gi] = v;
+        p.drift_posm[gi] = x;
     };
     auto pairs_in = [&](int t) {
         const int64_t left = hi - lo - (int64_t)t * kPairTile;
@@ -259,12 +287,14 @@ scf_coeff_pairs_kernel(ScfPairParams p) {
     };
 
     float4 cur = load(0);
+    if (DRIFT && ntb > 0) step(0, cur);
     if (ntb > 0) phase1(cur, Hb(0), Xb(0));
     cur = load(1);
     __syncthreads();
     int since = 0, b = 0;
     for (int t = 0; t < ntb; ++t, b ^= 1) {
         if (t + 1 < ntb) {
+            if (DRIFT) step(t + 1, cur);
             phase1(cur, Hb(b ^ 1), Xb(b ^ 1));
             cur = load(t + 2);
         }
@@ -318,10 +348,11 @@ inline size_t scf_pairs_workspace(int num_sms) {
 
 template <int NR, int LM, int CAP>
 inline int scf_coeffs_pairs_launch(const void* posm, int64_t N, double* coeffs, void* ws,
-                                   const LaunchCtx& ctx) {
+                                   DriftStep drift, const LaunchCtx& ctx) {
     constexpr int TH = PairConst<LM, CAP>::threads;
-    constexpr size_t smem = pair_smem_bytes<NR, LM, CAP>();
-    static_assert(smem <= 227 * 1024, "pairs kernel shared memory");
+    static_assert(pair_smem_bytes<NR, LM, CAP, true>() <= 227 * 1024, "pairs kernel shared memory");
+    const bool with = drift.posm != nullptr;
+    const size_t smem = with ? pair_smem_bytes<NR, LM, CAP, true>() : pair_smem_bytes<NR, LM, CAP, false>();
     const int ntiles = (int)((N + kPairTile - 1) / kPairTile);
     int grid = ctx.num_sms;
     if (grid > ntiles) grid = ntiles > 0 ? ntiles : 1;
@@ -331,13 +362,17 @@ inline int scf_coeffs_pairs_launch(const void* posm, int64_t N, double* coeffs, 
     int64_t per = (N + grid - 1) / grid;
     per += per & 1;
     ScfPairParams p{reinterpret_cast<const float4*>(posm), N, per,
-                    reinterpret_cast<double*>(ws), ctx.err};
+                    reinterpret_cast<double*>(ws), ctx.err, static_cast<float4*>(drift.posm),
+                    static_cast<float4*>(drift.vel), static_cast<const float4*>(drift.acc),
+                    (float)drift.dt};
     int nblocks = 0;
     if (ntiles > 0) {
-        auto k = scf_coeff_pairs_kernel<NR, LM, CAP>;
+        auto k = with ? scf_coeff_pairs_kernel<NR, LM, CAP, true>
+                      : scf_coeff_pairs_kernel<NR, LM, CAP, false>;
         // the function attributes are set once per device (a host call per
         // launch would sit between the caller's events and the kernel)
-        static std::atomic<uint64_t> attr_done{0};
+        static std::atomic<uint64_t> attr_done_of[2] = {{0}, {0}};
+        std::atomic<uint64_t>& attr_done = attr_done_of[with ? 1 : 0];
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return ETICS_ERR_CUDA;
         const uint64_t bit = uint64_t(1) << (dev & 63);

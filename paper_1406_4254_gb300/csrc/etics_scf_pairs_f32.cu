@@ -13,8 +13,8 @@ constexpr int kPairs106Cap = 4;
 size_t scf_pairs106_workspace_f32(int num_sms) {
     return scf_pairs_workspace<11, 6, kPairs106Cap>(num_sms);
 }
-int scf_coeffs_pairs106_f32(const void* posm, int64_t N, double* coeffs, void* ws,
+int scf_coeffs_pairs106_f32(const void* posm, int64_t N, double* coeffs, void* ws, DriftStep drift,
                             const LaunchCtx& ctx) {
-    return scf_coeffs_pairs_launch<11, 6, kPairs106Cap>(posm, N, coeffs, ws, ctx);
+    return scf_coeffs_pairs_launch<11, 6, kPairs106Cap>(posm, N, coeffs, ws, drift, ctx);
 }
 }  // namespace etics

@@ -1,6 +1,8 @@
 // etics_step.cu -- the kick and drift halves of the kick-drift-kick leapfrog
-// step that surrounds the force calculation (paper Secs. 3.4 and 5.4).
+// step that surrounds the force calculation (paper Secs. 3.4 and 5.4), where
+// the force passes do not do them themselves.
 #include "etics_internal.h"
+#include "etics_pair.cuh"
 
 namespace etics {
 
@@ -13,12 +15,7 @@ __global__ void kick_drift_kernel(Vec4<R>* __restrict__ posm, Vec4<R>* __restric
         Vec4<R> v = ld4(vel + i);
         const Vec4<R> a = ld4(acc + i);
         Vec4<R> x = ld4(posm + i);
-        v.x = fma(h, a.x, v.x);
-        v.y = fma(h, a.y, v.y);
-        v.z = fma(h, a.z, v.z);
-        x.x = fma(dt, v.x, x.x);
-        x.y = fma(dt, v.y, x.y);
-        x.z = fma(dt, v.z, x.z);
+        kick_drift(x, v, a, h, dt);
         st4(vel + i, v);
         st4(posm + i, x);
     }
