@@ -13,7 +13,7 @@
 //      of the block owning one "bin" (one level, up to three columns) of the
 //      instance's expansion (batch_pairs_kernel).  FP64: register tiles of
 //      four columns over a shared-memory radial basis (batch_coeff_kernel);
-//   2. finalize: one warp per output coefficient of any instance;
+//   2. finalize: one thread per output coefficient of any instance;
 //   3. field: one block per work item (a chunk of one instance's particles),
 //      the instance's coefficients staged in shared memory.
 // No grid-wide barrier is needed, so the three launches capture into a CUDA
@@ -440,24 +440,25 @@ batch_pairs_kernel(const float4* __restrict__ posm, const void* __restrict__ pla
 }
 
 // ---------------------------------------------------------------------------
-// 2. finalize: ordered sum of an instance's segments, times K_lm / J_nl
+// 2. finalize: ordered sum of an instance's segments, times K_lm / J_nl.  One
+// thread per output: FP64 additions are slow on this GPU, and a warp per
+// output spends most of them on its butterfly (256-system ensemble: 70 us).
 // ---------------------------------------------------------------------------
 __global__ void batch_finalize_kernel(const void* __restrict__ plan,
                                       const double* __restrict__ partial,
                                       double* __restrict__ coeffs) {
     const BatchHeader hd = *plan_table<BatchHeader>(plan, 0);
     const BatchInst* insts = plan_table<BatchInst>(plan, hd.off_inst);
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= hd.coef_total) return;
-    int lo = 0, hi = hd.ninst - 1;          // instance holding output `warp`
+    const int64_t out = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (out >= hd.coef_total) return;
+    int lo = 0, hi = hd.ninst - 1;          // instance holding this output
     while (lo < hi) {
         const int mid = (lo + hi + 1) / 2;
-        if (insts[mid].coef_offset <= warp) lo = mid; else hi = mid - 1;
+        if (insts[mid].coef_offset <= out) lo = mid; else hi = mid - 1;
     }
     const BatchInst in = insts[lo];
     const int nj = (in.l_max + 1) * (in.l_max + 1);
-    const int local = (int)(warp - in.coef_offset);
+    const int local = (int)(out - in.coef_offset);
     const int n = local / nj, jj = local % nj;
     int l = 0;
     while ((l + 1) * (l + 1) <= jj) ++l;
@@ -467,15 +468,12 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
     const int idx = hd.precision == ETICS_MIXED
                         ? n * kBpCols + l * l + col
                         : ((col_offset(l) / 4 + col / 4) * kBatchNR + n) * 4 + (col & 3);
+    const double* src = partial + (size_t)in.first_seg * hd.seg_stride + idx;
     double s = 0.0;
-    for (int k = lane; k < in.nseg; k += 32) s += partial[(size_t)(in.first_seg + k) * hd.seg_stride + idx];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        const int am = m < 0 ? -m : m;
-        coeffs[warp] = s * c_tab.knorm_fact[l * (l + 1) / 2 + am] * c_tab.inv_j[n][l] *
-                       geg_gamma(0, l, n);
-    }
+#pragma unroll 8
+    for (int k = 0; k < in.nseg; ++k) s += src[(size_t)k * hd.seg_stride];
+    const int am = m < 0 ? -m : m;
+    coeffs[out] = s * c_tab.knorm_fact[l * (l + 1) / 2 + am] * c_tab.inv_j[n][l] * geg_gamma(0, l, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -770,8 +768,7 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
     }
     stage_event(ctx, 1);
     if (hd.coef_total > 0) {
-        const int64_t threads = hd.coef_total * 32;
-        batch_finalize_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, ctx.stream>>>(
+        batch_finalize_kernel<<<(unsigned)((hd.coef_total + 127) / 128), 128, 0, ctx.stream>>>(
             plan_dev, static_cast<const double*>(ws), coeffs);
         if (cudaGetLastError()) return ETICS_ERR_CUDA;
         ++*ctx.launches;
