@@ -499,12 +499,9 @@ batch_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm,
     for (int w = blockIdx.x; w < hd.nfield; w += gridDim.x) {
         const BatchField it = items[w];
         const BatchInst in = insts[it.inst];
-        const int ncols = col_total(in.l_max);
         __syncthreads();
-        for (int e = threadIdx.x; e < (in.n_max + 1) * ncols; e += blockDim.x) {
-            const int n = e / ncols;
-            cs[e] = field_coeff<R>(coeffs + in.coef_offset, ETICS_BASIS_HO, n, e - n * ncols, in.l_max);
-        }
+        field_table(cs, col_offset_c(kBatchLM + 1), coeffs + in.coef_offset, ETICS_BASIS_HO, in.n_max,
+                    in.l_max);
         __syncthreads();
         for (int k = threadIdx.x * NP; k < it.count; k += blockDim.x * NP) {
             const int64_t i = in.offset + it.begin + k;
@@ -514,7 +511,7 @@ batch_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm,
                 pv[j] = k + j < it.count ? ld4(posm + i + j) : mk4<R>(R(0), R(0), R(0), R(0));
                 if (!finite4(pv[j].x, pv[j].y, pv[j].z, pv[j].w)) report(err, ETICS_ERR_NONFINITE);
             }
-            field_eval<P, kBatchLM, ACC, 0, 0>(pv, cs, ncols, in.n_max, in.l_max, ~0u, res);
+            field_eval<P, kBatchLM, ACC, 0, 0>(pv, cs, in.n_max, in.l_max, ~0u, res);
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
                 if (k + j >= it.count) continue;

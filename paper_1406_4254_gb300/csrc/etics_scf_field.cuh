@@ -57,18 +57,25 @@ constexpr FieldTable make_field_table() {
 }
 static __device__ const FieldTable g_field_tab = make_field_table();
 
-// table entry (row n, padded column c of all levels) of the coefficients: the
-// 2l+1 columns of a level, then at least one place of padding, the last of
-// which holds -bs_n, so that the recursion constant arrives with the columns
+// The table: row n holds the levels' 2l+1 columns, each level followed by at
+// least one place of padding, the last of which holds -bs_n, so that the
+// recursion constant arrives with the columns.  `stride` entries per row (a
+// constant of the kernel, so that a round's rows are at immediate offsets).
+// Warps take rows, lanes columns: one look for a column's level for all rows.
 template <typename R>
-__device__ __forceinline__ R field_coeff(const double* coeffs, int basis, int n, int c, int l_max) {
-    int l = 0;
-    while (c >= ncol_pad(l)) { c -= ncol_pad(l); ++l; }
-    if (c >= 2 * l + 1)   // padding; the last place carries the recursion constant
-        return c == ncol_pad(l) - 1 ? -geg_bs_of<R>(basis, l, n) : R(0);
-    const int am = (c + 1) / 2, m = (c & 1) ? am : -am;   // c = 0: m = 0
-    return (R)(__ldcg(coeffs + (size_t)n * (l_max + 1) * (l_max + 1) + l * l + l + m) *
-               g_field_tab.v[basis][n][l * (l + 1) / 2 + am]);
+__device__ __forceinline__ void field_table(R* cs, int stride, const double* coeffs, int basis,
+                                            int n_max, int l_max) {
+    const int nj = (l_max + 1) * (l_max + 1), ncols = col_total(l_max);
+    for (int c = threadIdx.x & 31; c < ncols; c += 32) {
+        int l = 0, k = c;
+        while (k >= ncol_pad(l)) { k -= ncol_pad(l); ++l; }
+        const int am = (k + 1) / 2, m = (k & 1) ? am : -am;   // k = 0: m = 0
+        for (int n = threadIdx.x >> 5; n <= n_max; n += blockDim.x >> 5)
+            cs[n * stride + c] =
+                k < 2 * l + 1 ? (R)(__ldcg(coeffs + (size_t)n * nj + l * l + l + m) *
+                                    g_field_tab.v[basis][n][l * (l + 1) / 2 + am])
+                : k == ncol_pad(l) - 1 ? -geg_bs_of<R>(basis, l, n) : R(0);
+    }
 }
 
 // NM1 > 0: specialised for n_max + 1 == NM1 and l_max == LM (n loop unrolled,
@@ -88,7 +95,7 @@ struct FieldEval {
     P vx, vy, vz, tau, xi, dxdr, st, pre, preR;
     P pot, gr, gx, gy, gz;   // gz at half its value
     const R* cs;
-    int ncols, n_max, l_max;
+    int n_max, l_max;
     unsigned levels;   // bit l: this thread adds level l
 
     // one row, v its table entries: acc[c] += v_c t, and (ACC) the sum of v_c Y_c
@@ -139,8 +146,7 @@ struct FieldEval {
             harm_scaled<R, L, P>(C[s1], S[s1], C[s2], S[s2], vx, vy, vz, C[s0], S[s0]);
             if (levels >> L & 1u) {
             constexpr int NC = 2 * L + 1;
-            constexpr int kStride = NM1 > 0 ? col_offset_c(LM + 1) : 0;
-            const int stride = NM1 > 0 ? kStride : ncols;
+            constexpr int stride = col_offset_c(LM + 1);
             const int nlim = NM1 > 0 ? NM1 - 1 : n_max;
             const R* r = cs + col_offset_c(L);
             P A[NC], Q = splat<P>(R(0));
@@ -233,8 +239,8 @@ __device__ __forceinline__ double half_of(const double& p, int) { return p; }
 // the levels not in `levels` are left out (a partial sum)
 template <typename P, int LM, bool ACC, int NM1, int BASIS>
 __device__ __forceinline__ void field_eval(const Vec4<typename FieldLane<P>::R> (&pv)[FieldLane<P>::kParticles],
-                                           const typename FieldLane<P>::R* cs, int ncols, int n_max,
-                                           int l_max, unsigned levels,
+                                           const typename FieldLane<P>::R* cs, int n_max, int l_max,
+                                           unsigned levels,
                                            Vec4<typename FieldLane<P>::R> (&res)[FieldLane<P>::kParticles]) {
     using R = typename FieldLane<P>::R;
     constexpr int NP = FieldLane<P>::kParticles;
@@ -263,7 +269,6 @@ __device__ __forceinline__ void field_eval(const Vec4<typename FieldLane<P>::R> 
     f.preR = mul2(f.preR, splat<P>(R(0.5 * kKappa)));
     f.pot = f.gr = f.gx = f.gy = f.gz = splat<P>(R(0));
     f.cs = cs;
-    f.ncols = ncols;
     f.n_max = n_max;
     f.l_max = l_max;
     f.levels = levels;
@@ -315,12 +320,9 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm, int64_
     constexpr int NP = FieldLane<P>::kParticles;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* cs = reinterpret_cast<R*>(smem_raw);
-    const int ncols = NM1 > 0 ? col_offset_c(LM + 1) : col_total(l_max);
+    constexpr int stride = col_offset_c(LM + 1);
     pdl_wait();   // the coefficients come from the previous kernel
-    for (int e = threadIdx.x; e < (n_max + 1) * ncols; e += blockDim.x) {
-        const int n = e / ncols;
-        cs[e] = field_coeff<R>(coeffs, B, n, e - n * ncols, l_max);
-    }
+    field_table(cs, stride, coeffs, B, n_max, l_max);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int part = split.parts > 1 ? warp % kFieldParts : 0;
@@ -335,10 +337,10 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm, int64_
             pv[j] = i + j < N ? ld4(posm + i + j) : mk4<R>(R(0), R(0), R(0), R(0));
             if (!finite4(pv[j].x, pv[j].y, pv[j].z, pv[j].w)) report(err, ETICS_ERR_NONFINITE);
         }
-        field_eval<P, LM, ACC, NM1, B>(pv, cs, ncols, n_max, l_max, split.level[part], res);
+        field_eval<P, LM, ACC, NM1, B>(pv, cs, n_max, l_max, split.level[part], res);
         if (split.parts > 1) {
             // parts 1.. leave their sums behind the table, part 0 adds them
-            Vec4<R>* sums = reinterpret_cast<Vec4<R>*>(cs + (n_max + 1) * ncols);
+            Vec4<R>* sums = reinterpret_cast<Vec4<R>*>(cs + (n_max + 1) * stride);
             if (part > 0) {
 #pragma unroll
                 for (int j = 0; j < NP; ++j) st4(sums + ((part - 1) * NP + j) * per + slot, res[j]);
@@ -397,7 +399,7 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     const int threads = warps * 32 * parts;
     const int64_t want = (lanes + warps * 32 - 1) / (warps * 32);
     const int grid = (int)(want < sms ? want : sms);
-    const size_t smem = (size_t)(n_max + 1) * col_total(l_max) * sizeof(R) +
+    const size_t smem = (size_t)(n_max + 1) * col_offset_c(LM + 1) * sizeof(R) +
                         (parts > 1 ? (size_t)(kFieldParts - 1) * FieldLane<P>::kParticles * warps * 32 *
                                          sizeof(Vec4<R>) : 0);
     auto k = (out_mask & ETICS_OUT_ACC) ? scf_field_kernel<P, LM, true, NM1, B>
