@@ -21,9 +21,10 @@
 // and have kernels of their own: the output layer with the loss, its backward
 // step, and the weight gradient of a narrow input.  The training step of the
 // shared network (8 -> 256 -> 256 -> 3, 19440 rows) went from 25 launches and
-// 437 us to 9 launches and 112 us (per kernel, cold: forward products 12 and
-// 14, output layer 12, its backward step 14, dH 10, dW 19, narrow dW 10,
-// reductions 18, Adam 4).
+// 437 us to 9 launches and 87 us: 112 one after the other (cold: forward
+// products 12 and 14, output layer 12, its backward step 14, dH 10, dW 19,
+// narrow dW 10, reductions 18, Adam 4), the rest by letting each kernel's launch
+// overlap the end of the one before (launch_pdl).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -243,6 +244,7 @@ mlp_narrow_out_kernel(const bf16* __restrict__ a, const bf16* __restrict__ W,
     __shared__ __align__(16) bf16 s_w[kThin][kThinInputs + kPadK];   // [output][input]
     __shared__ double s_loss[8], s_db[8][kThin];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    pdl_wait();
     for (int i = tid; i < din * kThin; i += 256) {
         const int n = i % kThin, k = i / kThin;
         s_w[n][k] = n < dout ? W[(size_t)k * dout + n] : __float2bfloat16_rn(0.0f);
@@ -347,6 +349,7 @@ mlp_narrow_back_kernel(const bf16* __restrict__ a, const float* __restrict__ h,
     const int m = (blockIdx.x * 64 + cg) * 4;
     const int r0 = blockIdx.y * rows, r1 = min(B, r0 + rows);
     const bool on = m < din;
+    pdl_wait();
     float w[4][DO], acc[4][DO], cs[4], ce[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -429,6 +432,7 @@ mlp_narrow_in_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dzb, i
     const int n = (blockIdx.x * 64 + cg) * 4;
     const int r0 = blockIdx.y * rows, r1 = min(B, r0 + rows);
     const bool on = n < dout;
+    pdl_wait();
     float acc[4][DI];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -478,7 +482,7 @@ struct ReduceItem {
     void* dst;
     int64_t n;
     int parts, block0;
-    int wide;        // src: 0 float, 1 double
+    int wide;        // src: 0 float, 1 double, 2 float with four outputs per lane
     double scale;    // dst is a double, sum * scale, if not 0; else a float
 };
 constexpr int kReduceItems = 2 * ETICS_MLP_MAX_LAYERS + 1;
@@ -489,10 +493,34 @@ struct ReduceList {
 __global__ void __launch_bounds__(256) mlp_reduce_kernel(const __grid_constant__ ReduceList list) {
     __shared__ double s_d[8][32];
     __shared__ float s_f[8][32];
+    __shared__ float4 s_f4[8][32];
     int k = 0;
     while (k + 1 < list.count && (int)blockIdx.x >= list.item[k + 1].block0) ++k;
     const ReduceItem it = list.item[k];
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (it.wide == 2) {   // FP32, four neighbouring outputs per lane
+        const int64_t j = ((int64_t)((int)blockIdx.x - it.block0) * 32 + lane) * 4;
+        float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (j < it.n) {
+            const float* p = static_cast<const float*>(it.src) + j;
+#pragma unroll 8
+            for (int i = warp; i < it.parts; i += 8) {
+                const float4 v = *reinterpret_cast<const float4*>(p + (size_t)i * it.n);
+                f.x += v.x; f.y += v.y; f.z += v.z; f.w += v.w;
+            }
+        }
+        s_f4[warp][lane] = f;
+        __syncthreads();
+        if (warp != 0 || j >= it.n) return;
+        for (int w = 1; w < 8; ++w) {
+            const float4 v = s_f4[w][lane];
+            f.x += v.x; f.y += v.y; f.z += v.z; f.w += v.w;
+        }
+        float* dst = static_cast<float*>(it.dst) + j;   // any alignment: a part of the gradient
+        dst[0] = f.x; dst[1] = f.y; dst[2] = f.z; dst[3] = f.w;
+        return;
+    }
     const int64_t j = (int64_t)((int)blockIdx.x - it.block0) * 32 + lane;
     double d = 0.0;
     float f = 0.0f;
@@ -525,6 +553,7 @@ __global__ void mlp_adam_kernel(float* __restrict__ p, const float* __restrict__
                                 float* __restrict__ m, float* __restrict__ v, int64_t n, float lr,
                                 float b1, float b2, float eps, float bc1, float bc2,
                                 bf16* __restrict__ pb) {
+    pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
@@ -897,12 +926,12 @@ __global__ void force_error_kernel(const Vec4<R>* __restrict__ a, const Vec4<R>*
 // while keeping >= 4 (mma.sync) or >= 2 (tcgen05) K steps per slice.
 struct GemmShape { int M, N, K, splits, kslice; bool tc; };
 
-GemmShape gemm_shape(int M, int N, int K) {
+GemmShape gemm_shape(int M, int N, int K, int target = kTargetBlocks) {
     GemmShape s{M, N, K, 1, 0, M >= 64 && N >= 64};
     const int bm = s.tc ? tc::kM : kBM, bn = s.tc ? tc::kN : kBN, bk = s.tc ? tc::kK : kBK;
     const int tiles = ((M + bm - 1) / bm) * ((N + bn - 1) / bn);
     const int ktiles = (K + bk - 1) / bk;
-    int splits = (kTargetBlocks + tiles - 1) / tiles;
+    int splits = (target + tiles - 1) / tiles;
     const int min_steps = s.tc ? 2 : 4;
     const int max_splits = ktiles / min_steps > 1 ? ktiles / min_steps : 1;
     if (splits > max_splits) splits = max_splits;
@@ -912,6 +941,12 @@ GemmShape gemm_shape(int M, int N, int K) {
     s.kslice = per * bk;
     s.splits = (ktiles + per - 1) / per;
     return s;
+}
+
+// A weight gradient: K is the batch, and each K slice leaves a partial product
+// to write and to add, so the tcgen05 kernel gets one block per SM, not two.
+GemmShape grad_shape(int din, int dout, int B) {
+    return gemm_shape(din, dout, B, din >= 64 && dout >= 64 ? kTargetBlocks / 2 : kTargetBlocks);
 }
 
 struct MlpLayout {
@@ -968,7 +1003,7 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
     }
     o.narrow_out = o.d[o.L] <= kThin && o.d[o.L - 1] % 16 == 0 && o.d[o.L - 1] <= kThinInputs;
     for (int i = 0; i < o.L; ++i) {
-        const GemmShape w = gemm_shape(o.d[i], o.d[i + 1], (int)Bz);
+        const GemmShape w = grad_shape(o.d[i], o.d[i + 1], (int)Bz);
         const size_t parts = (size_t)std::max(w.splits, kThinBlocks);
         const bool narrow = narrow_in(o, i) || (i == o.L - 1 && o.narrow_out);
         o.wpart[i] = off;
@@ -980,7 +1015,7 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
     size_t pmax = 0;
     for (int i = 0; i < o.L; ++i) {
         const GemmShape f = gemm_shape((int)Bz, o.d[i + 1], o.d[i]);            // forward
-        const GemmShape w = gemm_shape(o.d[i], o.d[i + 1], (int)Bz);            // dW
+        const GemmShape w = grad_shape(o.d[i], o.d[i + 1], (int)Bz);            // dW
         pmax = std::max(pmax, (size_t)f.splits * f.M * f.N);
         pmax = std::max(pmax, (size_t)w.splits * w.M * w.N);
         if (i > 0) {
@@ -1059,9 +1094,9 @@ struct GemmOut {
 };
 
 template <bool TA, bool TB>
-int gemm(const bf16* A, int64_t lda, const bf16* Bm, int64_t ldb, int M, int N, int K, float* part,
+int gemm(const bf16* A, int64_t lda, const bf16* Bm, int64_t ldb, const GemmShape& s, float* part,
          const GemmOut& g, const LaunchCtx& ctx) {
-    const GemmShape s = gemm_shape(M, N, K);
+    const int M = s.M, N = s.N, K = s.K;
     stage_event(ctx, 0);
     if (g.colsum_rows) *g.colsum_rows = 0;
     if (g.splits) *g.splits = s.splits;
@@ -1077,8 +1112,9 @@ int gemm(const bf16* A, int64_t lda, const bf16* Bm, int64_t ldb, int M, int N, 
             ep = tc::Epilogue{1, g.act, g.bias, g.h, g.out, g.out_b, g.colsum};
             if (g.colsum && g.colsum_rows) *g.colsum_rows = (int)grid.y;
         }
-        k<<<grid, tc::kTmaThreads, tc::kSmemTmaBytes, ctx.stream>>>(ma, mb, part, M, N, K, s.kslice,
-                                                                    ep, ctx.err);
+        if (launch_pdl(k, grid, dim3(tc::kTmaThreads), tc::kSmemTmaBytes, ctx.stream, ma, mb, part, M,
+                       N, K, s.kslice, ep, ctx.err))
+            return ETICS_ERR_CUDA;
     } else if (s.tc) {
         auto k = tc::gemm_kernel<TA, TB>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1105,17 +1141,18 @@ int gemm(const bf16* A, int64_t lda, const bf16* Bm, int64_t ldb, int M, int N, 
     return ETICS_OK;
 }
 
-// the narrow kernels for the run-time width W (1..kThin)
+// a narrow kernel for the run-time width W (1..kThin), arguments as launch_pdl;
+// sets rc
 #define ETICS_NARROW(W, KERNEL, ...)                                        \
     switch (W) {                                                            \
-        case 1: KERNEL<1> __VA_ARGS__; break;                               \
-        case 2: KERNEL<2> __VA_ARGS__; break;                               \
-        case 3: KERNEL<3> __VA_ARGS__; break;                               \
-        case 4: KERNEL<4> __VA_ARGS__; break;                               \
-        case 5: KERNEL<5> __VA_ARGS__; break;                               \
-        case 6: KERNEL<6> __VA_ARGS__; break;                               \
-        case 7: KERNEL<7> __VA_ARGS__; break;                               \
-        default: KERNEL<8> __VA_ARGS__; break;                              \
+        case 1: rc = launch_pdl(KERNEL<1>, __VA_ARGS__); break;                 \
+        case 2: rc = launch_pdl(KERNEL<2>, __VA_ARGS__); break;                 \
+        case 3: rc = launch_pdl(KERNEL<3>, __VA_ARGS__); break;                 \
+        case 4: rc = launch_pdl(KERNEL<4>, __VA_ARGS__); break;                 \
+        case 5: rc = launch_pdl(KERNEL<5>, __VA_ARGS__); break;                 \
+        case 6: rc = launch_pdl(KERNEL<6>, __VA_ARGS__); break;                 \
+        case 7: rc = launch_pdl(KERNEL<7>, __VA_ARGS__); break;                 \
+        default: rc = launch_pdl(KERNEL<8>, __VA_ARGS__); break;                \
     }
 
 // the narrow output layer: y, or with a target the loss and dy
@@ -1124,11 +1161,11 @@ int narrow_out(const MlpLayout& o, const float* params, const bf16* pb, const bf
                const LaunchCtx& ctx) {
     const int i = o.L - 1;
     const int blocks = std::min((B + 127) / 128, kThinBlocks);
-    mlp_narrow_out_kernel<<<blocks, 256, 0, ctx.stream>>>(
-        a, pb + o.woff[i], params + o.boff[i], target, B, o.d[i], o.d[o.L],
-        gemm_shape(B, o.d[o.L], o.d[i]).kslice, scale, y, dyb, at<double>(ws, o.loss_blocks),
-        at<double>(ws, o.bpart[i]));
-    if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    if (launch_pdl(mlp_narrow_out_kernel, dim3(blocks), dim3(256), 0, ctx.stream, a, pb + o.woff[i],
+                   params + o.boff[i], target, B, o.d[i], o.d[o.L],
+                   gemm_shape(B, o.d[o.L], o.d[i]).kslice, scale, y, dyb,
+                   at<double>(ws, o.loss_blocks), at<double>(ws, o.bpart[i])))
+        return ETICS_ERR_CUDA;
     ++*ctx.launches;
     *parts = blocks;
     return ETICS_OK;
@@ -1146,8 +1183,9 @@ int forward_impl(const MlpLayout& o, const float* params, const bf16* pb, const 
         g.act = last ? 0 : 1;
         g.out = last ? y : at<float>(ws, o.h32[i]);
         g.out_b = last ? nullptr : at<bf16>(ws, o.hb[i]);
-        const int rc = gemm<false, true>(a, o.d[i], pb + o.woff[i], o.d[i + 1], B, o.d[i + 1],
-                                         o.d[i], at<float>(ws, o.part), g, ctx);
+        const int rc = gemm<false, true>(a, o.d[i], pb + o.woff[i], o.d[i + 1],
+                                         gemm_shape(B, o.d[i + 1], o.d[i]), at<float>(ws, o.part),
+                                         g, ctx);
         if (rc) return rc;
         if (!last) a = at<bf16>(ws, o.hb[i]);
     }
@@ -1207,8 +1245,9 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
     // partial sums to be added at the end, all in one launch
     ReduceList list{};
     auto reduce = [&](const void* src, void* dst, int64_t n, int parts, int wide, double sc) {
+        if (!wide && n % 4 == 0) wide = 2;   // the partial sums are 256-byte aligned
         list.item[list.count++] = ReduceItem{src, dst, n, parts, list.blocks, wide, sc};
-        list.blocks += (int)((n + 31) / 32);
+        list.blocks += (int)(wide == 2 ? (n + 127) / 128 : (n + 31) / 32);
     };
     // rows per chunk of the narrow kernels
     const int rows = std::max(16, (B + kThinBlocks - 1) / kThinBlocks);
@@ -1226,12 +1265,11 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
         reduce(at<double>(ws, o.loss_blocks), loss, 1, parts, 1, 1.0 / (double)count);
         reduce(at<double>(ws, o.bpart[L - 1]), grads + o.boff[L - 1], dout, parts, 1, 0.0);
         const dim3 grid((din + 255) / 256, chunks);   // 64 threads of four columns
-        ETICS_NARROW(dout, mlp_narrow_back_kernel,
-                     <<<grid, 256, 0, ctx.stream>>>(
-                         a, L > 1 ? at<float>(ws, o.h32[L - 2]) : nullptr, pb + o.woff[L - 1], dyb, B,
-                         din, rows, at<bf16>(ws, o.dzb[cur ^ 1]), at<float>(ws, o.wpart[L - 1]),
-                         L > 1 ? at<double>(ws, o.bpart[L - 2]) : nullptr));
-        if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        ETICS_NARROW(dout, mlp_narrow_back_kernel, grid, dim3(256), 0, ctx.stream, a,
+                     L > 1 ? (const float*)at<float>(ws, o.h32[L - 2]) : nullptr, pb + o.woff[L - 1],
+                     (const bf16*)dyb, B, din, rows, at<bf16>(ws, o.dzb[cur ^ 1]),
+                     at<float>(ws, o.wpart[L - 1]), L > 1 ? at<double>(ws, o.bpart[L - 2]) : nullptr)
+        if (rc) return ETICS_ERR_CUDA;
         ++*ctx.launches;
         reduce(at<float>(ws, o.wpart[L - 1]), grads + o.woff[L - 1], (int64_t)din * dout, chunks, 0, 0.0);
         cur ^= 1;
@@ -1252,10 +1290,9 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
         // dW_i = a_in^T dz
         if (narrow_in(o, i)) {
             const dim3 grid((dout + 255) / 256, chunks);
-            ETICS_NARROW(din, mlp_narrow_in_kernel,
-                         <<<grid, 256, 0, ctx.stream>>>(a_in, dzb, B, dout, rows,
-                                                        at<float>(ws, o.wpart[i])));
-            if (cudaGetLastError()) return ETICS_ERR_CUDA;
+            ETICS_NARROW(din, mlp_narrow_in_kernel, grid, dim3(256), 0, ctx.stream, a_in, dzb, B, dout,
+                         rows, at<float>(ws, o.wpart[i]))
+            if (rc) return ETICS_ERR_CUDA;
             ++*ctx.launches;
             reduce(at<float>(ws, o.wpart[i]), grads + o.woff[i], (int64_t)din * dout, chunks, 0, 0.0);
         } else {
@@ -1263,7 +1300,8 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
             GemmOut g;
             g.out = grads + o.woff[i];
             g.splits = &splits;
-            rc = gemm<true, true>(a_in, din, dzb, dout, din, dout, B, at<float>(ws, o.wpart[i]), g, ctx);
+            rc = gemm<true, true>(a_in, din, dzb, dout, grad_shape(din, dout, B),
+                                  at<float>(ws, o.wpart[i]), g, ctx);
             if (rc) return rc;
             if (splits > 1)
                 reduce(at<float>(ws, o.wpart[i]), grads + o.woff[i], (int64_t)din * dout, splits, 0, 0.0);
@@ -1291,15 +1329,14 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
             g.out_b = at<bf16>(ws, o.dzb[nxt]);
             g.colsum = at<double>(ws, o.bpart[i - 1]);
             g.colsum_rows = &sums;
-            rc = gemm<false, false>(dzb, dout, pb + o.woff[i], dout, B, din, dout,
-                                    at<float>(ws, o.part), g, ctx);
+            rc = gemm<false, false>(dzb, dout, pb + o.woff[i], dout, gs, at<float>(ws, o.part), g, ctx);
             if (rc) return rc;
             if (sums == 0 && !g.out) return ETICS_ERR_CUDA;   // not reached: the test above is gemm's own
             cur = nxt;
         }
     }
-    mlp_reduce_kernel<<<list.blocks, 256, 0, ctx.stream>>>(list);
-    if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    if (launch_pdl(mlp_reduce_kernel, dim3(list.blocks), dim3(256), 0, ctx.stream, list))
+        return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;
 }
@@ -1310,9 +1347,9 @@ int mlp_adam(const etics_mlp_shape* s, float* params, const float* grads, float*
     const int64_t n = mlp_layout(s, 1).nparam;
     const double bc1 = 1.0 / (1.0 - pow((double)b1, (double)t));
     const double bc2 = 1.0 / (1.0 - pow((double)b2, (double)t));
-    mlp_adam_kernel<<<grid_1d(n, ctx), 256, 0, ctx.stream>>>(
-        params, grads, m, v, n, lr, b1, b2, eps, (float)bc1, (float)bc2, reinterpret_cast<bf16*>(pb));
-    if (cudaGetLastError()) return ETICS_ERR_CUDA;
+    if (launch_pdl(mlp_adam_kernel, dim3(grid_1d(n, ctx)), dim3(256), 0, ctx.stream, params, grads, m,
+                   v, n, lr, b1, b2, eps, (float)bc1, (float)bc2, reinterpret_cast<bf16*>(pb)))
+        return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;
 }

@@ -430,6 +430,7 @@ gemm_tma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
+    pdl_wait();   // operands, bias and outputs belong to the kernels before
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem;
