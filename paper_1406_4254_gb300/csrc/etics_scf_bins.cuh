@@ -95,9 +95,47 @@ struct BinConst {
     static constexpr BinPlan<LM> plan = make_bin_plan<LM>();
     static constexpr int nbins = plan.nbins;
 };
-// device copy of the column -> (bin, slot) map, read with run-time indices
+// A bin's columns in its lane's accumulators 0..6: cos and sin of one order are
+// neighbouring columns (c odd, c + 1) and form a pair, so that one paired FMA
+// updates both; accumulators 0..5 are three register pairs, 6 is single and
+// takes what has no partner in the bin, before the halves of free pairs do.
+struct BinItem { int l, c, q; };   // column c (of a pair: c, c + 1) of level l in accumulator q (, q + 1)
+struct BinRegs {
+    int np, ns;
+    BinItem pair[kBinCap / 2], single[kBinCap];
+};
+constexpr BinRegs make_bin_regs(const BinDef& b) {
+    BinRegs r{};
+    for (int s = 0; s < b.nseg; ++s)
+        for (int c = b.seg[s].c0; c < b.seg[s].c0 + b.seg[s].n; ++c) {
+            if (c % 2 == 1 && c + 1 < b.seg[s].c0 + b.seg[s].n) {
+                r.pair[r.np] = BinItem{b.seg[s].l, c, 2 * r.np};
+                ++r.np;
+                ++c;
+            } else {
+                r.single[r.ns++] = BinItem{b.seg[s].l, c, 0};
+            }
+        }
+    for (int i = 0; i < r.ns; ++i) r.single[i].q = i == 0 ? kBinCap - 1 : 2 * r.np + i - 1;
+    return r;
+}
 template <int LM>
-static __constant__ BinIndex<LM> c_bin_index = make_bin_index<LM>();
+constexpr BinIndex<LM> make_bin_acc_index() {   // column -> (bin, accumulator)
+    BinIndex<LM> ix = make_bin_index<LM>();
+    constexpr BinPlan<LM> p = make_bin_plan<LM>();
+    for (int b = 0; b < p.nbins; ++b) {
+        const BinRegs r = make_bin_regs(p.bin[b]);
+        for (int i = 0; i < r.np; ++i)
+            for (int h = 0; h < 2; ++h)
+                ix.slot[r.pair[i].l * r.pair[i].l + r.pair[i].c + h] = r.pair[i].q + h;
+        for (int i = 0; i < r.ns; ++i)
+            ix.slot[r.single[i].l * r.single[i].l + r.single[i].c] = r.single[i].q;
+    }
+    return ix;
+}
+// device copy of it, read with run-time indices
+template <int LM>
+static __constant__ BinIndex<LM> c_bin_index = make_bin_acc_index<LM>();
 
 struct ScfBinParams {
     const void* posm;
@@ -112,110 +150,146 @@ struct ScfBinParams {
     double dt;
 };
 
+// A lane's accumulators (or its columns' values) in the order of BinRegs
+struct BinValues {
+    float2 p[kBinCap / 2];
+    float s;
+};
+// The columns of a tile of T particles in shared memory: the (cos, sin) pairs
+// of (l, m), m >= 1, at (l (l-1) / 2 + m - 1) T as float2, the m = 0 columns
+// behind them at l T, then xi.
+template <int LM, int T>
+__device__ __forceinline__ const float* bin_zonal(const float2* Y) {
+    return reinterpret_cast<const float*>(Y + LM * (LM + 1) / 2 * T);
+}
+__host__ __device__ constexpr int bin_pair_column(int l, int c) { return l * (l - 1) / 2 + (c + 1) / 2 - 1; }
+
 // rows of segment S of bin B and the segments after it for one particle: the
 // Gegenbauer values of the segment's level times its columns y (harmonics
 // scaled by mass and radial prefactor)
-template <typename R, int NR, int LM, int B, int S>
-__device__ __forceinline__ void bin_segment(R (&acc)[NR][kBinCap], const R (&y)[kBinCap], R xi) {
+template <int NR, int LM, int B, int S>
+__device__ __forceinline__ void bin_segment(BinValues (&acc)[NR], const BinValues& y, float xi) {
     constexpr BinDef bd = BinConst<LM>::plan.bin[B];
     if constexpr (S < bd.nseg) {
-        constexpr BinSeg g = bd.seg[S];
-        constexpr int off = [] {
-            int o = 0;
-            for (int s = 0; s < S; ++s) o += BinConst<LM>::plan.bin[B].seg[s].n;
-            return o;
-        }();
-        R cm1 = R(0), cn = R(1);
+        constexpr int l = bd.seg[S].l;
+        constexpr BinRegs r = make_bin_regs(bd);
+        float cm1 = 0.0f, cn = 1.0f;
 #pragma unroll
         for (int n = 0; n < NR; ++n) {
             if (n == 1) {
                 cm1 = cn;
                 cn = xi;
             } else if (n > 1) {
-                const R cnew = fma(xi, cn, -geg_bs<R>(g.l, n) * cm1);   // rescaled
+                const float cnew = fma(xi, cn, -geg_bs<float>(l, n) * cm1);   // rescaled
                 cm1 = cn;
                 cn = cnew;
             }
 #pragma unroll
-            for (int c = 0; c < g.n; ++c)
-                acc[n][off + c] = n == 0 ? acc[n][off + c] + y[off + c]
-                                         : fma(cn, y[off + c], acc[n][off + c]);
+            for (int i = 0; i < r.np; ++i)
+                if (r.pair[i].l == l)
+                    acc[n].p[i] = n == 0 ? add2(acc[n].p[i], y.p[i])
+                                         : fma2(splat<float2>(cn), y.p[i], acc[n].p[i]);
+#pragma unroll
+            for (int i = 0; i < r.ns; ++i)
+                if (r.single[i].l == l) {
+                    const int q = r.single[i].q;
+                    if (q == kBinCap - 1) acc[n].s = fma(cn, y.s, acc[n].s);
+                    else if (q % 2 == 0) acc[n].p[q / 2].x = fma(cn, y.p[q / 2].x, acc[n].p[q / 2].x);
+                    else acc[n].p[q / 2].y = fma(cn, y.p[q / 2].y, acc[n].p[q / 2].y);
+                }
         }
-        bin_segment<R, NR, LM, B, S + 1>(acc, y, xi);
+        bin_segment<NR, LM, B, S + 1>(acc, y, xi);
     }
 }
-template <typename R, int LM, int T, int B, int S = 0>
-__device__ __forceinline__ void bin_load(R (&y)[kBinCap], const R* Ys, int k) {
-    constexpr BinDef bd = BinConst<LM>::plan.bin[B];
-    if constexpr (S < bd.nseg) {
-        constexpr BinSeg g = bd.seg[S];
-        constexpr int off = [] {
-            int o = 0;
-            for (int s = 0; s < S; ++s) o += BinConst<LM>::plan.bin[B].seg[s].n;
-            return o;
-        }();
+template <int LM, int T, int B>
+__device__ __forceinline__ void bin_load(BinValues& y, const float2* Y, int k) {
+    constexpr BinRegs r = make_bin_regs(BinConst<LM>::plan.bin[B]);
 #pragma unroll
-        for (int c = 0; c < g.n; ++c) y[off + c] = Ys[(g.l * g.l + g.c0 + c) * T + k];
-        bin_load<R, LM, T, B, S + 1>(y, Ys, k);
+    for (int i = 0; i < r.np; ++i) y.p[i] = Y[bin_pair_column(r.pair[i].l, r.pair[i].c) * T + k];
+#pragma unroll
+    for (int i = 0; i < r.ns; ++i) {
+        const int l = r.single[i].l, c = r.single[i].c, q = r.single[i].q;
+        const float v = c == 0 ? bin_zonal<LM, T>(Y)[l * T + k]
+                               : reinterpret_cast<const float*>(Y)[2 * (bin_pair_column(l, c) * T + k) +
+                                                                   (c + 1) % 2];
+        if (q == kBinCap - 1) y.s = v;
+        else if (q % 2 == 0) y.p[q / 2].x = v;
+        else y.p[q / 2].y = v;
     }
 }
 
 // the lane's particles of one tile of n; the next one's values are loaded
 // before this one's rows
-template <typename R, int NR, int LM, int T, int B>
-__device__ __forceinline__ void bin_tile(R (&acc)[NR][kBinCap], const R* Ys, const R* Xs, int lane,
-                                         int n) {
-    R y[kBinCap], xi = Xs[lane];
-    bin_load<R, LM, T, B>(y, Ys, lane);
+template <int NR, int LM, int T, int B>
+__device__ __forceinline__ void bin_tile(BinValues (&acc)[NR], const float2* Y, int lane, int n) {
+    const float* Xs = bin_zonal<LM, T>(Y) + (LM + 1) * T;
+    BinValues y = {};
+    float xi = Xs[lane];
+    bin_load<LM, T, B>(y, Y, lane);
 #pragma unroll 1
     for (int k = lane; k < n; k += 32) {
         const int kn = k + 32 < T ? k + 32 : lane;
-        R yn[kBinCap];
-        const R xn = Xs[kn];
-        bin_load<R, LM, T, B>(yn, Ys, kn);
-        bin_segment<R, NR, LM, B, 0>(acc, y, xi);
+        BinValues yn = {};
+        const float xn = Xs[kn];
+        bin_load<LM, T, B>(yn, Y, kn);
+        bin_segment<NR, LM, B, 0>(acc, y, xi);
         xi = xn;
-#pragma unroll
-        for (int c = 0; c < BinConst<LM>::plan.bin[B].ncol; ++c) y[c] = yn[c];
+        y = yn;
     }
 }
 
-template <typename R, int NR, int LM, int T, int B>
-__device__ __forceinline__ void bin_dispatch(int warp, R (&acc)[NR][kBinCap], const R* Ys,
-                                             const R* Xs, int lane, int n) {
+template <int NR, int LM, int T, int B>
+__device__ __forceinline__ void bin_dispatch(int warp, BinValues (&acc)[NR], const float2* Y, int lane,
+                                             int n) {
     if constexpr (B < BinConst<LM>::nbins) {
-        if (warp == B) bin_tile<R, NR, LM, T, B>(acc, Ys, Xs, lane, n);
-        else bin_dispatch<R, NR, LM, T, B + 1>(warp, acc, Ys, Xs, lane, n);
+        if (warp == B) bin_tile<NR, LM, T, B>(acc, Y, lane, n);
+        else bin_dispatch<NR, LM, T, B + 1>(warp, acc, Y, lane, n);
     }
 }
 
-// phase 1: w_l H_l^m of the columns of orders m in [M0, M1] into Ys, order by
-// order (the recursion in l at fixed m of harm_level_exact), so that two
-// threads share a particle and no thread holds more than two levels of one
-// order.  w[l] = m pre0 st^l; (c, s) the sectoral value of order M.
-template <typename R, int LM, int T, int M, int M1>
-__device__ __forceinline__ void bin_orders(const R (&w)[LM + 1], R ux, R uy, R uz, R c, R s, R* Ys) {
-    R c1 = c, s1 = s, c2 = R(0), s2 = R(0);   // level l - 1, l - 2 below
+// sectoral value (cos, sin) of order m from that of order m - 1
+__device__ __forceinline__ float2 bin_sectoral(int m, float2 cs, float ux, float uy) {
+    const float d = 2 * m - 1;
+    return mk2(d * (ux * cs.x - uy * cs.y), d * (ux * cs.y + uy * cs.x));
+}
+
+// phase 1: w_l H_l^m of the columns of orders m in [M, M1] of particle k into
+// Y, order by order (the recursion in l at fixed m of harm_level_exact, cos and
+// sin as one pair), so that two threads share a particle and no thread holds
+// more than two levels of one order.  w[l] = m pre0 st^l; cs the sectoral value
+// of order M.
+template <int LM, int T, int M, int M1>
+__device__ __forceinline__ void bin_orders(const float (&w)[LM + 1], float ux, float uy, float uz,
+                                           float2 cs, float2* Y, int k) {
+    if constexpr (M == 0) {
+        float* Z = const_cast<float*>(bin_zonal<LM, T>(Y));
+        float c1 = 1.0f, c2 = 0.0f;   // levels l - 1 and l - 2
 #pragma unroll
-    for (int l = M; l <= LM; ++l) {
-        if (l > M) {
-            const R d = R(2 * l - 1) * uz, b = R((l + M - 1) * (l - M - 1));
-            const R cn = l == M + 1 ? d * c1 : fma(d, c1, -b * c2);
-            const R sn = l == M + 1 ? d * s1 : fma(d, s1, -b * s2);
-            c2 = c1; s2 = s1;
-            c1 = cn; s1 = sn;
+        for (int l = 0; l <= LM; ++l) {
+            if (l > 0) {
+                const float d = (2 * l - 1) * uz;
+                const float cn = l == 1 ? d * c1 : fma(d, c1, -(float)((l - 1) * (l - 1)) * c2);
+                c2 = c1;
+                c1 = cn;
+            }
+            Z[l * T + k] = w[l] * c1;
         }
-        if constexpr (M == 0) {
-            Ys[l * l * T] = w[l] * c1;
-        } else {
-            Ys[(l * l + 2 * M - 1) * T] = w[l] * c1;
-            Ys[(l * l + 2 * M) * T] = w[l] * s1;
+    } else {
+        float2 v1 = cs, v2 = mk2(0.0f, 0.0f);
+#pragma unroll
+        for (int l = M; l <= LM; ++l) {
+            if (l > M) {
+                const float2 d = splat<float2>((2 * l - 1) * uz);
+                const float2 vn = l == M + 1 ? mul2(d, v1)
+                                             : fma2(d, v1, mul2(splat<float2>(-(float)((l + M - 1) * (l - M - 1))), v2));
+                v2 = v1;
+                v1 = vn;
+            }
+            Y[bin_pair_column(l, 2 * M) * T + k] = mul2(splat<float2>(w[l]), v1);
         }
     }
-    if constexpr (M < M1) {
-        constexpr R d = R(2 * M + 1);
-        bin_orders<R, LM, T, M + 1, M1>(w, ux, uy, uz, d * (ux * c - uy * s), d * (ux * s + uy * c), Ys);
-    }
+    if constexpr (M < M1)
+        bin_orders<LM, T, M + 1, M1>(w, ux, uy, uz, bin_sectoral(M + 1, cs, ux, uy), Y, k);
 }
 // orders 0..half-1 have about half of the columns
 template <int LM>
@@ -250,20 +324,22 @@ __device__ __forceinline__ void warp_scatter(float* v, int lane) {
 // and the two phases alternate.  Bound: FMA issue, NR x 7 updates and a
 // recursion of 2 NR per bin and particle.  (14, 8), 2^24 particles: 2645 us
 // with phase 1 on half of the warps and an FP64 addition per column in the
-// flush, 2158 without these and with two buffers of 192, 2050 so.
+// flush, 2158 without these and with two buffers of 192, 2050 with this tile,
+// 1390 with cos and sin updated by one paired FMA (fewer instructions to fetch
+// and to issue: the FMA pipe's share of busy cycles went from 45% to 56%).
 template <int LM>
 __host__ __device__ constexpr int bins_threads() { return BinConst<LM>::nbins * 32; }
 template <int LM>
 __host__ __device__ constexpr int bins_tile() { return bins_threads<LM>() * 3 / 2; }
-template <typename R, int NR, int LM, bool DRIFT>
+template <int NR, int LM, bool DRIFT>
 constexpr size_t bins_smem() {
     return ((size_t)BinConst<LM>::nbins * NR * kBinCap * sizeof(double) + 15) / 16 * 16 +
-           (size_t)bins_tile<LM>() * ((DRIFT ? 3 : 1) * sizeof(Vec4<R>) + ((LM + 1) * (LM + 1) + 1) * sizeof(R));
+           (size_t)bins_tile<LM>() * ((DRIFT ? 3 : 1) * sizeof(float4) + ((LM + 1) * (LM + 1) + 1) * sizeof(float));
 }
 // DRIFT: kick and drift the particles as they are read (the copies of a tile's
 // velocities and accelerations are hidden behind the contraction of the tile
 // before; a kick-drift kernel is bound by memory, 188 us at 2^24).
-template <typename R, int NR, int LM, bool DRIFT>
+template <int NR, int LM, bool DRIFT>
 __global__ void __launch_bounds__(bins_threads<LM>(), 1)
 scf_coeff_bins_kernel(ScfBinParams p) {
     constexpr int NB = BinConst<LM>::nbins;
@@ -271,35 +347,38 @@ scf_coeff_bins_kernel(ScfBinParams p) {
     constexpr int T = bins_tile<LM>();  // particles per tile
     constexpr int K1 = TH / 2;          // particles per round of phase 1
     static_assert(T % 32 == 0 && T % K1 == 0, "tile");
-    constexpr int NCOL = (LM + 1) * (LM + 1);
     constexpr int NOUT = NB * NR * kBinCap;
-    using V4 = Vec4<R>;
+    using V4 = float4;
     // dynamic shared memory: accd [NOUT] doubles, the next tile's particles
-    // P [T], (DRIFT) their velocities and accelerations V [T], A [T], then
-    // Ys [NCOL][T] and xi [T]
+    // P [T], (DRIFT) their velocities and accelerations V [T], A [T], then the
+    // columns and xi
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* accd = reinterpret_cast<double*>(smem_raw);
     V4* P = reinterpret_cast<V4*>(smem_raw + ((NOUT * sizeof(double) + 15) / 16) * 16);
     V4* V = P + T;
     V4* A = V + T;
-    R* Ys = reinterpret_cast<R*>(P + (DRIFT ? 3 : 1) * T);
+    float2* Y = reinterpret_cast<float2*>(P + (DRIFT ? 3 : 1) * T);   // see bin_zonal
+    float* Xs = const_cast<float*>(bin_zonal<LM, T>(Y)) + (LM + 1) * T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k1 = tid < K1 ? tid : tid - K1;   // phase 1: this thread's particle
     const V4* posm = reinterpret_cast<const V4*>(p.posm);
     for (int e = tid; e < NOUT; e += TH) accd[e] = 0.0;
-    R acc[NR][kBinCap];
+    BinValues acc[NR];
 #pragma unroll
-    for (int n = 0; n < NR; ++n)
-#pragma unroll
-        for (int c = 0; c < kBinCap; ++c) acc[n][c] = R(0);
+    for (int n = 0; n < NR; ++n) acc[n] = BinValues{};
 
     // FP64 additions are slow on this GPU: each total is one lane's, so that a
     // few warp-wide instructions add them all
     auto flush = [&]() {
         constexpr int kPerWarp = NR * kBinCap, K = (kPerWarp + 31) / 32 * 32;
-        R v[K];
+        float v[K];
 #pragma unroll
-        for (int i = 0; i < K; ++i) v[i] = i < kPerWarp ? acc[i / kBinCap][i % kBinCap] : R(0);
+        for (int i = 0; i < K; ++i) {
+            const int q = i % kBinCap;
+            if (i >= kPerWarp) { v[i] = 0.0f; continue; }
+            const BinValues& a = acc[i / kBinCap];
+            v[i] = q == kBinCap - 1 ? a.s : q % 2 == 0 ? a.p[q / 2].x : a.p[q / 2].y;
+        }
         warp_scatter<K, 16>(v, lane);
 #pragma unroll
         for (int i = 0; i < K / 32; ++i) {
@@ -307,9 +386,7 @@ scf_coeff_bins_kernel(ScfBinParams p) {
             if (idx < kPerWarp) accd[warp * kPerWarp + idx] += (double)v[i];
         }
 #pragma unroll
-        for (int n = 0; n < NR; ++n)
-#pragma unroll
-            for (int c = 0; c < kBinCap; ++c) acc[n][c] = R(0);
+        for (int n = 0; n < NR; ++n) acc[n] = BinValues{};
     };
     const int64_t lo = (int64_t)blockIdx.x * p.per;
     const int64_t hi = lo + p.per < p.N ? lo + p.per : p.N;
@@ -329,7 +406,7 @@ scf_coeff_bins_kernel(ScfBinParams p) {
     };
     // the thread's own copies have arrived: kick, drift, and back to memory
     auto step = [&](int64_t first) {
-        const R dt = (R)p.dt, h = R(0.5) * dt;
+        const float dt = (float)p.dt, h = 0.5f * dt;
         for (int i = tid; i < T && first + i < hi; i += TH) {
             V4 x = P[i], v = V[i];
             kick_drift(x, v, A[i], h, dt);
@@ -339,30 +416,26 @@ scf_coeff_bins_kernel(ScfBinParams p) {
         }
     };
     auto basis = [&](const V4& cur, int k) {
-        R x = R(0), y = R(0), z = R(0), m = R(0);
+        float x = 0.0f, y = 0.0f, z = 0.0f, m = 0.0f;
         if (finite4(cur.x, cur.y, cur.z, cur.w)) { x = cur.x; y = cur.y; z = cur.z; m = cur.w; }
         else report(p.err, ETICS_ERR_NONFINITE);
-        const R r = sqrt(x * x + y * y + z * z);
-        const R t = R(1) / (R(1) + r), st = r * t * t;
-        const R inv = r > R(0) ? R(1) / r : R(0);
-        R w[LM + 1];
+        const float r = sqrtf(x * x + y * y + z * z);
+        const float t = 1.0f / (1.0f + r), st = r * t * t;
+        const float inv = r > 0.0f ? 1.0f / r : 0.0f;
+        float w[LM + 1];
         w[0] = -m * t;
 #pragma unroll
         for (int l = 1; l <= LM; ++l) w[l] = w[l - 1] * st;
         constexpr int H = bin_half_order<LM>();
-        const R ux = x * inv, uy = y * inv, uz = z * inv;
+        const float ux = x * inv, uy = y * inv, uz = z * inv;
+        float2 cs = mk2(1.0f, 0.0f);
         if (tid < K1) {
-            Ys[NCOL * T + k] = R(1) - R(2) * t;
-            bin_orders<R, LM, T, 0, H - 1>(w, ux, uy, uz, R(1), R(0), Ys + k);
+            Xs[k] = 1.0f - 2.0f * t;
+            bin_orders<LM, T, 0, H - 1>(w, ux, uy, uz, cs, Y, k);
         } else {
-            R c = R(1), s = R(0);
 #pragma unroll
-            for (int m1 = 1; m1 <= H; ++m1) {
-                const R cn = R(2 * m1 - 1) * (ux * c - uy * s);
-                s = R(2 * m1 - 1) * (ux * s + uy * c);
-                c = cn;
-            }
-            bin_orders<R, LM, T, H, LM>(w, ux, uy, uz, c, s, Ys + k);
+            for (int m1 = 1; m1 <= H; ++m1) cs = bin_sectoral(m1, cs, ux, uy);
+            bin_orders<LM, T, H, LM>(w, ux, uy, uz, cs, Y, k);
         }
     };
 
@@ -377,7 +450,7 @@ scf_coeff_bins_kernel(ScfBinParams p) {
         for (int k = k1; k < n; k += K1) basis(P[k], k);
         __syncthreads();   // the columns are there; P is free
         if (first + T < hi) fetch(first + T);
-        bin_dispatch<R, NR, LM, T, 0>(warp, acc, Ys, Ys + NCOL * T, lane, n);
+        bin_dispatch<NR, LM, T, 0>(warp, acc, Y, lane, n);
         if (++since == kBinFlushTiles) { flush(); since = 0; }
     }
     if (since) flush();
@@ -414,12 +487,12 @@ __global__ void scf_finalize_bins_kernel(const double* __restrict__ partial, int
     }
 }
 
-template <typename R, int NR, int LM>
+template <int NR, int LM>
 inline size_t scf_bins_workspace(int num_sms) {
     return (size_t)num_sms * BinConst<LM>::nbins * NR * kBinCap * sizeof(double);
 }
 
-template <typename R, int NR, int LM>
+template <int NR, int LM>
 inline int scf_coeffs_bins_launch(const void* posm, int64_t N, double* coeffs, void* ws,
                                   DriftStep drift, const LaunchCtx& ctx) {
     constexpr int TH = bins_threads<LM>();
@@ -429,12 +502,12 @@ inline int scf_coeffs_bins_launch(const void* posm, int64_t N, double* coeffs, v
     const int grid = (int)((N + per - 1) / per);
     ScfBinParams p{posm, N, per, reinterpret_cast<double*>(ws), ctx.err,
                    drift.posm, drift.vel, drift.acc, drift.dt};
-    static_assert(bins_smem<R, NR, LM, true>() <= 227 * 1024, "bins kernel shared memory");
-    const size_t smem = drift.posm ? bins_smem<R, NR, LM, true>() : bins_smem<R, NR, LM, false>();
+    static_assert(bins_smem<NR, LM, true>() <= 227 * 1024, "bins kernel shared memory");
+    const size_t smem = drift.posm ? bins_smem<NR, LM, true>() : bins_smem<NR, LM, false>();
     int nblocks = 0;
     if (N > 0) {
-        auto k = drift.posm ? scf_coeff_bins_kernel<R, NR, LM, true>
-                            : scf_coeff_bins_kernel<R, NR, LM, false>;
+        auto k = drift.posm ? scf_coeff_bins_kernel<NR, LM, true>
+                            : scf_coeff_bins_kernel<NR, LM, false>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ||
             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100))
             return ETICS_ERR_CUDA;

@@ -10,10 +10,10 @@
 
 namespace etics {
 size_t scf_bins148_workspace_f32(int num_sms) {
-    return scf_bins_workspace<float, 15, 8>(num_sms);
+    return scf_bins_workspace<15, 8>(num_sms);
 }
 int scf_coeffs_bins148_f32(const void* posm, int64_t N, double* coeffs, void* ws, DriftStep drift,
                            const LaunchCtx& ctx) {
-    return scf_coeffs_bins_launch<float, 15, 8>(posm, N, coeffs, ws, drift, ctx);
+    return scf_coeffs_bins_launch<15, 8>(posm, N, coeffs, ws, drift, ctx);
 }
 }  // namespace etics
