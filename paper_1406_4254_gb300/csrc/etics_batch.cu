@@ -482,7 +482,8 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
 // (three blocks of 128 threads per SM at 168 registers: with one of 256 the
 // kernel takes 210 registers and leaves 8 warps per SM.  256 systems, 17
 // million particles: 1300 us with one particle per thread, 1200 with two and
-// 256 threads, 1160 so.)
+// 256 threads, 990 so; a launch per register class of l_max, 16 warps up to
+// l_max = 6, took 1070: more tails than it gained.)
 constexpr int kBatchFieldThreads = 128;
 template <typename P, bool ACC>
 __global__ void __launch_bounds__(kBatchFieldThreads, 3)

@@ -60,8 +60,10 @@ static __device__ const FieldTable g_field_tab = make_field_table();
 // The table: row n holds the levels' 2l+1 columns, each level followed by at
 // least one place of padding, the last of which holds -bs_n, so that the
 // recursion constant arrives with the columns.  `stride` entries per row (a
-// constant of the kernel, so that a round's rows are at immediate offsets).
+// constant of the kernel, so that a round's rows are at immediate offsets), at
+// least two rows.
 // Warps take rows, lanes columns: one look for a column's level for all rows.
+__host__ __device__ constexpr int field_rows(int n_max) { return n_max < 1 ? 2 : n_max + 1; }
 template <typename R>
 __device__ __forceinline__ void field_table(R* cs, int stride, const double* coeffs, int basis,
                                             int n_max, int l_max) {
@@ -70,9 +72,10 @@ __device__ __forceinline__ void field_table(R* cs, int stride, const double* coe
         int l = 0, k = c;
         while (k >= ncol_pad(l)) { k -= ncol_pad(l); ++l; }
         const int am = (k + 1) / 2, m = (k & 1) ? am : -am;   // k = 0: m = 0
-        for (int n = threadIdx.x >> 5; n <= n_max; n += blockDim.x >> 5)
+        for (int n = threadIdx.x >> 5; n < field_rows(n_max); n += blockDim.x >> 5)
             cs[n * stride + c] =
-                k < 2 * l + 1 ? (R)(__ldcg(coeffs + (size_t)n * nj + l * l + l + m) *
+                n > n_max ? R(0)   // at least two rows
+                : k < 2 * l + 1 ? (R)(__ldcg(coeffs + (size_t)n * nj + l * l + l + m) *
                                     g_field_tab.v[basis][n][l * (l + 1) / 2 + am])
                 : k == ncol_pad(l) - 1 ? -geg_bs_of<R>(basis, l, n) : R(0);
     }
@@ -149,19 +152,18 @@ struct FieldEval {
             constexpr int stride = col_offset_c(LM + 1);
             const int nlim = NM1 > 0 ? NM1 - 1 : n_max;
             const R* r = cs + col_offset_c(L);
-            P A[NC], Q = splat<P>(R(0));
+            P A[NC], Q;
             {
+                // rows 0 and 1 (always there): Ct_0 = 1, Dt_0 = 0, Ct_1 = xi,
+                // Dt_1 = 1; row 0 is the addend of the first FMAs, not a copy
                 V4 v[ncol_pad_c(L) / 4];
-                load_row<L>(r, v);                          // Ct_0 = 1, Dt_0 = 0
+                load_row<L>(r, v);
 #pragma unroll
                 for (int k = 0; k < NC; ++k) {
                     const V4 q = v[k / 4];
                     A[k] = splat<P>(k % 4 == 0 ? q.x : k % 4 == 1 ? q.y : k % 4 == 2 ? q.z : q.w);
                 }
-            }
-            if (nlim >= 1) {
-                r += stride;                                // Ct_1 = xi, Dt_1 = 1
-                V4 v[ncol_pad_c(L) / 4];
+                r += stride;
                 load_row<L>(r, v);
                 P sum;
                 add_row<L>(v, xi, A, C[s0], S[s0], sum);
@@ -340,7 +342,7 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm, int64_
         field_eval<P, LM, ACC, NM1, B>(pv, cs, n_max, l_max, split.level[part], res);
         if (split.parts > 1) {
             // parts 1.. leave their sums behind the table, part 0 adds them
-            Vec4<R>* sums = reinterpret_cast<Vec4<R>*>(cs + (n_max + 1) * stride);
+            Vec4<R>* sums = reinterpret_cast<Vec4<R>*>(cs + field_rows(n_max) * stride);
             if (part > 0) {
 #pragma unroll
                 for (int j = 0; j < NP; ++j) st4(sums + ((part - 1) * NP + j) * per + slot, res[j]);
@@ -399,7 +401,7 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     const int threads = warps * 32 * parts;
     const int64_t want = (lanes + warps * 32 - 1) / (warps * 32);
     const int grid = (int)(want < sms ? want : sms);
-    const size_t smem = (size_t)(n_max + 1) * col_offset_c(LM + 1) * sizeof(R) +
+    const size_t smem = (size_t)field_rows(n_max) * col_offset_c(LM + 1) * sizeof(R) +
                         (parts > 1 ? (size_t)(kFieldParts - 1) * FieldLane<P>::kParticles * warps * 32 *
                                          sizeof(Vec4<R>) : 0);
     auto k = (out_mask & ETICS_OUT_ACC) ? scf_field_kernel<P, LM, true, NM1, B>
