@@ -23,7 +23,10 @@
 //
 // All kernels are launched with programmatic dependent launch, so each launch
 // overlaps its predecessor's tail.
+#include <algorithm>
+#include <array>
 #include <atomic>
+#include <utility>
 #include <cstddef>
 
 #include "etics_internal.h"
@@ -679,6 +682,7 @@ __device__ __forceinline__ uint64_t r2_bits(const dvec4& v) {
 constexpr int kOversample = 16;
 constexpr int kMaxBuckets = 1024;
 constexpr int kPartThreads = 1024;          // one thread per bucket
+constexpr int kPartTiles = 151;             // one block per SM on a 152-SM part, less one
 constexpr int kBucketKpt = 12;              // members per thread at capacity
 constexpr int kSmallThreads = 256, kLargeThreads = 512;
 constexpr int kSmallMean = 1024, kLargeMean = 2048;
@@ -696,7 +700,12 @@ SamplePlan sample_plan(int64_t N) {
     if (N > kSampleMaxN) return p;
     p.mean = N <= int64_t(kMaxBuckets) * kSmallMean ? kSmallMean : kLargeMean;
     p.nbuckets = N <= kSingleMax ? 1 : (int)((N + p.mean - 1) / p.mean);
-    p.kpt = N <= (int64_t(1) << 18) ? 2 : N <= (int64_t(1) << 19) ? 4 : 8;
+    // as few particles per thread as let the tiles and the block with the table
+    // run at once, one block per SM (at 2^20 147 tiles of 7168 instead of 128
+    // of 8192)
+    p.kpt = (int)std::min<int64_t>(8, (N + int64_t(kPartTiles) * kPartThreads - 1) /
+                                          (int64_t(kPartTiles) * kPartThreads));
+    if (p.kpt < 1) p.kpt = 1;
     p.ntiles = (int)((N + (int64_t)kPartThreads * p.kpt - 1) / ((int64_t)kPartThreads * p.kpt));
     return p;
 }
@@ -1393,6 +1402,13 @@ static int launch_partition(const Vec4<R>* pp, int64_t N, const SamplePlan& sp,
     return ETICS_OK;
 }
 
+// for 1..8 particles per thread
+template <typename R, int... I>
+static constexpr auto partition_launchers(std::integer_sequence<int, I...>) {
+    return std::array<int (*)(const Vec4<R>*, int64_t, const SamplePlan&, const SortBuffers&,
+                              const LaunchCtx&), sizeof...(I)>{&launch_partition<R, I + 1>...};
+}
+
 template <typename R, int TH, int KPT>
 static int launch_buckets(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, const SortBuffers& b,
                           Vec4<R>* sorted, const LaunchCtx& ctx) {
@@ -1413,9 +1429,8 @@ template <typename R>
 static int sample_sort(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, const SortBuffers& b,
                        Vec4<R>* sorted, const LaunchCtx& ctx) {
     if (sp.nbuckets > 1) {
-        const int rc = sp.kpt == 2   ? launch_partition<R, 2>(pp, N, sp, b, ctx)
-                       : sp.kpt == 4 ? launch_partition<R, 4>(pp, N, sp, b, ctx)
-                                     : launch_partition<R, 8>(pp, N, sp, b, ctx);
+        static constexpr auto kRun = partition_launchers<R>(std::make_integer_sequence<int, 8>());
+        const int rc = kRun[sp.kpt - 1](pp, N, sp, b, ctx);
         if (rc) return rc;
     }
     stage_event(ctx, 1);
