@@ -949,6 +949,10 @@ GemmShape grad_shape(int din, int dout, int B) {
     return gemm_shape(din, dout, B, din >= 64 && dout >= 64 ? kTargetBlocks / 2 : kTargetBlocks);
 }
 
+// rows per chunk of the narrow kernels, and the chunks
+int thin_rows(int B) { return std::max(16, (B + kThinBlocks - 1) / kThinBlocks); }
+int thin_chunks(int B) { return (B + thin_rows(B) - 1) / thin_rows(B); }
+
 struct MlpLayout {
     int L;
     int d[6];
@@ -956,7 +960,7 @@ struct MlpLayout {
     int64_t nparam;
     int dmax;
     // workspace offsets (bytes)
-    size_t h32[5], hb[5], y32, dz32[2], dzb[2], part, loss_blocks, colsum;
+    size_t h32[5], hb[5], y32, dz32[2], dzb[2], part, loss_blocks;
     size_t wpart[5], bpart[5];         // a layer's partial weight and bias gradients
     size_t total;
     bool narrow_out;                   // the output layer runs on the narrow kernels
@@ -1004,12 +1008,15 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
     o.narrow_out = o.d[o.L] <= kThin && o.d[o.L - 1] % 16 == 0 && o.d[o.L - 1] <= kThinInputs;
     for (int i = 0; i < o.L; ++i) {
         const GemmShape w = grad_shape(o.d[i], o.d[i + 1], (int)Bz);
-        const size_t parts = (size_t)std::max(w.splits, kThinBlocks);
+        const size_t parts = (size_t)std::max(w.splits, thin_chunks((int)Bz));
         const bool narrow = narrow_in(o, i) || (i == o.L - 1 && o.narrow_out);
         o.wpart[i] = off;
         off += al256((narrow ? parts : (size_t)w.splits) * o.d[i] * o.d[i + 1] * 4);
         o.bpart[i] = off;
-        off += al256(std::max((size_t)kThinBlocks, (Bz + tc::kM - 1) / tc::kM) * o.d[i + 1] * 8);
+        // rows of column sums: of a narrow kernel, of a product's tiles, or of
+        // mlp_colsum_partial_kernel
+        off += al256(std::max({(size_t)thin_chunks((int)Bz), ((size_t)Bz + tc::kM - 1) / tc::kM,
+                               std::min((size_t)Bz, (size_t)kColChunks)}) * o.d[i + 1] * 8);
     }
     // the largest split-K partial buffer over all products
     size_t pmax = 0;
@@ -1025,7 +1032,6 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
     }
     o.part = off; off += al256(pmax * 4);
     o.loss_blocks = off; off += al256(std::max(kLossBlocks, kThinBlocks) * 8);
-    o.colsum = off; off += al256((size_t)kColChunks * o.dmax * 8);
     o.total = off;
     return o;
 }
@@ -1250,8 +1256,7 @@ int mlp_loss_grad(const etics_mlp_shape* s, const float* params, const uint16_t*
         list.blocks += (int)(wide == 2 ? (n + 127) / 128 : (n + 31) / 32);
     };
     // rows per chunk of the narrow kernels
-    const int rows = std::max(16, (B + kThinBlocks - 1) / kThinBlocks);
-    const int chunks = (B + rows - 1) / rows;
+    const int rows = thin_rows(B), chunks = thin_chunks(B);
     int cur = 0;
     int top = L - 1;       // the layer whose dz is in dz32/dzb[cur]
     int sums = 0;          // rows of its column sums in bpart[top]; 0: not made
