@@ -5,10 +5,10 @@
 #include "etics_scf_coeffs.cuh"
 
 namespace etics {
-size_t scf_coeffs_f32_a_workspace(int rows, int num_sms) {
-    if (rows == 3) return scf_coeff_plan_workspace<3>(num_sms);
-    if (rows == 5) return scf_coeff_plan_workspace<5>(num_sms);
-    if (rows == 7) return scf_coeff_plan_workspace<7>(num_sms);
+size_t scf_coeffs_f32_a_workspace(int rows, int l_max, int num_sms) {
+    if (rows == 3) return scf_coeff_plan_workspace<3>(l_max, num_sms);
+    if (rows == 5) return scf_coeff_plan_workspace<5>(l_max, num_sms);
+    if (rows == 7) return scf_coeff_plan_workspace<7>(l_max, num_sms);
     return 0;
 }
 int scf_coeffs_f32_a(int rows, const void* posm, int64_t N, int n_max, int l_max, int basis,

@@ -5,9 +5,9 @@
 #include "etics_scf_coeffs.cuh"
 
 namespace etics {
-size_t scf_coeffs_f32_b_workspace(int rows, int num_sms) {
-    if (rows == 9) return scf_coeff_plan_workspace<9>(num_sms);
-    if (rows == 11) return scf_coeff_plan_workspace<11>(num_sms);
+size_t scf_coeffs_f32_b_workspace(int rows, int l_max, int num_sms) {
+    if (rows == 9) return scf_coeff_plan_workspace<9>(l_max, num_sms);
+    if (rows == 11) return scf_coeff_plan_workspace<11>(l_max, num_sms);
     return 0;
 }
 int scf_coeffs_f32_b(int rows, const void* posm, int64_t N, int n_max, int l_max, int basis,

@@ -5,8 +5,8 @@
 #include "etics_scf_coeffs.cuh"
 
 namespace etics {
-size_t scf_coeffs_f32_d_workspace(int rows, int num_sms) {
-    if (rows == 17) return scf_coeff_plan_workspace<17>(num_sms);
+size_t scf_coeffs_f32_d_workspace(int rows, int l_max, int num_sms) {
+    if (rows == 17) return scf_coeff_plan_workspace<17>(l_max, num_sms);
     return 0;
 }
 int scf_coeffs_f32_d(int rows, const void* posm, int64_t N, int n_max, int l_max, int basis,

@@ -24,7 +24,7 @@ int scf_coeffs_f32(const void* posm, int64_t N, int n_max, int l_max, int basis,
                    void* ws, DriftStep drift, const LaunchCtx& ctx);
 // its parts, by the number of rows (n_max + 1 rounded up to an odd number)
 #define ETICS_COEFF_PART(k)                                                                      \
-    size_t scf_coeffs_f32_##k##_workspace(int rows, int num_sms);                                \
+    size_t scf_coeffs_f32_##k##_workspace(int rows, int l_max, int num_sms);                     \
     int scf_coeffs_f32_##k(int rows, const void* posm, int64_t N, int n_max, int l_max, int basis, \
                            double* coeffs, void* ws, const LaunchCtx& ctx)
 ETICS_COEFF_PART(a);

@@ -93,6 +93,23 @@ __device__ __forceinline__ void harm_scaled(const P* C1, const P* S1, const P* C
     }
 }
 
+// warp totals of v[0..K), K a multiple of 32, by a reduce-scatter (each step
+// halves the values a lane still holds): lane j ends with the totals of values
+// j K/32 .. in v[0..K/32)
+template <int K, int O>
+__device__ __forceinline__ void warp_scatter(float* v, int lane) {
+    if constexpr (O >= 1) {
+        const bool up = lane & O;
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) {
+            const float give = up ? v[i] : v[i + K / 2];
+            const float keep = up ? v[i + K / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, O);
+        }
+        warp_scatter<K / 2, O / 2>(v, lane);
+    }
+}
+
 // 16-byte asynchronous global -> shared copies
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);

@@ -299,23 +299,6 @@ __host__ __device__ constexpr int bin_half_order() {
     return m;
 }
 
-// warp totals of v[0..K), K a multiple of 32, by a reduce-scatter (each step
-// halves the values a lane still holds): lane j ends with the totals of values
-// j K/32 .. in v[0..K/32)
-template <int K, int O>
-__device__ __forceinline__ void warp_scatter(float* v, int lane) {
-    if constexpr (O >= 1) {
-        const bool up = lane & O;
-#pragma unroll
-        for (int i = 0; i < K / 2; ++i) {
-            const float give = up ? v[i] : v[i + K / 2];
-            const float keep = up ? v[i + K / 2] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, O);
-        }
-        warp_scatter<K / 2, O / 2>(v, lane);
-    }
-}
-
 // Two threads per particle in phase 1, one warp per bin in phase 2, one block
 // per SM: 105 accumulators a lane leave room for 12 warps.  Every bin is
 // straight-line code of its own, and so is phase 1: with tiles of 192

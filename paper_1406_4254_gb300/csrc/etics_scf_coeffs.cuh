@@ -65,6 +65,7 @@ struct CoeffGroup { int bin0, nbins, teams, l_lo, l_hi, block0, nblocks, pad; };
 struct CoeffPlan {
     int ngroups, nbins, warps, l_max;
     int nblocks;                       // of all groups
+    int slots;                         // bins a block has partial sums for, at most
     CoeffGroup group[kCoeffMaxGroups];
     CoeffBin bin[kCoeffMaxBins];
 };
@@ -73,7 +74,7 @@ struct ScfCoeffPairParams {
     const float4* posm;
     int64_t N;
     int basis;
-    double* partial;   // [block][warps][NR][CAP]
+    double* partial;   // [block][plan.slots][NR][CAP]
     unsigned* err;
     CoeffPlan plan;
 };
@@ -121,6 +122,12 @@ inline double coeff_bins(CoeffPlan& p, double* cost, int n_rows, int l_max, int 
 // the recursion more often but can occupy warps that would idle (l_max = 4: 9
 // bins of up to 4 columns or 15 of up to 2, for 16 warps).  Blocks per group in
 // proportion to its cost.
+// A bin has at least two columns where its level does: at most l + 1 bins of
+// level l, and in a group at most one per warp.
+inline int coeff_slots(int l_max, int warps) {
+    const int n = (l_max + 1) * (l_max + 2) / 2;
+    return n < warps ? n : warps;
+}
 inline CoeffPlan make_coeff_plan(int n_rows, int l_max, int cap, int warps, int64_t N, int num_sms) {
     CoeffPlan p, t;
     double cost[kCoeffMaxGroups], c[kCoeffMaxGroups], total = 1e301;
@@ -132,6 +139,7 @@ inline CoeffPlan make_coeff_plan(int n_rows, int l_max, int cap, int warps, int6
             for (int g = 0; g < p.ngroups; ++g) cost[g] = c[g];
         }
     }
+    p.slots = coeff_slots(l_max, warps);
     // at least 64 particles (one pair per lane) per block
     int64_t most = (N + 63) / 64;
     int left = num_sms;
@@ -222,22 +230,6 @@ __device__ __forceinline__ void pair_rows_nc(int nc, float2 (&acc)[NR][CAP], con
     }
 }
 
-// Reduce-scatter over the warp: v[0..K) per lane, K a multiple of 32; lane j
-// ends with the warp totals of values j K/32 ... in v[0..K/32).
-template <int K, int O>
-__device__ __forceinline__ void reduce_scatter(float* v, int lane) {
-    if constexpr (O >= 1) {
-        const bool up = lane & O;
-#pragma unroll
-        for (int i = 0; i < K / 2; ++i) {
-            const float give = up ? v[i] : v[i + K / 2];
-            const float keep = up ? v[i + K / 2] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, O);
-        }
-        reduce_scatter<K / 2, O / 2>(v, lane);
-    }
-}
-
 template <int NR, int LMU>
 __global__ void __launch_bounds__(PairShape<NR>::kWarps * 32, 1)
 scf_coeff_plan_kernel(const __grid_constant__ ScfCoeffPairParams p) {
@@ -277,7 +269,7 @@ scf_coeff_plan_kernel(const __grid_constant__ ScfCoeffPairParams p) {
 #pragma unroll
         for (int i = 0; i < K; ++i)
             v[i] = i < kPerWarp ? acc[i / CAP][i % CAP].x + acc[i / CAP][i % CAP].y : 0.0f;
-        reduce_scatter<K, 16>(v, lane);
+        warp_scatter<K, 16>(v, lane);
 #pragma unroll
         for (int i = 0; i < K / 32; ++i) {
             const int idx = lane * (K / 32) + i;
@@ -348,8 +340,13 @@ scf_coeff_plan_kernel(const __grid_constant__ ScfCoeffPairParams p) {
     }
     if (since && active) flush();
     __syncthreads();
-    double* out = p.partial + (size_t)blockIdx.x * PairShape<NR>::kWarps * kPerWarp;
-    for (int e = tid; e < PairShape<NR>::kWarps * kPerWarp; e += blockDim.x) out[e] = accd[e];
+    // the teams' sums of a bin, in team order
+    double* out = p.partial + (size_t)blockIdx.x * p.plan.slots * kPerWarp;
+    for (int e = tid; e < gr.nbins * kPerWarp; e += blockDim.x) {
+        double sum = accd[e];
+        for (int k = 1; k < gr.teams; ++k) sum += accd[k * gr.nbins * kPerWarp + e];
+        out[e] = sum;
+    }
 }
 
 // Block sums added in block order; one warp per output c[n][l*l+l+m], four
@@ -378,13 +375,11 @@ scf_finalize_plan_kernel(const __grid_constant__ ScfCoeffPairParams p, int n_max
     while (b >= p.plan.group[g].bin0 + p.plan.group[g].nbins) ++g;
     const CoeffGroup gr = p.plan.group[g];
     const int idx = ((b - gr.bin0) * NR + n) * CAP + col - p.plan.bin[b].c0;
-    const size_t stride = (size_t)PairShape<NR>::kWarps * NR * CAP;
+    const size_t stride = (size_t)p.plan.slots * NR * CAP;
+    const double* src = p.partial + (size_t)gr.block0 * stride + idx;
     double s = 0.0;
-    for (int team = 0; team < gr.teams; ++team) {
-        const double* src = p.partial + (size_t)gr.block0 * stride + (size_t)team * gr.nbins * NR * CAP + idx;
 #pragma unroll 4
-        for (int k = lane; k < gr.nblocks; k += 32) s += __ldcg(src + (size_t)k * stride);
-    }
+    for (int k = lane; k < gr.nblocks; k += 32) s += __ldcg(src + (size_t)k * stride);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
@@ -404,8 +399,9 @@ inline size_t coeff_smem(const CoeffPlan& p) {
 }
 
 template <int NR>
-inline size_t scf_coeff_plan_workspace(int num_sms) {
-    return (size_t)num_sms * PairShape<NR>::kWarps * NR * PairShape<NR>::kCap * sizeof(double);
+inline size_t scf_coeff_plan_workspace(int l_max, int num_sms) {
+    return (size_t)num_sms * coeff_slots(l_max, PairShape<NR>::kWarps) * NR * PairShape<NR>::kCap *
+           sizeof(double);
 }
 
 template <int NR, int LMU>

@@ -14,7 +14,7 @@ size_t scf_workspace_f32(int64_t N, int n_max, int l_max, int num_sms) {
     // at least what the register-tile kernel takes (the FP64 path's, and this
     // path's before it ran on particle pairs)
     size_t most = scf_workspace<float>(N, n_max, l_max, num_sms);
-    most = std::max(most, need(rows, num_sms));
+    most = std::max(most, need(rows, l_max, num_sms));
     if (n_max == 10 && l_max == 6) most = std::max(most, scf_pairs106_workspace_f32(num_sms));
     if (n_max == 14 && l_max == 8) most = std::max(most, scf_bins148_workspace_f32(num_sms));
     return most;

@@ -213,33 +213,27 @@ scf_coeff_pairs_kernel(ScfPairParams p) {
 #pragma unroll
         for (int c = 0; c < CAP; ++c) acc[n][c] = make_float2(0.0f, 0.0f);
 
-    // Flush: every warp total of the NR x CAP accumulators (pair halves
-    // added, then a butterfly over the lanes) is kept by lane (index % 32),
-    // so that the FP64 additions into the block sums run as a few warp-wide
-    // instructions instead of one instruction per value (FP64 issue is slow
-    // on this GPU).  Columns beyond the bin's width hold zeros.
+    // Flush: the warp totals of the NR x CAP accumulators (pair halves added)
+    // by a reduce-scatter, each total one lane's, so that the FP64 additions
+    // into the block sums run as a few warp-wide instructions (FP64 issue is
+    // slow on this GPU).  Columns beyond the bin's width hold zeros.
     constexpr int kPerWarp = NR * CAP;
-    constexpr int kRounds = (kPerWarp + 31) / 32;
     auto flush = [&]() {
-        float mine[kRounds];
+        constexpr int K = (kPerWarp + 31) / 32 * 32;
+        float v[K];
 #pragma unroll
-        for (int r = 0; r < kRounds; ++r) mine[r] = 0.0f;
+        for (int i = 0; i < K; ++i)
+            v[i] = i < kPerWarp ? acc[i / CAP][i % CAP].x + acc[i / CAP][i % CAP].y : 0.0f;
+        warp_scatter<K, 16>(v, lane);
+#pragma unroll
+        for (int i = 0; i < K / 32; ++i) {
+            const int idx = lane * (K / 32) + i;
+            if (idx < kPerWarp) accd[warp * kPerWarp + idx] += (double)v[i];
+        }
 #pragma unroll
         for (int n = 0; n < NR; ++n)
 #pragma unroll
-            for (int c = 0; c < CAP; ++c) {
-                float v = acc[n][c].x + acc[n][c].y;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                const int idx = n * CAP + c;
-                if (lane == (idx & 31)) mine[idx >> 5] = v;
-                acc[n][c] = make_float2(0.0f, 0.0f);
-            }
-#pragma unroll
-        for (int r = 0; r < kRounds; ++r) {
-            const int idx = r * 32 + lane;
-            if (idx < kPerWarp) accd[warp * kPerWarp + idx] += (double)mine[r];
-        }
+            for (int c = 0; c < CAP; ++c) acc[n][c] = make_float2(0.0f, 0.0f);
     };
     // this block's particles: one contiguous range, so that every block has
     // the same work up to one particle pair (the last tile may be partial;

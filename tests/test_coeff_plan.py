@@ -35,12 +35,12 @@ template <int NR> void check(int64_t N, int num_sms) {
         CHECK(p.warps == W);
         CHECK((coeff_tile<NR, 8>() <= W * 32 && coeff_tile<NR, kLmaxLimit>() <= W * 32));
         CHECK((l_max <= 8 ? coeff_smem<NR, 8>(p) : coeff_smem<NR, kLmaxLimit>(p)) <= 227 * 1024);
-        CHECK((size_t)p.nblocks * W * NR * CAP * 8 <= scf_coeff_plan_workspace<NR>(num_sms));
+        CHECK((size_t)p.nblocks * p.slots * NR * CAP * 8 <= scf_coeff_plan_workspace<NR>(l_max, num_sms));
         int bin = 0, block = 0;
         for (int g = 0; g < p.ngroups; ++g) {
             const CoeffGroup& q = p.group[g];
             CHECK(q.bin0 == bin && q.block0 == block && q.nblocks >= 1 && q.teams >= 1);
-            CHECK(q.nbins * q.teams <= p.warps);
+            CHECK(q.nbins * q.teams <= p.warps && q.nbins <= p.slots);
             for (int b = q.bin0; b < q.bin0 + q.nbins; ++b)
                 CHECK(p.bin[b].l >= q.l_lo && p.bin[b].l <= q.l_hi);
             bin += q.nbins;
