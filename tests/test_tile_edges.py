@@ -44,12 +44,14 @@ def order_of(pm):
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_radial_order_across_the_sort_paths(precision):
     """The order is exact on both sides of every line the sort draws by size:
-    one block up to 8192, buckets of mean 1024 up to 2^20 and of mean 2048 up
+    one block up to 8192, one to eight particles per thread (154624 each) in
+    the partition, buckets of mean 1024 up to 2^20 and of mean 2048 up
     to 2^21, the radix passes above; particles already in radial order, in two
     interleaved populations, and with one radius crowding (more equal keys
     than a bucket or a bin holds)."""
     rng = np.random.default_rng(3)
-    for n in (1023, 8191, 8192, 8193, 9217, (1 << 18) + 1, (1 << 20) + 1, (1 << 21) + 1):
+    for n in (1023, 8191, 8192, 8193, 9217, 154625, (1 << 18) + 1, 400001, 800001, (1 << 20) + 1,
+              (1 << 21) + 1):
         pm = hernquist(n, seed=5)
         if n == 8193:
             pm = pm[order_of(pm)]                      # sorted already
@@ -103,3 +105,30 @@ def test_scf_coefficient_tile_edges(nl, basis):
         etics.check_error()
         tol = max(2e-6, (10 + 5 * l_max + 2 * n_max) * 2.0 ** -24)
         assert np.max(np.abs(got.reshape(want.shape) - want)) <= tol * np.max(np.abs(want)), n
+
+
+@pytest.mark.parametrize("tile", [0, 64, 320])
+def test_batch_step_edges(tile):
+    """The mixed-precision batch takes 256 particles a step, adds its FP32 sums
+    in FP64 every 16 steps and walks chunks of 16 tiles of the plan: sizes around
+    each, odd sizes, and every l_max (a layout of its own).  Tolerance as above."""
+    sizes = [1, 2, 255, 256, 257, 511, 513, 1023, 1025, 4095, 4096, 4097, 5119, 5121, 8191, 8193, 12289]
+    n_maxes = [14 - i % 15 for i in range(len(sizes))]
+    l_maxes = [i % 9 for i in range(len(sizes))]
+    pms = [hernquist(n, seed=n) for n in sizes]
+    tuning = etics.BatchTuning(tile, 0, 0, 0) if tile else None
+    plan = etics.BatchPlan(sizes, n_maxes, l_maxes, precision=etics.MIXED, tuning=tuning)
+    d = device_particles(np.concatenate(pms), "mixed")
+    packed, out = etics.scf_batch(d, plan)
+    etics.check_error()
+    out = out.cpu().numpy()
+    first = 0
+    for i, (n, n_max, l_max) in enumerate(zip(sizes, n_maxes, l_maxes)):
+        ref = rounded(pms[i], "mixed")
+        want = oracle.scf_coeffs(ref[:, :3], ref[:, 3], n_max, l_max)
+        got = plan.coeffs_of(packed, i).cpu().numpy().reshape(want.shape)
+        tol = max(2e-6, (10 + 5 * l_max + 2 * n_max) * 2.0 ** -24)
+        assert np.max(np.abs(got - want)) <= tol * np.max(np.abs(want)), (n, n_max, l_max)
+        acc, pot = oracle.scf_field(ref[:, :3], n_max, l_max, want)
+        close(out[first:first + n], acc, pot, "mixed", (n, n_max, l_max))
+        first += n
