@@ -511,50 +511,53 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
 }
 
 // ---------------------------------------------------------------------------
-// 3. field: one work item (a chunk of one instance) per block iteration
+// 3. field: one work item (a chunk of one instance), or a part of it, per block
 // ---------------------------------------------------------------------------
 // (three blocks of 128 threads per SM at 168 registers: with one of 256 the
 // kernel takes 210 registers and leaves 8 warps per SM.  256 systems, 17
 // million particles: 1300 us with one particle per thread, 1200 with two and
-// 256 threads, 990 so; a launch per register class of l_max, 16 warps up to
-// l_max = 6, took 1070: more tails than it gained.)
-constexpr int kBatchFieldThreads = 128;
+// 256 threads, 980 with 128 and blocks that walk several items, 835 with one
+// item per block)
+constexpr int kBatchFieldThreads = 128, kFieldWaves = 12;
 template <typename P, bool ACC>
 __global__ void __launch_bounds__(kBatchFieldThreads, 3)
 batch_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm,
-                   const void* __restrict__ plan, const double* coeffs,
+                   const void* __restrict__ plan, int parts, const double* coeffs,
                    Vec4<typename FieldLane<P>::R>* __restrict__ out, int out_mask, unsigned* err) {
     using R = typename FieldLane<P>::R;
     constexpr int NP = FieldLane<P>::kParticles;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* cs = reinterpret_cast<R*>(smem_raw);
-    const BatchHeader hd = *plan_table<BatchHeader>(plan, 0);
+    const BatchHeader& hd = *plan_table<BatchHeader>(plan, 0);
     const BatchInst* insts = plan_table<BatchInst>(plan, hd.off_inst);
     const BatchField* items = plan_table<BatchField>(plan, hd.off_field);
-    for (int w = blockIdx.x; w < hd.nfield; w += gridDim.x) {
-        const BatchField it = items[w];
-        const BatchInst in = insts[it.inst];
-        __syncthreads();
-        field_table(cs, col_offset_c(kBatchLM + 1), coeffs + in.coef_offset, ETICS_BASIS_HO, in.n_max,
-                    in.l_max);
-        __syncthreads();
-        for (int k = threadIdx.x * NP; k < it.count; k += blockDim.x * NP) {
-            const int64_t i = in.offset + it.begin + k;
-            Vec4<R> pv[NP], res[NP];
+    // one part of an item per block: the hardware hands out the blocks, and
+    // items differ in cost by a factor of 20
+    BatchField it = items[blockIdx.x / parts];
+    const BatchInst in = insts[it.inst];
+    const int share = (it.count + parts - 1) / parts, skip = (int)(blockIdx.x % parts) * share;
+    it.begin += skip;
+    it.count = it.count - skip < share ? it.count - skip : share;
+    if (it.count <= 0) return;
+    field_table(cs, col_offset_c(kBatchLM + 1), coeffs + in.coef_offset, ETICS_BASIS_HO, in.n_max,
+                in.l_max);
+    __syncthreads();
+    for (int k = threadIdx.x * NP; k < it.count; k += blockDim.x * NP) {
+        const int64_t i = in.offset + it.begin + k;
+        Vec4<R> pv[NP], res[NP];
 #pragma unroll
-            for (int j = 0; j < NP; ++j) {
-                pv[j] = k + j < it.count ? ld4(posm + i + j) : mk4<R>(R(0), R(0), R(0), R(0));
-                if (!finite4(pv[j].x, pv[j].y, pv[j].z, pv[j].w)) report(err, ETICS_ERR_NONFINITE);
-            }
-            field_eval<P, kBatchLM, ACC, 0, 0>(pv, cs, in.n_max, in.l_max, ~0u, res);
+        for (int j = 0; j < NP; ++j) {
+            pv[j] = k + j < it.count ? ld4(posm + i + j) : mk4<R>(R(0), R(0), R(0), R(0));
+            if (!finite4(pv[j].x, pv[j].y, pv[j].z, pv[j].w)) report(err, ETICS_ERR_NONFINITE);
+        }
+        field_eval<P, kBatchLM, ACC, 0, 0>(pv, cs, in.n_max, in.l_max, ~0u, res);
 #pragma unroll
-            for (int j = 0; j < NP; ++j) {
-                if (k + j >= it.count) continue;
-                if (!(out_mask & ETICS_OUT_POT)) res[j].w = R(0);
-                if (!finite4(res[j].x, res[j].y, res[j].z, res[j].w))
-                    report(err, ETICS_ERR_NONFINITE);
-                st4(out + i + j, res[j]);
-            }
+        for (int j = 0; j < NP; ++j) {
+            if (k + j >= it.count) continue;
+            if (!(out_mask & ETICS_OUT_POT)) res[j].w = R(0);
+            if (!finite4(res[j].x, res[j].y, res[j].z, res[j].w))
+                report(err, ETICS_ERR_NONFINITE);
+            st4(out + i + j, res[j]);
         }
     }
 }
@@ -601,10 +604,18 @@ int batch_plan_build(const etics_batch_item* items, int ninst, const etics_batch
         ctot += (int64_t)(it.n_max + 1) * (it.l_max + 1) * (it.l_max + 1);
         const int64_t nt = (it.n + tn.tile - 1) / tn.tile;
         ntiles += nt;
-        nchunks += (nt + kBpChunkTiles - 1) / kBpChunkTiles;
         nfield += (it.n + tn.field_chunk - 1) / tn.field_chunk;
     }
     if (ntot >= (int64_t(1) << 30) || ntiles >= (int64_t(1) << 30)) return ETICS_ERR_ARG;
+    // chunks of up to kBpChunkTiles tiles, fewer where that would leave the
+    // resident blocks (two per SM) less than about eight chunks each
+    int chunk_tiles = (int)(ntot / ((int64_t)num_sms * 2 * 8) / tn.tile);
+    if (chunk_tiles > kBpChunkTiles) chunk_tiles = kBpChunkTiles;
+    if (chunk_tiles < 2) chunk_tiles = 2;
+    for (int i = 0; i < ninst; ++i) {
+        const int64_t nt = (items[i].n + tn.tile - 1) / tn.tile;
+        nchunks += (nt + chunk_tiles - 1) / chunk_tiles;
+    }
     const bool mixed = precision == ETICS_MIXED;
     // FP64: persistent blocks over static tile ranges, one segment per
     // (block, instance).  Mixed: blocks claim chunks, one segment per chunk
@@ -718,8 +729,8 @@ int batch_plan_build(const etics_batch_item* items, int ninst, const etics_batch
             BatchInst& in = insts[i];
             in.first_seg = c;
             in.nseg = 0;
-            for (int k0 = 0; k0 < in.ntiles; k0 += kBpChunkTiles) {
-                const int k1 = k0 + kBpChunkTiles < in.ntiles ? k0 + kBpChunkTiles : in.ntiles;
+            for (int k0 = 0; k0 < in.ntiles; k0 += chunk_tiles) {
+                const int k1 = k0 + chunk_tiles < in.ntiles ? k0 + chunk_tiles : in.ntiles;
                 chunks[c++] = BatchChunk{i, in.first_tile + k0, in.first_tile + k1, 0};
                 ++in.nseg;
             }
@@ -814,7 +825,10 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
     if (out && hd.nfield > 0) {
         using FieldP = std::conditional_t<sizeof(R) == 4, float2, double>;
         const size_t smem = (size_t)(kBatchNR) * col_total(kBatchLM) * sizeof(R);
-        int grid = hd.nfield < ctx.num_sms * 8 ? hd.nfield : ctx.num_sms * 8;
+        // items are split while fewer than kFieldWaves rounds of resident blocks
+        int parts = 1;
+        while (parts < 4 && (int64_t)hd.nfield * parts < (int64_t)kFieldWaves * 3 * ctx.num_sms) parts *= 2;
+        const int grid = hd.nfield * parts;
         const int threads = std::min(hd.field_threads, kBatchFieldThreads);
         if (out_mask & ETICS_OUT_ACC) {
             auto k = batch_field_kernel<FieldP, true>;
@@ -822,7 +836,7 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
                 cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
                 return ETICS_ERR_CUDA;
             k<<<grid, threads, smem, ctx.stream>>>(
-                reinterpret_cast<const Vec4<R>*>(posm), plan_dev, coeffs,
+                reinterpret_cast<const Vec4<R>*>(posm), plan_dev, parts, coeffs,
                 reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err);
         } else {
             auto k = batch_field_kernel<FieldP, false>;
@@ -830,7 +844,7 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
                 cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
                 return ETICS_ERR_CUDA;
             k<<<grid, threads, smem, ctx.stream>>>(
-                reinterpret_cast<const Vec4<R>*>(posm), plan_dev, coeffs,
+                reinterpret_cast<const Vec4<R>*>(posm), plan_dev, parts, coeffs,
                 reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err);
         }
         if (cudaGetLastError()) return ETICS_ERR_CUDA;

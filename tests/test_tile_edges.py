@@ -110,7 +110,7 @@ def test_scf_coefficient_tile_edges(nl, basis):
 @pytest.mark.parametrize("tile", [0, 64, 320])
 def test_batch_step_edges(tile):
     """The mixed-precision batch takes 256 particles a step, adds its FP32 sums
-    in FP64 every 16 steps and walks chunks of 16 tiles of the plan: sizes around
+    in FP64 every 16 steps and walks chunks of 2 to 16 tiles of the plan: sizes around
     each, odd sizes, and every l_max (a layout of its own).  Tolerance as above."""
     sizes = [1, 2, 255, 256, 257, 511, 513, 1023, 1025, 4095, 4096, 4097, 5119, 5121, 8191, 8193, 12289]
     n_maxes = [14 - i % 15 for i in range(len(sizes))]
