@@ -83,9 +83,9 @@ def kernel_traffic():
 
 
 def mex_bytes(fp64=False):
-    # keys 16R+12W, 4 sort passes (8R+8W), tie pass 4R, gather 4R+16R+16W,
-    # pass2 16R+4R+16W  (per particle, FP32 particles)
-    b = 16 + 12 + 4 * 16 + 4 + (4 + 16 + 16) + (16 + 4 + 16)
+    # partition 16R+8W, bucket sort 8R+16R+4W+16W, pass1 16R, pass2
+    # 16R+4R+16W  (per particle, FP32 particles; up to 2^21 of them)
+    b = (16 + 8) + (8 + 16 + 4 + 16) + 16 + (16 + 4 + 16)
     return b + (3 * 16 if fp64 else 0)
 
 
@@ -1290,9 +1290,9 @@ def main():
         "scf_coeff_pairs_kernel": ("alu", st["coef_kernel"], scf_coeff_flops(N_MAX, L_MAX)),
         "scf_field_kernel": ("alu", st["field_kernel"], scf_field_flops(N_MAX, L_MAX)),
         "mex_pass2_kernel": ("alu", st["mex_pass2"], mex_flops(L_MAX)),
-        "mex_sort (keys + 4 radix passes + ties)": ("hbm", st["mex_keys"] + st["mex_sort"],
-                                                    16 + 4 + 4 * 16 + 4),
-        "mex_pass1_kernel": ("hbm", st["mex_tile_sums"], 4 + 16 + 16),
+        "mex_sort (partition + bucket sort)": ("hbm", st["mex_keys"] + st["mex_sort"],
+                                               (16 + 8) + (8 + 16 + 4 + 16)),
+        "mex_pass1_kernel": ("hbm", st["mex_tile_sums"], 16),
     }
     table = {}
     for name, (bound, ms_k, work) in kern.items():
@@ -1308,11 +1308,8 @@ def main():
                            "unit": "GB/s", "frac": ach / peaks["hbm_gbs"],
                            "work_per_particle": work, "work_unit": "byte"}
         if name.startswith("mex_sort"):
-            # the group's launches: keygen, the 4 radix passes, the tie fix-up
-            parts = [traffic.get("keygen_kernel"), traffic.get("onesweep_kernel"),
-                     traffic.get("tie_fixup_kernel")]
-            table[name]["traffic"] = (None if None in parts
-                                      else parts[0] + 4 * parts[1] + parts[2])
+            parts = [traffic.get("partition_kernel"), traffic.get("bucket_sort_kernel")]
+            table[name]["traffic"] = None if None in parts else sum(parts)
         else:
             table[name]["traffic"] = traffic.get(name)
     # the SCF pass as a whole (coefficient kernel + finalize + field kernel),
