@@ -79,8 +79,6 @@ constexpr double csqrt(double x) {
 struct BasisTables {
     // Gegenbauer recursion C_n = a[l][n] xi C_{n-1} - b[l][n] C_{n-2}, alpha = 2l + 3/2:
     //   a = 2 (n + alpha - 1) / n,  b = (n + 2 alpha - 2) / n   (n >= 1; C_{-1} = 0)
-    float ga_f[kLmaxLimit + 1][kNmaxLimit + 1];
-    float gb_f[kLmaxLimit + 1][kNmaxLimit + 1];
     double ga_d[kLmaxLimit + 1][kNmaxLimit + 1];
     double gb_d[kLmaxLimit + 1][kNmaxLimit + 1];
     // real orthonormal normalisation of the unnormalised harmonics used on
@@ -96,8 +94,6 @@ struct BasisTables {
     // Clutton-Brock basis (Plummer zeroth term): Gegenbauer alpha = l + 1 and
     // 1/J_nl, J_nl = -K_nl 2^-(4l+6) (n+2l+1)! / (n! (n+l+1) (l!)^2),
     // K_nl = 4n(n+2l+2) + (2l+1)(2l+3)
-    float ga_cb_f[kLmaxLimit + 1][kNmaxLimit + 1];
-    float gb_cb_f[kLmaxLimit + 1][kNmaxLimit + 1];
     double ga_cb_d[kLmaxLimit + 1][kNmaxLimit + 1];
     double gb_cb_d[kLmaxLimit + 1][kNmaxLimit + 1];
     double inv_j_cb[kNmaxLimit + 1][kLmaxLimit + 1];
@@ -124,8 +120,6 @@ constexpr BasisTables make_tables() {
             }
             t.ga_d[l][n] = a;
             t.gb_d[l][n] = b;
-            t.ga_f[l][n] = (float)a;
-            t.gb_f[l][n] = (float)b;
         }
         for (int m = 0; m <= l; ++m) {
             double ratio = 1.0;   // (l-m)!/(l+m)!
@@ -160,8 +154,6 @@ constexpr BasisTables make_tables() {
             }
             t.ga_cb_d[l][n] = a;
             t.gb_cb_d[l][n] = b;
-            t.ga_cb_f[l][n] = (float)a;
-            t.gb_cb_f[l][n] = (float)b;
             const double K = 4.0 * n * (n + 2.0 * l + 2.0) + (2.0 * l + 1.0) * (2.0 * l + 3.0);
             double num = 1.0;                         // (n+2l+1)!/n!
             for (int k = n + 1; k <= n + 2 * l + 1; ++k) num *= (double)k;
@@ -256,42 +248,15 @@ struct RadialSeed {
 //   Z_m^m     = (2m-1) (ux + i uy) Z_{m-1}^{m-1}
 //   Z_{m+1}^m = (2m+1) uz Z_m^m
 //   (l-m) Z_l^m = (2l-1) uz Z_{l-1}^m - (l+m-1) |u|^2 Z_{l-2}^m
-// Gradient (homogeneous of degree l-1) from level l-1 by the ladder relations
-//   d/dz Z_l^m = (l+m) Z_{l-1}^m,
-//   (d/dx - i d/dy) Z_l^m = (l+m)(l+m-1) Z_{l-1}^{m-1},
-//   (d/dx + i d/dy) Z_l^m = -Z_{l-1}^{m+1}   (m >= 1),
-// and for m = 0: grad C_l^0 = (-C_{l-1}^1, -S_{l-1}^1, l C_{l-1}^0).
 // Arrays are indexed by m and must be used with compile-time l (unrolled).
 // ---------------------------------------------------------------------------
-template <typename R, int L>
-__device__ __forceinline__ void harm_level(const R* C1, const R* S1, const R* C2, const R* S2,
-                                           R ux, R uy, R uz, R uu, R* C, R* S) {
-    if constexpr (L == 0) {
-        C[0] = R(1);
-        S[0] = R(0);
-    } else {
-        constexpr R d = R(2 * L - 1);
-        C[L] = d * (ux * C1[L - 1] - uy * S1[L - 1]);
-        S[L] = d * (ux * S1[L - 1] + uy * C1[L - 1]);
-        C[L - 1] = d * uz * C1[L - 1];
-        S[L - 1] = (L - 1 == 0) ? R(0) : d * uz * S1[L - 1];
-#pragma unroll
-        for (int m = 0; m + 2 <= L; ++m) {
-            const R a = R(2 * L - 1) / R(L - m);
-            const R b = R(L + m - 1) / R(L - m);
-            C[m] = a * uz * C1[m] - b * uu * C2[m];
-            S[m] = (m == 0) ? R(0) : a * uz * S1[m] - b * uu * S2[m];
-        }
-    }
-}
-
-// The same harmonics scaled by (L-m)!, for the coefficient passes:
+// Scaled by (L-m)!, for the coefficient passes:
 //   H_L^m = (L-m)! Z_L^m(u) on the unit sphere (|u| = 1 taken exactly),
 //   H_m^m     = (2m-1) (ux + i uy) H_{m-1}^{m-1}
 //   H_{m+1}^m = (2m+1) uz H_m^m
 //   H_L^m     = (2L-1) uz H_{L-1}^m - (L+m-1)(L-m-1) H_{L-2}^m.
 // Every recursion constant is an integer, exact in FP32.  With the ratios
-// (2L-1)/(L-m) and (L+m-1)/(L-m) rounded to FP32 (harm_level above) the
+// (2L-1)/(L-m) and (L+m-1)/(L-m) rounded to FP32 the
 // rounding of the constants leaks into lower harmonics and, through
 // uz Z_1^0, into a constant: a bias of about -2e-8 in P_l (l >= 3, m = 0)
 // with a non-zero mean over the sphere, which every particle adds
@@ -316,74 +281,6 @@ __device__ __forceinline__ void harm_level_exact(const R* C1, const R* S1, const
             const R b = R((L + m - 1) * (L - m - 1));
             C[m] = fma(duz, C1[m], -b * C2[m]);
             S[m] = (m == 0) ? R(0) : fma(duz, S1[m], -b * S2[m]);
-        }
-    }
-}
-
-// gradient of C_L^m (gc) and S_L^m (gs) from level L-1 values (C1, S1; m <= L-1)
-template <typename R, int L>
-__device__ __forceinline__ void harm_grad(const R* C1, const R* S1, int m, R gc[3], R gs[3]) {
-    // values of level L-1 outside 0..L-1 are zero
-    auto c1 = [&](int k) -> R { return (k >= 0 && k <= L - 1) ? C1[k] : R(0); };
-    auto s1 = [&](int k) -> R { return (k >= 1 && k <= L - 1) ? S1[k] : R(0); };
-    if (m == 0) {
-        gc[0] = -c1(1);
-        gc[1] = -s1(1);
-        gc[2] = R(L) * c1(0);
-        gs[0] = gs[1] = gs[2] = R(0);
-    } else {
-        const R a = R((L + m) * (L + m - 1));
-        gc[0] = R(0.5) * (a * c1(m - 1) - c1(m + 1));
-        gc[1] = R(-0.5) * (a * s1(m - 1) + s1(m + 1));
-        gc[2] = R(L + m) * c1(m);
-        gs[0] = R(0.5) * (a * s1(m - 1) - s1(m + 1));
-        gs[1] = R(0.5) * (a * c1(m - 1) + c1(m + 1));
-        gs[2] = R(L + m) * s1(m);
-    }
-}
-
-// v += grad sum_m (ac[m] C_L^m + as[m] S_L^m) (as[0] unused), from the level
-// L-1 values.  The ladder relations above, regrouped by the level L-1
-// harmonic they multiply: each direction becomes one dot product with lowered
-// coefficients, 2L-1 terms instead of 2L+1 gradient triples.
-template <typename R, int L>
-__device__ __forceinline__ void grad_contract(const R* C1, const R* S1, const R* ac, const R* as,
-                                              R& vx, R& vy, R& vz) {
-    if constexpr (L >= 1) {
-#pragma unroll
-        for (int k = 0; k <= L - 1; ++k) {
-            // coefficients of C_{L-1}^k
-            R xc = R(0), yc = R(0);
-            if (k + 1 <= L) {
-                const R h = R(0.5 * (L + k + 1) * (L + k));
-                xc = h * ac[k + 1];
-                yc = (k + 1 >= 1) ? h * as[k + 1] : R(0);
-            }
-            if (k >= 2) {
-                xc = fma(R(-0.5), ac[k - 1], xc);
-                yc = fma(R(0.5), as[k - 1], yc);
-            }
-            if (k == 1) xc -= ac[0];
-            vx = fma(xc, C1[k], vx);
-            vy = fma(yc, C1[k], vy);
-            vz = fma(R(L + k) * ac[k], C1[k], vz);
-            if (k >= 1) {
-                // coefficients of S_{L-1}^k
-                R xs = R(0), ys = R(0);
-                if (k + 1 <= L) {
-                    const R h = R(0.5 * (L + k + 1) * (L + k));
-                    xs = h * as[k + 1];
-                    ys = -h * ac[k + 1];
-                }
-                if (k >= 2) {
-                    xs = fma(R(-0.5), as[k - 1], xs);
-                    ys = fma(R(-0.5), ac[k - 1], ys);
-                }
-                if (k == 1) ys -= ac[0];
-                vx = fma(xs, S1[k], vx);
-                vy = fma(ys, S1[k], vy);
-                vz = fma(R(L + k) * as[k], S1[k], vz);
-            }
         }
     }
 }
