@@ -147,8 +147,9 @@ typedef struct { int64_t n; int n_max; int l_max; } etics_batch_item;
  * precision: 8..512, rounded up to a multiple of 64 (default 512); FP64:
  * multiple of 4, 8..128 (default 32; tiles > 64 exceed one block's shared
  * memory and are rejected with ETICS_ERR_UNSUPPORTED) -- coefficient blocks
- * per SM (1..8), field threads per block (multiple of 32, <= 256; at most 128
- * used), particles per field work item (>= 1). */
+ * per SM (1..8; FP64, mixed precision runs two), field threads per block
+ * (multiple of 32, <= 256; at most 128 used), particles per field work item
+ * (>= 1). */
 typedef struct { int tile; int blocks_per_sm; int field_threads; int field_chunk; } etics_batch_tuning;
 
 /* Builds the batch plan in HOST memory.  With plan == NULL only the sizes are

@@ -10,20 +10,21 @@ namespace etics {
 constexpr int kBatchNR = 15;    // n_max <= 14
 constexpr int kBatchLM = 8;     // l_max <= 8
 
-// Mixed-precision coefficient pass (batch_pairs_kernel).  A block of
-// kBpThreads lanes handles one tile of up to kBpMaxTile particles of one
-// instance at a time.  The instance's expansion is cut into bins -- each
-// level's 2l+1 columns split evenly into ceil((2l+1)/kBpCap) bins -- and the
-// lanes are shared out evenly among the bins: lane j owns bin b(j) and takes
-// the particle pairs p = rank, rank + nlanes, ... of the tile.  The layout
-// depends only on l_max and is built on the host (batch_layout).  Blocks take
-// chunks of at most kBpChunkTiles tiles of one instance at a time.
+// Mixed-precision coefficient pass (batch_pairs_kernel).  An instance's
+// expansion is cut into bins -- each level's 2l+1 columns split evenly into
+// ceil((2l+1)/kBpCap) bins -- and the lanes of a block are shared out evenly
+// among the bins: lane j owns bin b(j) and takes the particle pairs p = rank,
+// rank + nlanes, ... of a step.  The bins depend only on l_max and are built on
+// the host (batch_layout).  Blocks take chunks of at most kBpChunkTiles tiles of
+// one instance at a time.  The plan also holds the shares of a block of
+// kBpThreads lanes, part of its format; the kernel, whose blocks are smaller,
+// derives its own from the bins.
 constexpr int kBpThreads = 512;
 constexpr int kBpMaxTile = 512;
 constexpr int kBpCap = 3;
 constexpr int kBpCols = (kBatchLM + 1) * (kBatchLM + 1);
 constexpr int kBpMaxBins = 30;        // sum over l <= 8 of ceil((2l+1)/3)
-constexpr int kBpChunkTiles = 16;     // tiles per claimed chunk (one FP32 accumulation window)
+constexpr int kBpChunkTiles = 16;     // tiles per claimed chunk, at most
 constexpr int kBpNbStride = 17;       // shared recursion constants per level (bank padding)
 constexpr size_t kBpNbBytes = ((size_t)(kBatchLM + 1) * kBpNbStride * sizeof(float) + 15) / 16 * 16;
 constexpr int64_t kBpRedFloats = (int64_t)kBatchNR * kBpCap * kBpThreads;
