@@ -484,7 +484,10 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
     const BatchHeader hd = *plan_table<BatchHeader>(plan, 0);
     const BatchInst* insts = plan_table<BatchInst>(plan, hd.off_inst);
     const int64_t out = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (out >= hd.coef_total) return;
+    if (out >= hd.coef_total) {
+        pdl_wait();
+        return;
+    }
     int lo = 0, hi = hd.ninst - 1;          // instance holding this output
     while (lo < hi) {
         const int mid = (lo + hi + 1) / 2;
@@ -503,9 +506,10 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
                         ? n * kBpCols + l * l + col
                         : ((col_offset(l) / 4 + col / 4) * kBatchNR + n) * 4 + (col & 3);
     const double* src = partial + (size_t)in.first_seg * hd.seg_stride + idx;
+    pdl_wait();   // the segments come from the coefficient kernel
     double s = 0.0;
 #pragma unroll 8
-    for (int k = 0; k < in.nseg; ++k) s += src[(size_t)k * hd.seg_stride];
+    for (int k = 0; k < in.nseg; ++k) s += __ldcg(src + (size_t)k * hd.seg_stride);
     const int am = m < 0 ? -m : m;
     coeffs[out] = s * c_tab.knorm_fact[l * (l + 1) / 2 + am] * c_tab.inv_j[n][l] * geg_gamma(0, l, n);
 }
@@ -538,6 +542,7 @@ batch_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm,
     const int share = (it.count + parts - 1) / parts, skip = (int)(blockIdx.x % parts) * share;
     it.begin += skip;
     it.count = it.count - skip < share ? it.count - skip : share;
+    pdl_wait();   // the coefficients come from the finalize
     if (it.count <= 0) return;
     field_table(cs, col_offset_c(kBatchLM + 1), coeffs + in.coef_offset, ETICS_BASIS_HO, in.n_max,
                 in.l_max);
@@ -816,9 +821,9 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
     }
     stage_event(ctx, 1);
     if (hd.coef_total > 0) {
-        batch_finalize_kernel<<<(unsigned)((hd.coef_total + 127) / 128), 128, 0, ctx.stream>>>(
-            plan_dev, static_cast<const double*>(ws), coeffs);
-        if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        if (launch_pdl(batch_finalize_kernel, dim3((unsigned)((hd.coef_total + 127) / 128)), dim3(128), 0,
+                       ctx.stream, plan_dev, static_cast<const double*>(ws), coeffs))
+            return ETICS_ERR_CUDA;
         ++*ctx.launches;
     }
     stage_event(ctx, 2);
@@ -830,24 +835,13 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
         while (parts < 4 && (int64_t)hd.nfield * parts < (int64_t)kFieldWaves * 3 * ctx.num_sms) parts *= 2;
         const int grid = hd.nfield * parts;
         const int threads = std::min(hd.field_threads, kBatchFieldThreads);
-        if (out_mask & ETICS_OUT_ACC) {
-            auto k = batch_field_kernel<FieldP, true>;
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-                return ETICS_ERR_CUDA;
-            k<<<grid, threads, smem, ctx.stream>>>(
-                reinterpret_cast<const Vec4<R>*>(posm), plan_dev, parts, coeffs,
-                reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err);
-        } else {
-            auto k = batch_field_kernel<FieldP, false>;
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-                return ETICS_ERR_CUDA;
-            k<<<grid, threads, smem, ctx.stream>>>(
-                reinterpret_cast<const Vec4<R>*>(posm), plan_dev, parts, coeffs,
-                reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err);
-        }
-        if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        auto k = out_mask & ETICS_OUT_ACC ? batch_field_kernel<FieldP, true>
+                                          : batch_field_kernel<FieldP, false>;
+        static_assert((size_t)kBatchNR * col_offset_c(kBatchLM + 1) * sizeof(R) <= 48 * 1024, "table");
+        if (launch_pdl(k, dim3(grid), dim3(threads), smem, ctx.stream,
+                       reinterpret_cast<const Vec4<R>*>(posm), plan_dev, parts, (const double*)coeffs,
+                       reinterpret_cast<Vec4<R>*>(out), out_mask, ctx.err))
+            return ETICS_ERR_CUDA;
         ++*ctx.launches;
     }
     stage_event(ctx, 3);
