@@ -84,7 +84,7 @@ def kernel_traffic():
 
 def mex_bytes(fp64=False):
     # partition 16R+8W, bucket sort 8R+16R+4W+16W, pass1 16R, pass2
-    # 16R+4R+16W  (per particle, FP32 particles; up to 2^21 of them)
+    # 16R+4R+16W  (per particle, FP32 particles; up to 1867776 of them)
     b = (16 + 8) + (8 + 16 + 4 + 16) + 16 + (16 + 4 + 16)
     return b + (3 * 16 if fp64 else 0)
 

@@ -9,7 +9,7 @@
 // into buckets of about 1024 (by a table of the keys' cumulative distribution,
 // from a sample), then one block per bucket sorts it in shared memory by the
 // 64-bit pattern of r^2 and writes the order and the particles themselves.  Up
-// to 8192 particles the last kernel alone does it.  Two dependent launches
+// to kSingleMax particles the last kernel alone does it.  Two dependent launches
 // instead of the radix path's six, and three passes over the particles instead
 // of ten over keys.
 //
@@ -688,12 +688,17 @@ constexpr int kSmallThreads = 256, kLargeThreads = 512;
 constexpr int kSmallMean = 1024, kLargeMean = 2048;
 static_assert(3 * kSmallMean == kSmallThreads * kBucketKpt && 3 * kLargeMean == kLargeThreads * kBucketKpt,
               "a bucket's capacity is three times its mean");
-constexpr int kSingleMax = 8192, kSingleKpt = kSingleMax / kLargeThreads;   // one block, no partition
+// One block, no partition, up to kSingleMax: MEX (l_max 4) takes 31.9 us at 6000
+// particles and 36.8 at 8192 so, 35.0 and 33.9 with a partition.
+constexpr int kSingleMax = 7168, kSingleKpt = kSingleMax / kLargeThreads;
 
 // How many buckets, of which mean, and how many particles per thread of the
-// partition: enough tiles for the SMs at each size (2^20: 128 tiles of 8192).
-// Above kSampleMaxN: the radix path.
-constexpr int64_t kSampleMaxN = int64_t(kMaxBuckets) * kLargeMean;
+// partition.  Above kSampleMaxN: the radix path.  The line lies where the large
+// buckets, two blocks per SM, start a fourth round on 152 SMs: MEX (l_max 4)
+// takes 195 us at 1.8 million particles and 256 at 2.0 million with buckets, 228
+// and 244 with the radix passes (2^20: 118 and 138).
+constexpr int64_t kSampleMaxN = int64_t(912) * kLargeMean;
+static_assert(kSampleMaxN <= int64_t(kMaxBuckets) * kLargeMean, "buckets");
 struct SamplePlan { int nbuckets, mean, kpt, ntiles; };
 SamplePlan sample_plan(int64_t N) {
     SamplePlan p{};

@@ -44,14 +44,14 @@ def order_of(pm):
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_radial_order_across_the_sort_paths(precision):
     """The order is exact on both sides of every line the sort draws by size:
-    one block up to 8192, one to eight particles per thread (154624 each) in
+    one block up to 7168, one to eight particles per thread (154624 each) in
     the partition, buckets of mean 1024 up to 2^20 and of mean 2048 up
-    to 2^21, the radix passes above; particles already in radial order, in two
+    to 1867776, the radix passes above; particles already in radial order, in two
     interleaved populations, and with one radius crowding (more equal keys
     than a bucket or a bin holds)."""
     rng = np.random.default_rng(3)
-    for n in (1023, 8191, 8192, 8193, 9217, 154625, (1 << 18) + 1, 400001, 800001, (1 << 20) + 1,
-              (1 << 21) + 1):
+    for n in (1023, 7167, 7168, 7169, 8193, 9217, 154625, (1 << 18) + 1, 400001, 800001, (1 << 20) + 1,
+              1867776, 1867777):
         pm = hernquist(n, seed=5)
         if n == 8193:
             pm = pm[order_of(pm)]                      # sorted already
