@@ -479,8 +479,8 @@ batch_pairs_kernel(const float4* __restrict__ posm, const void* __restrict__ pla
 // output spends most of them on its butterfly (256-system ensemble: 70 us).
 // ---------------------------------------------------------------------------
 __global__ void batch_finalize_kernel(const void* __restrict__ plan,
-                                      const double* __restrict__ partial,
-                                      double* __restrict__ coeffs) {
+                                      const double* partial,
+                                      double* coeffs) {
     const BatchHeader hd = *plan_table<BatchHeader>(plan, 0);
     const BatchInst* insts = plan_table<BatchInst>(plan, hd.off_inst);
     const int64_t out = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -509,7 +509,7 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
     pdl_wait();   // the segments come from the coefficient kernel
     double s = 0.0;
 #pragma unroll 8
-    for (int k = 0; k < in.nseg; ++k) s += __ldcg(src + (size_t)k * hd.seg_stride);
+    for (int k = 0; k < in.nseg; ++k) s += ld_cg(src + (size_t)k * hd.seg_stride);
     const int am = m < 0 ? -m : m;
     coeffs[out] = s * c_tab.knorm_fact[l * (l + 1) / 2 + am] * c_tab.inv_j[n][l] * geg_gamma(0, l, n);
 }
@@ -525,9 +525,9 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
 constexpr int kBatchFieldThreads = 128, kFieldWaves = 12;
 template <typename P, bool ACC>
 __global__ void __launch_bounds__(kBatchFieldThreads, 3)
-batch_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm,
+batch_field_kernel(const Vec4<typename FieldLane<P>::R>* posm,
                    const void* __restrict__ plan, int parts, const double* coeffs,
-                   Vec4<typename FieldLane<P>::R>* __restrict__ out, int out_mask, unsigned* err) {
+                   Vec4<typename FieldLane<P>::R>* out, int out_mask, unsigned* err) {
     using R = typename FieldLane<P>::R;
     constexpr int NP = FieldLane<P>::kParticles;
     extern __shared__ __align__(16) unsigned char smem_raw[];

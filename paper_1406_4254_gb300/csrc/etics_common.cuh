@@ -305,7 +305,38 @@ __host__ __device__ __forceinline__ int col_total(int lmax) { return col_offset(
 // explicitly: the implicit trigger at block exit keeps waiting blocks from
 // holding SM slots that a concurrent stream could use.  pdl_wait() is a
 // no-op in a kernel launched the ordinary way.
-__device__ __forceinline__ void pdl_wait() { cudaGridDependencySynchronize(); }
+//
+// Such a kernel takes no __restrict__ pointers: they would promise that nothing
+// else touches the data while it runs, and let the compiler move loads to the
+// read-only path and above the wait (the radix sort once read a histogram that
+// way before it was complete).  Through plain pointers the wait is a barrier
+// for every load and store.  Loads past the L1 cache are ld_cg's: volatile, so
+// that they keep their place as well.
+__device__ __forceinline__ void pdl_wait() {
+    cudaGridDependencySynchronize();
+    asm volatile("" ::: "memory");
+}
+__device__ __forceinline__ uint32_t ld_cg(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_cg(const double* p) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_cg(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_cg(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,

@@ -335,8 +335,8 @@ constexpr int mex_pass2_blocks() { return sizeof(R) == 4 ? (NG == 1 ? 4 : 3) : 2
 // ---------------------------------------------------------------------------
 template <typename R, int NG>
 __global__ void __launch_bounds__(kMexThreads, mex_pass1_blocks<R>())
-mex_pass1_kernel(const Vec4<R>* __restrict__ sorted, int64_t N, int l_max,
-                 double* __restrict__ tile_agg, int stride, unsigned* err) {
+mex_pass1_kernel(const Vec4<R>* sorted, int64_t N, int l_max,
+                 double* tile_agg, int stride, unsigned* err) {
     extern __shared__ __align__(16) unsigned char mex_smem[];
     R* rows = reinterpret_cast<R*>(mex_smem);
     __shared__ R s_end[2];
@@ -401,8 +401,8 @@ constexpr int kCarryThreads = 256;
 constexpr int kCarryWarps = kCarryThreads / 32;
 constexpr int kCarryRun = 16;
 static __global__ void __launch_bounds__(kCarryThreads)
-mex_carry_kernel(const double* __restrict__ tile_agg, int ntiles, int stride, int ncomp,
-                 double* __restrict__ carry) {
+mex_carry_kernel(const double* tile_agg, int ntiles, int stride, int ncomp,
+                 double* carry) {
     __shared__ double s_w[kCarryWarps + 1];
     pdl_wait();   // the tile sums come from pass 1
     const int c = blockIdx.x;
@@ -421,7 +421,7 @@ mex_carry_kernel(const double* __restrict__ tile_agg, int ntiles, int stride, in
 #pragma unroll
         for (int k = 0; k < kCarryRun; ++k) {
             const int o = o0 + k;
-            v[k] = k < run && o < ntiles ? __ldcg(src + (rev ? ntiles - 1 - o : o)) : 0.0;
+            v[k] = k < run && o < ntiles ? ld_cg(src + (rev ? ntiles - 1 - o : o)) : 0.0;
         }
         double local = v[0];
 #pragma unroll
@@ -530,9 +530,9 @@ constexpr int kMexLeftover = 8;
 
 template <typename R, int NG, bool ACC>
 __global__ void __launch_bounds__(kMexThreads, mex_pass2_blocks<R, NG>())
-mex_pass2_kernel(const Vec4<R>* __restrict__ sorted, const uint32_t* __restrict__ perm, int64_t N,
-                 int l_max, const double* __restrict__ carry, int stride,
-                 Vec4<R>* __restrict__ out, int out_mask, unsigned* err) {
+mex_pass2_kernel(const Vec4<R>* sorted, const uint32_t* perm, int64_t N,
+                 int l_max, const double* carry, int stride,
+                 Vec4<R>* out, int out_mask, unsigned* err) {
     extern __shared__ __align__(16) unsigned char mex_smem[];
     R* rows = reinterpret_cast<R*>(mex_smem);
     __shared__ R s_end[2];

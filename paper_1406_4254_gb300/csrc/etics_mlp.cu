@@ -236,11 +236,11 @@ __device__ __forceinline__ float bf(bf16 v) { return __bfloat162float(v); }
 // same bits).  With a target: dy = scale (y - t) in bf16 and per block the sums
 // of (y - t)^2 and of dy (FP32 pairs); else y itself.
 __global__ void __launch_bounds__(256)
-mlp_narrow_out_kernel(const bf16* __restrict__ a, const bf16* __restrict__ W,
-                      const float* __restrict__ bias, const float* __restrict__ target, int B,
-                      int din, int dout, int kslice, float scale, float* __restrict__ y,
-                      bf16* __restrict__ dyb, double* __restrict__ loss_part,
-                      double* __restrict__ db_part) {
+mlp_narrow_out_kernel(const bf16* a, const bf16* W,
+                      const float* bias, const float* target, int B,
+                      int din, int dout, int kslice, float scale, float* y,
+                      bf16* dyb, double* loss_part,
+                      double* db_part) {
     __shared__ __align__(16) bf16 s_w[kThin][kThinInputs + kPadK];   // [output][input]
     __shared__ double s_loss[8], s_db[8][kThin];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
@@ -325,8 +325,7 @@ mlp_narrow_out_kernel(const bf16* __restrict__ a, const bf16* __restrict__ W,
 // bound by the latency of the activations), added in group order at the end.
 constexpr int kThinRows = 128;   // rows of dy (or x) staged at a time
 
-__device__ __forceinline__ void load4(const bf16* p, float (&v)[4]) {
-    const uint2 raw = *reinterpret_cast<const uint2*>(p);
+__device__ __forceinline__ void unpack4(uint2 raw, float (&v)[4]) {
     const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.x));
     const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.y));
     v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
@@ -338,10 +337,10 @@ __device__ __forceinline__ void load4(const bf16* p, float (&v)[4]) {
 // the rows for all three.  din a multiple of 4.
 template <int DO>
 __global__ void __launch_bounds__(256)
-mlp_narrow_back_kernel(const bf16* __restrict__ a, const float* __restrict__ h,
-                       const bf16* __restrict__ W, const bf16* __restrict__ dyb, int B, int din,
-                       int rows, bf16* __restrict__ dzb, float* __restrict__ dw_part,
-                       double* __restrict__ db_part) {
+mlp_narrow_back_kernel(const bf16* a, const float* h,
+                       const bf16* W, const bf16* dyb, int B, int din,
+                       int rows, bf16* dzb, float* dw_part,
+                       double* db_part) {
     __shared__ float s_dy[kThinRows][DO];
     __shared__ float s_acc[3][64][4][DO];
     __shared__ double s_db[3][64][4];
@@ -367,34 +366,44 @@ mlp_narrow_back_kernel(const bf16* __restrict__ a, const float* __restrict__ h,
             (&s_dy[0][0])[i] = bf(dyb[(size_t)c0 * DO + i]);
         __syncthreads();
         if (!on) continue;
-#pragma unroll 4
-        for (int r = rg; r < n; r += 4) {
-            const size_t at = (size_t)(c0 + r) * din + m;
-            float av[4], hv[4];
-            load4(a + at, av);
-            if (h) {
-                const float4 t = *reinterpret_cast<const float4*>(h + at);
-                hv[0] = t.x; hv[1] = t.y; hv[2] = t.z; hv[3] = t.w;
+        // the loads of four rows are issued before the first row's store
+        for (int rb = rg; rb < n; rb += 16) {
+            uint2 ar[4];
+            float4 hr[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const size_t at = (size_t)(c0 + rb + 4 * u) * din + m;
+                if (rb + 4 * u < n) {
+                    ar[u] = *reinterpret_cast<const uint2*>(a + at);
+                    if (h) hr[u] = *reinterpret_cast<const float4*>(h + at);
+                }
             }
-            float z[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                z[j] = 0.0f;
+            for (int u = 0; u < 4; ++u) {
+                const int r = rb + 4 * u;
+                if (r >= n) break;
+                float av[4], hv[4] = {hr[u].x, hr[u].y, hr[u].z, hr[u].w}, z[4];
+                unpack4(ar[u], av);
 #pragma unroll
-                for (int o = 0; o < DO; ++o) {
-                    const float g = s_dy[r][o];
-                    acc[j][o] = fmaf(av[j], g, acc[j][o]);
-                    z[j] = fmaf(g, w[j][o], z[j]);
+                for (int j = 0; j < 4; ++j) {
+                    z[j] = 0.0f;
+#pragma unroll
+                    for (int o = 0; o < DO; ++o) {
+                        const float g = s_dy[r][o];
+                        acc[j][o] = fmaf(av[j], g, acc[j][o]);
+                        z[j] = fmaf(g, w[j][o], z[j]);
+                    }
+                    if (h) {
+                        z[j] *= 1.0f - hv[j] * hv[j];
+                        tc::add_exact(cs[j], ce[j], z[j]);
+                    }
                 }
                 if (h) {
-                    z[j] *= 1.0f - hv[j] * hv[j];
-                    tc::add_exact(cs[j], ce[j], z[j]);
+                    __nv_bfloat162 b2[2] = {__floats2bfloat162_rn(z[0], z[1]),
+                                            __floats2bfloat162_rn(z[2], z[3])};
+                    *reinterpret_cast<uint2*>(dzb + (size_t)(c0 + r) * din + m) =
+                        *reinterpret_cast<uint2*>(b2);
                 }
-            }
-            if (h) {
-                __nv_bfloat162 b2[2] = {__floats2bfloat162_rn(z[0], z[1]),
-                                        __floats2bfloat162_rn(z[2], z[3])};
-                *reinterpret_cast<uint2*>(dzb + at) = *reinterpret_cast<uint2*>(b2);
             }
         }
     }
@@ -424,8 +433,8 @@ mlp_narrow_back_kernel(const bf16* __restrict__ a, const float* __restrict__ h,
 // inputs; dout a multiple of 4
 template <int DI>
 __global__ void __launch_bounds__(256)
-mlp_narrow_in_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dzb, int B, int dout,
-                     int rows, float* __restrict__ dw_part) {
+mlp_narrow_in_kernel(const bf16* x, const bf16* dzb, int B, int dout,
+                     int rows, float* dw_part) {
     __shared__ float s_x[kThinRows][DI];
     __shared__ float s_acc[3][64][4][DI];
     const int cg = threadIdx.x & 63, rg = threadIdx.x >> 6;
@@ -448,7 +457,7 @@ mlp_narrow_in_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dzb, i
 #pragma unroll 8
         for (int r = rg; r < cnt; r += 4) {
             float g[4];
-            load4(dzb + (size_t)(c0 + r) * dout + n, g);
+            unpack4(*reinterpret_cast<const uint2*>(dzb + (size_t)(c0 + r) * dout + n), g);
 #pragma unroll
             for (int i = 0; i < DI; ++i) {
                 const float xv = s_x[r][i];
@@ -549,10 +558,10 @@ __global__ void __launch_bounds__(256) mlp_reduce_kernel(const __grid_constant__
     }
 }
 
-__global__ void mlp_adam_kernel(float* __restrict__ p, const float* __restrict__ g,
-                                float* __restrict__ m, float* __restrict__ v, int64_t n, float lr,
+__global__ void mlp_adam_kernel(float* p, const float* g,
+                                float* m, float* v, int64_t n, float lr,
                                 float b1, float b2, float eps, float bc1, float bc2,
-                                bf16* __restrict__ pb) {
+                                bf16* pb) {
     pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {

@@ -356,7 +356,7 @@ constexpr int kFinThreads = 128;
 template <int NR>
 __global__ void __launch_bounds__(kFinThreads)
 scf_finalize_plan_kernel(const __grid_constant__ ScfCoeffPairParams p, int n_max,
-                          double* __restrict__ coeffs) {
+                          double* coeffs) {
     constexpr int CAP = PairShape<NR>::kCap;
     const int nj = (p.plan.l_max + 1) * (p.plan.l_max + 1);
     pdl_wait();   // the partials come from the coefficient kernel
@@ -379,7 +379,7 @@ scf_finalize_plan_kernel(const __grid_constant__ ScfCoeffPairParams p, int n_max
     const double* src = p.partial + (size_t)gr.block0 * stride + idx;
     double s = 0.0;
 #pragma unroll 4
-    for (int k = lane; k < gr.nblocks; k += 32) s += __ldcg(src + (size_t)k * stride);
+    for (int k = lane; k < gr.nblocks; k += 32) s += ld_cg(src + (size_t)k * stride);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {

@@ -75,7 +75,7 @@ __device__ __forceinline__ void field_table(R* cs, int stride, const double* coe
         for (int n = threadIdx.x >> 5; n < field_rows(n_max); n += blockDim.x >> 5)
             cs[n * stride + c] =
                 n > n_max ? R(0)   // at least two rows
-                : k < 2 * l + 1 ? (R)(__ldcg(coeffs + (size_t)n * nj + l * l + l + m) *
+                : k < 2 * l + 1 ? (R)(ld_cg(coeffs + (size_t)n * nj + l * l + l + m) *
                                     g_field_tab.v[basis][n][l * (l + 1) / 2 + am])
                 : k == ncol_pad(l) - 1 ? -geg_bs_of<R>(basis, l, n) : R(0);
     }
@@ -314,9 +314,9 @@ template <int LM> constexpr int field_threads() { return LM <= 6 ? 512 : LM <= 8
 // acceleration still in registers
 template <typename P, int LM, bool ACC, int NM1, int B>
 __global__ void __launch_bounds__(field_threads<LM>(), 1)
-scf_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm, int64_t N, int n_max,
-                 int l_max, const double* coeffs, Vec4<typename FieldLane<P>::R>* __restrict__ out,
-                 int out_mask, Vec4<typename FieldLane<P>::R>* __restrict__ vel,
+scf_field_kernel(const Vec4<typename FieldLane<P>::R>* posm, int64_t N, int n_max,
+                 int l_max, const double* coeffs, Vec4<typename FieldLane<P>::R>* out,
+                 int out_mask, Vec4<typename FieldLane<P>::R>* vel,
                  typename FieldLane<P>::R kick, FieldSplit split, unsigned* err) {
     using R = typename FieldLane<P>::R;
     constexpr int NP = FieldLane<P>::kParticles;
@@ -359,6 +359,12 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm, int64_
             __syncthreads();
             if (part > 0) continue;
         }
+        Vec4<R> v[NP];
+        if (vel) {
+#pragma unroll
+            for (int j = 0; j < NP; ++j)
+                if (i + j < N) v[j] = ld4(vel + i + j);
+        }
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
             if (i + j >= N) continue;
@@ -366,11 +372,10 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* __restrict__ posm, int64_
             if (!finite4(res[j].x, res[j].y, res[j].z, res[j].w)) report(err, ETICS_ERR_NONFINITE);
             st4(out + i + j, res[j]);
             if (vel) {
-                Vec4<R> v = ld4(vel + i + j);
-                v.x = fma(kick, res[j].x, v.x);
-                v.y = fma(kick, res[j].y, v.y);
-                v.z = fma(kick, res[j].z, v.z);
-                st4(vel + i + j, v);
+                v[j].x = fma(kick, res[j].x, v[j].x);
+                v[j].y = fma(kick, res[j].y, v[j].y);
+                v[j].z = fma(kick, res[j].z, v[j].z);
+                st4(vel + i + j, v[j]);
             }
         }
     }

@@ -308,8 +308,8 @@ scf_coeff_pairs_kernel(ScfPairParams p) {
 constexpr int kFinThreads = 128;
 template <int NR, int LM, int CAP>
 __global__ void __launch_bounds__(kFinThreads)
-scf_finalize_pairs_kernel(const double* __restrict__ partial, int nblocks,
-                          double* __restrict__ coeffs) {
+scf_finalize_pairs_kernel(const double* partial, int nblocks,
+                          double* coeffs) {
     constexpr int NJ = (LM + 1) * (LM + 1);
     constexpr int NOUT = PairConst<LM, CAP>::nbins * NR * CAP;
     pdl_wait();   // the partials come from the coefficient kernel
@@ -325,7 +325,7 @@ scf_finalize_pairs_kernel(const double* __restrict__ partial, int nblocks,
                     c_pair_plan<LM, CAP>.slot_of[col];
     double s = 0.0;
 #pragma unroll 4
-    for (int k = lane; k < nblocks; k += 32) s += __ldcg(partial + (size_t)k * NOUT + idx);
+    for (int k = lane; k < nblocks; k += 32) s += ld_cg(partial + (size_t)k * NOUT + idx);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {

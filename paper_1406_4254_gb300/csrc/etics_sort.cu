@@ -288,10 +288,10 @@ __device__ __forceinline__ uint32_t lookback(const uint32_t* st, size_t stride, 
 // Launched with programmatic stream serialisation: nothing global is touched
 // before griddepcontrol.wait.
 __global__ void __launch_bounds__(kSortThreads, 2)
-onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
-                uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
+onesweep_kernel(const uint32_t* keys_in, const uint32_t* vals_in,
+                uint32_t* keys_out, uint32_t* vals_out,
                 const uint32_t* hist, uint32_t* status, uint32_t* counter, int shift,
-                int64_t N, int64_t spin_limit, uint32_t* __restrict__ next_hist, unsigned* err) {
+                int64_t N, int64_t spin_limit, uint32_t* next_hist, unsigned* err) {
     __shared__ uint32_t s_keys[kSortTile];
     __shared__ uint32_t s_vals[kSortTile];
     __shared__ uint32_t s_whist[kSortThreads / 32][256];
@@ -309,7 +309,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     // the histogram may have been completed by the kernel just before this
     // one (a programmatic dependent launch): a coherent load after the wait,
     // never the non-coherent read-only path
-    const uint32_t gcount = __ldcg(hist + dig);
+    const uint32_t gcount = ld_cg(hist + dig);
     // digits present in this pass over all keys: few -> rank with match_any
     const int ndig = __syncthreads_count(gcount != 0u);
     const uint32_t tile = s_tile;
@@ -541,8 +541,8 @@ __device__ void sort_run_block(const Vec4<R>* posm, int64_t N, uint32_t* val, ui
 // other run starts inside it, so no other block touches its positions.
 template <typename R>
 __global__ void __launch_bounds__(kFixThreads)
-tie_fixup_kernel(const uint32_t* __restrict__ key, const Vec4<R>* __restrict__ posm,
-                 uint32_t* __restrict__ val, uint32_t* __restrict__ tmp, int64_t N,
+tie_fixup_kernel(const uint32_t* key, const Vec4<R>* posm,
+                 uint32_t* val, uint32_t* tmp, int64_t N,
                  unsigned* err) {
     __shared__ uint32_t s_key[kFixTile + 2];
     __shared__ int s_runs[kFixTile / 2];
@@ -652,11 +652,11 @@ __device__ __forceinline__ Vec4<R> gather_particle(const Vec4<R>* posm, uint32_t
 
 template <typename R>
 __global__ void __launch_bounds__(256)
-gather_kernel(const Vec4<R>* __restrict__ posm, const uint32_t* perm, int64_t N,
-              Vec4<R>* __restrict__ sorted, unsigned* err) {
+gather_kernel(const Vec4<R>* posm, const uint32_t* perm, int64_t N,
+              Vec4<R>* sorted, unsigned* err) {
     pdl_wait();   // the order comes from the kernel before
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) st4(sorted + i, gather_particle<R>(posm, __ldcg(perm + i), N, err));
+    if (i < N) st4(sorted + i, gather_particle<R>(posm, ld_cg(perm + i), N, err));
 }
 
 // ---------------------------------------------------------------------------
@@ -1027,8 +1027,8 @@ __device__ __forceinline__ void make_cdf(const Vec4<R>* posm, int64_t N, int nbu
 constexpr int kPartHeader = 64;
 template <typename R, int KPT>
 __global__ void __launch_bounds__(kPartThreads, 1)
-partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int cap,
-                 uint64_t stride, KeyCdf* cdf, uint32_t* part, uint2* __restrict__ region,
+partition_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, int cap,
+                 uint64_t stride, KeyCdf* cdf, uint32_t* part, uint2* region,
                  int64_t spin_limit, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
     __shared__ uint32_t s_hist[kMaxBuckets];
@@ -1078,10 +1078,10 @@ partition_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, int 
     KeyCdf& t = *reinterpret_cast<KeyCdf*>(sort_smem);
     if (ok) {
         // without the rows of divided bins that are not there
-        const uint32_t nfine = __ldcg(&cdf->nfine);
+        const uint32_t nfine = ld_cg(&cdf->nfine);
         const int pieces = (int)((offsetof(KeyCdf, row) + nfine * sizeof(t.row[0])) / 16);
         for (int i = tid; i < pieces; i += kPartThreads)
-            reinterpret_cast<uint4*>(&t)[i] = __ldcg(reinterpret_cast<const uint4*>(cdf) + i);
+            reinterpret_cast<uint4*>(&t)[i] = ld_cg(reinterpret_cast<const uint4*>(cdf) + i);
     }
     __syncthreads();
     uint32_t at[KPT];   // bucket, then place within the tile's share (16 bits each)
@@ -1219,9 +1219,9 @@ __device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, 
 // block whatever its size, hidden only by other blocks.
 template <typename R, int TH, int KPT>
 __global__ void __launch_bounds__(TH)
-bucket_sort_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, const KeyCdf* cdf,
+bucket_sort_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, const KeyCdf* cdf,
                    const uint32_t* sizes, const uint2* region, uint32_t* perm, uint32_t* tmp,
-                   Vec4<R>* __restrict__ sorted, unsigned* err) {
+                   Vec4<R>* sorted, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
     using Sort = BlockSort<TH, KPT>;
     constexpr int CAP = Sort::CAP;
@@ -1237,13 +1237,13 @@ bucket_sort_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, co
         const uint2* mem = region + (size_t)b * CAP + tid;
 #pragma unroll
         for (int s = 0; s < kAhead; ++s) {
-            const uint2 m = __ldcg(mem + s * TH);
+            const uint2 m = ld_cg(mem + s * TH);
             k[s] = m.x;
             id[s] = m.y;
         }
         uint32_t before = 0;
-        for (int i = tid; i < b; i += TH) before += __ldcg(sizes + i);
-        len = __ldcg(sizes + b);
+        for (int i = tid; i < b; i += TH) before += ld_cg(sizes + i);
+        len = ld_cg(sizes + b);
         before = __reduce_add_sync(0xffffffffu, before);
         if (lane == 0) s_base[warp] = before;
         __syncthreads();
@@ -1262,7 +1262,7 @@ bucket_sort_kernel(const Vec4<R>* __restrict__ posm, int64_t N, int nbuckets, co
 #pragma unroll
         for (int s = kAhead; s < KPT; ++s)
             if (tid + s * TH < (int)len) {
-                const uint2 m = __ldcg(mem + s * TH);
+                const uint2 m = ld_cg(mem + s * TH);
                 k[s] = m.x;
                 id[s] = m.y;
             }

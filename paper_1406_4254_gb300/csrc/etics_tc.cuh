@@ -406,7 +406,7 @@ constexpr int kStageRow = kN + 4;   // floats; rows 16 bytes apart in the banks
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(kTmaThreads, 2)
 gemm_tma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                float* __restrict__ part, int M, int N, int K, int kslice, Epilogue ep,
+                float* part, int M, int N, int K, int kslice, Epilogue ep,
                 unsigned* err) {
     extern __shared__ unsigned char smem_raw[];
     SmemTma& sm = *reinterpret_cast<SmemTma*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
