@@ -821,9 +821,19 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
     }
     stage_event(ctx, 1);
     if (hd.coef_total > 0) {
-        if (launch_pdl(batch_finalize_kernel, dim3((unsigned)((hd.coef_total + 127) / 128)), dim3(128), 0,
-                       ctx.stream, plan_dev, static_cast<const double*>(ws), coeffs))
-            return ETICS_ERR_CUDA;
+        // The finalize reads the plan before its wait: the coefficient kernel,
+        // launched the ordinary way, began after whatever wrote it.  Without
+        // that kernel (no particles) the finalize has to do so itself.
+        const dim3 blocks((unsigned)((hd.coef_total + 127) / 128));
+        const double* partial = static_cast<const double*>(ws);
+        if (hd.ntiles > 0) {
+            if (launch_pdl(batch_finalize_kernel, blocks, dim3(128), 0, ctx.stream, plan_dev, partial,
+                           coeffs))
+                return ETICS_ERR_CUDA;
+        } else {
+            batch_finalize_kernel<<<blocks, 128, 0, ctx.stream>>>(plan_dev, partial, coeffs);
+            if (cudaGetLastError()) return ETICS_ERR_CUDA;
+        }
         ++*ctx.launches;
     }
     stage_event(ctx, 2);

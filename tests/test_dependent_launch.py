@@ -73,3 +73,34 @@ def test_dependent_kernels_make_no_promise_about_their_inputs(path):
 @pytest.mark.parametrize("path", FILES, ids=os.path.basename)
 def test_cached_loads_go_through_the_ordered_helper(path):
     assert not re.search(r"\b__ld(cg|g|ca|cs)\s*\(", _code(path))
+
+
+def test_a_plan_is_read_early_only_behind_the_coefficient_kernel():
+    """The batch's finalize reads the plan before its wait.  That is safe behind
+    the coefficient kernel, an ordinary launch that began after whatever wrote
+    the plan; a batch without particles has no such kernel and its finalize must
+    be an ordinary launch itself."""
+    code = _code(os.path.join(CSRC, "etics_batch.cu"))
+    body = next(b for n, _, b in kernels(code) if n == "batch_finalize_kernel")
+    assert body.index("plan_table") < body.index("pdl_wait()")
+    at = code.index("launch_pdl(batch_finalize_kernel")
+    guard = re.findall(r"if \(hd\.ntiles > 0\) \{\s*if \($", code[:at])
+    assert guard, "dependent launch of the finalize without a coefficient kernel before it"
+
+
+@pytest.mark.gpu
+def test_batch_without_particles_whose_plan_a_kernel_wrote():
+    import torch
+
+    from paper_1406_4254_gb300 import etics
+    plan = etics.BatchPlan([0, 0, 0], [10, 4, 14], [6, 0, 8])
+    filler = torch.ones(1 << 24, device="cuda")
+    host = plan.dev.clone()
+    for _ in range(20):
+        plan.dev.zero_()
+        coeffs = torch.full((plan.coeff_count,), 3.0, dtype=torch.float64, device="cuda")
+        filler.mul_(1.0)
+        torch.add(host, 0, out=plan.dev)   # a kernel, not a copy
+        etics.scf_batch(filler[:4].reshape(1, 4)[:0], plan, coeffs=coeffs, with_field=False)
+        assert etics.get_error() == 0
+        assert torch.all(coeffs == 0)
