@@ -1272,6 +1272,7 @@ bucket_sort_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, const KeyCdf* c
             const int i = tid + s * TH;
             if (i < (int)len) {
                 k[s] = sort_key<R>(ld4(posm + i));
+                if (k[s] == 0xffffffffu) report(err, ETICS_ERR_NONFINITE);
                 id[s] = (uint32_t)i;
             }
         }
