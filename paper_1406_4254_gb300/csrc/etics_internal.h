@@ -69,10 +69,11 @@ struct SortBuffers {
     uint32_t *hist, *status, *counters;
     void* zero_base;
     size_t zero_bytes;
-    // sample path: bucket contents, table of the keys' distribution, and
-    // ticket, flag and bucket sizes
+    // sample path: bucket contents, table of the keys' distribution, ticket,
+    // flag and bucket sizes, and what is beyond a bucket's room with its runs
     uint8_t *region, *cdf;
-    uint32_t* part;
+    uint32_t *part, *spill;
+    uint8_t* runs;
 };
 // carve the sort buffers from ws (ws may be null to only compute *total)
 SortBuffers sort_buffers(void* ws, int64_t N, size_t* total);

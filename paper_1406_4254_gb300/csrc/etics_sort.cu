@@ -198,12 +198,12 @@ __device__ __forceinline__ void st_volatile(uint32_t* p, uint32_t v) {
 // either with __match_any_sync (fast when a warp holds few distinct digits)
 // or with one ballot per digit bit plus one for validity (a cost independent
 // of how many distinct digits there are).
-template <bool kMatch>
-__device__ __forceinline__ void rank_in_warp(const uint32_t (&d)[kSortKpt], uint32_t (&rank)[kSortKpt],
+template <bool kMatch, int K>
+__device__ __forceinline__ void rank_in_warp(const uint32_t (&d)[K], uint32_t (&rank)[K],
                                              uint32_t* whist, int lane) {
     const unsigned below = (1u << lane) - 1u;
 #pragma unroll
-    for (int s = 0; s < kSortKpt; ++s) {
+    for (int s = 0; s < K; ++s) {
         unsigned mask;
         if (kMatch) {
             mask = __match_any_sync(0xffffffffu, d[s]);
@@ -699,6 +699,8 @@ constexpr int kSingleMax = 7168, kSingleKpt = kSingleMax / kLargeThreads;
 // and 244 with the radix passes (2^20: 118 and 138).
 constexpr int64_t kSampleMaxN = int64_t(912) * kLargeMean;
 static_assert(kSampleMaxN <= int64_t(kMaxBuckets) * kLargeMean, "buckets");
+constexpr int kMaxTiles = (int)((kSampleMaxN + 8 * kPartThreads - 1) / (8 * kPartThreads));
+static_assert(kMaxTiles >= kPartTiles, "tiles");
 struct SamplePlan { int nbuckets, mean, kpt, ntiles; };
 SamplePlan sample_plan(int64_t N) {
     SamplePlan p{};
@@ -1017,21 +1019,22 @@ __device__ __forceinline__ void make_cdf(const Vec4<R>* posm, int64_t N, int nbu
 // particles per bucket in shared memory, takes its places in the buckets with
 // one addition per bucket to the bucket sizes, and writes the particles' keys
 // and indices to region[b * cap + place].  The order inside a bucket's region is
-// whatever the additions give: the bucket sort orders by (r^2, index).  A place
-// beyond the capacity is not written (sort_bucket_global finds those particles
-// again).  A tile whose wait runs out (ETICS_ERR_TIMEOUT) counts its particles
-// in bucket 0: the sizes still add up to N, so that everything after stays
-// inside the buffers.
-// part (zero at launch): [0] ticket counter, [1] flag, from word kPartHeader
-// on the bucket sizes.
+// whatever the additions give: the bucket sort orders by (r^2, index).  A tile's
+// particles beyond a bucket's capacity go to a run of places of their own in
+// `spill`, runs[tile][bucket] = (first place, count), so that a crowded bucket is
+// collected in time proportional to its size.  A tile whose wait runs out
+// (ETICS_ERR_TIMEOUT) counts its particles in bucket 0: the sizes still add up
+// to N, so that everything after stays inside the buffers.
+// part (zero at launch): [0] ticket counter, [1] flag, [2] places of `spill`
+// taken, from word kPartHeader on the bucket sizes.
 constexpr int kPartHeader = 64;
 template <typename R, int KPT>
 __global__ void __launch_bounds__(kPartThreads, 1)
 partition_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, int cap,
-                 uint64_t stride, KeyCdf* cdf, uint32_t* part, uint2* region,
-                 int64_t spin_limit, unsigned* err) {
+                 uint64_t stride, KeyCdf* cdf, uint32_t* part, uint2* region, uint32_t* spill,
+                 uint2* runs, int64_t spin_limit, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
-    __shared__ uint32_t s_hist[kMaxBuckets];
+    __shared__ uint32_t s_hist[kMaxBuckets], s_spill[kMaxBuckets];
     __shared__ uint32_t s_ticket;
     __shared__ int s_ok;
     const int tid = threadIdx.x;
@@ -1094,8 +1097,16 @@ partition_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, int cap,
         }
     }
     __syncthreads();
-    if (tid < nbuckets && s_hist[tid])
-        s_hist[tid] = atomicAdd(part + kPartHeader + tid, s_hist[tid]);
+    if (tid < nbuckets) {
+        const uint32_t count = s_hist[tid], room = (uint32_t)cap;
+        const uint32_t first = count ? atomicAdd(part + kPartHeader + tid, count) : 0u;
+        const uint32_t from = first > room ? first : room;   // first place beyond the capacity
+        const uint32_t over = first + count > from ? first + count - from : 0u;
+        const uint32_t place = over ? atomicAdd(part + 2, over) : 0u;
+        s_hist[tid] = first;
+        s_spill[tid] = place - from;
+        runs[(size_t)(s_ticket - 1u) * nbuckets + tid] = make_uint2(place, over);
+    }
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < KPT; ++s) {
@@ -1103,99 +1114,117 @@ partition_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, int cap,
         if (i < N) {
             const uint32_t b = at[s] & 0xffffu, slot = s_hist[b] + (at[s] >> 16);
             if (slot < (uint32_t)cap) region[(size_t)b * cap + slot] = make_uint2(key[s], (uint32_t)i);
+            else spill[s_spill[b] + slot] = (uint32_t)i;
         }
     }
 }
 
 // A bucket larger than a block's shared memory (keys that crowd on one high
-// word, or, rarely, an unlucky sample): the block collects its members in
-// index order from all particles, then sorts them in place by the 64-bit
-// pattern with stable 8-bit passes (sort_run_block's, over both words),
-// passes whose digit is the same for all members left out.
+// word, or, rarely, an unlucky sample): the block collects its members, `mem`
+// holding the first `cap` and `spill` the rest in one run per tile (runs: this
+// bucket's of tile 0, `stride` further that of the next), and sorts them by
+// (64-bit pattern of r^2, index) with stable 8-bit passes between val and tmp,
+// kCrowdKpt members per thread at a time; passes over a digit that is the same
+// for all are left out.  The order of 2^20 particles on 300 thin shells takes
+// 430 us (5.5 ms when each such bucket's block read all particles again, 86
+// for a Hernquist sphere); 1.87 million on 1 / 100 / 300 / 1000 shells 31.7 ms
+// / 660 / 530 / 450 us, by the radix path 60.6 ms / 1260 / 870 / 490.
+constexpr int kCrowdKpt = 8;
 template <typename R, int TH>
-__device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, const KeyCdf* cdf,
-                                                int nbuckets, int bucket, uint32_t* val,
-                                                uint32_t* tmp, int64_t len, uint32_t* scratch) {
+__device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, const uint2* mem,
+                                                int cap, const uint32_t* spill, const uint2* runs,
+                                                int ntiles, int stride, uint32_t* val, uint32_t* tmp,
+                                                int64_t len, uint32_t* scratch) {
     constexpr int NW = TH / 32;
     uint32_t (*s_cnt)[256] = reinterpret_cast<uint32_t (*)[256]>(scratch);   // [NW][256]
-    uint32_t* s_off = scratch + NW * 256;                                    // [256]
-    uint32_t* s_wsum = s_off + 256;                                          // [NW]
+    __shared__ uint32_t s_wsum[NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int64_t found = 0;
-    for (int64_t c0 = 0; c0 < N; c0 += TH) {
-        bool mine = false;
-        if (c0 + tid < N)
-            mine = bucket_of(*cdf, sort_key<R>(ld4(posm + c0 + tid)), nbuckets) == bucket;
-        const unsigned bal = __ballot_sync(0xffffffffu, mine);
-        if (lane == 0) s_wsum[warp] = (uint32_t)__popc(bal);
-        __syncthreads();
-        uint32_t before = 0, total = 0;
-        for (int w = 0; w < NW; ++w) {
-            if (w < warp) before += s_wsum[w];
-            total += s_wsum[w];
-        }
-        const int64_t pos = found + before + __popc(bal & ((1u << lane) - 1u));
-        if (mine && pos < len) val[pos] = (uint32_t)(c0 + tid);
-        found += total;
-        __syncthreads();
-    }
-    auto digit = [&](uint32_t i, int shift) -> uint32_t {
-        const uint64_t b = (int64_t)i < N ? r2_bits(ld4(posm + i)) : ~uint64_t(0);
-        return (uint32_t)(b >> shift) & 255u;
-    };
-    uint32_t *src = val, *dst = tmp;
-    for (int pass = 0; pass < 8; ++pass) {
-        const int shift = 8 * pass;
-        for (int i = tid; i < NW * 256; i += TH) (&s_cnt[0][0])[i] = 0u;
-        __syncthreads();
-        for (int64_t i = tid; i < len; i += TH) atomicAdd(&s_cnt[0][digit(src[i], shift)], 1u);
-        __syncthreads();
-        const uint32_t c = tid < 256 ? s_cnt[0][tid] : 0u;
-        if (__syncthreads_or(tid < 256 && (int64_t)c == len)) continue;   // one digit only
-        uint32_t x = c;
+    // exclusive sum of x over the threads
+    auto scan = [&](uint32_t x) -> uint32_t {
+        uint32_t y = x;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += t;
-        }
-        if (lane == 31) s_wsum[warp] = x;
-        __syncthreads();
-        if (tid < 256) {
-            uint32_t b = 0;
-            for (int w = 0; w < warp; ++w) b += s_wsum[w];
-            s_off[tid] = b + x - c;
-            s_cnt[0][tid] = 0u;
+            const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += t;
         }
         __syncthreads();
-        for (int64_t c0 = 0; c0 < len; c0 += TH) {
-            const bool valid = c0 + tid < len;
-            const uint32_t v = valid ? src[c0 + tid] : 0u;
-            const uint32_t d = valid ? digit(v, shift) : 256u;
-            const unsigned vb = __ballot_sync(0xffffffffu, valid);
-            unsigned mask = valid ? vb : ~vb;
-#pragma unroll
-            for (int bit = 0; bit < 8; ++bit) {
-                const bool on = (d >> bit) & 1u;
-                const unsigned bal = __ballot_sync(0xffffffffu, on);
-                mask &= on ? bal : ~bal;
+        if (lane == 31) s_wsum[warp] = y;
+        __syncthreads();
+        return y - x + __reduce_add_sync(0xffffffffu, lane < warp ? s_wsum[lane] : 0u);
+    };
+    for (int i = tid; i < cap; i += TH) val[i] = ld_cg(mem + i).y;
+    // the runs, a warp each (their places in s_cnt, dead here)
+    uint32_t *s_at = scratch, *s_first = scratch + TH, *s_n = scratch + 2 * TH;
+    static_assert(3 * TH <= NW * 256, "room for the runs");
+    int64_t have = cap;
+    for (int t0 = 0; t0 < ntiles; t0 += TH) {
+        const uint2 r = t0 + tid < ntiles ? ld_cg(runs + (size_t)(t0 + tid) * stride) : make_uint2(0u, 0u);
+        const uint32_t first = scan(r.y);
+        s_at[tid] = r.x;
+        s_first[tid] = first;
+        s_n[tid] = r.y;
+        __syncthreads();
+        for (int q = warp; q < TH; q += NW)
+            for (uint32_t j = lane; j < s_n[q]; j += 32) {
+                const int64_t pos = have + s_first[q] + j;
+                if (pos < len) val[pos] = ld_cg(spill + s_at[q] + j);
             }
-            const unsigned lower = mask & ((1u << lane) - 1u);
-            if (valid && lower == 0u) s_cnt[warp][d] = (uint32_t)__popc(mask);
+        have += s_first[TH - 1] + s_n[TH - 1];
+    }
+    // the digits of (index, pattern) counted for all passes in one look
+    constexpr int kDigits = 12;   // 0..3 of the index, 4..11 of the pattern
+    uint32_t (*s_off)[256] = reinterpret_cast<uint32_t (*)[256]>(scratch + NW * 256);
+    auto bits = [&](uint32_t i) -> uint64_t {
+        return (int64_t)i < N ? r2_bits(ld4(posm + i)) : ~uint64_t(0);
+    };
+    for (int i = tid; i < kDigits * 256; i += TH) (&s_off[0][0])[i] = 0u;
+    __syncthreads();
+#pragma unroll 2
+    for (int64_t i = tid; i < len; i += TH) {
+        const uint32_t v = val[i];
+        const uint64_t w = bits(v);
+#pragma unroll
+        for (int p = 0; p < kDigits; ++p)
+            atomicAdd(&s_off[p][(p < 4 ? v >> 8 * p : (uint32_t)(w >> 8 * (p - 4 & 7))) & 255u], 1u);
+    }
+    __syncthreads();
+    uint32_t *src = val, *dst = tmp;
+    for (int pass = 0; pass < kDigits; ++pass) {
+        const uint32_t count = tid < 256 ? s_off[pass][tid] : 0u;
+        if (__syncthreads_or((int64_t)count == len)) continue;   // one digit only
+        const uint32_t start = scan(count);
+        if (tid < 256) s_off[pass][tid] = start;
+        for (int64_t c0 = 0; c0 < len; c0 += TH * kCrowdKpt) {
+            for (int i = tid; i < NW * 256; i += TH) (&s_cnt[0][0])[i] = 0u;
             __syncthreads();
-            uint32_t total = 0;   // thread = digit: exclusive prefix over the warps
-            if (tid < 256)
+            uint32_t v[kCrowdKpt], d[kCrowdKpt], rank[kCrowdKpt];
+#pragma unroll
+            for (int s = 0; s < kCrowdKpt; ++s) {
+                const int64_t i = c0 + (int64_t)warp * kCrowdKpt * 32 + s * 32 + lane;
+                v[s] = i < len ? src[i] : 0u;
+            }
+#pragma unroll
+            for (int s = 0; s < kCrowdKpt; ++s) {
+                const int64_t i = c0 + (int64_t)warp * kCrowdKpt * 32 + s * 32 + lane;
+                d[s] = 256u;
+                if (i < len)
+                    d[s] = (pass < 4 ? v[s] >> 8 * pass : (uint32_t)(bits(v[s]) >> 8 * (pass - 4))) & 255u;
+            }
+            rank_in_warp<false>(d, rank, s_cnt[warp], lane);
+            __syncthreads();
+            if (tid < 256) {   // thread = digit: where each warp's members go
+                uint32_t at = s_off[pass][tid];
                 for (int w = 0; w < NW; ++w) {
                     const uint32_t t = s_cnt[w][tid];
-                    s_cnt[w][tid] = total;
-                    total += t;
+                    s_cnt[w][tid] = at;
+                    at += t;
                 }
-            __syncthreads();
-            if (valid) dst[s_off[d] + s_cnt[warp][d] + (uint32_t)__popc(lower)] = v;
-            __syncthreads();
-            if (tid < 256) {
-                s_off[tid] += total;
-                for (int w = 0; w < NW; ++w) s_cnt[w][tid] = 0u;
+                s_off[pass][tid] = at;
             }
+            __syncthreads();
+#pragma unroll
+            for (int s = 0; s < kCrowdKpt; ++s)
+                if (d[s] < 256u) dst[s_cnt[warp][d[s]] + rank[s]] = v[s];
             __syncthreads();
         }
         uint32_t* t = src;
@@ -1204,8 +1233,8 @@ __device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, 
     }
     if (src != val) {
         for (int64_t i = tid; i < len; i += TH) val[i] = src[i];
-        __syncthreads();
     }
+    __syncthreads();
 }
 
 // One block per bucket: its place in the order from the bucket sizes, the sort
@@ -1218,10 +1247,10 @@ __device__ __noinline__ void sort_bucket_global(const Vec4<R>* posm, int64_t N, 
 // it.  Latency-bound: a chain of loads and block-wide steps, about 12 us per
 // block whatever its size, hidden only by other blocks.
 template <typename R, int TH, int KPT>
-__global__ void __launch_bounds__(TH)
-bucket_sort_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, const KeyCdf* cdf,
-                   const uint32_t* sizes, const uint2* region, uint32_t* perm, uint32_t* tmp,
-                   Vec4<R>* sorted, unsigned* err) {
+__global__ void __launch_bounds__(TH, 1024 / TH)   // 64 registers
+bucket_sort_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, int ntiles, const uint32_t* sizes,
+                   const uint2* region, const uint32_t* spill, const uint2* runs, uint32_t* perm,
+                   uint32_t* tmp, Vec4<R>* sorted, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
     using Sort = BlockSort<TH, KPT>;
     constexpr int CAP = Sort::CAP;
@@ -1252,7 +1281,8 @@ bucket_sort_kernel(const Vec4<R>* posm, int64_t N, int nbuckets, const KeyCdf* c
         if (base + len > N) len = N - base;
         if (len == 0) return;
         if (len > CAP) {
-            sort_bucket_global<R, TH>(posm, N, cdf, nbuckets, b, perm + base, tmp + base, len,
+            sort_bucket_global<R, TH>(posm, N, region + (size_t)b * CAP, CAP, spill, runs + b, ntiles,
+                                      nbuckets, perm + base, tmp + base, len,
                                       reinterpret_cast<uint32_t*>(sort_smem));
             if (sorted)
                 for (int64_t i = tid; i < len; i += TH)
@@ -1370,6 +1400,11 @@ SortBuffers sort_buffers(void* ws, int64_t N, size_t* total) {
         b.region = take((size_t)sp.nbuckets * 3 * sp.mean * sizeof(uint2));
         b.cdf = take(sizeof(KeyCdf));
         b.part = reinterpret_cast<uint32_t*>(take((kPartHeader + kMaxBuckets) * 4));
+        b.spill = reinterpret_cast<uint32_t*>(take(n4));
+        // (bounds of the tiles and buckets that grow with N, as the sizes asked for should)
+        const size_t tiles = (size_t)std::min<int64_t>((N + kPartThreads - 1) / kPartThreads, kMaxTiles);
+        const size_t buckets = (size_t)std::min<int64_t>((N + kSmallMean - 1) / kSmallMean, kMaxBuckets);
+        b.runs = take(tiles * buckets * sizeof(uint2));
     }
     if (radix_end > off) off = radix_end;
     if (total) *total = off;
@@ -1402,7 +1437,8 @@ static int launch_partition(const Vec4<R>* pp, int64_t N, const SamplePlan& sp,
     const uint64_t stride = ((uint64_t)N << 32) / (uint64_t)(kOversample * sp.nbuckets);
     if (launch_pdl(k, dim3(sp.ntiles + 1), dim3(kPartThreads), smem, ctx.stream, pp, N, sp.nbuckets,
                    3 * sp.mean, stride, reinterpret_cast<KeyCdf*>(b.cdf), b.part,
-                   reinterpret_cast<uint2*>(b.region), ctx.wait_limit > 0 ? ctx.wait_limit : kSpinLimit, ctx.err))
+                   reinterpret_cast<uint2*>(b.region), b.spill, reinterpret_cast<uint2*>(b.runs),
+                   ctx.wait_limit > 0 ? ctx.wait_limit : kSpinLimit, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;
@@ -1422,10 +1458,10 @@ static int launch_buckets(const Vec4<R>* pp, int64_t N, const SamplePlan& sp, co
     constexpr size_t smem = BlockSort<TH, KPT>::kSmem;
     auto k = bucket_sort_kernel<R, TH, KPT>;
     if (allow_smem(k, done, smem)) return ETICS_ERR_CUDA;
-    if (launch_pdl(k, dim3(sp.nbuckets), dim3(TH), smem, ctx.stream, pp, N, sp.nbuckets,
-                   reinterpret_cast<const KeyCdf*>(b.cdf),
+    if (launch_pdl(k, dim3(sp.nbuckets), dim3(TH), smem, ctx.stream, pp, N, sp.nbuckets, sp.ntiles,
                    (const uint32_t*)(b.part ? b.part + kPartHeader : nullptr),
-                   reinterpret_cast<const uint2*>(b.region), b.vals_a, b.vals_b, sorted, ctx.err))
+                   reinterpret_cast<const uint2*>(b.region), (const uint32_t*)b.spill,
+                   reinterpret_cast<const uint2*>(b.runs), b.vals_a, b.vals_b, sorted, ctx.err))
         return ETICS_ERR_CUDA;
     ++*ctx.launches;
     return ETICS_OK;

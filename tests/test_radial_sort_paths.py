@@ -13,6 +13,31 @@ DTYPES = {"mixed": torch.float32, "fp64": torch.float64}
 ONE_BLOCK, BUCKETS, RADIX = 7168, 1867776, 1867777
 
 
+def oracle_order(pm):
+    x = pm[:, :3]
+    r2 = (x[:, 0] * x[:, 0] + x[:, 1] * x[:, 1]) + x[:, 2] * x[:, 2]
+    return np.lexsort((np.arange(len(x)), r2))
+
+
+def seen(pm, precision):
+    return pm.astype(np.float32).astype(np.float64) if precision == "mixed" else pm
+
+
+def shells(n, count, seed, same=False):
+    """n particles on `count` thin shells (r^2 of a shell within a few ulps) or,
+    same=True, at `count` points (equal r^2: ordered by index alone), shuffled."""
+    rng = np.random.default_rng(seed)
+    u = rng.normal(size=(n, 3))
+    which = rng.integers(0, count, n)
+    if same:
+        u = rng.normal(size=(count, 3))[which]
+    r = np.geomspace(0.05, 20.0, count)[which]
+    pm = np.empty((n, 4))
+    pm[:, :3] = u / np.linalg.norm(u, axis=1)[:, None] * r[:, None]
+    pm[:, 3] = 1.0 / n
+    return pm
+
+
 def device(pm, precision):
     return torch.tensor(pm, dtype=DTYPES[precision], device="cuda")
 
@@ -32,3 +57,47 @@ def test_order_reports_a_nonfinite_particle(n, bad, precision):
         assert etics.get_error() == etics.ERR_NONFINITE, (at, column)
     etics.radial_order(x)
     assert etics.get_error() == 0
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("same", [False, True])
+@pytest.mark.parametrize("n,count", [(7169, 1), (7169, 2), (12289, 3), (154625, 7), (300007, 40),
+                                     (1048577, 150), (BUCKETS, 300)])
+def test_order_of_crowded_buckets(n, count, same, precision):
+    """Buckets beyond a block's room: their first places, the runs of every tile
+    and the sort of the lot, at the edges of the tile and bucket sizes."""
+    pm = shells(n, count, 17 + count, same)
+    pm[: n // 20] = inputs.hernquist(n // 20, seed=5)      # and ordinary ones beside them
+    got = etics.radial_order(device(pm, precision)).cpu().numpy()
+    etics.check_error()
+    assert np.array_equal(got, oracle_order(seen(pm, precision)))
+
+
+@pytest.mark.parametrize("same", [False, True])
+def test_crowded_buckets_cost_what_they_hold(same):
+    """2^20 particles on 300 shells: every shell of 3500 is more than its bucket
+    has room for.  A bucket's block then goes over its own members at most 13 times (a
+    count of all digits, a placement for each of up to 12) in steps of 2048: about
+    25 steps of a few us beside the ordinary sort of as many particles, so at most
+    ten times that.  Reading all particles for each such bucket would take 4096
+    steps."""
+    n = 1 << 20
+
+    def best(pm):
+        x = device(pm, "mixed")
+        for _ in range(3):
+            etics.radial_order(x)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        times = []
+        for _ in range(10):
+            t0.record()
+            etics.radial_order(x)
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        etics.check_error()
+        return min(times)
+
+    plain, crowded = best(inputs.hernquist(n, seed=1)), best(shells(n, 300, 2, same))
+    print(f"plain {plain * 1e3:.0f} us, crowded {crowded * 1e3:.0f} us")
+    assert crowded <= 10 * plain, (plain, crowded)
