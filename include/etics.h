@@ -72,7 +72,8 @@ enum etics_out { ETICS_OUT_ACC = 1, ETICS_OUT_POT = 2 };   /* force/potential/bo
 /* Bytes of device workspace a call of `method` (ETICS_SCF: etics_scf_coeffs
  * and etics_leapfrog_step with SCF; ETICS_MEX: etics_mex_field,
  * etics_radial_sort and etics_leapfrog_step with MEX) needs on the current
- * device.  Returns 0 for invalid arguments. */
+ * device.  It does not decrease with N, so a workspace sized for the largest
+ * call serves every smaller one.  Returns 0 for invalid arguments. */
 size_t etics_workspace_bytes(int64_t N, int n_max, int l_max, int method, int precision);
 
 /* SCF coefficient pass (Sec. 3.3, first part; eq. 18):

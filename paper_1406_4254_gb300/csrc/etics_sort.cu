@@ -1407,7 +1407,11 @@ SortBuffers sort_buffers(void* ws, int64_t N, size_t* total) {
         b.runs = take(tiles * buckets * sizeof(uint2));
     }
     if (radix_end > off) off = radix_end;
-    if (total) *total = off;
+    // at least what the largest bucket sort takes: a workspace sized for the
+    // largest call serves every smaller one
+    size_t least = 0;
+    if (total && N > kSampleMaxN) sort_buffers(nullptr, kSampleMaxN, &least);
+    if (total) *total = std::max(off, least);
     return b;
 }
 

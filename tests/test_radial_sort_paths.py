@@ -101,3 +101,27 @@ def test_crowded_buckets_cost_what_they_hold(same):
     plain, crowded = best(inputs.hernquist(n, seed=1)), best(shells(n, 300, 2, same))
     print(f"plain {plain * 1e3:.0f} us, crowded {crowded * 1e3:.0f} us")
     assert crowded <= 10 * plain, (plain, crowded)
+
+
+def test_workspace_does_not_shrink_with_more_particles():
+    """A workspace sized for the largest call serves every smaller one, across
+    the lines between the paths and between their tile and bucket sizes."""
+    sizes = sorted({max(1, c + d) for c in (1, 1024, ONE_BLOCK, 154624, 309248, 463872, 1 << 20,
+                                            (1 << 20) + 2048, 1300000, 1800000, BUCKETS, 2500000,
+                                            4000000)
+                    for d in (-1025, -1, 0, 1, 1025)})
+    for method, l_max in ((etics.MEX, 0), (etics.MEX, 6), (etics.MEX, 10), (etics.SCF, 6)):
+        for prec in (etics.MIXED, etics.FP64):
+            need = [etics.workspace_bytes(n, 10, l_max, method, prec) for n in sizes]
+            assert all(b >= a for a, b in zip(need, need[1:])), (method, l_max, prec)
+
+
+def test_a_workspace_for_more_particles_is_accepted():
+    n, most = 1800000, 2500000
+    x = device(inputs.hernquist(n, seed=9), "mixed")
+    ws = torch.empty(etics.workspace_bytes(most, 0, 4, etics.MEX, etics.MIXED) + 256,
+                     dtype=torch.uint8, device="cuda")
+    ref = etics.mex_field(x, 4)
+    out = etics.mex_field(x, 4, ws=ws)
+    etics.check_error()
+    assert torch.equal(out, ref)
