@@ -228,6 +228,8 @@ __global__ void mlp_colsum_partial_kernel(const float* __restrict__ dz, int M, i
 constexpr int kThin = 8;
 constexpr int kThinBlocks = kTargetBlocks;   // row chunks, and so partial sums, at most
 constexpr int kThinInputs = 1024;            // inputs of a narrow output layer, at most
+constexpr int kThinOutputs = 1024;           // outputs of a narrow input layer, at most (every
+                                             // chunk of rows leaves a partial gradient)
 
 __device__ __forceinline__ float bf(bf16 v) { return __bfloat162float(v); }
 
@@ -976,7 +978,9 @@ struct MlpLayout {
 };
 
 // whether the weight gradient of layer i runs on the narrow kernel
-bool narrow_in(const MlpLayout& o, int i) { return o.d[i] <= kThin && o.d[i + 1] % 4 == 0; }
+bool narrow_in(const MlpLayout& o, int i) {
+    return o.d[i] <= kThin && o.d[i + 1] % 4 == 0 && o.d[i + 1] <= kThinOutputs;
+}
 
 bool valid_shape(const etics_mlp_shape* s) {
     if (!s || s->nlayers < 1 || s->nlayers > ETICS_MLP_MAX_LAYERS) return false;
@@ -1027,13 +1031,11 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
         off += al256(std::max({(size_t)thin_chunks((int)Bz), ((size_t)Bz + tc::kM - 1) / tc::kM,
                                std::min((size_t)Bz, (size_t)kColChunks)}) * o.d[i + 1] * 8);
     }
-    // the largest split-K partial buffer over all products
+    // the largest split-K partial buffer over the forward and dH products
     size_t pmax = 0;
     for (int i = 0; i < o.L; ++i) {
         const GemmShape f = gemm_shape((int)Bz, o.d[i + 1], o.d[i]);            // forward
-        const GemmShape w = grad_shape(o.d[i], o.d[i + 1], (int)Bz);            // dW
         pmax = std::max(pmax, (size_t)f.splits * f.M * f.N);
-        pmax = std::max(pmax, (size_t)w.splits * w.M * w.N);
         if (i > 0) {
             const GemmShape h = gemm_shape((int)Bz, o.d[i], o.d[i + 1]);        // dH
             pmax = std::max(pmax, (size_t)h.splits * h.M * h.N);
