@@ -228,7 +228,7 @@ typedef struct { int nlayers; int dims[ETICS_MLP_MAX_LAYERS + 1]; } etics_mlp_sh
  * width outside 1..2^20). */
 int64_t etics_mlp_param_count(const etics_mlp_shape *shape);
 /* Device workspace of etics_mlp_forward / etics_mlp_loss_grad for `batch` rows
- * (0 for an invalid shape). */
+ * (0 for an invalid shape); it does not decrease with the batch. */
 size_t etics_mlp_workspace_bytes(const etics_mlp_shape *shape, int batch);
 /* y = network(x). */
 int etics_mlp_forward(const etics_mlp_shape *shape, const float *params,

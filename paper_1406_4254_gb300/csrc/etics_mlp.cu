@@ -935,10 +935,11 @@ __global__ void force_error_kernel(const Vec4<R>* __restrict__ a, const Vec4<R>*
 // output dimensions fill a tile at least half, else on the mma.sync kernel
 // (64 x 64 tiles, K step 32).  Split-K brings the block count near two per SM
 // while keeping >= 4 (mma.sync) or >= 2 (tcgen05) K steps per slice.
-struct GemmShape { int M, N, K, splits, kslice; bool tc; };
+// most: at least splits, and never smaller for a larger K.
+struct GemmShape { int M, N, K, splits, kslice, most; bool tc; };
 
 GemmShape gemm_shape(int M, int N, int K, int target = kTargetBlocks) {
-    GemmShape s{M, N, K, 1, 0, M >= 64 && N >= 64};
+    GemmShape s{M, N, K, 1, 0, 1, M >= 64 && N >= 64};
     const int bm = s.tc ? tc::kM : kBM, bn = s.tc ? tc::kN : kBN, bk = s.tc ? tc::kK : kBK;
     const int tiles = ((M + bm - 1) / bm) * ((N + bn - 1) / bn);
     const int ktiles = (K + bk - 1) / bk;
@@ -948,10 +949,31 @@ GemmShape gemm_shape(int M, int N, int K, int target = kTargetBlocks) {
     if (splits > max_splits) splits = max_splits;
     if (splits > 64) splits = 64;
     if (splits < 1) splits = 1;
+    s.most = splits;
     const int per = (ktiles + splits - 1) / splits;
     s.kslice = per * bk;
     s.splits = (ktiles + per - 1) / per;
     return s;
+}
+
+// Floats of the K slices of a product with B rows, the most of any B' <= B (it
+// is cut into fewer slices where it has more rows).
+size_t slice_floats(int B, int N, int K) {
+    size_t most = 0;
+    auto look = [&](int64_t rows) {
+        const GemmShape s = gemm_shape((int)std::min<int64_t>(B, rows), N, K);
+        most = std::max(most, (size_t)s.splits * s.M * s.N);
+    };
+    look(B);
+    look(63);   // below the tcgen05 kernel's least
+    const int bm = N >= 64 ? tc::kM : kBM, bn = N >= 64 ? tc::kN : kBN;
+    const int cols = (N + bn - 1) / bn;
+    // the most rows with so many slices or more (a slice has 128 values of K)
+    for (int splits = 2; splits <= std::min(64, K / 128 + 1); ++splits) {
+        const int64_t tiles = (kTargetBlocks - 1) / (splits - 1) / cols;
+        if (tiles > 0) look(tiles * bm);
+    }
+    return most;
 }
 
 // A weight gradient: K is the batch, and each K slice leaves a partial product
@@ -963,6 +985,8 @@ GemmShape grad_shape(int din, int dout, int B) {
 // rows per chunk of the narrow kernels, and the chunks
 int thin_rows(int B) { return std::max(16, (B + kThinBlocks - 1) / kThinBlocks); }
 int thin_chunks(int B) { return (B + thin_rows(B) - 1) / thin_rows(B); }
+// at least as many, never fewer for more rows
+int thin_most(int B) { return std::min((B + 15) / 16, kThinBlocks); }
 
 struct MlpLayout {
     int L;
@@ -1021,25 +1045,23 @@ MlpLayout mlp_layout(const etics_mlp_shape* s, int B) {
     o.narrow_out = o.d[o.L] <= kThin && o.d[o.L - 1] % 16 == 0 && o.d[o.L - 1] <= kThinInputs;
     for (int i = 0; i < o.L; ++i) {
         const GemmShape w = grad_shape(o.d[i], o.d[i + 1], (int)Bz);
-        const size_t parts = (size_t)std::max(w.splits, thin_chunks((int)Bz));
+        // (sized by bounds that grow with the batch: a workspace for many rows
+        // serves fewer)
+        const size_t parts = (size_t)std::max(w.most, thin_most((int)Bz));
         const bool narrow = narrow_in(o, i) || (i == o.L - 1 && o.narrow_out);
         o.wpart[i] = off;
-        off += al256((narrow ? parts : (size_t)w.splits) * o.d[i] * o.d[i + 1] * 4);
+        off += al256((narrow ? parts : (size_t)w.most) * o.d[i] * o.d[i + 1] * 4);
         o.bpart[i] = off;
         // rows of column sums: of a narrow kernel, of a product's tiles, or of
         // mlp_colsum_partial_kernel
-        off += al256(std::max({(size_t)thin_chunks((int)Bz), ((size_t)Bz + tc::kM - 1) / tc::kM,
+        off += al256(std::max({(size_t)thin_most((int)Bz), ((size_t)Bz + tc::kM - 1) / tc::kM,
                                std::min((size_t)Bz, (size_t)kColChunks)}) * o.d[i + 1] * 8);
     }
     // the largest split-K partial buffer over the forward and dH products
     size_t pmax = 0;
     for (int i = 0; i < o.L; ++i) {
-        const GemmShape f = gemm_shape((int)Bz, o.d[i + 1], o.d[i]);            // forward
-        pmax = std::max(pmax, (size_t)f.splits * f.M * f.N);
-        if (i > 0) {
-            const GemmShape h = gemm_shape((int)Bz, o.d[i], o.d[i + 1]);        // dH
-            pmax = std::max(pmax, (size_t)h.splits * h.M * h.N);
-        }
+        pmax = std::max(pmax, slice_floats((int)Bz, o.d[i + 1], o.d[i]));              // forward
+        if (i > 0) pmax = std::max(pmax, slice_floats((int)Bz, o.d[i], o.d[i + 1]));   // dH
     }
     o.part = off; off += al256(pmax * 4);
     o.loss_blocks = off; off += al256(std::max(kLossBlocks, kThinBlocks) * 8);

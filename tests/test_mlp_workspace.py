@@ -24,6 +24,15 @@ def test_a_wide_layer_needs_no_sums_per_chunk_of_rows(width, batch):
     assert need([8, width], batch) <= rows + width * (columns + narrow) + (1 << 16)
 
 
+@pytest.mark.parametrize("dims", [[8, 64, 64, 3], [8, 1024], [64, 64, 64, 64, 64], [4, 8, 8],
+                                  [8, 4096, 8], [16, 3], [8, 16, 1], [8, 256, 256, 3], [256, 256],
+                                  [9720, 256, 256, 1215], [1000, 70, 500, 63], [2000, 64]])
+def test_workspace_does_not_shrink_with_more_rows(dims):
+    """A workspace sized for the largest batch serves every smaller one."""
+    sizes = [need(dims, b) for b in range(1, 42000)]
+    assert all(b >= a for a, b in zip(sizes, sizes[1:]))
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("dims,batch", [([8, 1024, 3], 33), ([8, 1028, 3], 33), ([3, 2048], 130)])
 def test_layers_around_the_widest_narrow_one_match_oracle(dims, batch):
