@@ -235,8 +235,8 @@ __device__ __forceinline__ float bf(bf16 v) { return __bfloat162float(v); }
 
 // y = a W + bias for dout <= kThin outputs on m16n8k16 MMAs, one warp per 16
 // rows, the K slices and the order inside them those of mlp_gemm_kernel (the
-// same bits).  With a target: dy = scale (y - t) in bf16 and per block the sums
-// of (y - t)^2 and of dy (FP32 pairs); else y itself.
+// same bits).  With a target: dy = scale (y - t) in bf16 and per block the FP64
+// sums of (y - t)^2 and of dy; else y itself.
 __global__ void __launch_bounds__(256)
 mlp_narrow_out_kernel(const bf16* a, const bf16* W,
                       const float* bias, const float* target, int B,
@@ -253,7 +253,7 @@ mlp_narrow_out_kernel(const bf16* a, const bf16* W,
     }
     __syncthreads();
     const float b0 = 2 * t < dout ? bias[2 * t] : 0.0f, b1 = 2 * t + 1 < dout ? bias[2 * t + 1] : 0.0f;
-    float ls = 0.0f, le = 0.0f, gs[2] = {0.0f, 0.0f}, ge[2] = {0.0f, 0.0f};
+    double l = 0.0, db[2] = {0.0, 0.0};
     for (int r0 = ((int)blockIdx.x * 8 + warp) * 16; r0 < B; r0 += (int)gridDim.x * 8 * 16) {
         const bool v0 = r0 + g < B, v1 = r0 + g + 8 < B;
         const bf16* p0 = a + (size_t)(r0 + g) * din + 2 * t;
@@ -283,19 +283,16 @@ mlp_narrow_out_kernel(const bf16* a, const bf16* W,
             const size_t at = (size_t)row * dout + n;
             const float v = total[e] + ((e & 1) ? b1 : b0);
             if (target) {
-                const float d = v - target[at], gr = scale * d, sq = d * d;
+                const float d = v - target[at], gr = scale * d;
                 dyb[at] = __float2bfloat16_rn(gr);
-                tc::add_exact(ls, le, sq);
-                le += fmaf(d, d, -sq);
-                tc::add_exact(gs[e & 1], ge[e & 1], gr);
+                l += (double)d * (double)d;
+                db[e & 1] += (double)gr;
             } else {
                 y[at] = v;
             }
         }
     }
     if (!target) return;
-    double l = (double)ls + (double)le;
-    double db[2] = {(double)gs[0] + (double)ge[0], (double)gs[1] + (double)ge[1]};
 #pragma unroll
     for (int o = 16; o >= 4; o >>= 1) {   // over the rows (lanes of equal t)
         l += __shfl_xor_sync(0xffffffffu, l, o);
@@ -414,7 +411,7 @@ mlp_narrow_back_kernel(const bf16* a, const float* h,
         for (int j = 0; j < 4; ++j) {
 #pragma unroll
             for (int o = 0; o < DO; ++o) s_acc[rg - 1][cg][j][o] = acc[j][o];
-            s_db[rg - 1][cg][j] = (double)cs[j] + (double)ce[j];
+            s_db[rg - 1][cg][j] = tc::exact_sum(cs[j], ce[j]);
         }
     }
     __syncthreads();
@@ -427,7 +424,7 @@ mlp_narrow_back_kernel(const bf16* a, const float* h,
                 ((acc[j][o] + s_acc[0][cg][j][o]) + s_acc[1][cg][j][o]) + s_acc[2][cg][j][o];
         if (h)
             db_part[(size_t)blockIdx.y * din + m + j] =
-                (((double)cs[j] + (double)ce[j]) + s_db[0][cg][j]) + (s_db[1][cg][j] + s_db[2][cg][j]);
+                (tc::exact_sum(cs[j], ce[j]) + s_db[0][cg][j]) + (s_db[1][cg][j] + s_db[2][cg][j]);
     }
 }
 
