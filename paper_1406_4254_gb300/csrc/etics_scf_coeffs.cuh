@@ -20,7 +20,7 @@
 //     load brings both particles' values of a column, and each of the NR x ncol
 //     updates is one paired FMA.  Accumulators are FP32 register pairs;
 //     the recursion constants of the bin's level are scalar registers.
-//   * every kPairFlushTiles tiles each warp adds its accumulators over its
+//   * every 2048 particles (coeff_flush_tiles) each warp adds its accumulators over its
 //     lanes (a reduce-scatter: each step halves the values a lane still holds)
 //     and the totals to its FP64 block sums in shared memory.  The per-block
 //     sums are added in a fixed order by the finalize kernel: deterministic.
@@ -42,7 +42,6 @@
 
 namespace etics {
 
-constexpr int kPairFlushTiles = 16;   // tiles between FP64 flushes
 constexpr int kCoeffMaxBins = 80;      // sum over l <= 14 of ceil((2l+1)/CAP) <= 64
 constexpr int kCoeffMaxGroups = 8;
 
@@ -59,6 +58,9 @@ template <int NR> struct PairShape {
 template <int NR, int LMU> constexpr int coeff_tile() {
     return LMU <= 8 ? PairShape<NR>::kWarps * 32 : 256;
 }
+
+// tiles between FP64 flushes: the FP32 partial sums span at most 2048 particles
+template <int NR, int LMU> constexpr int coeff_flush_tiles() { return 2048 / coeff_tile<NR, LMU>(); }
 
 struct CoeffBin { int16_t l, c0, nc, pad; };
 struct CoeffGroup { int bin0, nbins, teams, l_lo, l_hi, block0, nblocks, pad; };
@@ -332,7 +334,7 @@ scf_coeff_plan_kernel(const __grid_constant__ ScfCoeffPairParams p) {
                                            reinterpret_cast<const float2*>(Hb(b)) + (size_t)col0 * TP,
                                            reinterpret_cast<const float2*>(Xb(b)),
                                            lane + 32 * team, pairs_in(t), 32 * gr.teams);
-        if (++since == kPairFlushTiles) {
+        if (++since == coeff_flush_tiles<NR, LMU>()) {
             if (active) flush();
             since = 0;
         }
