@@ -32,7 +32,6 @@ namespace etics {
 constexpr int kBatchThreads = 256;
 
 constexpr int kBatchMagic = 0x45544232;   // "ETB2"
-constexpr size_t kMaxDynSmem = 227 * 1024;  // opt-in shared memory per block on sm_103a
 
 struct BatchHeader {
     int magic, precision;
@@ -335,6 +334,10 @@ struct BpShare {
 inline int64_t bp_region(int l_max) {
     const int64_t cols = (int64_t)(l_max + 1) * (l_max + 1) * kBpStep;
     return std::max(cols, (int64_t)kBatchNR * kBpCap * kBpBlock);
+}
+
+inline size_t bp_smem(int l_max) {
+    return kBpNbBytes + (size_t)(bp_region(l_max) + kBpStep) * sizeof(float) + kBpStep * sizeof(float4);
 }
 
 __global__ void __launch_bounds__(kBpBlock, 2)
@@ -797,11 +800,9 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
             int l_max = 0;
             for (int i = 0; i < hd.ninst; ++i) l_max = std::max(l_max, insts[i].l_max);
             const int64_t region = bp_region(l_max);
-            const size_t smem = kBpNbBytes + (size_t)(region + kBpStep) * sizeof(float) +
-                                kBpStep * sizeof(float4);
+            const size_t smem = bp_smem(l_max);
             auto k = batch_pairs_kernel;
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-                return ETICS_ERR_CUDA;
+            if (allow_dynamic_smem(k, bp_smem(kBatchLM))) return ETICS_ERR_CUDA;
             unsigned* counter =
                 reinterpret_cast<unsigned*>(static_cast<unsigned char*>(ws) + hd.counter_off);
             if (cudaMemsetAsync(counter, 0, sizeof(unsigned), ctx.stream)) return ETICS_ERR_CUDA;
@@ -810,9 +811,7 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
                 static_cast<double*>(ws), counter, ctx.err);
         } else {
             auto k = batch_coeff_kernel<R>;
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)hd.smem_coef))
-                return ETICS_ERR_CUDA;
+            if (allow_dynamic_smem(k)) return ETICS_ERR_CUDA;
             k<<<hd.nblocks, kBatchThreads, hd.smem_coef, ctx.stream>>>(
                 reinterpret_cast<const Vec4<R>*>(posm), plan_dev, static_cast<double*>(ws), ctx.err);
         }

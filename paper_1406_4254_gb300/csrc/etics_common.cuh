@@ -295,6 +295,13 @@ __host__ __device__ __forceinline__ int col_offset(int l) {
 }
 __host__ __device__ __forceinline__ int col_total(int lmax) { return col_offset(lmax + 1); }
 
+// Shared memory a kernel may ask for: set to the same bound by every call, never
+// to what one call needs, which another host thread's launch could find too small.
+constexpr size_t kMaxDynSmem = 227 * 1024;   // opt-in shared memory per block on sm_103a
+template <typename K> inline cudaError_t allow_dynamic_smem(K kernel, size_t most = kMaxDynSmem) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // launch context handed from the C ABI to the kernel launchers
 // Programmatic dependent launch.  A kernel started by launch_pdl may be
 // scheduled while the previous kernel in its stream drains (its launch

@@ -411,9 +411,7 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
                                          sizeof(Vec4<R>) : 0);
     auto k = (out_mask & ETICS_OUT_ACC) ? scf_field_kernel<P, LM, true, NM1, B>
                                         : scf_field_kernel<P, LM, false, NM1, B>;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-        return ETICS_ERR_CUDA;
+    if (smem > 48 * 1024 && allow_dynamic_smem(k)) return ETICS_ERR_CUDA;
     // launched as a programmatic dependent of the coefficient finalize (or
     // whatever precedes it): its launch overlaps the predecessor's tail
     if (launch_pdl(k, dim3(grid), dim3(threads), smem, ctx.stream,

@@ -319,13 +319,11 @@ inline int launch_coeff_nr(const ScfCoeffParams& p, int lmu, int grid, size_t sm
                            cudaStream_t s) {
     if (lmu <= 6) {
         auto k = scf_coeff_kernel<R, NR, 6, B>;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-            return ETICS_ERR_CUDA;
+        if (allow_dynamic_smem(k)) return ETICS_ERR_CUDA;
         k<<<grid, ScfCfg<R>::kThreads, smem, s>>>(p);
     } else {
         auto k = scf_coeff_kernel<R, NR, kLmaxLimit, B>;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-            return ETICS_ERR_CUDA;
+        if (allow_dynamic_smem(k)) return ETICS_ERR_CUDA;
         k<<<grid, ScfCfg<R>::kThreads, smem, s>>>(p);
     }
     return cudaGetLastError() == cudaSuccess ? ETICS_OK : ETICS_ERR_CUDA;
