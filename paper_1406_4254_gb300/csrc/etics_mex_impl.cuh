@@ -60,7 +60,8 @@ constexpr int kMexGroups = 3;
 __host__ __device__ constexpr int mex_group_l0(int g) { return g == 0 ? 0 : (g == 1 ? 7 : 9); }
 __host__ __device__ constexpr int mex_group_l1(int g) { return g == 0 ? 6 : (g == 1 ? 8 : 10); }
 __host__ __device__ constexpr int mex_ncomp(int l_max) { return (l_max + 1) * (l_max + 1); }
-// components per side in the buffers: one layout for all l_max <= 6
+// components per side that the workspace has room for (one size for all
+// l_max <= 6); the passes use mex_ncomp of them
 __host__ __device__ constexpr int mex_layout_ncomp(int l_max) {
     return l_max <= 6 ? kMexNC : mex_ncomp(l_max);
 }
@@ -352,7 +353,7 @@ mex_pass1_kernel(const Vec4<R>* sorted, int64_t N, int l_max,
     const int e = mex_tile_exponent<R>(v[0], v[1], nt, s_end);
     MexPair<R> p;
     p.init(v[0], v[1], ldexp(R(1), -e), ldexp(R(1), e));
-    const int ncomp = mex_layout_ncomp(l_max);
+    const int ncomp = mex_ncomp(l_max);
     for (int g = 0; g < NG; ++g) {
         const int L0 = mex_group_l0(g), L1 = mex_group_l1(g);
         if (L0 > l_max) break;
@@ -555,7 +556,7 @@ mex_pass2_kernel(const Vec4<R>* sorted, const uint32_t* perm, int64_t N,
     MexField<R> f;
     const Pair<R> zero = splat<Pair<R>>(R(0));
     f.s0 = f.s1 = f.rad = f.vx = f.vy = f.vz0 = f.vz1 = f.pot0 = zero;
-    const int ncomp = mex_layout_ncomp(l_max);
+    const int ncomp = mex_ncomp(l_max);
     for (int g = 0; g < NG; ++g) {
         const int L0 = mex_group_l0(g), L1 = mex_group_l1(g);
         if (L0 > l_max) break;
@@ -624,7 +625,7 @@ template <typename R>
 struct MexBuffers {
     SortBuffers sort;
     Vec4<R>* sorted;
-    double* tile_agg;    // [2 * ncomp][tile]: inner then outer sums (ncomp: mex_layout_ncomp)
+    double* tile_agg;    // [2 * ncomp][tile]: inner then outer sums (ncomp: mex_ncomp)
     double* carry;       // [2 * ncomp][tile]
 };
 
@@ -676,7 +677,7 @@ template <typename R, int NG>
 inline int mex_passes(const MexBuffers<R>& b, int64_t N, int l_max, void* out, int out_mask,
                       const LaunchCtx& ctx) {
     const int nt = mex_tiles(N);
-    const int ncomp = mex_layout_ncomp(l_max);
+    const int ncomp = mex_ncomp(l_max);
     constexpr size_t smem_max = (size_t)2 * kMexNC * kMexRow * sizeof(R);
     const size_t smem = (size_t)2 * mex_row_comps(l_max) * kMexRow * sizeof(R);
     static std::atomic<uint64_t> done1{0}, done2{0}, done3{0};

@@ -125,3 +125,25 @@ def test_a_workspace_for_more_particles_is_accepted():
     out = etics.mex_field(x, 4, ws=ws)
     etics.check_error()
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("l_max", [0, 3, 5])
+def test_scans_only_the_components_there_are(l_max, precision):
+    """The workspace has room for 49 components per side up to l_max = 6; the
+    carry scan of fewer must not read the rest of it, which nothing writes, nor
+    write sums of that: the end of the workspace, which holds the last
+    components' carries, stays as it was."""
+    n = 100000
+    x = device(inputs.hernquist(n, seed=5), precision)
+    prec = etics.MIXED if precision == "mixed" else etics.FP64
+    need = etics.workspace_bytes(n, 0, l_max, etics.MEX, prec)
+    ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+    ws.fill_(0x11)
+    out = etics.mex_field(x, l_max, ws=ws)
+    etics.check_error()
+    assert torch.isfinite(out).all()
+    at = (-ws.data_ptr()) % 256
+    tiles = (n + 255) // 256
+    missing = 49 - (l_max + 1) ** 2
+    assert (ws[at + need - missing * tiles * 8:] == 0x11).all()
