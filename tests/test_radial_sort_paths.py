@@ -147,3 +147,87 @@ def test_scans_only_the_components_there_are(l_max, precision):
     tiles = (n + 255) // 256
     missing = 49 - (l_max + 1) ** 2
     assert (ws[at + need - missing * tiles * 8:] == 0x11).all()
+
+
+# ---- the radix path, and calls that no other test makes on it --------------------
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_radix_path_orders_long_runs(precision):
+    """Above the buckets: two shell halves of 100000 equal keys each, sorted by
+    one block across many tiles, 3000 copies of a point, runs of 17 to 300, and
+    then nothing but coincident points and few distinct radii in sorted order."""
+    from test_parity_mex import long_tie_particles
+    shell, copies = 200000, 3000
+    pm = long_tie_particles(shell, copies, RADIX - shell - copies, seed=41)
+    assert len(pm) >= RADIX
+    got = etics.radial_order(device(pm, precision)).cpu().numpy()
+    etics.check_error()
+    assert np.array_equal(got, oracle_order(seen(pm, precision)))
+    few = shells(RADIX + 5, 300, 43, same=True)
+    few = few[oracle_order(few)[::-1]]           # radii falling: every run reversed
+    got = etics.radial_order(device(few, precision)).cpu().numpy()
+    etics.check_error()
+    assert np.array_equal(got, oracle_order(seen(few, precision)))
+
+
+def test_both_paths_give_the_same_field():
+    """One massless particle far outside takes the call to the radix path and
+    changes nothing else (the carry scan is cut into other runs: FP64 roundings)."""
+    pm = inputs.hernquist(BUCKETS, seed=21, axes=(1.0, 0.8, 0.6))
+    pm[:, :3] = np.clip(pm[:, :3], -5e5, 5e5)
+    far = np.concatenate([pm, [[1e6, 0.0, 0.0, 0.0]]])
+    a = etics.mex_field(device(pm, "mixed"), 4)
+    b = etics.mex_field(device(far, "mixed"), 4)
+    etics.check_error()
+    rel = (b[:-1] - a).norm(dim=1) / a.norm(dim=1)
+    assert rel.max().item() < 1e-5 and rel.median().item() == 0.0
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [RADIX, 1 << 21])
+def test_radix_path_with_a_one_poll_lookback_bound_returns_and_reports(n, precision):
+    x = device(inputs.hernquist(n, seed=11), precision)
+    ref = etics.mex_field(x, 2)
+    assert etics.get_error() == 0
+    outcomes = []
+    try:
+        etics.set_wait_limit(1)
+        for _ in range(20):
+            etics.mex_field(x, 2)
+            outcomes.append(etics.get_error())
+            if etics.ERR_TIMEOUT in outcomes:
+                break
+    finally:
+        etics.set_wait_limit(0)
+    assert etics.ERR_TIMEOUT in outcomes, outcomes
+    assert set(outcomes) <= {0, etics.ERR_TIMEOUT}, outcomes
+    again = etics.mex_field(x, 2)
+    assert etics.get_error() == 0
+    assert torch.equal(again, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [5000, 100003, RADIX])
+def test_captured_call_gives_the_same_bits(n, precision):
+    """One block, buckets and radix passes (the latter two behind a memset node)
+    in a CUDA graph, replayed on other particles in the same buffers."""
+    x = device(inputs.hernquist(n, seed=7), precision)
+    y = device(inputs.hernquist(n, seed=8), precision)
+    prec = etics.MIXED if precision == "mixed" else etics.FP64
+    ws = torch.empty(etics.workspace_bytes(n, 0, 3, etics.MEX, prec) + 256, dtype=torch.uint8,
+                     device="cuda")
+    want = [etics.mex_field(x, 3), etics.mex_field(y, 3)]
+    posm, out = x.clone(), torch.empty_like(x)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        etics.mex_field(posm, 3, out=out, ws=ws)
+    torch.cuda.current_stream().wait_stream(side)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        etics.mex_field(posm, 3, out=out, ws=ws)
+    for particles, ref in zip((x, y, x), (want[0], want[1], want[0])):
+        posm.copy_(particles)
+        out.zero_()
+        graph.replay()
+        assert etics.get_error() == 0
+        assert torch.equal(out, ref)
