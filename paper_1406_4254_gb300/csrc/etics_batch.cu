@@ -13,7 +13,7 @@
 //      of the block owning one "bin" (one level, up to three columns) of the
 //      instance's expansion (batch_pairs_kernel).  FP64: register tiles of
 //      four columns over a shared-memory radial basis (batch_coeff_kernel);
-//   2. finalize: one thread per output coefficient of any instance;
+//   2. finalize: one to 32 threads per output coefficient of any instance;
 //   3. field: one block per work item (a chunk of one instance's particles),
 //      the instance's coefficients staged in shared memory.
 // No grid-wide barrier is needed, so the three launches capture into a CUDA
@@ -477,20 +477,29 @@ batch_pairs_kernel(const float4* __restrict__ posm, const void* __restrict__ pla
 }
 
 // ---------------------------------------------------------------------------
-// 2. finalize: ordered sum of an instance's segments, times K_lm / J_nl.  One
-// thread per output: FP64 additions are slow on this GPU, and a warp per
-// output spends most of them on its butterfly (256-system ensemble: 70 us).
+// 2. finalize: ordered sum of an instance's segments, times K_lm / J_nl.
+// `lanes` neighbouring threads (a power of two up to 32) share an output: one
+// where every system has at most kFinSegments segments, since FP64 additions are
+// slow on this GPU and a warp per output spends most of them on its butterfly
+// (256-system ensemble: 70 us, 21 with one thread); more where there are more, a
+// thread's share being a chain of loads and additions (one system of 2^20
+// particles: 1024 segments, 240 us with one thread, 14 with 16).
 // ---------------------------------------------------------------------------
-__global__ void batch_finalize_kernel(const void* __restrict__ plan,
+constexpr int kFinSegments = 64;
+inline int batch_fin_lanes(int nseg) {
+    int lanes = 1;
+    while (lanes < 32 && nseg > kFinSegments * lanes) lanes *= 2;
+    return lanes;
+}
+__global__ void batch_finalize_kernel(const void* __restrict__ plan, int lanes,
                                       const double* partial,
                                       double* coeffs) {
     const BatchHeader hd = *plan_table<BatchHeader>(plan, 0);
     const BatchInst* insts = plan_table<BatchInst>(plan, hd.off_inst);
-    const int64_t out = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (out >= hd.coef_total) {
-        pdl_wait();
-        return;
-    }
+    const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int sub = (int)(thread & (lanes - 1));
+    const bool valid = thread / lanes < hd.coef_total;
+    const int64_t out = valid ? thread / lanes : hd.coef_total - 1;
     int lo = 0, hi = hd.ninst - 1;          // instance holding this output
     while (lo < hi) {
         const int mid = (lo + hi + 1) / 2;
@@ -511,10 +520,21 @@ __global__ void batch_finalize_kernel(const void* __restrict__ plan,
     const double* src = partial + (size_t)in.first_seg * hd.seg_stride + idx;
     pdl_wait();   // the segments come from the coefficient kernel
     double s = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < in.nseg; ++k) s += ld_cg(src + (size_t)k * hd.seg_stride);
+    const int nseg = valid ? in.nseg : 0;
+    constexpr int kAhead = 8;   // loads in flight
+    int k = sub;
+    for (; k + (kAhead - 1) * lanes < nseg; k += kAhead * lanes) {
+        double v[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) v[j] = ld_cg(src + (size_t)(k + j * lanes) * hd.seg_stride);
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) s += v[j];
+    }
+    for (; k < nseg; k += lanes) s += ld_cg(src + (size_t)k * hd.seg_stride);
+    for (int o = lanes / 2; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
     const int am = m < 0 ? -m : m;
-    coeffs[out] = s * c_tab.knorm_fact[l * (l + 1) / 2 + am] * c_tab.inv_j[n][l] * geg_gamma(0, l, n);
+    if (valid && sub == 0)
+        coeffs[out] = s * c_tab.knorm_fact[l * (l + 1) / 2 + am] * c_tab.inv_j[n][l] * geg_gamma(0, l, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -823,14 +843,18 @@ int batch_launch(const void* posm, const void* plan_host, const void* plan_dev, 
         // The finalize reads the plan before its wait: the coefficient kernel,
         // launched the ordinary way, began after whatever wrote it.  Without
         // that kernel (no particles) the finalize has to do so itself.
-        const dim3 blocks((unsigned)((hd.coef_total + 127) / 128));
+        const BatchInst* insts = plan_table<BatchInst>(plan_host, hd.off_inst);
+        int nseg = 0;
+        for (int i = 0; i < hd.ninst; ++i) nseg = std::max(nseg, insts[i].nseg);
+        const int lanes = batch_fin_lanes(nseg);
+        const dim3 blocks((unsigned)((hd.coef_total * lanes + 127) / 128));
         const double* partial = static_cast<const double*>(ws);
         if (hd.ntiles > 0) {
-            if (launch_pdl(batch_finalize_kernel, blocks, dim3(128), 0, ctx.stream, plan_dev, partial,
-                           coeffs))
+            if (launch_pdl(batch_finalize_kernel, blocks, dim3(128), 0, ctx.stream, plan_dev, lanes,
+                           partial, coeffs))
                 return ETICS_ERR_CUDA;
         } else {
-            batch_finalize_kernel<<<blocks, 128, 0, ctx.stream>>>(plan_dev, partial, coeffs);
+            batch_finalize_kernel<<<blocks, 128, 0, ctx.stream>>>(plan_dev, lanes, partial, coeffs);
             if (cudaGetLastError()) return ETICS_ERR_CUDA;
         }
         ++*ctx.launches;
