@@ -202,7 +202,8 @@ __device__ __forceinline__ void mex_group_moments(const MexPair<R>& p, int l_max
 // + p rho^(l-1) (both already weighted), l >= 1:
 //   Phi = -(1/s) [ rho sum s R + q_00 / rho + p_00 ]
 //   a   = (1/s^2) [ kappa sum s grad R - u (sum (2l+1) q rho^-(l+2) R + q_00 / rho^2) ]
-// so one gradient contraction serves both parts.  The column holds the sums
+// so one gradient contraction serves both parts.  The potential alone takes
+// s_lm = q rho^-(l+1) + p rho^l, which stays in range for wider tiles.  The column holds the sums
 // over the particles before (after) the pair; the second particle's q also
 // holds the first, the first one's p the second (own: the first particle's
 // m rho^l and the second one's m rho^-(l+1); ownf: their factors per level).
@@ -289,7 +290,7 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                 }
             }
         }
-        // a_l = rho^-(l+2); b_l = rho^(l-1), b_1 = 1
+        // a_l = rho^-(l+2); b_l = rho^(l-1), b_1 = 1 (without the force: once more rho)
         const P bn = L == 0 ? b : mul2(b, p.rho);
         mex_eval<R, L0, L1, L + 1, ACC>(C, S, p, l_max, mul2(a, p.irho), bn, mul2(own, ownf), ownf,
                                         col, nc, f);
@@ -301,7 +302,8 @@ __device__ __forceinline__ void mex_group_eval(const MexPair<R>& p, int l_max, c
                                                MexField<R>& f) {
     constexpr int L0 = mex_group_l0(G), L1 = mex_group_l1(G);
     Pair<R> C[3][L1 + 1], S[3][L1 + 1];
-    mex_eval<R, L0, L1, 0, ACC>(C, S, p, l_max, mul2(p.irho, p.irho), splat<Pair<R>>(R(1)),
+    mex_eval<R, L0, L1, 0, ACC>(C, S, p, l_max, ACC ? mul2(p.irho, p.irho) : p.irho,
+                                ACC ? splat<Pair<R>>(R(1)) : p.rho,
                                 mk2(p.m.x, p.m.y * p.irho.y), mk2(p.rho.x, p.irho.y), col, nc, f);
 }
 
@@ -603,7 +605,8 @@ mex_pass2_kernel(const Vec4<R>* sorted, const uint32_t* perm, int64_t N,
         auto at = [&](const Pair<R>& q) { return j == 0 ? q.x : q.y; };
         const int i = 2 * tid + j;
         if (i >= nt) continue;
-        const R pot = fma(at(p.rho), fma(two, at(f.s1), at(f.s0)), at(f.pot0));
+        const R sum = fma(two, at(f.s1), at(f.s0));
+        const R pot = ACC ? fma(at(p.rho), sum, at(f.pot0)) : sum + at(f.pot0);
         const R potv = (out_mask & ETICS_OUT_POT) ? -pot * s1 : R(0);
         R fx = R(0), fy = R(0), fz = R(0);
         if (ACC) {
