@@ -320,7 +320,7 @@ int etics_get_error(void *stream);
  *
  * Bound, in polls, of the waits of the MEX radial sort's decoupled lookback
  * (a tile waiting for an earlier tile to publish its digit counts) and of its
- * partition's wait for the splitters, in later calls on any stream; 0 restores
+ * partition's wait for the table of the keys' distribution, in later calls on any stream; 0 restores
  * the default (2^22 polls of >= 32 ns).
  * When a wait runs out, the error word records ETICS_ERR_TIMEOUT, the tile
  * goes on with a partial prefix, and every later kernel of the call keeps its

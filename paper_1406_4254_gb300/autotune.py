@@ -4,7 +4,8 @@ Times every candidate :class:`~paper_1406_4254_gb300.etics.BatchTuning`
 (particles per coefficient tile, coefficient blocks per SM, field threads per
 block, particles per field work item) on a given batch with CUDA events and
 records the fastest in a JSON table keyed by the batch's largest n_max, largest
-l_max and total-N bucket (log2).  :func:`lookup` reads the table back.
+l_max and total-N bucket (log2).  Field threads beyond 128 are not used, and
+mixed-precision plans run two coefficient blocks per SM whatever blocks_per_sm says.  :func:`lookup` reads the table back.
 
     python -m paper_1406_4254_gb300.autotune      # tunes the 256-system ensemble
 """

@@ -202,9 +202,8 @@ batch_coeff_kernel(const Vec4<R>* __restrict__ posm, const void* __restrict__ pl
                 } else {
                     const R inv = r > R(0) ? R(1) / r : R(0);
                     const R ux = x * inv, uy = y * inv, uz = z * inv;
-                    const R uu = ux * ux + uy * uy + uz * uz;
                     R C[3][LMU + 1], S[3][LMU + 1];
-                    angular_levels<R, 0, LMU>(C, S, ux, uy, uz, uu, l_max, Ys, T, k);
+                    angular_levels<R, 0, LMU>(C, S, ux, uy, uz, l_max, Ys, T, k);
                     radial_levels<R, NR, 0, LMU>(Rs, T, k, n_max, l_split, l_max, -m * t, st, xi);
                 }
             }

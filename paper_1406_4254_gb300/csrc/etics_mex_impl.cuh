@@ -26,12 +26,14 @@
 // both access patterns, thread = particle pair and thread = component, are
 // free of bank conflicts); one thread per component then runs down its row.
 // Nothing per particle but the sorted copy reaches memory between the passes.
-// What bounds them: instruction issue (pass 2), the gather's latency (pass 1).
-// Measured against the form it replaced (seven particles per thread, all 98
-// sums of l_max = 6 in registers, every thread's prefix sums through memory):
-// N = 2^20, l_max = 6: pass 1 51 -> 37 us, pass 2 61 -> 52 us; N = 500009,
-// l_max = 10 (the whole call): 291 -> 167 us; N = 100003, l_max = 6, FP64:
-// 450 -> 341 us (256-particle tiles also fill the SMs more evenly).
+// What bounds them: instruction issue (pass 2), latency and shared memory (pass
+// 1, which reads the copy in radial order that the sort leaves).  Measured
+// against the form it replaced (seven particles per thread, all 98 sums of
+// l_max = 6 in registers, every thread's prefix sums through memory, the
+// particles gathered in pass 1): N = 2^20, l_max = 6: pass 1 51 -> 25 us, pass 2
+// 61 -> 51 us.  Whole calls with the sort by buckets: N = 500009, l_max = 10:
+// 291 -> 145 us; N = 100003, l_max = 6, FP64: 450 -> 323 us (256-particle tiles
+// also fill the SMs more evenly).
 //
 // Harmonics: the scaled ones of etics_pair.cuh, at kappa u.  The product of an
 // evaluated and a summed harmonic needs the weight (l-m)!(l+m)! kappa^-2l

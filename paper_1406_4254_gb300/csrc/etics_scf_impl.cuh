@@ -1,6 +1,7 @@
-// etics_scf_impl.cuh -- SCF coefficient kernel (templated on the arithmetic
-// type; instantiated for float in etics_scf_f32.cu and for double in
-// etics_scf_f64.cu).  The field pass is in etics_scf_field.cuh.
+// etics_scf_impl.cuh -- the FP64 SCF coefficient kernel (instantiated in
+// etics_scf_f64.cu and etics_scf_cb_f64.cu; mixed precision runs the kernels of
+// etics_scf_pairs.cuh, etics_scf_bins.cuh and etics_scf_coeffs.cuh) and the
+// finalize.  The field pass is in etics_scf_field.cuh.
 //
 // Method (paper Sec. 2.4 eq. 18, basis of Sec. 2.5, two passes of Sec. 3.3):
 //   c_nlm = (1/J_nl) sum_k m_k phi_nl(r_k) Y_lm(x_k)             (coefficients)
@@ -15,9 +16,9 @@
 //     contraction c[n][l,col] += sum_k R[l][n][k] Y[l,col][k] is then done
 //     with each thread owning an (n_rows x 4 columns) register tile of one l
 //     over a strided subset of the tile's particles (4 particles per 16-byte
-//     shared load).  FP32 partial sums are flushed into per-block FP64
-//     accumulators every few tiles; per-block FP64 partials are summed in a
-//     fixed order by a finalize kernel (deterministic).
+//     shared load).  The partial sums are flushed into per-block accumulators
+//     every few tiles; those are summed in a fixed order by a finalize kernel
+//     (deterministic).
 #pragma once
 
 #include "etics_scf_field.cuh"
@@ -25,7 +26,7 @@
 namespace etics {
 
 template <typename R> struct ScfCfg;
-template <> struct ScfCfg<float> {
+template <> struct ScfCfg<float> {   // for a workspace size only (scf_workspace_f32)
     static constexpr int kThreads = 256;   // coefficient kernel block
     static constexpr int kTile = 128;      // particles per tile (2 threads each in phase 1)
 };
@@ -61,25 +62,23 @@ __host__ inline size_t scf_coeff_smem(int NR, int l_max, int T, int W, int G) {
 
 // phase 1, angular half: write the factorial-scaled harmonics (l-m)! Z_l^m
 // (harm_level_exact; the finalize applies knorm_fact) of level 0..l_max for
-// particle k into Ys[col][k] (compile-time recursion over the level).
-// PAD: levels padded to multiples of 4 columns (col_offset_c); otherwise the
-// dense layout, level l starting at column l*l.  uu is unused: the
-// harmonics are taken on the unit sphere.
-template <typename R, int L, int LMU, bool PAD = true>
+// particle k into Ys[col][k] (compile-time recursion over the level), levels
+// padded to multiples of 4 columns (col_offset_c).
+template <typename R, int L, int LMU>
 __device__ __forceinline__ void angular_levels(R (&C)[3][LMU + 1], R (&S)[3][LMU + 1], R ux, R uy,
-                                               R uz, R uu, int l_max, R* Ys, int T, int k) {
+                                               R uz, int l_max, R* Ys, int T, int k) {
     if constexpr (L <= LMU) {
         if (L > l_max) return;
         constexpr int s0 = L % 3, s1 = (L + 2) % 3, s2 = (L + 1) % 3;
         harm_level_exact<R, L>(C[s1], S[s1], C[s2], S[s2], ux, uy, uz, C[s0], S[s0]);
-        constexpr int co = PAD ? col_offset_c(L) : L * L;
+        constexpr int co = col_offset_c(L);
         Ys[(size_t)(co + 0) * T + k] = C[s0][0];
 #pragma unroll
         for (int m = 1; m <= L; ++m) {
             Ys[(size_t)(co + 2 * m - 1) * T + k] = C[s0][m];
             Ys[(size_t)(co + 2 * m) * T + k] = S[s0][m];
         }
-        angular_levels<R, L + 1, LMU, PAD>(C, S, ux, uy, uz, uu, l_max, Ys, T, k);
+        angular_levels<R, L + 1, LMU>(C, S, ux, uy, uz, l_max, Ys, T, k);
     }
 }
 
@@ -201,9 +200,8 @@ scf_coeff_kernel(ScfCoeffParams p) {
                 // angular basis of every level, then radial levels [l_split, l_max]
                 const R inv = r > R(0) ? R(1) / r : R(0);
                 const R ux = x * inv, uy = y * inv, uz = z * inv;
-                const R uu = ux * ux + uy * uy + uz * uz;
                 R C[3][LMU + 1], S[3][LMU + 1];
-                angular_levels<R, 0, LMU>(C, S, ux, uy, uz, uu, p.l_max, Ys, T, k);
+                angular_levels<R, 0, LMU>(C, S, ux, uy, uz, p.l_max, Ys, T, k);
                 radial_levels<R, NR, 0, LMU, B>(Rs, T, k, p.n_max, p.l_split, p.l_max,
                                                 m * rs.pre0, rs.st, rs.xi);
             }

@@ -1,8 +1,8 @@
 // etics_scf_pairs_f32.cu -- the particle-pair SCF coefficient pass (see
 // etics_scf_pairs.cuh) at (n_max, l_max) = (10, 6), the expansion of the
 // paper's timing runs (Sec. 3.4): bins of at most 4 columns of one level, 16
-// warps of up to 128 registers (measured on GB300 at N = 2^20: 60.0 us against
-// 62.1 us with 3-column bins and 19 warps).  Its own translation unit so that
+// warps of up to 128 registers (46 us at N = 2^20; an early form took 60.0 us
+// so and 62.1 with 3-column bins and 19 warps).  Its own translation unit so that
 // it compiles in parallel with the other SCF kernels.
 #include "etics_internal.h"
 #include "etics_scf_pairs.cuh"
