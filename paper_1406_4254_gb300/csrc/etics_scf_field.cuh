@@ -288,18 +288,18 @@ __device__ __forceinline__ void field_eval(const Vec4<typename FieldLane<P>::R> 
 }
 
 // Few particles leave the SMs with a warp or two each, waiting on their own
-// results: then kFieldParts warps share the levels of the same particles and
-// their partial sums are added through shared memory.  level[w]: warp w's.
+// results: then two or kFieldParts warps share the levels of the same particles
+// and their partial sums are added through shared memory.  level[w]: warp w's.
 constexpr int kFieldParts = 4;
 struct FieldSplit { int parts; unsigned level[kFieldParts]; };
 inline FieldSplit field_split(int l_max, int parts) {
     FieldSplit s{parts, {~0u, ~0u, ~0u, ~0u}};
     if (parts == 1) return s;
     int load[kFieldParts] = {};
-    for (int w = 0; w < kFieldParts; ++w) s.level[w] = 0u;
+    for (int w = 0; w < parts; ++w) s.level[w] = 0u;
     for (int l = l_max; l >= 0; --l) {   // largest level first, to the least loaded
         int best = 0;
-        for (int w = 1; w < kFieldParts; ++w)
+        for (int w = 1; w < parts; ++w)
             if (load[w] < load[best]) best = w;
         s.level[best] |= 1u << l;
         load[best] += 2 * (2 * l + 1) + 6;
@@ -327,7 +327,7 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* posm, int64_t N, int n_ma
     field_table(cs, stride, coeffs, B, n_max, l_max);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int part = split.parts > 1 ? warp % kFieldParts : 0;
+    const int part = warp % split.parts;
     const int per = blockDim.x / split.parts;   // lanes of particles per block
     const int slot = (warp / split.parts) * 32 + lane;
     for (int64_t first = (int64_t)blockIdx.x * per * NP; first < N;
@@ -349,7 +349,7 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* posm, int64_t N, int n_ma
             }
             __syncthreads();
             if (part == 0) {
-                for (int w = 0; w < kFieldParts - 1; ++w)
+                for (int w = 0; w < split.parts - 1; ++w)
 #pragma unroll
                     for (int j = 0; j < NP; ++j) {
                         const Vec4<R> t = ld4(sums + (w * NP + j) * per + slot);
@@ -390,15 +390,16 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     // this GPU) is built once per SM; as many threads as give every block the
     // same number of rounds over the particles, so that neither a few large
     // blocks on part of the SMs (small N) nor a last round that is nearly
-    // empty leaves the GPU idle.  Where a quarter of the threads would do, the
-    // levels are split over four warps (mixed precision: the FP64 kernel is
-    // bound by the FP64 pipe at any size, and repeats the harmonics): (10, 6)
-    // 13 us up to 38912 particles, 17 with one warp for all levels; (14, 8) 17
-    // to 21 and 23 to 25 around 29184; l_max 10 19 and 27 around 19456.
+    // empty leaves the GPU idle.  Where a quarter or half of the threads would
+    // do, the levels are split over four or two warps (mixed precision: the FP64
+    // kernel is bound by the FP64 pipe at any size, and repeats the harmonics).
+    // 19456 | 19500 | 38912 particles at (16, 12), four | two | two warps: 20.3 |
+    // 23.5 | 23.9 us, with one warp 31.9 and 29.7 for the latter two; (14, 8) at
+    // 29200 12.8 us with two, 15.6 with one; (10, 6) at 38912 8 us with four.
     constexpr int kMost = field_threads<LM>();
     const int64_t lanes = (N + FieldLane<P>::kParticles - 1) / FieldLane<P>::kParticles;
-    const int parts = sizeof(R) == 4 && l_max >= 2 &&
-                              lanes * kFieldParts <= (int64_t)ctx.num_sms * kMost ? kFieldParts : 1;
+    int parts = sizeof(R) == 4 && l_max >= 2 ? kFieldParts : 1;
+    while (parts > 1 && lanes * parts > (int64_t)ctx.num_sms * kMost) parts /= 2;
     const int64_t sms = ctx.num_sms, most = kMost / parts;
     const int64_t rounds = (lanes + sms * most - 1) / (sms * most);
     const int64_t per = (lanes + sms * rounds - 1) / (sms * rounds);
@@ -407,8 +408,7 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     const int64_t want = (lanes + warps * 32 - 1) / (warps * 32);
     const int grid = (int)(want < sms ? want : sms);
     const size_t smem = (size_t)field_rows(n_max) * col_offset_c(LM + 1) * sizeof(R) +
-                        (parts > 1 ? (size_t)(kFieldParts - 1) * FieldLane<P>::kParticles * warps * 32 *
-                                         sizeof(Vec4<R>) : 0);
+                        (size_t)(parts - 1) * FieldLane<P>::kParticles * warps * 32 * sizeof(Vec4<R>);
     auto k = (out_mask & ETICS_OUT_ACC) ? scf_field_kernel<P, LM, true, NM1, B>
                                         : scf_field_kernel<P, LM, false, NM1, B>;
     if (smem > 48 * 1024 && allow_dynamic_smem(k)) return ETICS_ERR_CUDA;
