@@ -307,13 +307,18 @@ inline FieldSplit field_split(int l_max, int parts) {
     return s;
 }
 
-// threads per block the registers are sized for, one block per SM
+// threads per block the registers are sized for, and blocks per SM: two where the
+// potential alone of the smallest expansions leaves nothing but memory to wait for
+// (2^21 particles: (0, 0) 13.8 us, (2, 2) 17.3; 19.6 and 24.2 with one)
 template <int LM> constexpr int field_threads() { return LM <= 6 ? 512 : LM <= 8 ? 384 : 256; }
+template <typename P, int LM, bool ACC> constexpr int field_blocks() {
+    return FieldLane<P>::kParticles > 1 && LM <= 2 && !ACC ? 2 : 1;
+}
 
 // vel (nullable): the second kick of a leapfrog step, v += kick a, with the
 // acceleration still in registers
 template <typename P, int LM, bool ACC, int NM1, int B>
-__global__ void __launch_bounds__(field_threads<LM>(), 1)
+__global__ void __launch_bounds__(field_threads<LM>(), (field_blocks<P, LM, ACC>()))
 scf_field_kernel(const Vec4<typename FieldLane<P>::R>* posm, int64_t N, int n_max,
                  int l_max, const double* coeffs, Vec4<typename FieldLane<P>::R>* out,
                  int out_mask, Vec4<typename FieldLane<P>::R>* vel,
@@ -332,11 +337,16 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* posm, int64_t N, int n_ma
     const int slot = (warp / split.parts) * 32 + lane;
     for (int64_t first = (int64_t)blockIdx.x * per * NP; first < N;
          first += (int64_t)gridDim.x * per * NP) {
-        const int64_t i = first + (int64_t)slot * NP;
+        // particle j of the thread: a neighbour, or (kApart) as far on as the
+        // block has lanes, so that neighbouring lanes take neighbouring particles
+        constexpr bool kApart = field_blocks<P, LM, ACC>() > 1;
+        auto at = [&](int j) -> int64_t {
+            return kApart ? first + (int64_t)j * per + slot : first + (int64_t)slot * NP + j;
+        };
         Vec4<R> pv[NP], res[NP];
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
-            pv[j] = i + j < N ? ld4(posm + i + j) : mk4<R>(R(0), R(0), R(0), R(0));
+            pv[j] = at(j) < N ? ld4(posm + at(j)) : mk4<R>(R(0), R(0), R(0), R(0));
             if (!finite4(pv[j].x, pv[j].y, pv[j].z, pv[j].w)) report(err, ETICS_ERR_NONFINITE);
         }
         field_eval<P, LM, ACC, NM1, B>(pv, cs, n_max, l_max, split.level[part], res);
@@ -363,19 +373,19 @@ scf_field_kernel(const Vec4<typename FieldLane<P>::R>* posm, int64_t N, int n_ma
         if (vel) {
 #pragma unroll
             for (int j = 0; j < NP; ++j)
-                if (i + j < N) v[j] = ld4(vel + i + j);
+                if (at(j) < N) v[j] = ld4(vel + at(j));
         }
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
-            if (i + j >= N) continue;
+            if (at(j) >= N) continue;
             if (!(out_mask & ETICS_OUT_POT)) res[j].w = R(0);
             if (!finite4(res[j].x, res[j].y, res[j].z, res[j].w)) report(err, ETICS_ERR_NONFINITE);
-            st4(out + i + j, res[j]);
+            st4(out + at(j), res[j]);
             if (vel) {
                 v[j].x = fma(kick, res[j].x, v[j].x);
                 v[j].y = fma(kick, res[j].y, v[j].y);
                 v[j].z = fma(kick, res[j].z, v[j].z);
-                st4(vel + i + j, v[j]);
+                st4(vel + at(j), v[j]);
             }
         }
     }
@@ -398,9 +408,12 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     // 29200 12.8 us with two, 15.6 with one; (10, 6) at 38912 8 us with four.
     constexpr int kMost = field_threads<LM>();
     const int64_t lanes = (N + FieldLane<P>::kParticles - 1) / FieldLane<P>::kParticles;
+    const bool acc = out_mask & ETICS_OUT_ACC;
+    const int64_t sms = (int64_t)ctx.num_sms *
+                        (acc ? field_blocks<P, LM, true>() : field_blocks<P, LM, false>());
     int parts = sizeof(R) == 4 && l_max >= 2 ? kFieldParts : 1;
     while (parts > 1 && lanes * parts > (int64_t)ctx.num_sms * kMost) parts /= 2;
-    const int64_t sms = ctx.num_sms, most = kMost / parts;
+    const int64_t most = kMost / parts;
     const int64_t rounds = (lanes + sms * most - 1) / (sms * most);
     const int64_t per = (lanes + sms * rounds - 1) / (sms * rounds);
     const int warps = (int)((per + 31) / 32);
@@ -409,8 +422,7 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     const int grid = (int)(want < sms ? want : sms);
     const size_t smem = (size_t)field_rows(n_max) * col_offset_c(LM + 1) * sizeof(R) +
                         (size_t)(parts - 1) * FieldLane<P>::kParticles * warps * 32 * sizeof(Vec4<R>);
-    auto k = (out_mask & ETICS_OUT_ACC) ? scf_field_kernel<P, LM, true, NM1, B>
-                                        : scf_field_kernel<P, LM, false, NM1, B>;
+    auto k = acc ? scf_field_kernel<P, LM, true, NM1, B> : scf_field_kernel<P, LM, false, NM1, B>;
     if (smem > 48 * 1024 && allow_dynamic_smem(k)) return ETICS_ERR_CUDA;
     // launched as a programmatic dependent of the coefficient finalize (or
     // whatever precedes it): its launch overlaps the predecessor's tail
