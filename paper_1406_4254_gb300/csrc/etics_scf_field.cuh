@@ -22,6 +22,8 @@
 // the SMs).
 #pragma once
 
+#include <algorithm>
+
 #include "etics_internal.h"
 #include "etics_pair.cuh"
 
@@ -416,7 +418,10 @@ inline int launch_field_lm(const void* posm, int64_t N, int n_max, int l_max,
     const int64_t most = kMost / parts;
     const int64_t rounds = (lanes + sms * most - 1) / (sms * most);
     const int64_t per = (lanes + sms * rounds - 1) / (sms * rounds);
-    const int warps = (int)((per + 31) / 32);
+    // (the one warp of a small call's block would load the table's rows one after
+    // the other: l_max = 0, n_max = 16, 4219 particles 9.3 us, 6.0 with four)
+    const int least = sizeof(R) == 4 ? 4 / parts : 1;
+    const int warps = std::max((int)((per + 31) / 32), least);
     const int threads = warps * 32 * parts;
     const int64_t want = (lanes + warps * 32 - 1) / (warps * 32);
     const int grid = (int)(want < sms ? want : sms);

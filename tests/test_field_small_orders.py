@@ -48,3 +48,18 @@ def test_potential_alone_is_bound_by_memory():
     field = _best(lambda: etics.scf_field(x, c, 0, 0, out=out, out_mask=etics.OUT_POT))
     print(f"copy {copy * 1e3:.1f} us, field {field * 1e3:.1f} us")
     assert field <= 1.8 * copy, (field, copy)
+
+
+@pytest.mark.parametrize("n", [500, 4219])
+def test_many_rows_cost_a_small_call_little(n):
+    """l_max = 0: the block builds a table of 17 rows instead of two and walks them,
+    half a microsecond beside a launch of five; a table loaded row by row by one
+    warp cost more than half as much again."""
+    x = torch.tensor(inputs.hernquist(n, seed=2), dtype=torch.float32, device="cuda")
+    out = torch.empty_like(x)
+    times = {}
+    for n_max in (1, 16):
+        c = etics.scf_coeffs(x, n_max, 0)
+        times[n_max] = _best(lambda: etics.scf_field(x, c, n_max, 0, out=out))
+    print({k: round(v * 1e3, 1) for k, v in times.items()})
+    assert times[16] <= 1.3 * times[1], times
