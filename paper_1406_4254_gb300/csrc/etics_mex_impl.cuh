@@ -235,6 +235,29 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                 const P q2 = mk2(q, q + own.x), p2 = mk2(pp + own.y, pp);
                 f.pot0 = fma2(q2, p.irho, p2);
                 if (ACC) f.rad = mul2(q2, a);
+            } else if constexpr (!ACC) {
+                // the level's sums of q R and p R before their powers of the radius
+                P q0, p0, q1, p1;
+#pragma unroll
+                for (int m = 0; m <= L; ++m) {
+                    const P wm = mul2(own, splat<P>(mex_w<R>(L * (L + 1) / 2 + m)));
+#pragma unroll
+                    for (int s = 0; s < (m > 0 ? 2 : 1); ++s) {
+                        const int cc = o + (m == 0 ? 0 : 2 * m - 1 + s);
+                        const R q = col[cc * kMexRow], pp = col[(nc + cc) * kMexRow];
+                        const P h = s == 0 ? C[s0][m] : S[s0][m];
+                        const P q2 = mk2(q, fma(wm.x, h.x, q)), p2 = mk2(fma(wm.y, h.y, pp), pp);
+                        if (m == 0) {
+                            q0 = mul2(q2, h);
+                            p0 = mul2(p2, h);
+                        } else {
+                            q1 = m == 1 && s == 0 ? mul2(q2, h) : fma2(q2, h, q1);
+                            p1 = m == 1 && s == 0 ? mul2(p2, h) : fma2(p2, h, p1);
+                        }
+                    }
+                }
+                f.s0 = fma2(a, q0, fma2(b, p0, f.s0));
+                f.s1 = fma2(a, q1, fma2(b, p1, f.s1));
             } else {
                 P ac[L + 1], as[L + 1];
                 P r0 = splat<Pair<R>>(R(0)), r1 = splat<Pair<R>>(R(0));
@@ -250,10 +273,8 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                         ac[m] = fma2(mk2(fma(wm.y, h.y, pp), pp), b, qa);
                         if (m == 0) f.s0 = fma2(ac[m], h, f.s0);
                         else f.s1 = fma2(ac[m], h, f.s1);
-                        if (ACC) {
-                            if (m == 0) r0 = mul2(qa, h);
-                            else r1 = fma2(qa, h, r1);
-                        }
+                        if (m == 0) r0 = mul2(qa, h);
+                        else r1 = fma2(qa, h, r1);
                     }
                     as[m] = splat<Pair<R>>(R(0));
                     if (m > 0) {
@@ -263,31 +284,29 @@ __device__ __forceinline__ void mex_eval(Pair<R> (&C)[3][L1 + 1], Pair<R> (&S)[3
                         const P qa = mul2(mk2(q, fma(wm.x, h.x, q)), a);
                         as[m] = fma2(mk2(fma(wm.y, h.y, pp), pp), b, qa);
                         f.s1 = fma2(as[m], h, f.s1);
-                        if (ACC) r1 = fma2(qa, h, r1);
+                        r1 = fma2(qa, h, r1);
                     }
                 }
-                if (ACC) {
-                    f.rad = fma2(splat<Pair<R>>(R(2 * L + 1)), r0, f.rad);
-                    f.rad = fma2(splat<Pair<R>>(R(2 * (2 * L + 1))), r1, f.rad);
-                    // gradient from the level below (the ladder regrouped by the
-                    // harmonic it multiplies)
-                    const P* C1 = C[s1];
-                    const P* S1 = S[s1];
+                f.rad = fma2(splat<Pair<R>>(R(2 * L + 1)), r0, f.rad);
+                f.rad = fma2(splat<Pair<R>>(R(2 * (2 * L + 1))), r1, f.rad);
+                // gradient from the level below (the ladder regrouped by the
+                // harmonic it multiplies)
+                const P* C1 = C[s1];
+                const P* S1 = S[s1];
 #pragma unroll
-                    for (int k = 0; k <= L - 1; ++k) {
-                        const P xc = k >= 1 ? sub2(ac[k + 1], ac[k - 1]) : ac[k + 1];
-                        const P yc = k >= 2 ? add2(as[k + 1], as[k - 1]) : as[k + 1];
-                        f.vx = fma2(xc, C1[k], f.vx);
-                        f.vy = fma2(yc, C1[k], f.vy);
-                        if (k == 0) f.vz0 = fma2(ac[k], C1[k], f.vz0);
-                        if (k >= 1) {
-                            const P xs = k >= 2 ? sub2(as[k + 1], as[k - 1]) : as[k + 1];
-                            const P ys = add2(ac[k + 1], ac[k - 1]);
-                            f.vz1 = fma2(ac[k], C1[k], f.vz1);
-                            f.vx = fma2(xs, S1[k], f.vx);
-                            f.vy = fma2(neg2(ys), S1[k], f.vy);
-                            f.vz1 = fma2(as[k], S1[k], f.vz1);
-                        }
+                for (int k = 0; k <= L - 1; ++k) {
+                    const P xc = k >= 1 ? sub2(ac[k + 1], ac[k - 1]) : ac[k + 1];
+                    const P yc = k >= 2 ? add2(as[k + 1], as[k - 1]) : as[k + 1];
+                    f.vx = fma2(xc, C1[k], f.vx);
+                    f.vy = fma2(yc, C1[k], f.vy);
+                    if (k == 0) f.vz0 = fma2(ac[k], C1[k], f.vz0);
+                    if (k >= 1) {
+                        const P xs = k >= 2 ? sub2(as[k + 1], as[k - 1]) : as[k + 1];
+                        const P ys = add2(ac[k + 1], ac[k - 1]);
+                        f.vz1 = fma2(ac[k], C1[k], f.vz1);
+                        f.vx = fma2(xs, S1[k], f.vx);
+                        f.vy = fma2(neg2(ys), S1[k], f.vy);
+                        f.vz1 = fma2(as[k], S1[k], f.vz1);
                     }
                 }
             }
@@ -329,11 +348,15 @@ __device__ __forceinline__ int mex_tile_exponent(const Vec4<R>& a, const Vec4<R>
 }
 
 // resident blocks per SM the registers are sized for
-// (FP32 pass 2: 118 registers for l_max <= 6, 158 with the later level groups)
+// (FP32 pass 2: 118 registers for l_max <= 6, 158 with the later level groups;
+// FP64 218, and 168 for the potential alone, which three blocks fill the FP64 pipe
+// with while one scans: l_max = 2 at 2^20 840 -> 724 us)
 template <typename R>
 constexpr int mex_pass1_blocks() { return sizeof(R) == 4 ? 4 : 2; }
-template <typename R, int NG>
-constexpr int mex_pass2_blocks() { return sizeof(R) == 4 ? (NG == 1 ? 4 : 3) : 2; }
+template <typename R, int NG, bool ACC>
+constexpr int mex_pass2_blocks() {
+    return sizeof(R) == 4 ? (NG == 1 ? 4 : 3) : NG == 1 && !ACC ? 3 : 2;
+}
 
 // ---------------------------------------------------------------------------
 // pass 1: per-tile FP64 moment sums
@@ -534,7 +557,7 @@ __device__ __forceinline__ void mex_scan_row_warp(Vec4<R>* row, bool inner, R q0
 constexpr int kMexLeftover = 8;
 
 template <typename R, int NG, bool ACC>
-__global__ void __launch_bounds__(kMexThreads, mex_pass2_blocks<R, NG>())
+__global__ void __launch_bounds__(kMexThreads, (mex_pass2_blocks<R, NG, ACC>()))
 mex_pass2_kernel(const Vec4<R>* sorted, const uint32_t* perm, int64_t N,
                  int l_max, const double* carry, int stride,
                  Vec4<R>* out, int out_mask, unsigned* err) {
